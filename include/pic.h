@@ -74,7 +74,7 @@ extern "C" {
 /* Precision modes. */
 #define PIC_FP32_FIXED 0  /* float32 push, int64 fixed-point deposit (default) */
 #define PIC_FP32_ATOMIC 1 /* float32 push, float32 atomic deposit              */
-#define PIC_FP64 2        /* float64 push, float64 atomic deposit              */
+#define PIC_FP64 2        /* float64 push, float64 weights summed exactly      */
 
 /* Deposit-kernel variants of the fused push (PIC_FP32_FIXED only); all give
  * the same integers.  The values 3, 4 and 7 are not variants (PIC_EINVAL). */

@@ -26,11 +26,9 @@
 // shared memory, and block 0 reduces the diagnostics and writes the history
 // rows.
 //
-// Float modes (precision study): one block (one warp per 32 nodes, at most
-// kSolveThreads threads), float64 prefix scans of rho; the block then reduces
-// the diagnostics, writes the history rows, clears the density accumulator
-// and advances the step counter (finalize).  The paper's CG solver
-// (PIC_SOLVER_CG) runs on a thread-block cluster (below).
+// The float modes (precision study) solve their density sums as integers of
+// finer units by the same kernel (take_density).  The paper's CG solver
+// (PIC_SOLVER_CG) runs on a thread-block cluster too (below).
 //
 // Diagnostics: field energy (1/2) dx sum E^2 in float64; mode amplitudes
 // from the float32 field with float32 twiddles, summed per block in float32
@@ -53,101 +51,44 @@ constexpr int kClusterSolveThreads = 512;   // most nodes per block (one per thr
 constexpr int kSolveNodesPerBlock = 256;
 constexpr int kMaxSolveCluster = 16;        // blocks per cluster (16: non-portable)
 
-// The block's share of the diagnostics, written to a.dpart[blockIdx.x]; the
-// push's per-block sums are split over the solve blocks.
-__device__ void write_block_partials(const SolveArgs &a, NodeDiag &d, double charge,
-                                     unsigned long long cq) {
-    __shared__ float shf[32 * 2 * PIC_NMODES];
-    __shared__ double shd[32 * 3];
-    double kv[3] = {d.fe, 0.0, 0.0};
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < a.npartials;
-         i += gridDim.x * blockDim.x) {
-        kv[1] += a.partials[2 * i];
-        kv[2] += a.partials[2 * i + 1];
-    }
-    float md[2 * PIC_NMODES];
-#pragma unroll
-    for (int m = 0; m < PIC_NMODES; m++) { md[2 * m] = d.re[m]; md[2 * m + 1] = d.im[m]; }
-    block_sum_t<3, double>(kv, shd);
-    block_sum_t<2 * PIC_NMODES, float>(md, shf);
-    if (threadIdx.x == 0) {
-        DiagPartial &p = a.dpart[blockIdx.x];
-        p.v[kDiagFE] = kv[0];
-        p.v[kDiagKE] = kv[1];
-        p.v[kDiagMom] = kv[2];
-        p.v[kDiagCharge] = charge;
-        p.cq = cq;
-        for (int m = 0; m < 2 * PIC_NMODES; m++) p.v[kDiagModes + m] = (double)md[m];
-    }
+// ---- the density as integers --------------------------------------------------
+//
+// Every precision mode solves the same integers: node g's particle sum is q_g
+// units of 2^-B of a particle, and rho_g = K R_g with R_g = N 2^B - NG q_g and
+// K = rho_ion / (N 2^B).
+//   fixed point     B = 24: the deposit's own integers
+//   float32 atomic  B = 30: the float32 sum to the nearest 2^-30 (a sum of at
+//                   least 2^-6 converts exactly)
+//   float64         B = 53: the deposit's own integers, kept as two 64-bit sums
+//                   of the low 40 bits and of the rest (push.cu)
+// Bounds of the 128-bit arithmetic below, worst at B = 53, N < 2^32, NG = 2^13
+// with every particle in one cell: |P_g| <= NG N 2^53 < 2^98, |sum P| < 2^111,
+// |M_g| < 2^112 and the two terms of sum M below 2^125 each.
+// N 2^B (in 64 bits where it fits: N < 2^39 at B = 24)
+template <int MODE>
+__device__ __forceinline__ i128 whole_density(const SolveArgs &a) {
+    if (MODE == PIC_FP32_FIXED) return (i128)(a.npart_total << kFixBits);
+    constexpr int kBits = density_bits(MODE);
+    return (i128)a.npart_total << kBits;
 }
 
-// Last block: reduce the per-block partials in a fixed order, write the
-// history rows, clear the accumulator, advance the step counter.  Field f of
-// the partials is summed over the blocks by thread f.
-__device__ void finalize(const SolveArgs &a, long long step) {
-    __shared__ unsigned ticket;
-    __shared__ double tot[kDiagFields];
-    __shared__ unsigned long long tot_cq;
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) ticket = atomicAdd(a.counter, 1u);
-    __syncthreads();
-    if (ticket != gridDim.x - 1) return;
-    __threadfence();
-    // the accumulator is no longer read by any block
-    const int ng = a.ng;
-    for (int g = threadIdx.x; g < ng; g += blockDim.x) {
-        if (a.mode == PIC_FP32_FIXED) a.rho_q[g] = 0ull;
-        else if (a.mode == PIC_FP32_ATOMIC) a.rho_f32[g] = 0.0f;
-        else a.rho_f64[g] = 0.0;
+template <int MODE>
+__device__ __forceinline__ i128 take_density(const SolveArgs &a, int g) {
+    // read and cleared by this thread only
+    if (MODE == PIC_FP32_FIXED) {
+        const unsigned long long q = __ldcg(&a.rho_q[g]);
+        a.rho_q[g] = 0ull;
+        a.rho_q_last[g] = q;
+        return (i128)q;
     }
-    // all the partials' loads in flight at once, summed in block order
-    const int f = threadIdx.x;
-    const int nb = (int)gridDim.x;
-    if (f < kDiagFields) {
-        double part[kSolveMaxBlocks];
-#pragma unroll
-        for (int b = 0; b < kSolveMaxBlocks; b++) part[b] = b < nb ? __ldcg(&a.dpart[b].v[f]) : 0.0;
-        double acc = 0.0;
-#pragma unroll
-        for (int b = 0; b < kSolveMaxBlocks; b++) acc += part[b];
-        tot[f] = acc;
-    } else if (f == kDiagFields) {
-        unsigned long long part[kSolveMaxBlocks];
-#pragma unroll
-        for (int b = 0; b < kSolveMaxBlocks; b++) part[b] = b < nb ? __ldcg(&a.dpart[b].cq) : 0ull;
-        unsigned long long acc = 0;
-#pragma unroll
-        for (int b = 0; b < kSolveMaxBlocks; b++) acc += part[b];
-        tot_cq = acc;
+    if (MODE == PIC_FP32_ATOMIC) {
+        const float acc = __ldcg(&a.rho_f32[g]);
+        a.rho_f32[g] = 0.0f;
+        return (i128)__float2ll_rn(acc * 0x1p30f);
     }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        long long n = step;
-        if (a.npartials > 0) {
-            pic_diag_row *row = &a.hist[n % a.hist_len];
-            row->kinetic = 0.5 * a.mass * tot[kDiagKE];
-            row->momentum = a.mass * tot[kDiagMom];
-            n = step + 1;
-            *a.dstep = n;
-        }
-        pic_diag_row *row = &a.hist[n % a.hist_len];
-        const double qnan = __longlong_as_double(0x7ff8000000000000ll);
-        row->step = n;
-        row->kinetic = qnan;
-        row->momentum = qnan;
-        row->field = 0.5 * a.dx * tot[kDiagFE];
-        row->charge = tot[kDiagCharge];
-        row->charge_q = (long long)tot_cq;
-        *a.counter = 0u;
-    }
-    // the mode amplitudes one lane each (warp 1 when there is one)
-    const int mt = blockDim.x >= 64 ? (int)threadIdx.x - 32 : (int)threadIdx.x;
-    if (mt >= 0 && mt < PIC_NMODES) {
-        const long long n = a.npartials > 0 ? step + 1 : step;
-        const double re = tot[kDiagModes + 2 * mt], im = tot[kDiagModes + 2 * mt + 1];
-        a.hist[n % a.hist_len].mode[mt] = sqrt(re * re + im * im) * a.k_mode;
-    }
+    const ulonglong2 w = __ldcg(reinterpret_cast<const ulonglong2 *>(a.rho_w) + g);
+    reinterpret_cast<ulonglong2 *>(a.rho_w)[g] = make_ulonglong2(0ull, 0ull);
+    return (i128)w.x + ((i128)w.y << 40);
 }
 
 // ---- the cluster solves' common parts -------------------------------------
@@ -309,6 +250,7 @@ struct SliceSums {
     i128 s0, s1;                  // slice sums of R and k R
 };
 
+template <int MODE>
 __global__ void __launch_bounds__(kClusterSolveThreads) pic_solve_cluster_kernel(SolveArgs a) {
     cg::cluster_group cl = cg::this_cluster();
     __shared__ SliceSums ex;
@@ -318,21 +260,17 @@ __global__ void __launch_bounds__(kClusterSolveThreads) pic_solve_cluster_kernel
     const int C = (int)cl.num_blocks(), r = (int)cl.block_rank();
     const int ng = a.ng, t = threadIdx.x;
     const long long step = *a.dstep;
-    const long long ntot = a.weight_total;
+    const i128 ntot = whole_density<MODE>(a);
     const int per = (ng + C - 1) / C;
     const int b0 = r * per;
     const int b1 = min(ng, b0 + per);
     const int g = b0 + t;
     const bool mine = g < b1;
-    unsigned long long q = 0ull;
-    if (mine) {
-        q = __ldcg(&a.rho_q[g]);
-        a.rho_q[g] = 0ull;            // read by this thread only
-        a.rho_q_last[g] = q;
-    }
+    i128 q = 0;
+    if (mine) q = take_density<MODE>(a, g);
     double kv[2];
     push_sums_share(a, C, r, kv);
-    const i128 R = mine ? (i128)ntot - (i128)ng * (i128)q : (i128)0;
+    const i128 R = mine ? ntot - (i128)ng * q : (i128)0;
     // one pass of the slice's inclusive scans of R_k and k R_k
     const I128Pair sc = block_inclusive_scan2_i128(R, R * (i128)g, scan64);
     if (t == 0) {
@@ -385,7 +323,8 @@ __global__ void __launch_bounds__(kClusterSolveThreads) pic_solve_cluster_kernel
         node_diag(d, g, ng, E, E32);
     }
     const double charge = r == 0 ? a.dx * a.k_rho * i128_to_f64(SR) : 0.0;
-    cluster_finish(a, cl, cd, kv, d, charge, q, step);                // #2, #3
+    cluster_finish(a, cl, cd, kv, d, charge,
+                   MODE == PIC_FP32_FIXED ? (unsigned long long)q : 0ull, step);   // #2, #3
 }
 
 // ---- CG: the paper's field solver, on one thread-block cluster ------------
@@ -419,7 +358,7 @@ struct CgExchange {
     double v0, v1, r0, r1;        // v (before the update) and r (after) at the
                                   // slice's first and last node
     double x0, x1;                // Phi at the slice's first and last node
-    i128 sr;                      // fixed point: slice sum of R
+    i128 sr;                      // slice sum of R
 };
 
 __device__ __forceinline__ double warp_div(double num, double den) {
@@ -428,6 +367,7 @@ __device__ __forceinline__ double warp_div(double num, double den) {
     return __shfl_sync(kFull, q, 0);
 }
 
+template <int MODE>
 __global__ void __launch_bounds__(kClusterSolveThreads) pic_solve_cg_kernel(SolveArgs a) {
     cg::cluster_group cl = cg::this_cluster();
     __shared__ double sv[kClusterSolveThreads + 2];   // v of the slice, ghost-padded
@@ -447,27 +387,14 @@ __global__ void __launch_bounds__(kClusterSolveThreads) pic_solve_cg_kernel(Solv
     double kv[2];
     push_sums_share(a, C, r, kv);
     double rh = 0.0;
-    unsigned long long q = 0ull;
-    i128 R = 0;
+    i128 q = 0, R = 0;
     if (mine) {
-        if (a.mode == PIC_FP32_FIXED) {
-            q = __ldcg(&a.rho_q[g]);
-            a.rho_q[g] = 0ull;
-            a.rho_q_last[g] = q;
-            R = (i128)a.weight_total - (i128)ng * (i128)q;
-            rh = a.k_rho * i128_to_f64(R);
-        } else if (a.mode == PIC_FP32_ATOMIC) {
-            const float acc = a.rho_f32[g];
-            a.rho_f32[g] = 0.0f;
-            rh = a.rho_ion + a.q_over_dx * (double)acc;
-        } else {
-            const double acc = a.rho_f64[g];
-            a.rho_f64[g] = 0.0;
-            rh = a.rho_ion + a.q_over_dx * acc;
-        }
+        q = take_density<MODE>(a, g);
+        R = whole_density<MODE>(a) - (i128)ng * q;
+        rh = a.k_rho * i128_to_f64(R);
         a.rho[g] = rh;
     }
-    if (a.mode == PIC_FP32_FIXED) {
+    {
         i128 z1 = 0, z2 = 0, sr = R;
         block_sum3_i128(sr, z1, z2, sh);
         if (t == 0) ex.sr = sr;
@@ -545,7 +472,6 @@ __global__ void __launch_bounds__(kClusterSolveThreads) pic_solve_cg_kernel(Solv
     __syncthreads();
     NodeDiag dg;
     node_diag_reset(dg);
-    double pcharge = 0.0;
     if (mine) {
         const double E = -(sv[t + 2] - sv[t]) / (2.0 * dx);
         const float E32 = (float)E;
@@ -553,111 +479,27 @@ __global__ void __launch_bounds__(kClusterSolveThreads) pic_solve_cg_kernel(Solv
         a.E64[g] = E;
         a.E32[g] = E32;
         node_diag(dg, g, ng, E, E32);
-        pcharge = rh;
     }
-    double charge;
-    if (a.mode == PIC_FP32_FIXED) {
-        i128 sr = 0;
-        if (r == 0)
-            for (int b = 0; b < C; b++) sr += cl.map_shared_rank(&ex, b)->sr;
-        charge = r == 0 ? dx * a.k_rho * i128_to_f64(sr) : 0.0;
-    } else {
-        charge = dx * block_sum_f64(pcharge, slot);
-    }
-    cluster_finish(a, cl, cd, kv, dg, charge, q, step);
+    i128 sr = 0;
+    if (r == 0)
+        for (int b = 0; b < C; b++) sr += cl.map_shared_rank(&ex, b)->sr;
+    const double charge = r == 0 ? dx * a.k_rho * i128_to_f64(sr) : 0.0;
+    cluster_finish(a, cl, cd, kv, dg, charge,
+                   MODE == PIC_FP32_FIXED ? (unsigned long long)q : 0ull, step);
 }
 
-// ---- float modes: one block, float64 prefix scans ---------------------------
+using SolveKernel = void (*)(SolveArgs);
 
-constexpr int kMaxPerThread = (PIC_NCELL_MAX + kSolveThreads - 1) / kSolveThreads;
-
-__device__ double block_exclusive_scan_f64(double val, double *warp_tot, double &total) {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    double inc = val;
-    for (int o = 1; o < 32; o <<= 1) {
-        const double u = __shfl_up_sync(kFull, inc, o);
-        if (lane >= o) inc += u;
+SolveKernel pick_solve(int mode, int solver) {
+    const bool c = solver == PIC_SOLVER_CG;
+    switch (mode) {
+        case PIC_FP32_FIXED:
+            return c ? &pic_solve_cg_kernel<PIC_FP32_FIXED> : &pic_solve_cluster_kernel<PIC_FP32_FIXED>;
+        case PIC_FP32_ATOMIC:
+            return c ? &pic_solve_cg_kernel<PIC_FP32_ATOMIC> : &pic_solve_cluster_kernel<PIC_FP32_ATOMIC>;
+        default:
+            return c ? &pic_solve_cg_kernel<PIC_FP64> : &pic_solve_cluster_kernel<PIC_FP64>;
     }
-    if (lane == 31) warp_tot[w] = inc;
-    __syncthreads();
-    double off = 0.0, tot = 0.0;
-    for (int i = 0; i < nw; i++) {
-        if (i < w) off += warp_tot[i];
-        tot += warp_tot[i];
-    }
-    __syncthreads();
-    total = tot;
-    return off + inc - val;
-}
-
-__global__ void __launch_bounds__(kSolveThreads) pic_solve_float_kernel(SolveArgs a) {
-    __shared__ double wt[32];
-    __shared__ double last_of_warp[32];
-    const int ng = a.ng, T = blockDim.x, t = threadIdx.x;
-    const int k = (ng + T - 1) / T;
-    const int g0 = t * k;
-    const long long step = *a.dstep;
-    double r[kMaxPerThread], S[kMaxPerThread];
-    double lsum = 0.0;
-#pragma unroll
-    for (int j = 0; j < kMaxPerThread; j++) {
-        const int g = g0 + j;
-        double rho = 0.0;
-        if (j < k && g < ng) {
-            const double acc = (a.mode == PIC_FP32_ATOMIC) ? (double)a.rho_f32[g] : a.rho_f64[g];
-            rho = a.rho_ion + a.q_over_dx * acc;
-            a.rho[g] = rho;
-        }
-        r[j] = rho;
-        lsum += rho;
-    }
-    double total_rho;
-    double run = block_exclusive_scan_f64(lsum, wt, total_rho);
-    double ssum = 0.0;
-#pragma unroll
-    for (int j = 0; j < kMaxPerThread; j++) {
-        run += r[j];
-        S[j] = run;
-        if (j < k && g0 + j < ng) ssum += run;
-    }
-    double stot;
-    block_exclusive_scan_f64(ssum, wt, stot);
-    const double Sbar = stot / (double)ng;
-    // S_{g0-1}: previous thread's last S; S_{-1} = S_{NG-1} = total
-    double prev_last = __shfl_up_sync(kFull, S[kMaxPerThread - 1], 1);
-    const int lane = t & 31, w = t >> 5;
-    if (lane == 31) last_of_warp[w] = S[kMaxPerThread - 1];
-    __syncthreads();
-    if (lane == 0) prev_last = (w == 0) ? total_rho : last_of_warp[w - 1];
-    double dsum = 0.0;
-#pragma unroll
-    for (int j = 0; j < kMaxPerThread; j++)
-        if (j < k && g0 + j < ng) dsum += S[j] - Sbar;
-    double dtot;
-    double doff = block_exclusive_scan_f64(dsum, wt, dtot);
-    const double half_dx = 0.5 * a.dx, dx2 = a.dx * a.dx;
-    NodeDiag d;
-    node_diag_reset(d);
-    double sprev = prev_last, charge = 0.0;
-#pragma unroll
-    for (int j = 0; j < kMaxPerThread; j++) {
-        const int g = g0 + j;
-        if (j < k && g < ng) {
-            const double E = half_dx * ((S[j] - Sbar) + (sprev - Sbar));
-            const float E32 = (float)E;
-            a.E64[g] = E;
-            a.E32[g] = E32;
-            a.phi[g] = -dx2 * doff;
-            doff += S[j] - Sbar;
-            charge += r[j];
-            node_diag(d, g, ng, E, E32);
-        }
-        sprev = S[j];
-    }
-    double ch[1] = {charge};
-    block_sum_t<1, double>(ch, wt);
-    write_block_partials(a, d, a.dx * ch[0], 0ull);
-    finalize(a, step);
 }
 
 }  // namespace
@@ -675,38 +517,31 @@ void solve_cluster_shape(int ng, int per_block, int *C, int *threads) {
 }
 
 cudaError_t solve_prepare_attributes() {
-    cudaError_t e = cudaFuncSetAttribute(&pic_solve_cluster_kernel,
-                                         cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(&pic_solve_cg_kernel,
-                                cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    for (int mode : {PIC_FP32_FIXED, PIC_FP32_ATOMIC, PIC_FP64})
+        for (int solver : {PIC_SOLVER_EXACT, PIC_SOLVER_CG}) {
+            const cudaError_t e = cudaFuncSetAttribute(
+                pick_solve(mode, solver), cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+            if (e != cudaSuccess) return e;
+        }
+    return cudaSuccess;
 }
 
 cudaError_t launch_solve(const SolveArgs &a, cudaStream_t s) {
-    if (a.solver == PIC_SOLVER_CG || a.mode == PIC_FP32_FIXED) {
-        int C = 1, threads = 32;
-        solve_cluster_shape(a.ng, a.solver == PIC_SOLVER_CG ? 32 : kSolveNodesPerBlock, &C,
-                            &threads);
-        cudaLaunchConfig_t cfg = {};
-        cudaLaunchAttribute attr[1];
-        cfg.gridDim = dim3((unsigned)C, 1, 1);
-        cfg.blockDim = dim3((unsigned)threads, 1, 1);
-        cfg.dynamicSmemBytes = 0;
-        cfg.stream = s;
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = (unsigned)C;
-        attr[0].val.clusterDim.y = 1;
-        attr[0].val.clusterDim.z = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        if (a.solver == PIC_SOLVER_CG) return cudaLaunchKernelEx(&cfg, pic_solve_cg_kernel, a);
-        return cudaLaunchKernelEx(&cfg, pic_solve_cluster_kernel, a);
-    }
-    // one block, one warp per 32 nodes up to kSolveThreads (the float64
-    // scans cost per warp, not per node)
-    const int threads = a.ng >= kSolveThreads ? kSolveThreads : ((a.ng + 31) / 32) * 32;
-    pic_solve_float_kernel<<<1, threads, 0, s>>>(a);
-    return cudaGetLastError();
+    int C = 1, threads = 32;
+    solve_cluster_shape(a.ng, a.solver == PIC_SOLVER_CG ? 32 : kSolveNodesPerBlock, &C, &threads);
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    cfg.gridDim = dim3((unsigned)C, 1, 1);
+    cfg.blockDim = dim3((unsigned)threads, 1, 1);
+    cfg.dynamicSmemBytes = 0;
+    cfg.stream = s;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)C;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, pick_solve(a.mode, a.solver), a);
 }
 
 }  // namespace pic

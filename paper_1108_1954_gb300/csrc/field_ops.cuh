@@ -88,11 +88,6 @@ static __device__ void block_sum3_i128(i128 &a, i128 &b, i128 &c, i128 *sh /*[96
     __syncthreads();
 }
 
-// Block sum of K values per thread, fixed order; result valid in thread 0
-// (in fact in every lane of warp 0).  Warp sums by shuffles; the cross-warp
-// sum of each value by warp 0: for float64 (a slow pipe on GB300, so the
-// dependent chain matters) a butterfly over the warp sums, one value at a
-// time; for float32 lane i adds value i over the warps.
 // Sums of 16 float32 values over the 32 lanes of a warp by recursive
 // halving: at offset o = 16, 8, 4, 2 a lane keeps the half of its values
 // that bit o of its lane index selects, adds the partner's (lane ^ o) copy
@@ -127,41 +122,11 @@ __device__ __forceinline__ float warp_sum16_halving(const float (&v)[16], int la
     return h1 + __shfl_xor_sync(kFull, h1, 1);
 }
 
-template <int K, typename T>
-static __device__ void block_sum_t(T (&v)[K], T *sh /*[32*K]*/) {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-    for (int i = 0; i < K; i++)
-        for (int o = 16; o > 0; o >>= 1) v[i] += __shfl_down_sync(kFull, v[i], o);
-    if (lane == 0)
-#pragma unroll
-        for (int i = 0; i < K; i++) sh[w * K + i] = v[i];
-    __syncthreads();
-    if (w == 0) {
-        static_assert(K <= 32, "one lane per value");
-        if (sizeof(T) == 8) {
-#pragma unroll
-            for (int i = 0; i < K; i++) {
-                T s = lane < nw ? sh[lane * K + i] : (T)0;
-                for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(kFull, s, o);
-                v[i] = s;
-            }
-        } else {
-            T s = 0;
-            if (lane < K)
-                for (int j = 0; j < nw; j++) s += sh[j * K + lane];
-#pragma unroll
-            for (int i = 0; i < K; i++) v[i] = __shfl_sync(kFull, s, i);
-        }
-    }
-    __syncthreads();
-}
-
 // Sums of K float64 values per thread over a block (warp trees, then warp 0
 // over the warp sums), valid in lane 0 of warp 0.  The adds run in the
 // predicated lanes only (31 lane-adds per warp and value instead of 160):
-// GB300 issues float64 at 2 lanes per clock per SM, so the full butterfly
-// of block_sum_t costs more than the rest of a small solve.
+// GB300 issues float64 at 2 lanes per clock per SM, so a full butterfly
+// costs more than the rest of a small solve.
 template <int K>
 __device__ __forceinline__ void block_sum_f64k(double (&v)[K], double *slot /*[32*K]*/) {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;

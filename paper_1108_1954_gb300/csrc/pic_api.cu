@@ -63,9 +63,9 @@ namespace {
 
 struct Layout {
     size_t x[2], v[2];
-    size_t rho_q, rho_q_last, rho_f32, rho_f64;
+    size_t rho_q, rho_q_last, rho_f32, rho_w;
     size_t rho, phi, E64, E32;
-    size_t partials, dpart, hist, dev, tune_rho, phase;
+    size_t partials, hist, dev, tune_rho, phase;
     size_t s_hist, s_segtot, s_base;
     size_t total;
     int hist_len;
@@ -77,7 +77,7 @@ struct Layout {
 struct DevScalars {
     long long step;
     unsigned err;
-    unsigned counter;
+    unsigned unused;
 };
 
 // Chunks of the counting sort: 2048 particles (one scatter tile) or more
@@ -112,13 +112,12 @@ void make_layout(const pic_params *p, Layout *L) {
     L->rho_q = take(ng * 8);
     L->rho_q_last = take(ng * 8);
     L->rho_f32 = take(ng * 4);
-    L->rho_f64 = take(ng * 8);
+    L->rho_w = take(ng * 16);
     L->rho = take(ng * 8);
     L->phi = take(ng * 8);
     L->E64 = take(ng * 8);
     L->E32 = take(ng * 4);
     L->partials = take((size_t)kMaxPushGrid * 2 * 8);
-    L->dpart = take((size_t)kSolveMaxBlocks * sizeof(DiagPartial));
     L->hist_len = p->history > 0 ? p->history : kDefaultHistory;
     L->hist = take((size_t)L->hist_len * sizeof(pic_diag_row));
     L->dev = take(sizeof(DevScalars));
@@ -161,7 +160,7 @@ struct pic_run {
     cudaGraphExec_t period[2] = {nullptr, nullptr};   // S steps from x parity 0/1
     cudaGraphExec_t plain = nullptr;                  // kPlainBlock steps, no sort
     PushConsts pc{};
-    double dx = 0, mass = 0, q_over_dx = 0, k_rho = 0, k_e = 0, k_phi = 0;
+    double dx = 0, mass = 0, k_rho = 0, k_e = 0, k_phi = 0;
     double to_cells = 0, to_phys = 0;  // NG/L and L/NG (float32 positions)
     int64_t npart_total = 0;           // particles of the whole plasma (a shard holds npart)
     float length32 = 0;                // (float)L: positions lie in [0, length32)
@@ -182,9 +181,8 @@ void set_solve_constants(pic_run *r, int64_t n_total) {
     r->npart_total = n_total;
     r->dx = p->length / (double)p->ncell;
     const double q0 = (p->rho_ion * p->length / (double)n_total) * (p->qm / std::fabs(p->qm));
-    r->q_over_dx = q0 / r->dx;
     r->mass = q0 / p->qm;
-    r->k_rho = p->rho_ion / std::ldexp((double)n_total, kFixBits);
+    r->k_rho = p->rho_ion / std::ldexp((double)n_total, density_bits(p->precision));
     r->k_e = 0.5 * r->dx * r->k_rho / (double)p->ncell;
     r->k_phi = -r->dx * r->dx * r->k_rho / (double)p->ncell;
 }
@@ -225,7 +223,7 @@ cudaError_t enqueue_push(pic_run *r, cudaStream_t s, bool push) {
         a.v = (double *)r->vs(c);
         a.n = r->p.npart;
         a.E64 = r->at<double>(r->lay.E64);
-        a.rho_acc = r->at<double>(r->lay.rho_f64);
+        a.rho_w = r->at<unsigned long long>(r->lay.rho_w);
         a.partials = r->at<double>(r->lay.partials);
         a.err = &r->dev()->err;
         a.ng = r->p.ncell;
@@ -243,22 +241,18 @@ cudaError_t enqueue_solve(pic_run *r, cudaStream_t s, bool after_push) {
     a.rho_q = r->at<unsigned long long>(r->lay.rho_q);
     a.rho_q_last = r->at<unsigned long long>(r->lay.rho_q_last);
     a.rho_f32 = r->at<float>(r->lay.rho_f32);
-    a.rho_f64 = r->at<double>(r->lay.rho_f64);
+    a.rho_w = r->at<unsigned long long>(r->lay.rho_w);
     a.rho = r->at<double>(r->lay.rho);
     a.phi = r->at<double>(r->lay.phi);
     a.E64 = r->at<double>(r->lay.E64);
     a.E32 = r->at<float>(r->lay.E32);
     a.partials = r->at<double>(r->lay.partials);
     a.npartials = after_push ? r->grid : 0;
-    a.dpart = r->at<DiagPartial>(r->lay.dpart);
-    a.counter = &r->dev()->counter;
     a.hist = r->at<pic_diag_row>(r->lay.hist);
     a.hist_len = r->lay.hist_len;
     a.dstep = &r->dev()->step;
     a.ng = r->p.ncell;
-    a.weight_total = (long long)r->npart_total << kFixBits;
-    a.rho_ion = r->p.rho_ion;
-    a.q_over_dx = r->q_over_dx;
+    a.npart_total = r->npart_total;
     a.k_rho = r->k_rho;
     a.k_e = r->k_e;
     a.k_phi = r->k_phi;
@@ -350,14 +344,28 @@ int push_grid(const pic_run *r, int variant, int block, int unroll, int bps_cap)
     if (bps_cap && bps_cap < bps) bps = bps_cap;
     long long want = (long long)r->sms * bps;
     const int gw = group_width(variant);
-    const long long units = r->p.precision == PIC_FP32_FIXED ? (r->p.npart + gw - 1) / gw
-                                                             : r->p.npart;
+    const long long units = (r->p.npart + gw - 1) / gw;
     const long long per_block = (long long)block * unroll;
     const long long need = (units + per_block - 1) / per_block;
     if (want > need) want = need;
     if (want > kMaxPushGrid) want = kMaxPushGrid;
     if (want < 1) want = 1;
     return (int)want;
+}
+
+// Threads per block of the push when the caller leaves them open.  Every
+// block stages E and flushes a tile of NG nodes with one or two global adds
+// each, so large runs take few large blocks (512 threads; 1024 where the
+// float64 tile leaves room for one block per SM); a run with less than a
+// block of 512 for every SM takes smaller ones, down to 64 threads, so that
+// all SMs share it.
+int default_block(const pic_run *r) {
+    if (r->p.precision == PIC_FP32_FIXED) return 512;
+    const long long groups = (r->p.npart + 3) / 4;
+    const int most = push_smem_bytes(r->p.precision, r->p.ncell) > 100 * 1024 ? 1024 : 512;
+    int b = 64;
+    while (b < most && groups > (long long)b * r->sms) b *= 2;
+    return b;
 }
 
 // Work on the private stream after everything enqueued on the run's stream
@@ -400,7 +408,7 @@ int prepare_loaded(pic_run *r, int64_t step, Units units, bool aux_copy = false)
                                     &r->dev()->err, r->sms, r->stream));
     PIC_CUDA(cudaMemsetAsync(r->ws + r->lay.rho_q, 0, (size_t)r->p.ncell * 8, r->stream));
     PIC_CUDA(cudaMemsetAsync(r->ws + r->lay.rho_f32, 0, (size_t)r->p.ncell * 4, r->stream));
-    PIC_CUDA(cudaMemsetAsync(r->ws + r->lay.rho_f64, 0, (size_t)r->p.ncell * 8, r->stream));
+    PIC_CUDA(cudaMemsetAsync(r->ws + r->lay.rho_w, 0, (size_t)r->p.ncell * 16, r->stream));
     PIC_CUDA(cudaMemsetAsync(r->ws + r->lay.hist, 0xFF, (size_t)r->lay.hist_len * sizeof(pic_diag_row), r->stream));
     PIC_CUDA(enqueue_push(r, r->stream, false));
     PIC_CUDA(enqueue_solve(r, r->stream, false));
@@ -475,7 +483,7 @@ int pic_create(const pic_params *p, void *workspace, size_t workspace_bytes,
     r->stream = (cudaStream_t)stream;
     cudaError_t e = cudaGetDevice(&r->device);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&r->sms, cudaDevAttrMultiProcessorCount, r->device);
-    if (e == cudaSuccess) e = push_prepare_attributes(p->precision, p->ncell);
+    if (e == cudaSuccess) e = push_prepare_attributes(p->precision);
     if (e == cudaSuccess) e = sort_prepare_attributes(p->ncell);
     if (e == cudaSuccess) e = solve_prepare_attributes();
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&r->cap, cudaStreamNonBlocking);
@@ -498,7 +506,7 @@ int pic_create(const pic_params *p, void *workspace, size_t workspace_bytes,
     r->variant = p->deposit_variant ? p->deposit_variant : PIC_DEPOSIT_QUAD;
     if (p->precision != PIC_FP32_FIXED) r->variant = PIC_DEPOSIT_ATOMIC;
     if (p->shape == PIC_SHAPE_NGP) r->variant = kDepositNgp;
-    r->block = p->block_size ? p->block_size : (p->precision == PIC_FP32_FIXED ? 512 : 256);
+    r->block = p->block_size ? p->block_size : default_block(r);
     r->unroll = p->unroll ? p->unroll : 1;
     if (p->precision != PIC_FP32_FIXED) r->unroll = 1;
     r->grid = push_grid(r, r->variant, r->block, r->unroll, p->blocks_per_sm);
@@ -569,7 +577,7 @@ int pic_deposit(pic_run *run) {
     const size_t ng = (size_t)run->p.ncell;
     PIC_CUDA(cudaMemsetAsync(run->ws + run->lay.rho_q, 0, ng * 8, run->stream));
     PIC_CUDA(cudaMemsetAsync(run->ws + run->lay.rho_f32, 0, ng * 4, run->stream));
-    PIC_CUDA(cudaMemsetAsync(run->ws + run->lay.rho_f64, 0, ng * 8, run->stream));
+    PIC_CUDA(cudaMemsetAsync(run->ws + run->lay.rho_w, 0, ng * 16, run->stream));
     PIC_CUDA(enqueue_push(run, run->stream, false));
     return PIC_OK;
 }

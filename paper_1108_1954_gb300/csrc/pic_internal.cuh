@@ -59,10 +59,11 @@ struct PushArgs {
 
 // Float64 push (PIC_FP64) and float32 push with float32 atomic deposit.
 struct PushArgs64 {
-    double *x, *v;
+    double *x, *v;                // 32-byte aligned
     long long n;
     const double *E64;
-    double *rho_acc;              // sum of weights per node [NG]
+    unsigned long long *rho_w;    // density sums in 2^-53: [NG][2], the low 40
+                                  // bits of the blocks' sums and the rest
     double *partials;
     unsigned int *err;
     int ng;
@@ -70,46 +71,37 @@ struct PushArgs64 {
 };
 
 struct PushArgsF32Atomic {
-    float *x, *v;
+    float *x, *v;                 // 16-byte aligned
     long long n;
     const float *E32;
     float *rho_acc;               // sum of float32 weights per node [NG]
     double *partials;
     unsigned int *err;
+    int copies;                   // sums per node of a block's tile (set by the launcher)
     PushConsts c;
 };
 
-// Per-block share of the step diagnostics, reduced by the solve's last block.
+// Per-block share of the step diagnostics.
 enum { kDiagFE = 0, kDiagKE, kDiagMom, kDiagCharge, kDiagModes,
        kDiagFields = kDiagModes + 2 * PIC_NMODES };
-struct DiagPartial {
-    double v[kDiagFields];         // field energy sum, KE and momentum sums,
-                                   // charge, mode sums (re, im) x 8
-    unsigned long long cq;         // fixed-point charge sum
-};
 
-// Field solve (fixed point: one cluster of up to 16 blocks; float modes and
-// CG: one block).
+// Field solve (one cluster of up to 16 blocks).
 struct SolveArgs {
     int mode;                     // PIC_FP32_FIXED / PIC_FP32_ATOMIC / PIC_FP64
     unsigned long long *rho_q;    // FIXED: accumulator (read, then zeroed)
     unsigned long long *rho_q_last; // FIXED: copy of the consumed sums
     float *rho_f32;               // FP32_ATOMIC accumulator
-    double *rho_f64;              // FP64 accumulator
+    unsigned long long *rho_w;    // FP64 accumulator, [NG][2]
     double *rho, *phi, *E64;      // outputs [NG]
     float *E32;                   // output copy for the gather [NG]
     const double *partials;       // per-block sums of the push that ran
     int npartials;                // 0: no push ran since the last solve
-    DiagPartial *dpart;           // [kSolveMaxBlocks]
-    unsigned *counter;            // last-block ticket (0 between launches)
     pic_diag_row *hist;           // history ring
     int hist_len;
     long long *dstep;             // device step counter
     int ng;
-    long long weight_total;       // N 2^24
-    double rho_ion;
-    double q_over_dx;             // Q0/dx = -rho_ion NG / N (float modes)
-    double k_rho;                 // rho_ion / (N 2^24)
+    long long npart_total;        // N
+    double k_rho;                 // rho_ion / (N 2^B)
     double k_e;                   // (dx/2) k_rho / NG
     double k_phi;                 // -dx^2 k_rho / NG
     double k_mode;                // 2 / NG: mode amplitude of the mode sums
@@ -118,6 +110,11 @@ struct SolveArgs {
     int solver;                   // PIC_SOLVER_EXACT / PIC_SOLVER_CG
     int cg_maxit;                 // CG: iterations per solve
 };
+
+// B by precision mode: a density sum counts 2^-B of a particle.
+__host__ __device__ constexpr int density_bits(int mode) {
+    return mode == PIC_FP32_FIXED ? kFixBits : mode == PIC_FP32_ATOMIC ? 30 : 53;
+}
 
 // Counting sort by cell.
 template <typename T>
@@ -227,18 +224,16 @@ int validate_params(const pic_params *p);
 // Launchers (each returns the launch's cudaError_t).
 cudaError_t launch_push_fixed(const PushArgs &a, int grid, int block,
                               int variant, int unroll, bool push, cudaStream_t s);
-cudaError_t launch_push_f32_atomic(const PushArgsF32Atomic &a, int grid,
-                                   int block, bool push, cudaStream_t s);
+cudaError_t launch_push_f32_atomic(PushArgsF32Atomic a, int grid, int block, bool push,
+                                   cudaStream_t s);
 cudaError_t launch_push_f64(const PushArgs64 &a, int grid, int block,
                             bool push, cudaStream_t s);
 size_t push_smem_bytes(int mode, int ng);
-cudaError_t push_prepare_attributes(int mode, int ng);
+cudaError_t push_prepare_attributes(int mode);
 int push_max_blocks_per_sm(int mode, int variant, int unroll, int block, int ng);
 
 cudaError_t launch_solve(const SolveArgs &a, cudaStream_t s);
 cudaError_t solve_prepare_attributes();
-constexpr int kSolveThreads = 1024;
-constexpr int kSolveMaxBlocks = 32;
 
 cudaError_t launch_sort_f32(const SortArgs<float> &a, cudaStream_t s);
 cudaError_t launch_sort_f64(const SortArgs<double> &a, cudaStream_t s);

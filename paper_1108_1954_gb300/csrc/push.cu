@@ -245,6 +245,26 @@ __global__ void __launch_bounds__(512) pic_push_oct_kernel(PushArgs a) {
 }
 
 // ---- float32 push with float32 atomic deposit (precision study) -------------
+//
+// Groups of 4 particles per thread and loads ahead, as the fixed-point push.
+// A float32 add on shared memory is a compare-and-swap loop, and lanes that hit
+// one node go through it one after the other: that is what bounds the kernel.
+// So two open runs per thread are summed in registers first (PAIR), and the
+// block keeps `copies` sums per node, side by side, lane l adding to copy
+// l mod copies: lanes of one cell then meet on an address copies times less
+// often.  As many copies as fit beside E in kAtomicTile bytes, at most 32 (one
+// per lane).  Measured (2^24 particles, 1024 cells, 16 copies): 61 us a push,
+// the mean over sort periods, against 295 us with one copy and a shuffle sum
+// where a whole warp holds one run, and 140 us (sorted) to 380 us (lattice
+// order) with two adds per particle.
+// (72 KB: two 512-thread blocks of 53 registers per SM keep their place.)
+constexpr size_t kAtomicTile = 72 * 1024;
+
+int atomic_copies(int ng) {
+    int k = 32;
+    while (k > 1 && (size_t)(ng + 2) * 4 * k > kAtomicTile) k /= 2;
+    return k;
+}
 
 template <bool PUSH>
 __global__ void __launch_bounds__(1024) pic_push_f32atomic_kernel(PushArgsF32Atomic a) {
@@ -252,26 +272,73 @@ __global__ void __launch_bounds__(1024) pic_push_f32atomic_kernel(PushArgsF32Ato
     __shared__ double red[64];
     const PushConsts c = a.c;
     const int ng = c.ng;
-    float *sRho = reinterpret_cast<float *>(smem_raw);   // ng + 2, ghost-padded
-    float *sE = sRho + ng + 2;                            // ng + 2, ghost-padded
-    const int tid = threadIdx.x, bs = blockDim.x;
-    for (int j = tid; j < ng + 2; j += bs) {
-        sRho[j] = 0.0f;
+    float *sE = reinterpret_cast<float *>(smem_raw);      // ng + 2, ghost-padded
+    float *sRho = sE + ng + 2;                            // [ng + 2][copies], ghost-padded
+    const int tid = threadIdx.x, bs = blockDim.x, K = a.copies;
+    for (int j = tid; j < ng + 2; j += bs)
         if (PUSH) sE[j] = a.E32[j == 0 ? ng - 1 : (j == ng + 1 ? 0 : j - 1)];
-    }
+    for (int j = tid; j < (ng + 2) * K; j += bs) sRho[j] = 0.0f;
     __syncthreads();
+    float *mine = sRho + (tid & (K - 1));                 // this lane's copy
+    auto add = [&](unsigned key, float l, float r) {
+        atomicAdd(&mine[key * K], l);
+        atomicAdd(&mine[(key + 1) * K], r);
+    };
     float ke = 0.0f, mom = 0.0f;
+    const long long n4 = a.n >> 2;
     const long long stride = (long long)gridDim.x * bs;
-    for (long long i = (long long)blockIdx.x * bs + tid; i < a.n; i += stride) {
+    float4 *x4 = reinterpret_cast<float4 *>(a.x);
+    float4 *v4 = reinterpret_cast<float4 *>(a.v);
+    const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
+    const long long q00 = (long long)blockIdx.x * bs;
+    float4 cx = q00 + tid < n4 ? __ldcs(x4 + q00 + tid) : zero4;
+    float4 cv = PUSH && q00 + tid < n4 ? __ldcs(v4 + q00 + tid) : zero4;
+    for (long long q = q00 + tid; q < n4; q += stride) {
+        const long long qn = q + stride;
+        const float4 nx = qn < n4 ? __ldcs(x4 + qn) : zero4;
+        const float4 nv = PUSH && qn < n4 ? __ldcs(v4 + qn) : zero4;
+        float xs[4] = {cx.x, cx.y, cx.z, cx.w}, vs[4] = {cv.x, cv.y, cv.z, cv.w};
+        unsigned ka = 0xffffffffu, kb = 0xffffffffu;      // open runs' left nodes + 1
+        float la = 0.0f, ra = 0.0f, lb = 0.0f, rb = 0.0f;
+        bool bad = false;
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            if (PUSH) push_particle(xs[k], vs[k], sE, c, ke, mom);
+            const Loc l = locate(xs[k]);
+            const bool ok = l.j <= (unsigned)ng;
+            bad |= !ok;
+            if (!ok) continue;
+            const float wl = 1.0f - l.f;
+            if (l.j == ka) {
+                la += wl;
+                ra += l.f;
+            } else if (l.j == kb) {
+                lb += wl;
+                rb += l.f;
+            } else {
+                if (kb != 0xffffffffu) add(kb, lb, rb);
+                kb = ka; lb = la; rb = ra;
+                ka = l.j; la = wl; ra = l.f;
+            }
+        }
+        if (PUSH) {
+            __stcs(x4 + q, make_float4(xs[0], xs[1], xs[2], xs[3]));
+            __stcs(v4 + q, make_float4(vs[0], vs[1], vs[2], vs[3]));
+        }
+        if (ka != 0xffffffffu) add(ka, la, ra);
+        if (kb != 0xffffffffu) add(kb, lb, rb);
+        if (bad) atomicOr(a.err, kErrPosition);
+        cx = nx;
+        cv = nv;
+    }
+    // the last N mod 4 particles
+    if (blockIdx.x == 0 && tid < (int)(a.n & 3)) {
+        const long long i = n4 * 4 + tid;
         float x = a.x[i], v = PUSH ? a.v[i] : 0.0f;
         if (PUSH) push_particle(x, v, sE, c, ke, mom);
         const Loc l = locate(x);
-        if (l.j <= (unsigned)ng) {
-            atomicAdd(&sRho[l.j], 1.0f - l.f);
-            atomicAdd(&sRho[l.j + 1], l.f);
-        } else {
-            atomicOr(a.err, kErrPosition);
-        }
+        if (l.j <= (unsigned)ng) add(l.j, 1.0f - l.f, l.f);
+        else atomicOr(a.err, kErrPosition);
         if (PUSH) { a.x[i] = x; a.v[i] = v; }
     }
     if (PUSH) {
@@ -285,87 +352,230 @@ __global__ void __launch_bounds__(1024) pic_push_f32atomic_kernel(PushArgsF32Ato
     }
     __syncthreads();
     for (int j = tid; j < ng + 2; j += bs) {
-        const float t = sRho[j];
+        float t = 0.0f;
+        for (int k = 0; k < K; k++) t += sRho[j * K + ((k + tid) & (K - 1))];
         if (t == 0.0f) continue;
         const int node = j == 0 ? ng - 1 : (j == ng + 1 ? 0 : j - 1);
         atomicAdd(&a.rho_acc[node], t);
     }
 }
 
-// ---- float64 push with float64 atomic deposit (precision study) ------------
+// ---- float64 push and deposit (precision study) --------------------------------
+//
+// GB300 issues float64 at 2 lanes per clock per SM, so a float64 instruction
+// of a warp takes the pipe for 16 clocks, the time of some 40 integer
+// instructions.  The kernel keeps five per particle -- gather, kick, v v', sum
+// v', drift -- and does the rest in integers:
+//   locate    u = x NG/L as the high 64 bits of the product of the two
+//             mantissas, shifted to F = 62 - floor(log2(NG)) bits after the binary
+//             point (float64 keeps 52 - log2(u)); plus 1/2, its integer part is
+//             the tile index and the rest the fraction;
+//   gather    E_l + f (E_r - E_l) = fma(1 + f, dE, E_l - dE): 1 + f is the
+//             fraction's bits under the exponent of 1, dE and E_l - dE are
+//             kept as pairs in shared memory;
+//   deposit   the weights are integers of 2^-53 (f to within 2^-54, which a
+//             float64 sum of one particle or more does not resolve either),
+//             summed exactly: runs of equal cell in registers (two open runs
+//             of a thread's 4 particles, as PAIR), then in a tile of three
+//             32-bit words per node.  Native 32-bit shared adds take the place
+//             of float64 compare-and-swap loops, and the density no longer
+//             depends on the order of the adds.
+// The tile goes to global memory as two 64-bit sums per node, of the low 40
+// bits and of the rest: at most 4096 blocks of less than 2^40 each, so neither
+// needs a carry.
+// Measured (2^24 particles, 1024 cells, sorted every 20 steps): 178 us a push,
+// 145 us of it the five float64 instructions at the pipe's rate; 353 us with
+// the two s = x NG/L + 1/2 as float64 FMAs and the wrap predicated (9.3 float64
+// instructions), 1509 us with float64 floors, a segmented shuffle sum of the
+// weights and float64 shared adds.
+struct Loc64 {
+    unsigned j;                   // tile index (left node + 1)
+    unsigned fh, fl;              // fraction in 2^-64
+    bool ok;
+};
+
+struct Push64 {
+    const double2 *pair;          // (E_l - dE, dE) of tile index j
+    u64 lbits;                    // bits of L
+    u64 wide;                     // mantissa of NG/L, its top bit set
+    int frac_bits;                // F
+    int shift;                    // u = high(mantissa(x) wide) >> (shift - exponent bits of x)
+};
+
+__device__ __forceinline__ Push64 push64_consts(const PushArgs64 &a, const double2 *pair) {
+    Push64 c;
+    c.pair = pair;
+    c.lbits = (u64)__double_as_longlong(a.length);
+    const u64 w = (u64)__double_as_longlong(a.inv_dx);
+    c.wide = ((w & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull) << 11;
+    // U = u 2^F must hold NG + 1/2 in 64 bits: F = 63 - (bits of NG)
+    c.frac_bits = 31 + __clz(a.ng);
+    // x = M 2^(ex - 63), NG/L = W 2^(k - 63): u 2^F = high64(M W) 2^(ex + k - 62 + F)
+    const int k = (int)(w >> 52) - 1023;
+    c.shift = 62 - c.frac_bits - k + 1023;
+    return c;
+}
+
+__device__ __forceinline__ Loc64 locate64(double x, double inv_dx, int ng, const Push64 &c) {
+    const u64 b = (u64)__double_as_longlong(x);
+    Loc64 l;
+    u64 U;
+    if (b < c.lbits) {                               // 0 <= x < L
+        const u64 m = ((b & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull) << 11;
+        const unsigned r = (unsigned)(c.shift - (int)(b >> 52));
+        U = r < 64u ? __umul64hi(m, c.wide) >> r : 0ull;   // u < 2^-F: 0
+        U += 1ull << (c.frac_bits - 1);
+        l.ok = true;
+    } else {
+        // outside the box: what lies within half a cell of it (left of node 0 or
+        // right of node NG - 1) still has two nodes
+        const double s = fma(x, inv_dx, 0.5);
+        l.ok = s >= 0.0 && s < (double)(ng + 1);
+        U = l.ok ? __double2ull_rz(scalbn(s, c.frac_bits)) : 0ull;
+    }
+    l.j = (unsigned)(U >> c.frac_bits);
+    const u64 f = U << (64 - c.frac_bits);
+    l.fh = (unsigned)(f >> 32);
+    l.fl = (unsigned)f;
+    return l;
+}
+
+struct Tile96 {
+    unsigned *lo, *mid, *hi;
+};
+
+__device__ __forceinline__ void tile_add96(const Tile96 &t, unsigned j, u64 val) {
+    const unsigned vl = (unsigned)val;
+    const unsigned ol = atomicAdd(&t.lo[j], vl);
+    const unsigned vm = (unsigned)(val >> 32) + (ol + vl < ol ? 1u : 0u);   // < 2^27
+    const unsigned om = atomicAdd(&t.mid[j], vm);
+    if (om + vm < om) atomicAdd(&t.hi[j], 1u);
+}
+
+constexpr u64 kOne53 = 1ull << 53;
+
+struct Run64 {
+    unsigned key, cnt;            // left node + 1 (0xffffffff: none open), particles
+    u64 r;                        // sum of the right weights
+};
+
+__device__ __forceinline__ void close_run(const Tile96 &t, const Run64 &w) {
+    if (w.key == 0xffffffffu) return;
+    tile_add96(t, w.key, w.cnt * kOne53 - w.r);
+    tile_add96(t, w.key + 1, w.r);
+}
+
+struct D4 {
+    double v[4];
+};
+
+__device__ __forceinline__ D4 ld4d(const double *p) {
+    D4 r;
+    asm volatile("ld.global.cs.v4.f64 {%0, %1, %2, %3}, [%4];"
+                 : "=d"(r.v[0]), "=d"(r.v[1]), "=d"(r.v[2]), "=d"(r.v[3]) : "l"(p));
+    return r;
+}
+
+__device__ __forceinline__ void st4d(double *p, const D4 &r) {
+    asm volatile("st.global.cs.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(p), "d"(r.v[0]), "d"(r.v[1]),
+                 "d"(r.v[2]), "d"(r.v[3]) : "memory");
+}
+
+__device__ __forceinline__ void push_particle64(double &x, double &v, const PushArgs64 &a,
+                                                const Push64 &c, double &ke, double &mom) {
+    const Loc64 l = locate64(x, a.inv_dx, a.ng, c);
+    const double g = __hiloint2double((int)(0x3FF00000u | (l.fh >> 12)),
+                                      (int)__funnelshift_l(l.fl, l.fh, 20));
+    const double2 p = c.pair[l.j];
+    const double ep = l.ok ? fma(g, p.y, p.x) : 0.0;
+    const double vn = fma(a.qmdt, ep, v);
+    ke = fma(v, vn, ke);
+    mom += vn;
+    double xn = fma(vn, a.dt, x);
+    // x < 0, x >= L and NaN all have bits of at least those of L (the vote
+    // keeps it a branch: as predicated instructions the three comparisons and
+    // two adds took the float64 pipe for every particle)
+    const bool out = (u64)__double_as_longlong(xn) >= c.lbits;
+    if (__any_sync(__activemask(), out) && out) {
+        if (xn < 0.0) xn += a.length;
+        else if (xn >= a.length) xn -= a.length;
+        if (xn >= a.length) xn = 0.0;
+    }
+    x = xn;
+    v = vn;
+}
 
 template <bool PUSH>
 __global__ void __launch_bounds__(1024) pic_push_f64_kernel(PushArgs64 a) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ double red[64];
-    double *sRho = reinterpret_cast<double *>(smem_raw);
-    double *sE = sRho + a.ng;
     const int tid = threadIdx.x, bs = blockDim.x, ng = a.ng;
-    for (int g = tid; g < ng; g += bs) {
-        sRho[g] = 0.0;
-        if (PUSH) sE[g] = a.E64[g];
+    double2 *pair = reinterpret_cast<double2 *>(smem_raw);           // ng + 1
+    Tile96 t;                                                        // ng + 2 each
+    t.lo = reinterpret_cast<unsigned *>(pair + ng + 1);
+    t.mid = t.lo + ng + 2;
+    t.hi = t.mid + ng + 2;
+    for (int j = tid; j < ng + 2; j += bs) {
+        t.lo[j] = 0u;
+        t.mid[j] = 0u;
+        t.hi[j] = 0u;
+        if (PUSH && j <= ng) {
+            const double el = a.E64[j == 0 ? ng - 1 : j - 1], er = a.E64[j == ng ? 0 : j];
+            const double de = er - el;
+            pair[j] = make_double2(el - de, de);
+        }
     }
     __syncthreads();
+    const Push64 c = push64_consts(a, pair);
     double ke = 0.0, mom = 0.0;
+    const long long n4 = a.n >> 2;
     const long long stride = (long long)gridDim.x * bs;
-    const int lane = tid & 31;
-    // the trip count is uniform over a warp (base is), so every lane takes
-    // part in the deposit's shuffles
-    for (long long base = (long long)blockIdx.x * bs + (tid & ~31); base < a.n; base += stride) {
-        const long long i = base + lane;
-        const bool valid = i < a.n;
-        double x = valid ? a.x[i] : 0.0;
-        double s = x * a.inv_dx - 0.5;
-        double fl = floor(s);
-        bool ok = valid && fl >= -1.0 && fl <= (double)(ng - 1);
-        if (PUSH && valid) {
-            double v = a.v[i];
-            int j = ok ? (int)fl : 0;
-            int il = j < 0 ? j + ng : j, ir = j + 1 >= ng ? j + 1 - ng : j + 1;
-            double f = s - fl;
-            double ep = ok ? (1.0 - f) * sE[il] + f * sE[ir] : 0.0;
-            double vn = v + a.qmdt * ep;
-            ke += v * vn;
-            mom += vn;
-            x = x + vn * a.dt;
-            if (x < 0.0) x += a.length;
-            else if (x >= a.length) x -= a.length;
-            if (x >= a.length) x = 0.0;
-            a.x[i] = x;
-            a.v[i] = vn;
-            s = x * a.inv_dx - 0.5;
-            fl = floor(s);
-            ok = fl >= -1.0 && fl <= (double)(ng - 1);
-        }
-        // Deposit.  Lanes with equal left node in a row (particles in
-        // lattice or sorted order share nodes) first add their weights in a
-        // segmented shuffle sum, and the segment's first lane does the two
-        // adds; a float64 add on shared memory is a compare-and-swap loop,
-        // which lanes hitting one node would otherwise serialise.
-        const int j = ok ? (int)fl : 0;
-        const int il = j < 0 ? j + ng : j, ir = j + 1 >= ng ? j + 1 - ng : j + 1;
-        const double f = s - fl;
-        const unsigned key = ok ? (unsigned)il : 0xffffffffu;
-        const unsigned kprev = __shfl_up_sync(kFull, key, 1);
-        const bool head = ok && (lane == 0 || kprev != key);
-        const unsigned heads = __ballot_sync(kFull, head || !ok);
-        const unsigned above = lane == 31 ? 0u : heads & (0xffffffffu << (lane + 1));
-        const int end = above ? __ffs(above) - 1 : 32;       // this lane's segment ends before
-        double sl = ok ? 1.0 - f : 0.0, sr = ok ? f : 0.0;
+    for (long long q = (long long)blockIdx.x * bs + tid; q < n4; q += stride) {
+        D4 x = ld4d(a.x + 4 * q), v;
+        if (PUSH) v = ld4d(a.v + 4 * q);
+        Run64 ra = {0xffffffffu, 0u, 0ull}, rb = {0xffffffffu, 0u, 0ull};
+        bool bad = false;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const double tl = __shfl_down_sync(kFull, sl, o);
-            const double tr = __shfl_down_sync(kFull, sr, o);
-            if (lane + o < end) {
-                sl += tl;
-                sr += tr;
+        for (int k = 0; k < 4; k++) {
+            if (PUSH) push_particle64(x.v[k], v.v[k], a, c, ke, mom);
+            const Loc64 l = locate64(x.v[k], a.inv_dx, ng, c);
+            bad |= !l.ok;
+            if (!l.ok) continue;
+            const u64 w = (((u64)l.fh << 32) | l.fl) >> 11;
+            if (l.j == ra.key) {
+                ra.cnt++;
+                ra.r += w;
+            } else if (l.j == rb.key) {
+                rb.cnt++;
+                rb.r += w;
+            } else if (rb.key == 0xffffffffu) {
+                rb = ra;
+                ra = Run64{l.j, 1u, w};
+            } else {
+                close_run(t, ra);
+                ra = Run64{l.j, 1u, w};
             }
         }
-        if (head) {
-            atomicAdd(&sRho[il], sl);
-            atomicAdd(&sRho[ir], sr);
+        if (PUSH) {
+            st4d(a.x + 4 * q, x);
+            st4d(a.v + 4 * q, v);
         }
-        if (valid && !ok) atomicOr(a.err, kErrPosition);
+        close_run(t, ra);
+        close_run(t, rb);
+        if (bad) atomicOr(a.err, kErrPosition);
+    }
+    if (blockIdx.x == 0 && tid < (int)(a.n & 3)) {          // the last N mod 4 particles
+        const long long i = n4 * 4 + tid;
+        double x = a.x[i], v = 0.0;
+        if (PUSH) {
+            v = a.v[i];
+            push_particle64(x, v, a, c, ke, mom);
+            a.x[i] = x;
+            a.v[i] = v;
+        }
+        const Loc64 l = locate64(x, a.inv_dx, ng, c);
+        if (l.ok) close_run(t, Run64{l.j, 1u, (((u64)l.fh << 32) | l.fl) >> 11});
+        else atomicOr(a.err, kErrPosition);
     }
     if (PUSH) {
         __syncthreads();
@@ -376,8 +586,14 @@ __global__ void __launch_bounds__(1024) pic_push_f64_kernel(PushArgs64 a) {
         }
     }
     __syncthreads();
-    for (int g = tid; g < ng; g += bs)
-        if (sRho[g] != 0.0) atomicAdd(&a.rho_acc[g], sRho[g]);
+    for (int j = tid; j < ng + 2; j += bs) {
+        const unsigned lo = t.lo[j], mid = t.mid[j];
+        const u64 low40 = ((u64)(mid & 0xFFu) << 32) | lo;
+        const u64 rest = ((u64)t.hi[j] << 24) | (mid >> 8);
+        const int node = j == 0 ? ng - 1 : (j == ng + 1 ? 0 : j - 1);
+        if (low40) atomicAdd(&a.rho_w[2 * node], low40);
+        if (rest) atomicAdd(&a.rho_w[2 * node + 1], rest);
+    }
 }
 
 using FixedKernel = void (*)(PushArgs);
@@ -419,17 +635,18 @@ FixedKernel pick_fixed(int variant, bool push, int unroll) {
 }  // namespace
 
 size_t push_smem_bytes(int mode, int ng) {
-    if (mode == PIC_FP64) return (size_t)ng * 16;
-    if (mode == PIC_FP32_ATOMIC) return (size_t)(ng + 2) * 8;
+    if (mode == PIC_FP64) return (size_t)(ng + 1) * 16 + (size_t)(ng + 2) * 12;
+    if (mode == PIC_FP32_ATOMIC) return (size_t)(ng + 2) * 4 * (1 + atomic_copies(ng));
     return (size_t)(ng + 2) * 12;
 }
 
 // Shared memory of a fused fixed-point push launch.
 size_t fixed_smem_bytes(int ng) { return push_smem_bytes(PIC_FP32_FIXED, ng); }
 
-cudaError_t push_prepare_attributes(int mode, int ng) {
-    const int bytes = (int)push_smem_bytes(mode, PIC_NCELL_MAX);
-    (void)ng;
+cudaError_t push_prepare_attributes(int mode) {
+    // the atomic tile is largest where 32 copies just fit
+    const int bytes = mode == PIC_FP32_ATOMIC ? (int)(2 * kAtomicTile)
+                                              : (int)push_smem_bytes(mode, PIC_NCELL_MAX);
     cudaError_t e = cudaSuccess;
     if (mode == PIC_FP32_FIXED) {
         const int unrolls[3] = {1, 2, 4};
@@ -489,9 +706,10 @@ cudaError_t launch_push_fixed(const PushArgs &a, int grid, int block, int varian
     return cudaGetLastError();
 }
 
-cudaError_t launch_push_f32_atomic(const PushArgsF32Atomic &a, int grid, int block,
-                                   bool push, cudaStream_t s) {
+cudaError_t launch_push_f32_atomic(PushArgsF32Atomic a, int grid, int block, bool push,
+                                   cudaStream_t s) {
     const size_t smem = push_smem_bytes(PIC_FP32_ATOMIC, a.c.ng);
+    a.copies = atomic_copies(a.c.ng);
     if (push) pic_push_f32atomic_kernel<true><<<grid, block, smem, s>>>(a);
     else pic_push_f32atomic_kernel<false><<<grid, block, smem, s>>>(a);
     return cudaGetLastError();

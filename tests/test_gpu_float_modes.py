@@ -1,0 +1,98 @@
+"""The float64 and float32-atomic pushes at the sizes where their groups, tiles
+and integer locate can go wrong, against the FP64 oracle.
+
+float64: the deposit is exact integers of 2^-53, so the density is compared with
+exactly summed weights (the oracle's own sums are rounded at every add): what
+is left is the result's rounding, n/ng 2^-52 a node at most, and the cell
+fraction's ng 2^-52 per particle.  float32 atomic: a node's float32
+sum is off by at most its number of adds times its size times 2^-24, and the
+fraction by ng 2^-24."""
+import math
+
+import numpy as np
+import pytest
+
+import oracle as O
+import paper_1108_1954_gb300 as pic
+import torch  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+L = 3.7
+
+
+def state(n, ng, seed):
+    """Random particles, with some on nodes, cell edges and the box's ends."""
+    rng = np.random.default_rng(seed)
+    x = rng.uniform(0.0, L, n)
+    dx = L / ng
+    edge = [0.0, np.nextafter(0.0, 1.0), np.nextafter(L, 0.0), 0.5 * dx, np.nextafter(0.5 * dx, 0.0),
+            L - 0.5 * dx, (ng // 2) * dx]
+    k = min(n, len(edge))
+    x[:k] = edge[:k]
+    return np.clip(x, 0.0, np.nextafter(L, 0.0)), rng.normal(0.0, 0.3, n)
+
+
+def exact_density(x, ng):
+    """rho from the CIC weights of x, summed without rounding: the weights as
+    multiples of 2^-52, their halves of 26 bits summed exactly in float64."""
+    s = x * (ng / L) - 0.5
+    left = np.floor(s).astype(np.int64)
+    w = np.rint((s - left) * 2.0 ** 52).astype(np.int64)
+    total = np.zeros(ng)
+    for node, q in ((left % ng, (1 << 52) - w), ((left + 1) % ng, w)):
+        total += np.bincount(node, (q >> 26).astype(float), ng) * 2.0 ** -26 \
+            + np.bincount(node, (q & ((1 << 26) - 1)).astype(float), ng) * 2.0 ** -52
+    return 1.0 - total * (ng / x.size)
+
+
+@pytest.mark.parametrize("n", [1, 2, 3, 4, 5, 7, 255, 256, 257, 2051, 40003])
+@pytest.mark.parametrize("ng", [1, 2, 3, 64, 127, 128, 1000, 8191, 8192])
+def test_fp64_step_at_the_edges(n, ng):
+    x, v = state(n, ng, 31 * n + ng)
+    run = pic.Run(pic.Params(npart=n, ncell=ng, length=L, precision=pic.PIC_FP64), device="cuda:0")
+    run.init(x, v)
+    ref = O.State(O.params(ng, n, L, 0.1), x, v)
+    tol = (n / ng + ng * math.sqrt(n) + 8) * 2.0 ** -50 * (ng / n)
+    assert np.abs(run.get_field()["rho"] - exact_density(x, ng)).max() <= tol
+    assert abs(run.get_field()["rho"].sum()) <= 1e-12          # every particle whole
+    run.push()
+    run.solve_field()
+    ref.step()
+    x1, v1 = run.get_state()
+    d = np.abs(x1 - ref.x)
+    assert np.minimum(d, L - d).max() <= 1e-12 * L
+    assert np.abs(v1 - ref.v).max() <= 1e-11
+    assert abs(run.get_field()["rho"].sum()) <= 1e-12
+
+
+@pytest.mark.parametrize("n", [1, 3, 4, 5, 257, 40003])
+@pytest.mark.parametrize("ng", [1, 64, 574, 575, 1150, 8192])     # 32, 16, 8 and 2 copies
+def test_atomic_deposit_at_the_edges(n, ng):
+    x, v = state(n, ng, 17 * n + ng)
+    x32 = np.minimum(x.astype(np.float32), np.nextafter(np.float32(L), np.float32(0)))
+    run = pic.Run(pic.Params(npart=n, ncell=ng, length=L, precision=pic.PIC_FP32_ATOMIC),
+                  device="cuda:0")
+    run.init(x32, v.astype(np.float32))
+    ref = O.State(O.params(ng, n, L, 0.1), x32.astype(np.float64), v)
+    most = float((1.0 - ref.rho).max() / (ng / n))              # the fullest node's particles
+    tol = (ng / n) * 2.0 ** -24 * (2.0 * (most + 1) ** 2 + 2.0 * ng * (most + 1))
+    assert np.abs(run.get_field()["rho"] - ref.rho).max() <= tol
+    run.push()
+    run.solve_field()
+    u1, _ = run.get_cells()
+    assert ((u1 >= 0) & (u1 < ng)).all()
+
+
+@pytest.mark.parametrize("precision", [pic.PIC_FP64, pic.PIC_FP32_ATOMIC])
+@pytest.mark.parametrize("bad", [float("nan"), float("-inf"), -1e4])   # (beyond the far end is the point 0)
+def test_a_particle_thrown_out_of_the_box_is_flagged(precision, bad):
+    n = 1001
+    x, v = state(n, 64, 5)
+    v[n - 1] = v[500] = bad                                     # in a group and in the tail
+    run = pic.Run(pic.Params(npart=n, ncell=64, length=L, precision=precision), device="cuda:0")
+    dt = run.p.dtype
+    run.init(np.minimum(x.astype(dt), np.nextafter(dt(L), dt(0))), v.astype(dt))
+    run.push()
+    with pytest.raises(pic.PicError) as e:
+        run.sync()
+    assert e.value.code == pic.PIC_EDEVICE
