@@ -420,12 +420,13 @@ typedef struct pic_pool_config {
     int32_t ncell_max;     /* largest NG admitted (<= PIC_NCELL_MAX)            */
     int32_t history;       /* diagnostics rows kept per run (>= 1)              */
     int32_t variant;       /* PIC_DEPOSIT_ATOMIC | _MATCH | _QUAD | _PAIR
-                              (0 = MATCH); + 16: kernel built for two
+                              (0 = ATOMIC + 16); + 16: kernel built for two
                               512-thread blocks per SM (64 registers)
                               instead of one                                 */
     int32_t cluster;       /* blocks per cluster: 1, 2, 4, 8 (0 = 8)            */
-    int32_t block;         /* threads per block: 128 .. 512 (0 = 256); the
-                              shape needs ceil(ncell_max / cluster) <= block   */
+    int32_t block;         /* threads per block: 128 .. 512 (0 = 256, or 512
+                              while few runs are active); the shape needs
+                              ceil(ncell_max / cluster) <= block (0: <= 256)   */
 } pic_pool_config;
 
 /* Arena bytes one run with parameters *p takes in a pool with `history`
@@ -472,7 +473,8 @@ int pic_pool_finished(const pic_pool *pool, int32_t *slots, int32_t max, int32_t
 int pic_pool_step_count(const pic_pool *pool, int32_t slot, int64_t *step);
 
 /* Results of a run (synchronise): state (positions converted from cell
- * units on the host, by the same two float64-rounded steps as pic_get_state),
+ * units by the same two float64-rounded steps as pic_get_state: on the device
+ * through free space of the arena, on the host when there is none),
  * the state in cell units as held on the device, field of its last step,
  * history. */
 int pic_pool_get_state(pic_pool *pool, int32_t slot, void *x, void *v);
