@@ -65,9 +65,9 @@ extern "C" {
 #define PIC_EINVAL (-1)   /* bad argument or parameter                       */
 #define PIC_ENOMEM (-2)   /* workspace too small / pool budget exhausted      */
 #define PIC_ECUDA (-3)    /* a CUDA runtime call failed                       */
-#define PIC_ETIMEOUT (-4) /* reserved: no call waits on the device with a
-                             time limit (every device wait is a hardware
-                             block or cluster barrier)                      */
+#define PIC_ETIMEOUT (-4) /* a grid barrier of a pic_step_n launch ran out of
+                             its limit (some seconds); the run needs
+                             pic_init or pic_set_state                       */
 #define PIC_EDEVICE (-5)  /* a kernel flagged bad particle data                */
 #define PIC_ESTATE (-6)   /* call out of order (e.g. push before init)         */
 
@@ -207,7 +207,11 @@ int pic_push(pic_run *run);
  * their order).  Changes no physical quantity.  Asynchronous. */
 int pic_sort(pic_run *run);
 
-/* n whole steps: [sort if due] + push + solve, replayed from CUDA graphs.
+/* n whole steps: [sort if due] + push + solve.  Fixed-point runs with the
+ * exact solver, up to 12.5e6 particles and 4096 cells, whose launch shape is
+ * left open (pic_params, pic_set_launch) take many steps per cooperative
+ * launch; others replay CUDA graphs.  The results are the same.  While the
+ * stream is being captured single launches are enqueued.
  * A step n with n % S == 0 (S = sort_interval > 0, n > 0) sorts first.
  * Asynchronous. */
 int pic_step_n(pic_run *run, int64_t n);

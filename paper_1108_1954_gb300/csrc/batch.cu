@@ -77,16 +77,16 @@ __device__ __forceinline__ unsigned sort_key(float u, int ng) {
 // Block r owns the contiguous particle chunk [c0, c1) (the chunks in rank
 // order cover the run) and the cell slice [b0, b1) of at most one cell per
 // thread.  Four cluster barriers:
-//   count    each block counts the cells of its chunk into tile.lo;
+//   count    each block counts the cells of its chunk into tile.w;
 //   #1       the owner of cell g reads the C blocks' counts of g and forms
 //            the per-block exclusive prefixes and the cell total; a block
 //            scan over its slice gives the slice-local bases and the slice
 //            total, published in ex.sort_total;
 //   #2       every owner adds the totals of the slices before its own and
 //            writes its table T[r'][g - b0] = first slot of block r' in cell
-//            g into tile.hi;
+//            g into tile.n;
 //   #3       every block reads its first slot of every cell from the owners'
-//            tables into tile.lo and scatters its chunk in order, 256
+//            tables into tile.w and scatters its chunk in order, 256
 //            particles at a time (lanes of one cell ranked by match, warps
 //            taking their slots one after the other), into xa, va;
 //   #4       the scattered particles are visible to the whole cluster.
@@ -101,14 +101,14 @@ __device__ void cluster_sort(const BatchArgs &a, cg::cluster_group &cl, Exchange
     const int tid = threadIdx.x, bs = blockDim.x, lane = tid & 31, warp = tid >> 5;
     const int nwarp = bs >> 5;
     // count (the tile is empty at the start of a step)
-    for (long long i = c0 + tid; i < c1; i += bs) atomicAdd(&tile.lo[sort_key(X[i], ng)], 1u);
+    for (long long i = c0 + tid; i < c1; i += bs) atomicAdd(&tile.w[sort_key(X[i], ng)], 1u);
     cl.sync();                                                        // #1
     const int g = b0 + tid;
     const bool mine = g < b1;
     unsigned cnt[kMaxCluster];
 #pragma unroll
     for (int b = 0; b < kMaxCluster; b++)
-        cnt[b] = (mine && b < C) ? cl.map_shared_rank(tile.lo, b)[g] : 0u;
+        cnt[b] = (mine && b < C) ? cl.map_shared_rank(tile.w, b)[g] : 0u;
     unsigned tot = 0;
 #pragma unroll
     for (int b = 0; b < kMaxCluster; b++) tot += cnt[b];
@@ -142,7 +142,7 @@ __device__ void cluster_sort(const BatchArgs &a, cg::cluster_group &cl, Exchange
         unsigned slot = before + local;
 #pragma unroll
         for (int b = 0; b < kMaxCluster; b++) {
-            if (b < C) tile.hi[b * P + tid] = slot;
+            if (b < C) tile.n[b * P + tid] = slot;
             slot += cnt[b];
         }
     }
@@ -150,7 +150,7 @@ __device__ void cluster_sort(const BatchArgs &a, cg::cluster_group &cl, Exchange
     // this block's first slot of every cell, from the cell's owner
     for (int h = tid; h < ng; h += bs) {
         const int o = h / P;
-        tile.lo[h] = cl.map_shared_rank(tile.hi, o)[r * P + (h - o * P)];
+        tile.w[h] = cl.map_shared_rank(tile.n, o)[r * P + (h - o * P)];
     }
     __syncthreads();
     const unsigned lt = (1u << lane) - 1u;
@@ -164,8 +164,8 @@ __device__ void cluster_sort(const BatchArgs &a, cg::cluster_group &cl, Exchange
         unsigned base = 0;
         for (int w = 0; w < nwarp; w++) {
             if (w == warp && valid && lane == leader) {
-                base = tile.lo[key];
-                tile.lo[key] = base + (unsigned)__popc(peers);
+                base = tile.w[key];
+                tile.w[key] = base + (unsigned)__popc(peers);
             }
             __syncthreads();
         }
@@ -183,8 +183,8 @@ __device__ void cluster_sort(const BatchArgs &a, cg::cluster_group &cl, Exchange
     cl.sync();                                                        // #4
     // the tile empty again for the push (hi held the table: C P words)
     for (int j = tid; j < ng + kTilePad; j += bs) {
-        tile.lo[j] = 0u;
-        tile.hi[j] = 0u;
+        tile.w[j] = 0u;
+        tile.n[j] = 0u;
     }
     __syncthreads();
 }
@@ -207,8 +207,8 @@ __device__ void run_steps(const BatchArgs &a, const BatchRun &R, cg::cluster_gro
     // E of the current step, ghost-padded; empty tile
     for (int j = tid; j < ng + 2; j += bs) {
         sE[j] = R.E32[j == 0 ? ng - 1 : (j == ng + 1 ? 0 : j - 1)];
-        tile.lo[j] = 0u;
-        tile.hi[j] = 0u;
+        tile.w[j] = 0u;
+        tile.n[j] = 0u;
     }
     __syncthreads();
 
@@ -331,8 +331,8 @@ __device__ void run_steps(const BatchArgs &a, const BatchRun &R, cg::cluster_gro
             unsigned lo[kMaxCluster], hi[kMaxCluster];
 #pragma unroll
             for (int b = 0; b < kMaxCluster; b++) {
-                lo[b] = b < C ? cl.map_shared_rank(tile.lo, b)[g + 1] : 0u;
-                hi[b] = b < C ? cl.map_shared_rank(tile.hi, b)[g + 1] : 0u;
+                lo[b] = b < C ? cl.map_shared_rank(tile.w, b)[g + 1] : 0u;
+                hi[b] = b < C ? cl.map_shared_rank(tile.n, b)[g + 1] : 0u;
             }
 #pragma unroll
             for (int b = 0; b < kMaxCluster; b++)
@@ -347,8 +347,8 @@ __device__ void run_steps(const BatchArgs &a, const BatchRun &R, cg::cluster_gro
                 unsigned glo[kMaxCluster], ghi[kMaxCluster];
 #pragma unroll
                 for (int b = 0; b < kMaxCluster; b++) {
-                    glo[b] = b < C ? cl.map_shared_rank(tile.lo, b)[jg] : 0u;
-                    ghi[b] = b < C ? cl.map_shared_rank(tile.hi, b)[jg] : 0u;
+                    glo[b] = b < C ? cl.map_shared_rank(tile.w, b)[jg] : 0u;
+                    ghi[b] = b < C ? cl.map_shared_rank(tile.n, b)[jg] : 0u;
                 }
 #pragma unroll
                 for (int b = 0; b < kMaxCluster; b++)
@@ -497,8 +497,8 @@ __device__ void run_steps(const BatchArgs &a, const BatchRun &R, cg::cluster_gro
                 }
             }
             for (int j = tid; j < ng + 2; j += bs) {
-                tile.lo[j] = 0u;
-                tile.hi[j] = 0u;
+                tile.w[j] = 0u;
+                tile.n[j] = 0u;
             }
         }
         __syncthreads();                          // sE and the tile complete
@@ -517,10 +517,8 @@ __global__ void __launch_bounds__(512, MINB) pic_batch_kernel(BatchArgs a) {
     __shared__ __align__(16) float shf[32 * 2 * PIC_NMODES];
     cg::cluster_group cl = cg::this_cluster();
     const int ngm = a.ng_max;
-    Tile tile;
-    tile.lo = reinterpret_cast<unsigned *>(smem_raw);
-    tile.hi = tile.lo + ngm + kTilePad;
-    float *sE = reinterpret_cast<float *>(tile.hi + ngm + kTilePad);
+    Tile tile = make_tile(smem_raw, ngm + kTilePad, false);
+    float *sE = reinterpret_cast<float *>(tile.n + ngm + kTilePad);
     for (;;) {
         if (cl.block_rank() == 0 && threadIdx.x == 0) ex.ticket = (int)atomicAdd(a.next, 1u);
         cl.sync();

@@ -110,6 +110,7 @@ __device__ __forceinline__ double cluster_total(cg::cluster_group &cl, const dou
 
 // The part of a block's shared memory that block 0 reads for the diagnostics.
 struct ClusterDiag {
+    double fe[kClusterSolveThreads / 32];   // field energy sums of the warps
     double kv[2];                 // the block's share of the push sums
     double diag[kDiagFields];     // slice diagnostics
     unsigned long long cq;        // slice sum of rho_q
@@ -143,24 +144,20 @@ __device__ __forceinline__ void push_sums_share(const SolveArgs &a, int C, int r
 __device__ void cluster_finish(const SolveArgs &a, cg::cluster_group &cl, ClusterDiag &cd,
                                const double (&kv)[2], const NodeDiag &d, double charge,
                                unsigned long long q, long long step) {
-    __shared__ __align__(16) double shd[32];
+    __shared__ __align__(16) double shd[8];
     __shared__ __align__(16) float shf[2 * PIC_NMODES][32];       // [value][warp]
     __shared__ __align__(16) unsigned long long cqw[32];
     const int C = (int)cl.num_blocks(), r = (int)cl.block_rank();
     const int t = threadIdx.x, lane = t & 31, w = t >> 5, nw = blockDim.x >> 5;
-    // The block's sums of the field energy (float64), the mode sums (float32)
-    // and the integer charge with one barrier: warp sums by shuffles (the 16
-    // mode sums by recursive halving), then warp 0 across the warps -- the
-    // field energy by the predicated float64 tree, each mode sum by one lane
-    // in warp order.
-    double fe = d.fe;
+    // The warps' sums of the field energy (float64, published: block 0 adds them
+    // in node order, below) and the block's sums of the mode sums (float32) and
+    // the integer charge, with one barrier: warp sums by shuffles (the 16 mode
+    // sums by recursive halving), then warp 0 across the warps, each mode sum by
+    // one lane in warp order.
+    const double fe = warp_sum_f64(d.fe);
     unsigned long long cqb = q;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const double u = __shfl_down_sync(kFull, fe, o);
-        if (lane < o) fe += u;
-        cqb += __shfl_down_sync(kFull, cqb, o);
-    }
+    for (int o = 16; o > 0; o >>= 1) cqb += __shfl_down_sync(kFull, cqb, o);
     float md[2 * PIC_NMODES];
 #pragma unroll
     for (int m = 0; m < PIC_NMODES; m++) { md[2 * m] = d.re[m]; md[2 * m + 1] = d.im[m]; }
@@ -168,18 +165,11 @@ __device__ void cluster_finish(const SolveArgs &a, cg::cluster_group &cl, Cluste
     const float msum = warp_sum16_halving(md, lane);   // value lane/2 in lanes 2i, 2i+1
     if ((lane & 1) == 0) shf[lane >> 1][w] = msum;
     if (lane == 0) {
-        shd[w] = fe;
+        cd.fe[w] = fe;
         cqw[w] = cqb;
     }
     __syncthreads();
     if (w == 0) {
-        double sf = lane < nw ? shd[lane] : 0.0;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            if (o >= nw) continue;                // warp-uniform
-            const double u = __shfl_down_sync(kFull, sf, o);
-            if (lane < o) sf += u;
-        }
         if (lane < 2 * PIC_NMODES) {
             float sm = 0.0f;
             for (int j = 0; j < nw; j++) sm += shf[lane][j];
@@ -191,7 +181,7 @@ __device__ void cluster_finish(const SolveArgs &a, cg::cluster_group &cl, Cluste
             cd.cq = sc;
             cd.kv[0] = kv[0];
             cd.kv[1] = kv[1];
-            cd.diag[kDiagFE] = sf;
+            cd.diag[kDiagFE] = 0.0;
             cd.diag[kDiagKE] = 0.0;
             cd.diag[kDiagMom] = 0.0;
             cd.diag[kDiagCharge] = charge;
@@ -202,7 +192,9 @@ __device__ void cluster_finish(const SolveArgs &a, cg::cluster_group &cl, Cluste
         __shared__ double tot[kDiagFields + 2];
         __shared__ unsigned long long tot_cq;
         cluster_diag_sums<kMaxSolveCluster>(cl, cd, tot, &tot_cq);
-        __syncthreads();
+        // the warps' field energies in node order (C nw <= 32 nw threads)
+        const double fes = t < C * nw ? cl.map_shared_rank(&cd, t / nw)->fe[t % nw] : 0.0;
+        const double fe_total = chunk_sum_f64(fes, C * nw, shd);
         const long long n = a.npartials > 0 ? step + 1 : step;
         pic_diag_row *row = &a.hist[n % a.hist_len];
         if (t == 0) {
@@ -216,7 +208,7 @@ __device__ void cluster_finish(const SolveArgs &a, cg::cluster_group &cl, Cluste
             row->step = n;
             row->kinetic = qnan;
             row->momentum = qnan;
-            row->field = 0.5 * a.dx * tot[kDiagFE];
+            row->field = 0.5 * a.dx * fe_total;
             row->charge = tot[kDiagCharge];
             row->charge_q = (long long)tot_cq;
         }
@@ -261,7 +253,7 @@ __global__ void __launch_bounds__(kClusterSolveThreads) pic_solve_cluster_kernel
     const int ng = a.ng, t = threadIdx.x;
     const long long step = *a.dstep;
     const i128 ntot = whole_density<MODE>(a);
-    const int per = (ng + C - 1) / C;
+    const int per = (int)blockDim.x;              // whole warps of nodes
     const int b0 = r * per;
     const int b1 = min(ng, b0 + per);
     const int g = b0 + t;
@@ -507,7 +499,9 @@ SolveKernel pick_solve(int mode, int solver) {
 
 // Cluster shape of the solves: C = ceil(NG / per_block) blocks (at most 16),
 // ceil(NG / C) nodes each, rounded up to whole warps.  The exact solve takes
-// up to 256 nodes per block, the CG 32 (both are float64-bound on GB300).
+// up to 256 nodes per block, the CG 32 (both are float64-bound on GB300).  The
+// exact solve's blocks take as many nodes as they have threads, so that every
+// warp holds 32 nodes from a multiple of 32 on.
 void solve_cluster_shape(int ng, int per_block, int *C, int *threads) {
     int c = (ng + per_block - 1) / per_block;
     c = c < 1 ? 1 : (c > kMaxSolveCluster ? kMaxSolveCluster : c);

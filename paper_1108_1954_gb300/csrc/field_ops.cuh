@@ -122,6 +122,40 @@ __device__ __forceinline__ float warp_sum16_halving(const float (&v)[16], int la
     return h1 + __shfl_xor_sync(kFull, h1, 1);
 }
 
+// Sum of a float64 value over a warp, in lane 0 (predicated adds, see
+// block_sum_f64k).
+__device__ __forceinline__ double warp_sum_f64(double v) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const double u = __shfl_down_sync(kFull, v, o);
+        if (lane < o) v += u;
+    }
+    return v;
+}
+
+// Field energy from the sums of 32 consecutive nodes each, of which thread c <
+// 256 holds number c (0 beyond the last): the one order in which the cluster
+// solve and the many-step launch add them, so that a run gives the same value
+// either way.  In thread 0; slot: 8 values; the whole block calls.
+__device__ __forceinline__ double chunk_sum_f64(double v, int chunks, double *slot) {
+    const int w = threadIdx.x >> 5, nw = (chunks + 31) >> 5;
+    if (w < nw) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            if (o >= chunks) continue;        // uniform: zeros only
+            const double u = __shfl_down_sync(kFull, v, o);
+            if ((threadIdx.x & 31) < o) v += u;
+        }
+        if ((threadIdx.x & 31) == 0) slot[w] = v;
+    }
+    __syncthreads();
+    double s = 0.0;
+    if (threadIdx.x == 0)
+        for (int i = 0; i < nw; i++) s += slot[i];
+    return s;
+}
+
 // Sums of K float64 values per thread over a block (warp trees, then warp 0
 // over the warp sums), valid in lane 0 of warp 0.  The adds run in the
 // predicated lanes only (31 lane-adds per warp and value instead of 160):

@@ -3,6 +3,7 @@
 // (batch.cu), so that a run gives bit-identical particles in either.
 //   locate         cell of a position by the fixed-point recipe
 //   fixed_weight   the right node's share trunc(f * 2^24)
+//   Tile           a block's private density in shared memory, and the deposits
 //   push_particle  gather (Sec. 2.3), kick (Eq. 3), drift (Eq. 2), wrap
 #pragma once
 
@@ -132,19 +133,102 @@ __device__ __forceinline__ void push_particle_ngp(float &u, float &v, const floa
     kick_drift_wrap(u, v, ep, c, ke, mom);
 }
 
-// Shared-memory density tiles.  GB300 has no single-instruction 64-bit
-// integer add on shared memory (it runs as a compare-and-swap loop, which
-// serialises badly when the lanes of a warp hit one node), so a tile keeps
-// each node's 64-bit sum as two 32-bit words: a 32-bit fetch-add on the low
-// word, and +1 on the high word from the one add that wraps it.  The tile is
-// ghost-padded: index j is node (j-1) mod NG, j = 0..NG+1.
-struct Tile {
-    unsigned *lo, *hi;      // 32-bit halves of the node sums
+// Shared-memory density tiles.  GB300 has no single-instruction 64-bit integer
+// add on shared memory (it is a compare-and-swap loop), so sums are kept in 32
+// bits by fetch-adds, and the one add that wraps a word counts a carry.
+//
+// Node tiles (the combining variants MATCH, QUAD, PAIR, and the batched kernel): per ghost-padded node j
+// = 0..NG+1 (node j - 1 mod NG) the low word w and the carries n of its sum; a
+// run of particles adds its left and its right weights.
+//
+// Cell tiles (kDepositCells: ATOMIC in the single run): a particle in the cell between nodes j - 1 and j (j =
+// 0..NG, locate) gives its left node 2^24 - W and its right node W, so per cell
+// the number of particles n and the sum w of W are kept, and the nodes formed
+// when the tile is read.  An add of the constant 1 that returns nothing is
+// counted over the lanes of a warp by the hardware: lanes on one word cost no
+// more than one lane, where other adds take a clock per lane.  Measured, clocks
+// per warp of particles on one SM (4 of them the loop's random numbers):
+//   distinct cells in the warp      1     2     4     8    16   many
+//   two fetch-adds per particle  63.0  36.2  22.2  14.5  10.1   9.1
+//   count and fetch-add          32.8  19.3  12.5   8.6   6.8   6.8
+// Runs add more than 1 at a time and gain nothing from it (QUAD 0.188 ms a push
+// of 2^26 particles with cell tiles, 0.184 with node tiles; PAIR8 takes 48
+// registers instead of 40), so they keep node tiles.
+// Carries of one cell number at most n / 256, so while a tile takes fewer than
+// 2^20 particles both fit the count's word: count below, carries from bit 20
+// (cinc = 2^20, c = n).  A tile of more has words of its own for the carries
+// (cinc = 1).
+//
+// The nearest-grid-point shape only counts, in n[j] for the node j - 1.
+template <int VARIANT>
+struct CellTile {
+    static constexpr bool value = VARIANT == kDepositCells;
 };
 
+struct Tile {
+    unsigned *w, *n, *c;    // low words; carries (node tiles) or counts; carries (cell tiles)
+    unsigned cinc;          // one carry
+    unsigned k;             // cell j's word is j << k (2^k copies of the tile, steps.cu)
+};
+
+constexpr int kCountBits = 20;
+// The most particles of a tile whose carries share the counts' words.
+constexpr long long kPackedCount = (1ll << kCountBits) - 1;
+
+// A tile of `words` words per array at mem; 8 or (wide) 12 bytes per word.
+__device__ __forceinline__ Tile make_tile(unsigned char *mem, int words, bool wide) {
+    Tile t;
+    t.w = reinterpret_cast<unsigned *>(mem);
+    t.n = t.w + words;
+    t.c = wide ? t.n + words : t.n;
+    t.cinc = wide ? 1u : 1u << kCountBits;
+    t.k = 0u;
+    return t;
+}
+
+// A node tile: val to node j.
 __device__ __forceinline__ void tile_add(const Tile &t, unsigned j, unsigned val) {
-    const unsigned old = atomicAdd(&t.lo[j], val);
-    if (old + val < old) atomicAdd(&t.hi[j], 1u);
+    const unsigned old = atomicAdd(&t.w[j], val);
+    if (old + val < old) atomicAdd(&t.n[j], 1u);
+}
+
+// A cell tile: one particle of right weight W in cell j.
+__device__ __forceinline__ void tile_add_one(const Tile &t, unsigned j, unsigned W) {
+    atomicAdd(&t.n[j << t.k], 1u);
+    const unsigned old = atomicAdd(&t.w[j << t.k], W);
+    if (old + W < old) atomicAdd(&t.c[j << t.k], t.cinc);
+}
+
+// A cell's count and sum of W from its three words (the carry word is the count
+// word unless wide).
+struct CellSum {
+    unsigned n;
+    u64 W;
+};
+__device__ __forceinline__ CellSum cell_sum(unsigned w, unsigned n, unsigned c, bool wide) {
+    CellSum s;
+    s.n = wide ? n : n & ((1u << kCountBits) - 1u);
+    s.W = ((u64)(wide ? c : n >> kCountBits) << 32) | w;
+    return s;
+}
+
+// (one copy)
+__device__ __forceinline__ CellSum tile_cell(const Tile &t, int j) {
+    return cell_sum(t.w[j], t.n[j], t.c[j], t.cinc == 1u);
+}
+
+// The tile's share of ghost-padded node j = 0..NG+1.
+template <int VARIANT>
+__device__ __forceinline__ u64 tile_node(const Tile &t, int j, int ng) {
+    if (VARIANT == kDepositNgp) return (u64)t.n[j] << kFixBits;
+    if (!CellTile<VARIANT>::value) return ((u64)t.n[j] << 32) | (u64)t.w[j];
+    u64 v = 0ull;
+    if (j <= ng) {
+        const CellSum s = tile_cell(t, j);
+        v = ((u64)s.n << kFixBits) - s.W;
+    }
+    if (j >= 1) v += tile_cell(t, j - 1).W;
+    return v;
 }
 
 // Deposit one particle (all 32 lanes of the warp call this together for the
@@ -156,16 +240,16 @@ __device__ __forceinline__ void deposit_one(const Tile &t, float x, bool valid,
         const unsigned j = locate_ngp(x);
         const bool ok = valid && j - 1u <= (unsigned)c.ng;
         if (valid && !ok) atomicOr(err, kErrPosition);
-        if (ok) tile_add(t, j, kFixOne);
+        if (ok) atomicAdd(&t.n[j << t.k], 1u);
         return;
     }
     const Loc l = locate(x);
     const bool ok = valid && l.j <= (unsigned)c.ng;
     if (valid && !ok) atomicOr(err, kErrPosition);
     const unsigned W = ok ? fixed_weight(l.f) : 0u;
-    if (VARIANT == PIC_DEPOSIT_ATOMIC || VARIANT == PIC_DEPOSIT_QUAD ||
-        VARIANT == PIC_DEPOSIT_PAIR || VARIANT == PIC_DEPOSIT_QUAD8 ||
-        VARIANT == PIC_DEPOSIT_PAIR8) {
+    if (CellTile<VARIANT>::value) {
+        if (ok) tile_add_one(t, l.j, W);
+    } else if (VARIANT != PIC_DEPOSIT_MATCH) {
         if (ok) {
             tile_add(t, l.j, kFixOne - W);
             tile_add(t, l.j + 1, W);
@@ -183,30 +267,57 @@ __device__ __forceinline__ void deposit_one(const Tile &t, float x, bool valid,
     }
 }
 
+// Deposit the first m of W particles into a cell tile: the fetch-adds in flight
+// together, their carries after them.
+template <int W>
+__device__ __forceinline__ void deposit_cells(const Tile &t, const float (&xs)[W], int m,
+                                              const PushConsts &c, unsigned *err) {
+    unsigned j[W], w[W], old[W];
+    bool ok[W], bad = false;
+#pragma unroll
+    for (int k = 0; k < W; k++) {
+        const Loc l = locate(xs[k]);
+        ok[k] = k < m && l.j <= (unsigned)c.ng;
+        bad |= k < m && !ok[k];
+        j[k] = l.j << t.k;
+        w[k] = fixed_weight(l.f);
+    }
+#pragma unroll
+    for (int k = 0; k < W; k++) {
+        old[k] = 0u;
+        if (ok[k]) {
+            atomicAdd(&t.n[j[k]], 1u);
+            old[k] = atomicAdd(&t.w[j[k]], w[k]);
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < W; k++)
+        if (ok[k] && old[k] + w[k] < old[k]) atomicAdd(&t.c[j[k]], t.cinc);
+    if (bad) atomicOr(err, kErrPosition);
+}
+
+// The first m of W particles of the nearest-grid-point shape.
+template <int W>
+__device__ __forceinline__ void deposit_ngp(const Tile &t, const float (&xs)[W], int m,
+                                            const PushConsts &c, unsigned *err) {
+    bool bad = false;
+#pragma unroll
+    for (int k = 0; k < W; k++) {
+        const unsigned j = locate_ngp(xs[k]);
+        const bool ok = k < m && j - 1u <= (unsigned)c.ng;
+        bad |= k < m && !ok;
+        if (ok) atomicAdd(&t.n[j << t.k], 1u);
+    }
+    if (bad) atomicOr(err, kErrPosition);
+}
+
 // Deposit a thread's W consecutive particles (W = 4: a float4 group; W = 8:
 // the 32-byte groups of the QUAD8 / PAIR8 variants), valid per lane.
 template <int VARIANT, int W>
 __device__ __forceinline__ void deposit_group(const Tile &t, const float (&xs)[W], bool valid,
                                               const PushConsts &c, unsigned *err, int lane) {
     if (VARIANT == kDepositNgp) {
-        // runs of equal cell among the W particles: count * 2^24 per run
-        unsigned key = 0xffffffffu, cnt = 0;
-        bool bad = false;
-#pragma unroll
-        for (int k = 0; k < W; k++) {
-            const unsigned j = locate_ngp(xs[k]);
-            const bool ok = valid && j - 1u <= (unsigned)c.ng;
-            bad |= valid && !ok;
-            if (ok && j == key) {
-                cnt += kFixOne;
-            } else if (ok) {
-                if (key != 0xffffffffu) tile_add(t, key, cnt);
-                key = j;
-                cnt = kFixOne;
-            }
-        }
-        if (key != 0xffffffffu) tile_add(t, key, cnt);
-        if (bad) atomicOr(err, kErrPosition);
+        deposit_ngp<W>(t, xs, valid ? W : 0, c, err);
     } else if (VARIANT == PIC_DEPOSIT_PAIR || VARIANT == PIC_DEPOSIT_PAIR8) {
         // two open runs (key, left, right); a third key closes run a
         unsigned ka = 0xffffffffu, la = 0, ra = 0, kb = 0xffffffffu, lb = 0, rb = 0;
@@ -266,6 +377,8 @@ __device__ __forceinline__ void deposit_group(const Tile &t, const float (&xs)[W
             tile_add(t, key + 1, right);
         }
         if (bad) atomicOr(err, kErrPosition);
+    } else if (CellTile<VARIANT>::value) {
+        deposit_cells<W>(t, xs, valid ? W : 0, c, err);
     } else {
 #pragma unroll
         for (int k = 0; k < W; k++) deposit_one<VARIANT>(t, xs[k], valid, c, err, lane);

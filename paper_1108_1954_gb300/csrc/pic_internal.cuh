@@ -33,6 +33,7 @@ enum : uint32_t {
     kErrPosition = 1u,   // a position outside [0, L) or not finite
     kErrSortKey = 4u,    // a sort key outside the grid
     kErrInput = 8u,      // an uploaded position outside [0, L) (pic_init, pic_set_state)
+    kErrWait = 16u,      // a grid barrier's wait ran out (steps.cu)
 };
 
 // Float32 constants of the push, formed once on the host.  In the float32
@@ -54,6 +55,7 @@ struct PushArgs {
     unsigned long long *rho_q;    // fixed-point density accumulator [NG]
     double *partials;             // per-block [sum v_old v_new, sum v_new]
     unsigned int *err;            // device error word
+    bool wide;                    // a block may take 2^20 particles or more
     PushConsts c;
 };
 
@@ -115,6 +117,38 @@ struct SolveArgs {
 __host__ __device__ constexpr int density_bits(int mode) {
     return mode == PIC_FP32_FIXED ? kFixBits : mode == PIC_FP32_ATOMIC ? 30 : 53;
 }
+
+// Many steps of a fixed-point run in one cooperative launch (steps.cu).
+struct StepsArgs {
+    float *x, *v;                 // N each, 16-byte aligned
+    long long n;
+    float *E32;                   // field of the first step in, of the last one out
+    double *E64, *phi, *rho;      // of the last step, out
+    unsigned long long *rho_q_last; // idem
+    unsigned long long *acc;      // [kStepsSlots][NG] density sums, 0 between launches
+    double *partials;             // [kStepsSlots][kStepsMaxGrid] float4: per-block push sums as
+                                  // float32 pairs (sum v_old v_new and its rest, sum v_new, rest)
+    unsigned *err;
+    unsigned *sync;               // [4], 16-byte aligned: arrivals of the workers, steps
+                                  // done by each diagnostics block; never reset ...
+    unsigned base[3];             // ... their values before this launch
+    int log_copies;               // copies of a block's tile (set by the launcher)
+    pic_diag_row *hist;
+    int hist_len;
+    long long step0;              // steps taken before this launch
+    long long *dstep;             // device step counter
+    int steps;
+    PushConsts c;
+    long long weight_total;       // N 2^24
+    double k_rho, k_e, k_phi, k_mode, dx, mass;   // as SolveArgs
+};
+constexpr int kStepsMaxGrid = 256;
+constexpr int kStepsSlots = 6;     // accumulators in turn
+constexpr int kStepsDiag = 2;      // blocks of the grid without particles
+constexpr int kStepsMaxCells = 4096;
+constexpr int64_t kStepsMaxParticles = 12500000;   // 100 MB of state
+cudaError_t steps_prepare(int variant, int ng, int block, int *per_sm);
+cudaError_t launch_steps(StepsArgs a, int variant, int grid, int block, cudaStream_t s);
 
 // Counting sort by cell.
 template <typename T>
@@ -181,6 +215,8 @@ int make_load_args(const pic_loading *ld, long long n, double length, float *x, 
 // Internal kernel choice of the fused push for the nearest-grid-point shape
 // (not a public deposit variant: PIC_SHAPE_NGP selects it).
 constexpr int kDepositNgp = 15;
+// The single run's kernels' form of PIC_DEPOSIT_ATOMIC (cell tiles).
+constexpr int kDepositCells = 14;
 
 // Phase-space histogram (phase.cu).
 constexpr int kPhaseMaxBins = 16384;
@@ -228,9 +264,10 @@ cudaError_t launch_push_f32_atomic(PushArgsF32Atomic a, int grid, int block, boo
                                    cudaStream_t s);
 cudaError_t launch_push_f64(const PushArgs64 &a, int grid, int block,
                             bool push, cudaStream_t s);
-size_t push_smem_bytes(int mode, int ng);
+size_t push_smem_bytes(int mode, int ng, bool wide);
+bool push_wide_tile(long long n, int sms);
 cudaError_t push_prepare_attributes(int mode);
-int push_max_blocks_per_sm(int mode, int variant, int unroll, int block, int ng);
+int push_max_blocks_per_sm(int mode, int variant, int unroll, int block, int ng, bool wide);
 
 cudaError_t launch_solve(const SolveArgs &a, cudaStream_t s);
 cudaError_t solve_prepare_attributes();

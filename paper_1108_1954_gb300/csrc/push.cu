@@ -33,18 +33,15 @@ namespace pic {
 namespace {
 
 
-// Add the block's tile to the global density and clear it (ghost nodes
-// folded onto their periodic images).
+// Add the block's tile to the global density (ghost nodes folded onto their
+// periodic images).
+template <int VARIANT>
 __device__ __forceinline__ void flush_tile(const Tile &t, u64 *rho_q, int ng) {
     __syncthreads();
     for (int j = threadIdx.x; j <= ng + 1; j += blockDim.x) {
-        const u64 w = ((u64)t.hi[j] << 32) | (u64)t.lo[j];
-        if (w == 0) continue;
-        t.lo[j] = 0u;
-        t.hi[j] = 0u;
-        atomicAdd(&rho_q[j == 0 ? ng - 1 : (j == ng + 1 ? 0 : j - 1)], w);
+        const u64 v = tile_node<VARIANT>(t, j, ng);
+        if (v) atomicAdd(&rho_q[j == 0 ? ng - 1 : (j == ng + 1 ? 0 : j - 1)], v);
     }
-    __syncthreads();
 }
 
 // Sum two per-thread values over the block in a fixed order; thread 0 gets it.
@@ -76,14 +73,13 @@ __global__ void __launch_bounds__(512) pic_push_fixed_kernel(PushArgs a) {
     __shared__ double red[64];
     const PushConsts c = a.c;
     const int ng = c.ng;
-    Tile tile;                                                       // 8 (ng + 2) B
-    tile.lo = reinterpret_cast<unsigned *>(smem_raw);
-    tile.hi = tile.lo + ng + 2;
-    float *sE = reinterpret_cast<float *>(smem_raw + 8 * (ng + 2));  // ng + 2
+    float *sE = reinterpret_cast<float *>(smem_raw);                 // ng + 2
+    const Tile tile = make_tile(smem_raw + 4 * (ng + 2), ng + 2, a.wide);
     const int tid = threadIdx.x, bs = blockDim.x, lane = tid & 31;
     for (int j = tid; j < ng + 2; j += bs) {
-        tile.lo[j] = 0u;
-        tile.hi[j] = 0u;
+        tile.w[j] = 0u;
+        tile.n[j] = 0u;
+        tile.c[j] = 0u;
         if (PUSH) sE[j] = a.E32[j == 0 ? ng - 1 : (j == ng + 1 ? 0 : j - 1)];
     }
     __syncthreads();
@@ -162,7 +158,7 @@ __global__ void __launch_bounds__(512) pic_push_fixed_kernel(PushArgs a) {
             a.partials[2 * blockIdx.x + 1] = dmom;
         }
     }
-    flush_tile(tile, a.rho_q, ng);
+    flush_tile<VARIANT>(tile, a.rho_q, ng);
 }
 
 // ---- the fused push on 8-particle groups (QUAD8, PAIR8) ---------------------
@@ -178,14 +174,13 @@ __global__ void __launch_bounds__(512) pic_push_oct_kernel(PushArgs a) {
     __shared__ double red[64];
     const PushConsts c = a.c;
     const int ng = c.ng;
-    Tile tile;                                                       // 8 (ng + 2) B
-    tile.lo = reinterpret_cast<unsigned *>(smem_raw);
-    tile.hi = tile.lo + ng + 2;
-    float *sE = reinterpret_cast<float *>(smem_raw + 8 * (ng + 2));  // ng + 2
+    float *sE = reinterpret_cast<float *>(smem_raw);                 // ng + 2
+    const Tile tile = make_tile(smem_raw + 4 * (ng + 2), ng + 2, a.wide);
     const int tid = threadIdx.x, bs = blockDim.x, lane = tid & 31;
     for (int j = tid; j < ng + 2; j += bs) {
-        tile.lo[j] = 0u;
-        tile.hi[j] = 0u;
+        tile.w[j] = 0u;
+        tile.n[j] = 0u;
+        tile.c[j] = 0u;
         if (PUSH) sE[j] = a.E32[j == 0 ? ng - 1 : (j == ng + 1 ? 0 : j - 1)];
     }
     __syncthreads();
@@ -241,7 +236,7 @@ __global__ void __launch_bounds__(512) pic_push_oct_kernel(PushArgs a) {
             a.partials[2 * blockIdx.x + 1] = dmom;
         }
     }
-    flush_tile(tile, a.rho_q, ng);
+    flush_tile<VARIANT>(tile, a.rho_q, ng);
 }
 
 // ---- float32 push with float32 atomic deposit (precision study) -------------
@@ -623,7 +618,7 @@ FixedKernel pick_fixed(int variant, bool push, int unroll) {
     switch (variant) {
         case PIC_DEPOSIT_QUAD8: return pick_oct<PIC_DEPOSIT_QUAD8>(push, unroll);
         case PIC_DEPOSIT_PAIR8: return pick_oct<PIC_DEPOSIT_PAIR8>(push, unroll);
-        case PIC_DEPOSIT_ATOMIC: return pick_unroll<PIC_DEPOSIT_ATOMIC>(push, unroll);
+        case PIC_DEPOSIT_ATOMIC: return pick_unroll<kDepositCells>(push, unroll);
         case PIC_DEPOSIT_MATCH: return pick_unroll<PIC_DEPOSIT_MATCH>(push, unroll);
         case PIC_DEPOSIT_QUAD: return pick_unroll<PIC_DEPOSIT_QUAD>(push, unroll);
         case PIC_DEPOSIT_PAIR: return pick_unroll<PIC_DEPOSIT_PAIR>(push, unroll);
@@ -634,19 +629,21 @@ FixedKernel pick_fixed(int variant, bool push, int unroll) {
 
 }  // namespace
 
-size_t push_smem_bytes(int mode, int ng) {
-    if (mode == PIC_FP64) return (size_t)(ng + 1) * 16 + (size_t)(ng + 2) * 12;
-    if (mode == PIC_FP32_ATOMIC) return (size_t)(ng + 2) * 4 * (1 + atomic_copies(ng));
-    return (size_t)(ng + 2) * 12;
+bool push_wide_tile(long long n, int sms) {
+    // a grid smaller than the SMs takes one group of particles per thread
+    return n / sms > kPackedCount - 512 * 32;
 }
 
-// Shared memory of a fused fixed-point push launch.
-size_t fixed_smem_bytes(int ng) { return push_smem_bytes(PIC_FP32_FIXED, ng); }
+size_t push_smem_bytes(int mode, int ng, bool wide) {
+    if (mode == PIC_FP64) return (size_t)(ng + 1) * 16 + (size_t)(ng + 2) * 12;
+    if (mode == PIC_FP32_ATOMIC) return (size_t)(ng + 2) * 4 * (1 + atomic_copies(ng));
+    return (size_t)(ng + 2) * (wide ? 16 : 12);
+}
 
 cudaError_t push_prepare_attributes(int mode) {
     // the atomic tile is largest where 32 copies just fit
     const int bytes = mode == PIC_FP32_ATOMIC ? (int)(2 * kAtomicTile)
-                                              : (int)push_smem_bytes(mode, PIC_NCELL_MAX);
+                                              : (int)push_smem_bytes(mode, PIC_NCELL_MAX, true);
     cudaError_t e = cudaSuccess;
     if (mode == PIC_FP32_FIXED) {
         const int unrolls[3] = {1, 2, 4};
@@ -658,8 +655,7 @@ cudaError_t push_prepare_attributes(int mode) {
                 for (int u : unrolls) {
                     FixedKernel k = pick_fixed(v, p != 0, u);
                     if (!k) continue;
-                    e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)fixed_smem_bytes(PIC_NCELL_MAX));
+                    e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
                     if (e != cudaSuccess) return e;
                 }
     } else if (mode == PIC_FP32_ATOMIC) {
@@ -678,14 +674,14 @@ cudaError_t push_prepare_attributes(int mode) {
     return e;
 }
 
-int push_max_blocks_per_sm(int mode, int variant, int unroll, int block, int ng) {
+int push_max_blocks_per_sm(int mode, int variant, int unroll, int block, int ng, bool wide) {
     int nb = 0;
-    const size_t smem = push_smem_bytes(mode, ng);
+    const size_t smem = push_smem_bytes(mode, ng, wide);
     cudaError_t e;
     if (mode == PIC_FP32_FIXED) {
         FixedKernel k = pick_fixed(variant, true, unroll);
         if (!k) return 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, block, fixed_smem_bytes(ng));
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, block, smem);
     }
     else if (mode == PIC_FP32_ATOMIC)
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, &pic_push_f32atomic_kernel<true>, block, smem);
@@ -702,13 +698,13 @@ cudaError_t launch_push_fixed(const PushArgs &a, int grid, int block, int varian
                               int unroll, bool push, cudaStream_t s) {
     FixedKernel k = pick_fixed(variant, push, unroll);
     if (!k) return cudaErrorInvalidValue;
-    k<<<grid, block, fixed_smem_bytes(a.c.ng), s>>>(a);
+    k<<<grid, block, push_smem_bytes(PIC_FP32_FIXED, a.c.ng, a.wide), s>>>(a);
     return cudaGetLastError();
 }
 
 cudaError_t launch_push_f32_atomic(PushArgsF32Atomic a, int grid, int block, bool push,
                                    cudaStream_t s) {
-    const size_t smem = push_smem_bytes(PIC_FP32_ATOMIC, a.c.ng);
+    const size_t smem = push_smem_bytes(PIC_FP32_ATOMIC, a.c.ng, false);
     a.copies = atomic_copies(a.c.ng);
     if (push) pic_push_f32atomic_kernel<true><<<grid, block, smem, s>>>(a);
     else pic_push_f32atomic_kernel<false><<<grid, block, smem, s>>>(a);
@@ -717,7 +713,7 @@ cudaError_t launch_push_f32_atomic(PushArgsF32Atomic a, int grid, int block, boo
 
 cudaError_t launch_push_f64(const PushArgs64 &a, int grid, int block, bool push,
                             cudaStream_t s) {
-    const size_t smem = push_smem_bytes(PIC_FP64, a.ng);
+    const size_t smem = push_smem_bytes(PIC_FP64, a.ng, false);
     if (push) pic_push_f64_kernel<true><<<grid, block, smem, s>>>(a);
     else pic_push_f64_kernel<false><<<grid, block, smem, s>>>(a);
     return cudaGetLastError();

@@ -1,0 +1,558 @@
+// steps.cu -- many steps of one fixed-point run in one cooperative launch.
+//
+// A step of a small or middling run is two short kernels whose times are
+// latency, not work: on GB300 the push of 5e4 particles takes 5.6 us and the
+// cluster solve 7.6 us, of which the arithmetic is well under a microsecond.
+// Here the blocks (one per SM) stay resident for all the steps of a call and a
+// step has one grid barrier:
+//
+//   push     each block pushes its contiguous part of the particles and deposits
+//            into its own tile (the device code of push.cu).  A thread keeps its
+//            first kResident groups of 4 particles in registers from step to step;
+//   flush    the tile is added to one of kStepsSlots global accumulators, used
+//            in turn;
+//   barrier  arrivals counted in global memory, a bounded spin;
+//   solve    every block reads the NG sums and solves for the whole grid itself,
+//            into its shared copy of E.  No second barrier: the solve is exact
+//            integer arithmetic, so all blocks get the same bits, and with one
+//            node per thread its cost hardly depends on NG.
+//
+// Two more blocks have no particles.  They take the steps in turn and, while
+// the workers go on, compute a step's diagnostics (float64 work that would hold
+// the workers up: at 64 clocks a dependent float64 add and 840 a square root,
+// a step's take 8 to 16 thousand clocks, up to twice a worker's step), then
+// clear the step's accumulator and give it back; a worker waits only if the
+// diagnostics fall kStepsSlots - 1 steps behind.  After the last step they
+// write E, Phi, rho and the consumed sums.
+//
+// What a step costs (GB300, us): launches of push and solve before, and here
+//   2e4 particles, 64 cells, one step a call   16.4   11.0
+//   5e4, 100 cells                             14.0    4.3
+//   5e5, 300 cells                             18.5    7.1
+//   1e6, 1024 cells, sorted every 20           22.5   10.7
+//   3e6, 777 cells, NGP, sorted every 10       27.4   17.8
+//   4.2e6, 2048 cells, sorted every 20         31.0   22.8
+//   1e6, 4096 cells                            24.8   17.5
+//   1.2e7, 2048 cells, sorted every 20         52.9   44.6
+// of which, at 5e4 (clocks): push 2300, sums 380, flush 1040, barrier 2400 (the
+// adds' release and a poll, each a trip to L2), solve 1300 (900 the sums' way
+// from L2), E 510.  Where the state no longer fits L2 (1.7e7 particles: 82
+// against 72 us) or a thread has 8 nodes (1e6 particles on 6000 cells: 31
+// against 28) the two launches are faster and are kept (set_steps_shape).
+//
+// The solve in 64 bits.  R_g = N 2^24 - NG rho_q[g] and its prefix sums P_g are
+// below N NG 2^24 in magnitude, so they fit 64 bits for N NG <= 2^38 (the
+// launch's runs stay below 2^36); sum_g P_g = sum_k (NG - k) R_k and M_g = NG P_g - sum P
+// take 128.  The sum over the lanes of a warp is taken in three 26-bit pieces by
+// redux.sync.  E_g = k_e (M_g + M_{g-1}) must be the same float32 as the
+// float64 chain of field.cu gives, (float)(k_e (double)(M_g + M_{g-1})):
+// GB300's float64 pipe takes 2 lanes per clock, so the product is formed from
+// the two 64-bit mantissas in integers and rounded once; within 2^14 units of
+// 2^-64 of a rounding boundary of float32, where the chain's own three
+// roundings (each 2^-53) could matter, the chain itself is evaluated.
+//
+// Every wait has a limit (kSpinLimit polls, some seconds), after which the block
+// sets kErrWait and all blocks return.
+#include "field_ops.cuh"
+#include "particle_ops.cuh"
+
+namespace pic {
+namespace {
+
+constexpr int kResident = 2;               // groups of 4 particles a thread keeps
+constexpr unsigned kSpinLimit = 1u << 23;  // polls of one grid barrier
+
+// The launch's counters, never reset: arrivals of the workers, and the steps
+// that each diagnostics block is done with (StepsArgs::sync, on 16 bytes).
+__device__ __forceinline__ uint4 ld_acquire(const unsigned *p) {
+    uint4 v;
+    asm volatile("ld.acquire.gpu.global.v4.u32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
+    return v;
+}
+
+__device__ __forceinline__ void red_release(unsigned *p) {
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(p) : "memory");
+}
+
+// Steps t <= last with t mod kStepsDiag == d.
+__device__ __forceinline__ unsigned steps_of(int last, int d) {
+    return last < d ? 0u : (unsigned)((last - d) / kStepsDiag + 1);
+}
+
+// Waits until all workers have arrived for step s, and, for a worker, until the
+// slot of step s + 1 has been given back by the diagnostics of step s + 1 -
+// kStepsSlots.  All threads of the block; false when the wait ran out.
+__device__ __forceinline__ bool wait_step(const StepsArgs &a, int s, int workers, bool worker,
+                                          int *dead) {
+    static_assert(kStepsDiag == 2, "two counters");
+    if (threadIdx.x == 0) {
+        const unsigned target = a.base[0] + (unsigned)workers * (unsigned)(s + 1);
+        const unsigned d0 = a.base[1] + steps_of(s + 1 - kStepsSlots, 0);
+        const unsigned d1 = a.base[2] + steps_of(s + 1 - kStepsSlots, 1);
+        unsigned polls = 0;
+        for (;;) {
+            const uint4 v = ld_acquire(a.sync);
+            if ((int)(v.x - target) >= 0 && (!worker || ((int)(v.y - d0) >= 0 && (int)(v.z - d1) >= 0)))
+                break;
+            if (++polls >= kSpinLimit) {
+                atomicOr(a.err, kErrWait);
+                *dead = 1;
+                break;
+            }
+        }
+    }
+    __syncthreads();
+    return *dead == 0;
+}
+
+// Sum over a warp of 78-bit signed integers, in every lane.
+__device__ __forceinline__ i128 warp_sum_i78(i128 v) {
+    const unsigned m = (1u << 26) - 1u;
+    const unsigned s0 = __reduce_add_sync(kFull, (unsigned)v & m);
+    const unsigned s1 = __reduce_add_sync(kFull, (unsigned)(v >> 26) & m);
+    const int s2 = __reduce_add_sync(kFull, (int)(v >> 52));
+    return (i128)s0 + ((i128)s1 << 26) + ((i128)s2 << 52);
+}
+
+__device__ __forceinline__ long long warp_sum_i64(long long v) {
+    const unsigned m = (1u << 26) - 1u;
+    const unsigned s0 = __reduce_add_sync(kFull, (unsigned)v & m);
+    const unsigned s1 = __reduce_add_sync(kFull, (unsigned)(v >> 26) & m);
+    const int s2 = __reduce_add_sync(kFull, (int)(v >> 52));
+    return (long long)s0 + ((long long)s1 << 26) + ((long long)s2 << 52);
+}
+
+// (float)(k (double)m), k > 0 (see above): kmant the mantissa of k with its top
+// bit set, k = kmant 2^(kexp - 63).
+__device__ __forceinline__ float scaled_f32(i128 m, double k, unsigned long long kmant, int kexp) {
+    const bool neg = m < 0;
+    const unsigned __int128 a = neg ? (unsigned __int128)(-m) : (unsigned __int128)m;
+    const unsigned long long hi = (unsigned long long)(a >> 64), lo = (unsigned long long)a;
+    if ((hi | lo) == 0ull) return 0.0f;
+    const int n = hi ? __clzll((long long)hi) : 64 + __clzll((long long)lo);
+    const unsigned long long A = n >= 64 ? lo << (n - 64) : n ? (hi << n) | (lo >> (64 - n)) : hi;
+    unsigned long long p = __umul64hi(A, kmant);
+    const int norm = __clzll((long long)p);              // 0 or 1
+    p <<= norm;
+    // a k = p 2^(65 - n - norm + kexp), p in [2^63, 2^64)
+    const int e = 63 + 65 - n - norm + kexp + 127;        // biased float32 exponent
+    const unsigned long long rem = p & ((1ull << 40) - 1ull), half = 1ull << 39;
+    const unsigned long long dist = rem > half ? rem - half : half - rem;
+    if (dist <= (1ull << 14) || e < 1 || e > 253) return (float)(k * i128_to_f64(m));
+    const unsigned mant = (unsigned)(p >> 40) + (rem > half ? 1u : 0u);   // 2^24: exponent + 1
+    const unsigned bits = ((unsigned)e << 23) + (mant - (1u << 23));
+    return __uint_as_float(bits | (neg ? 0x80000000u : 0u));
+}
+
+// s + e = a + b exactly (Knuth's two-sum); pairs (h, l) added over a warp
+__device__ __forceinline__ void add_pair(float &h, float &l, float h2, float l2) {
+    const float s = __fadd_rn(h, h2);
+    const float t = __fsub_rn(s, h);
+    const float e = __fadd_rn(__fsub_rn(h, __fsub_rn(s, t)), __fsub_rn(h2, t));
+    l = __fadd_rn(__fadd_rn(l, l2), e);
+    h = s;
+}
+
+// (x, y) and (z, w) summed over the first n lanes of a warp (the others hold
+// zeros), in lane 0.
+__device__ __forceinline__ void warp_sum_pairs(float4 &p, int n) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        if (o >= n) continue;                         // uniform
+        add_pair(p.x, p.y, __shfl_down_sync(kFull, p.x, o), __shfl_down_sync(kFull, p.y, o));
+        add_pair(p.z, p.w, __shfl_down_sync(kFull, p.z, o), __shfl_down_sync(kFull, p.w, o));
+    }
+}
+
+// Push and deposit the first m of a group's 4 particles.
+template <bool NGP>
+__device__ __forceinline__ void step4(float4 &x, float4 &v, int m, const float *sE, const Tile &t,
+                                      const PushConsts &c, unsigned *err, float &ke, float &mom) {
+    float xs[4] = {x.x, x.y, x.z, x.w}, vs[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+        if (k >= m) continue;
+        if (NGP) push_particle_ngp(xs[k], vs[k], sE, c, ke, mom);
+        else push_particle(xs[k], vs[k], sE, c, ke, mom);
+    }
+    if (NGP) deposit_ngp<4>(t, xs, m, c, err);
+    else deposit_cells<4>(t, xs, m, c, err);
+    x = make_float4(xs[0], xs[1], xs[2], xs[3]);
+    v = make_float4(vs[0], vs[1], vs[2], vs[3]);
+}
+
+// The field of the whole grid, in thread t's K nodes K t ... K t + K - 1.
+template <int K>
+struct NodeSolve {
+    long long R[K], P[K];         // R_g and its inclusive prefix sums
+    unsigned long long q[K];      // the consumed sums
+    long long SR;                 // sum of R (threads of warp 0)
+    i128 SP;                      // sum of P
+    i128 m[K];                    // M_g + M_{g-1}
+};
+
+template <int K>
+__device__ __forceinline__ void solve_nodes(NodeSolve<K> &s, const StepsArgs &a,
+                                            const unsigned long long *acc, int ng,
+                                            long long *wr, unsigned long long *ws) {
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5, nw = blockDim.x >> 5;
+    const int g0 = t * K;
+    long long r = 0;
+    i128 sp = 0;
+#pragma unroll
+    for (int j = 0; j < K; j++) s.q[j] = g0 + j < ng ? __ldcg(acc + g0 + j) : 0ull;
+#pragma unroll
+    for (int j = 0; j < K; j++) {
+        const bool in = g0 + j < ng;
+        s.R[j] = in ? a.weight_total - (long long)ng * (long long)s.q[j] : 0ll;
+        r += s.R[j];
+        sp += (i128)s.R[j] * (i128)(ng - (g0 + j));
+    }
+    long long inc = r;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const long long u = __shfl_up_sync(kFull, inc, o);
+        if (lane >= o) inc += u;
+    }
+    const i128 wsp = warp_sum_i78(sp);
+    if (lane == 31) {
+        wr[w] = inc;
+        ws[w] = (unsigned long long)wsp;
+        ws[32 + w] = (unsigned long long)(wsp >> 64);
+    }
+    __syncthreads();
+    const long long wv = lane < nw ? wr[lane] : 0ll;
+    const long long before = warp_sum_i64(w == 0 || lane < w ? wv : 0ll);
+    s.SR = before;                // in warp 0: the total
+    const i128 wq = lane < nw ? (i128)(((unsigned __int128)ws[32 + lane] << 64) | ws[lane]) : (i128)0;
+    s.SP = warp_sum_i78(wq);
+    long long run = (w == 0 ? 0ll : before) + inc - r;
+#pragma unroll
+    for (int j = 0; j < K; j++) {
+        // M_g = NG P_g - SP, M_{g-1} the same with P_{g-1}, M_{-1} = M_{NG-1}
+        const i128 prev = g0 + j == 0 ? (i128)s.SR : (i128)run;
+        run += s.R[j];
+        s.P[j] = run;
+        s.m[j] = (i128)ng * ((i128)run + prev) - 2 * s.SP;
+    }
+}
+
+template <int VARIANT, int K>
+__global__ void __launch_bounds__(1024, 1) pic_steps_kernel(StepsArgs a) {
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    __shared__ long long wr[32];
+    __shared__ unsigned long long ws[64];
+    __shared__ float4 kvs[32];                    // per warp: (ke, ke low, mom, mom low)
+    __shared__ int dead;
+    constexpr bool kNgp = VARIANT == kDepositNgp;
+    const PushConsts c = a.c;
+    const int ng = c.ng;
+    const int words = (ng + 2) << a.log_copies, K_ = 1 << a.log_copies;
+    const Tile tile0 = make_tile(smem_raw, words, false);
+    float *sE = reinterpret_cast<float *>(tile0.n + words);
+    Tile tile = tile0;                            // this lane's copy
+    tile.w += threadIdx.x & (K_ - 1);
+    tile.n += threadIdx.x & (K_ - 1);
+    tile.c = tile.n;
+    tile.k = a.log_copies;
+    const int tid = threadIdx.x, bs = blockDim.x, lane = tid & 31, w = tid >> 5, nw = bs >> 5;
+    const int workers = (int)gridDim.x - kStepsDiag, b = blockIdx.x;
+    const bool diag = b >= workers;
+    const unsigned long long kmant =
+        (((unsigned long long)__double_as_longlong(a.k_e) & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull) << 11;
+    const int kexp = (int)((unsigned long long)__double_as_longlong(a.k_e) >> 52) - 1023;
+    if (tid == 0) dead = 0;
+    auto clear_tile = [&] {
+        for (int j = tid; j < words; j += bs) {
+            if (!kNgp) tile0.w[j] = 0u;
+            tile0.n[j] = 0u;
+        }
+    };
+    clear_tile();
+    for (int j = tid; j < ng + 2; j += bs) sE[j] = a.E32[j == 0 ? ng - 1 : (j == ng + 1 ? 0 : j - 1)];
+    // this block's groups [q0, q1); the thread's groups q0 + tid + i bs, the first
+    // kResident of them in registers.  The run's last group may hold fewer than 4
+    // particles; its other words are padding of the arrays.
+    const int n4 = (int)((a.n + 3) >> 2), left = (int)(a.n - 4ll * (n4 - 1));    // n4 <= 2^30
+    const int q0 = diag ? 0 : (int)((long long)n4 * b / workers);
+    const int q1 = diag ? 0 : (int)((long long)n4 * (b + 1) / workers);
+    const unsigned h0 = diag ? (unsigned)(a.step0 % a.hist_len) : 0u;     // history slot of the first step
+    auto members = [&](int q) { return q >= q1 ? 0 : q == n4 - 1 ? left : 4; };
+    float4 *x4 = reinterpret_cast<float4 *>(a.x);
+    float4 *v4 = reinterpret_cast<float4 *>(a.v);
+    const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
+    float4 rx[kResident], rv[kResident];
+#pragma unroll
+    for (int i = 0; i < kResident; i++) {
+        const int q = q0 + tid + i * bs;
+        rx[i] = q < q1 ? __ldcg(x4 + q) : zero4;
+        rv[i] = q < q1 ? __ldcg(v4 + q) : zero4;
+    }
+    __syncthreads();
+    for (int s = diag ? b - workers : 0; s < a.steps; s += diag ? kStepsDiag : 1) {
+        const bool last = s == a.steps - 1;
+        const int slot = s % kStepsSlots;
+        unsigned long long *acc = a.acc + (size_t)slot * ng;
+        float4 *kv = reinterpret_cast<float4 *>(a.partials) + (size_t)slot * kStepsMaxGrid;
+        if (!diag) {
+            float ke = 0.0f, mom = 0.0f;
+            const int qs = q0 + tid + kResident * bs;
+            float4 cx = qs < q1 ? __ldcg(x4 + qs) : zero4, cv = qs < q1 ? __ldcg(v4 + qs) : zero4;
+#pragma unroll
+            for (int i = 0; i < kResident; i++) {
+                const int m = members(q0 + tid + i * bs);
+                if (m) step4<kNgp>(rx[i], rv[i], m, sE, tile, c, a.err, ke, mom);
+            }
+            for (int q = qs; q < q1; q += bs) {
+                float4 xx = cx, vv = cv;
+                const int qn = q + bs;
+                cx = qn < q1 ? __ldcg(x4 + qn) : zero4;
+                cv = qn < q1 ? __ldcg(v4 + qn) : zero4;
+                step4<kNgp>(xx, vv, members(q), sE, tile, c, a.err, ke, mom);
+                __stcg(x4 + q, xx);
+                __stcg(v4 + q, vv);
+            }
+            float4 sums = make_float4(ke, 0.0f, mom, 0.0f);
+            warp_sum_pairs(sums, 32);
+            if (lane == 0) kvs[w] = sums;
+            __syncthreads();
+            if (w == nw - 1) {                        // the block's sums, still as pairs
+                float4 p = lane < nw ? kvs[lane] : zero4;
+                warp_sum_pairs(p, nw);
+                if (lane == 0) kv[b] = p;
+            }
+            // node g: the left weights of cell g + 1 and the right ones of cell g
+            // (held by the lane below: a warp's first lane only reads them), node
+            // NG - 1 also cell 0's left ones, node 0 cell NG's right ones (NGP: the
+            // counts of word g + 1; word NG + 1 is node 0, word 0 stays empty)
+            auto cell = [&](int j) {
+                u64 n = 0ull, W = 0ull;
+#pragma unroll 4
+                for (int i = 0; i < K_; i++) {
+                    const int at = (j << a.log_copies) + ((i + lane) & (K_ - 1));
+                    if (kNgp) {
+                        n += tile0.n[at];
+                    } else {
+                        const CellSum cs = cell_sum(tile0.w[at], tile0.n[at], 0u, false);
+                        n += cs.n;
+                        W += cs.W;
+                    }
+                }
+                return ulonglong2{n, W};
+            };
+            constexpr int kPer = kNgp ? 32 : 31;                // nodes a warp
+            for (int g0 = kPer * w; g0 < ng; g0 += kPer * nw) {
+                const int g = kNgp ? g0 + lane : g0 + lane - 1;
+                const ulonglong2 own = g < ng ? cell(g + 1) : ulonglong2{0ull, 0ull};
+                u64 val = (own.x << kFixBits) - own.y;
+                if (!kNgp) val += __shfl_up_sync(kFull, own.y, 1);
+                if (g == (kNgp ? 0 : ng - 1)) {
+                    const ulonglong2 e = cell(kNgp ? ng + 1 : 0);
+                    val += (e.x << kFixBits) - e.y;
+                }
+                if (!kNgp && g == 0) val += cell(ng).y;
+                if ((kNgp || lane > 0) && g < ng && val) atomicAdd(&acc[g], val);
+            }
+            __syncthreads();
+            if (tid == 0) red_release(a.sync);        // the whole block's adds: after the barrier
+            if (last) break;                          // a diagnostics block writes the results
+            clear_tile();                             // while the others arrive
+        }
+        if (!wait_step(a, s, workers, !diag, &dead)) return;
+        NodeSolve<K> ns;
+        solve_nodes<K>(ns, a, acc, ng, wr, ws);
+        if (!diag) {
+#pragma unroll
+            for (int j = 0; j < K; j++) {
+                const int g = tid * K + j;
+                if (g >= ng) break;
+                const float e = scaled_f32(ns.m[j], a.k_e, kmant, kexp);
+                sE[g + 1] = e;
+                if (g == ng - 1) sE[0] = e;
+                if (g == 0) sE[ng + 1] = e;
+            }
+            __syncthreads();
+            continue;
+        }
+        // ---- a diagnostics block: those of the step, beside the workers' next ones
+        __shared__ float shf[2 * PIC_NMODES][32];
+        __shared__ double shd[8], fchunk[256], tot[2];
+        double *fe = reinterpret_cast<double *>(smem_raw);      // [ng], in the tile
+        NodeDiag d;
+        node_diag_reset(d);
+#pragma unroll
+        for (int j = 0; j < K; j++) {
+            const int g = tid * K + j;
+            if (g >= ng) break;
+            const double E = a.k_e * i128_to_f64(ns.m[j]);
+            d.fe = 0.0;
+            node_diag(d, g, ng, E, (float)E);
+            fe[g] = d.fe;
+            if (last) {
+                a.E64[g] = E;
+                a.E32[g] = (float)E;
+                a.rho[g] = a.k_rho * i128_to_f64((i128)ns.R[j]);
+                a.rho_q_last[g] = ns.q[j];
+            }
+        }
+        float md[2 * PIC_NMODES];
+#pragma unroll
+        for (int m = 0; m < PIC_NMODES; m++) { md[2 * m] = d.re[m]; md[2 * m + 1] = d.im[m]; }
+        static_assert(2 * PIC_NMODES == 16, "16 mode sums per warp");
+        const int used = (ng + 32 * K - 1) / (32 * K);          // warps with nodes
+        if (w < used) {
+            const float msum = warp_sum16_halving(md, lane);
+            if ((lane & 1) == 0) shf[lane >> 1][w] = msum;
+        }
+        __syncthreads();
+        const int chunks = (ng + 31) >> 5;
+        for (int i = w; i < chunks; i += nw) {                  // field energy of 32 nodes
+            const int g = 32 * i + lane;
+            const double sum = warp_sum_f64(g < ng ? fe[g] : 0.0);
+            if (lane == 0) fchunk[i] = sum;
+        }
+        if (w == nw - 1) {                                      // the push's sums
+            float4 p[kStepsMaxGrid / 32];                       // all loads in flight
+#pragma unroll
+            for (int i = 0; i < kStepsMaxGrid / 32; i++)
+                p[i] = 32 * i + lane < workers ? __ldcg(kv + 32 * i + lane) : zero4;
+#pragma unroll
+            for (int i = 1; i < kStepsMaxGrid / 32; i++) {
+                add_pair(p[0].x, p[0].y, p[i].x, p[i].y);
+                add_pair(p[0].z, p[0].w, p[i].z, p[i].w);
+            }
+            warp_sum_pairs(p[0], 32);
+            if (lane == 0) {
+                tot[0] = (double)p[0].x + (double)p[0].y;
+                tot[1] = (double)p[0].z + (double)p[0].w;
+            }
+        }
+        __syncthreads();
+        const double fe_total = chunk_sum_f64(tid < chunks ? fchunk[tid] : 0.0, chunks, shd);
+        if (w == 0) {
+            const long long n = a.step0 + s + 1;
+            pic_diag_row *prev = &a.hist[(h0 + s) % a.hist_len], *row = &a.hist[(h0 + s + 1) % a.hist_len];
+            // one value per lane: kinetic energy and momentum of the row before,
+            // field energy and charge of this one
+            const double coef = lane == 0 ? 0.5 * a.mass : lane == 1 ? a.mass
+                                : lane == 2 ? 0.5 * a.dx : a.dx * a.k_rho;
+            const double fe0 = __shfl_sync(kFull, fe_total, 0);
+            const double val = coef * (lane < 2 ? tot[lane] : lane == 2 ? fe0 : (double)ns.SR);
+            if (lane < 4) *(lane == 0 ? &prev->kinetic : lane == 1 ? &prev->momentum
+                            : lane == 2 ? &row->field : &row->charge) = val;
+            if (lane == 4) row->step = n;
+            // sum of rho_q: SR = NG (N 2^24 - it), 0 unless particles were lost
+            if (lane == 5) row->charge_q = ns.SR ? a.weight_total - ns.SR / ng : a.weight_total;
+            if (last && lane >= 6 && lane < 8)       // (otherwise the next step's, perhaps written already)
+                *(lane == 6 ? &row->kinetic : &row->momentum) = __longlong_as_double(0x7ff8000000000000ll);
+            if (last && lane == 8) *a.dstep = n;
+        } else if (w == 1) {
+            // mode sums: float32 over 8 warps, float64 over those
+            double sum = 0.0;
+            for (int i0 = 0; i0 < used; i0 += 8) {
+                float part = 0.0f;
+#pragma unroll
+                for (int i = 0; i < 8; i++)
+                    part += i0 + i < used ? shf[lane & 15][(i0 + i) & 31] : 0.0f;
+                sum += (double)part;
+            }
+            const double im = __shfl_down_sync(kFull, sum, 1);
+            if (lane < 2 * PIC_NMODES && !(lane & 1))
+                a.hist[(h0 + s + 1) % a.hist_len].mode[lane >> 1] =
+                    sqrt(sum * sum + im * im) * a.k_mode;
+        }
+        if (last) {
+            // Phi: sum_{k<g} M_k = NG (g P_g - sum_{j<=g} j R_j) - g SP
+            __shared__ unsigned long long scan64[4 * 32];
+            i128 jr = 0;
+#pragma unroll
+            for (int j = 0; j < K; j++) jr += (i128)ns.R[j] * (i128)(tid * K + j);
+            i128 run = block_inclusive_scan2_i128(jr, 0, scan64).a - jr;
+#pragma unroll
+            for (int j = 0; j < K; j++) {
+                const int g = tid * K + j;
+                if (g >= ng) break;
+                run += (i128)ns.R[j] * (i128)g;
+                const i128 sumM = (i128)ng * ((i128)g * (i128)ns.P[j] - run) - (i128)g * ns.SP;
+                a.phi[g] = a.k_phi * i128_to_f64(sumM);
+            }
+        }
+        // give the slot back, once no worker reads it any more
+        if (!last && !wait_step(a, s + 1, workers, false, &dead)) return;
+        for (int g = tid; g < ng; g += bs) acc[g] = 0ull;
+        __syncthreads();
+        if (tid == 0) red_release(a.sync + 1 + (b - workers));
+    }
+    if (!diag) {
+#pragma unroll
+        for (int i = 0; i < kResident; i++) {
+            const int q = q0 + tid + i * bs;
+            if (q >= q1) break;
+            __stcg(x4 + q, rx[i]);
+            __stcg(v4 + q, rv[i]);
+        }
+    }
+}
+
+using StepsKernel = void (*)(StepsArgs);
+
+template <int V>
+StepsKernel pick_nodes(int per_thread) {
+    switch (per_thread) {
+        case 1: return &pic_steps_kernel<V, 1>;
+        case 2: return &pic_steps_kernel<V, 2>;
+        case 4: return &pic_steps_kernel<V, 4>;
+        default: return nullptr;
+    }
+}
+
+StepsKernel pick_steps(int variant, int ng, int block) {
+    int k = 1;
+    while (k * block < ng) k *= 2;
+    return variant == kDepositNgp ? pick_nodes<kDepositNgp>(k) : pick_nodes<kDepositCells>(k);
+}
+
+// Copies of a block's tile, lanes alternating between them: lanes of one cell
+// then meet on a word half as often, for twice the words to clear and read.
+// Two pay in blocks of 1024 threads (1e6 Maxwellian particles on 1024 cells:
+// 10.7 against 11.2 us a step, 4e6 on 2048: 22.8 against 24.5; four 10.8 and
+// 23.2), not in small ones (4.3 us either way), and not where the deposit only
+// counts (NGP).
+int log_copies(int variant, int block) { return variant != kDepositNgp && block == 1024 ? 1 : 0; }
+
+size_t steps_smem(int variant, int ng, int block) {
+    return (size_t)(ng + 2) * (4 + (8 << log_copies(variant, block)));
+}
+
+}  // namespace
+
+cudaError_t steps_prepare(int variant, int ng, int block, int *per_sm) {
+    *per_sm = 0;
+    StepsKernel k = pick_steps(variant, ng, block);
+    if (!k) return cudaSuccess;
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)steps_smem(variant, kStepsMaxCells, block));
+    if (e != cudaSuccess) return e;
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, k, block,
+                                                         steps_smem(variant, ng, block));
+}
+
+cudaError_t launch_steps(StepsArgs a, int variant, int grid, int block, cudaStream_t s) {
+    StepsKernel k = pick_steps(variant, a.c.ng, block);
+    if (!k) return cudaErrorInvalidValue;
+    a.log_copies = log_copies(variant, block);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)block);
+    cfg.dynamicSmemBytes = steps_smem(variant, a.c.ng, block);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k, a);
+}
+
+}  // namespace pic

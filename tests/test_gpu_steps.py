@@ -1,0 +1,128 @@
+"""The many-step launch (a run whose launch shape is left open) against the
+push and solve kernels, which an explicit shape selects: the particles, the
+density, E and the histories' exact entries bit for bit, whatever the sizes
+and however the steps are split into calls."""
+import math
+
+import numpy as np
+import pytest
+
+import paper_1108_1954_gb300 as pic
+import torch  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+L = 4.0 * math.pi
+
+
+def state(n, seed):
+    rng = np.random.default_rng(seed)
+    x = rng.uniform(0.0, L, n).astype(np.float32)
+    x[x >= np.float32(L)] = 0.0
+    if n > 2:
+        x[0], x[1] = 0.0, np.nextafter(np.float32(L), np.float32(0))
+    return x, rng.normal(0.0, 0.4, n).astype(np.float32)
+
+
+def pair(n, ng, **kw):
+    a = pic.Run(pic.Params(npart=n, ncell=ng, length=L, **kw), device="cuda:0")
+    # an explicit block size (NGP: its one variant) keeps the two kernels
+    b = pic.Run(pic.Params(npart=n, ncell=ng, length=L, block_size=256, **kw), device="cuda:0")
+    x, v = state(n, 7 * n + ng)
+    a.init(x, v)
+    b.init(x, v)
+    return a, b
+
+
+def assert_same(a, b, n, ng):
+    for p, q in zip(a.get_cells(), b.get_cells()):
+        assert np.array_equal(p, q)
+    f, g = a.get_field(), b.get_field()
+    for k in ("rho_q", "E", "rho", "phi"):
+        assert np.array_equal(f[k], g[k]), k
+    d, e = a.diagnostics(), b.diagnostics()
+    for k in ("step", "charge_q", "charge", "field"):
+        assert np.array_equal(d[k], e[k]), k
+    assert np.isnan(d["kinetic"][-1]) and np.isnan(d["momentum"][-1])
+    # the kinetic sums and the modes add float32 terms in another order
+    np.testing.assert_allclose(d["kinetic"][:-1], e["kinetic"][:-1], rtol=1e-5)
+    scale = L / n * np.abs(a.get_cells()[1]).sum()
+    assert np.abs(d["momentum"][:-1] - e["momentum"][:-1]).max(initial=0.0) <= 1e-5 * scale
+    tol = 2.0 / ng * np.abs(f["E"]).sum() * 64 * 2.0 ** -24 + 1e-12
+    assert np.abs(d["mode"][-1] - e["mode"][-1]).max() <= tol
+
+
+@pytest.mark.parametrize("n", [1, 2, 3, 4, 5, 1023, 1024, 1025, 131072, 131073, 700001])
+@pytest.mark.parametrize("ng", [1, 2, 31, 32, 33, 256, 257, 512, 513, 1025, 4096])
+def test_steps_equal_the_two_kernels(n, ng):
+    a, b = pair(n, ng)
+    for k in (1, 6, 2, 9):             # more steps than accumulators, and fewer
+        a.step_n(k)
+        b.step_n(k)
+    assert_same(a, b, n, ng)
+
+
+@pytest.mark.parametrize("n,ng,S", [(20000, 64, 1), (50021, 100, 3), (300007, 777, 7), (1000003, 2048, 20)])
+@pytest.mark.parametrize("shape", [pic.PIC_SHAPE_CIC, pic.PIC_SHAPE_NGP])
+def test_sorted_steps_equal_the_two_kernels(n, ng, S, shape):
+    a, b = pair(n, ng, sort_interval=S, shape=shape)
+    for k in (5, 1, 20, 3):
+        a.step_n(k)
+        b.step_n(k)
+    assert_same(a, b, n, ng)
+    a.push(), a.solve_field(), b.push(), b.solve_field()      # single phases in between
+    a.step_n(4), b.step_n(4)
+    assert_same(a, b, n, ng)
+
+
+@pytest.mark.parametrize("n,ng", [(12500000, 512), (12500001, 512), (100003, 4096), (100003, 4097)])
+def test_steps_at_the_limits_of_the_launch(n, ng):
+    a, b = pair(n, ng)
+    a.step_n(3), b.step_n(3)
+    assert_same(a, b, n, ng)
+
+
+def test_crowded_cells_and_a_steep_field():
+    # all particles in one cell, and a plasma whose field spans its largest range
+    n, ng = 262147, 1000
+    for kw in (dict(), dict(rho_ion=1e-30), dict(rho_ion=1e25)):   # E32 near its smallest and largest
+        a, b = pair(n, ng, **kw)
+        x = np.full(n, 0.3, np.float32)
+        for r in (a, b):
+            r.set_state(x, np.zeros(n, np.float32), 5)
+            r.step_n(3)
+        for p, q in zip(a.get_cells(), b.get_cells()):
+            assert np.array_equal(p, q, equal_nan=True)
+        assert np.array_equal(a.get_field()["E"], b.get_field()["E"], equal_nan=True)
+
+
+@pytest.mark.parametrize("bad", [float("nan"), float("-inf")])
+def test_a_bad_particle_is_flagged_and_the_run_restarts(bad):
+    a, b = pair(5001, 64)
+    x, v = state(5001, 1)
+    w = v.copy()
+    w[5000] = bad
+    a.set_state(x, w, 0)
+    a.step_n(3)
+    with pytest.raises(pic.PicError) as e:
+        a.sync()
+    assert e.value.code == pic.PIC_EDEVICE
+    for r in (a, b):
+        r.set_state(x, v, 0)
+        r.step_n(7)
+    assert_same(a, b, 5001, 64)
+
+
+def test_a_captured_step_replays():
+    a, b = pair(20000, 64)
+    s = torch.cuda.Stream()
+    c = pic.Run(pic.Params(npart=20000, ncell=64, length=L), device="cuda:0", stream=s)
+    c.init(*state(20000, 7 * 20000 + 64))
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s):
+        c.step_n(1)
+    for _ in range(4):
+        g.replay()
+    torch.cuda.synchronize()
+    b.step_n(4)
+    for p, q in zip(c.get_cells(), b.get_cells()):
+        assert np.array_equal(p, q)
