@@ -65,9 +65,10 @@ extern "C" {
 #define PIC_EINVAL (-1)   /* bad argument or parameter                       */
 #define PIC_ENOMEM (-2)   /* workspace too small / pool budget exhausted      */
 #define PIC_ECUDA (-3)    /* a CUDA runtime call failed                       */
-#define PIC_ETIMEOUT (-4) /* a grid barrier of a pic_step_n launch ran out of
-                             its limit (some seconds); the run needs
-                             pic_init or pic_set_state                       */
+#define PIC_ETIMEOUT (-4) /* a wait between the blocks of a kernel ran out of
+                             its limit (pic_step_n's many-step launch, the
+                             CG solver); the run needs pic_init or
+                             pic_set_state                                   */
 #define PIC_EDEVICE (-5)  /* a kernel flagged bad particle data                */
 #define PIC_ESTATE (-6)   /* call out of order (e.g. push before init)         */
 

@@ -93,21 +93,6 @@ __device__ __forceinline__ i128 take_density(const SolveArgs &a, int g) {
 
 // ---- the cluster solves' common parts -------------------------------------
 
-// Sum over the cluster of the blocks' values *pub (each published by its
-// block before the caller's cluster barrier), the same fixed tree over the
-// ranks in every warp of every block: every thread gets the same total.
-__device__ __forceinline__ double cluster_total(cg::cluster_group &cl, const double *pub, int C) {
-    const int lane = threadIdx.x & 31;
-    double p = lane < C ? *cl.map_shared_rank(pub, lane) : 0.0;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        if (o >= C) continue;                 // uniform: only the levels C needs
-        const double u = __shfl_down_sync(kFull, p, o);
-        if (lane < o) p += u;
-    }
-    return __shfl_sync(kFull, p, 0);
-}
-
 // The part of a block's shared memory that block 0 reads for the diagnostics.
 struct ClusterDiag {
     double fe[kClusterSolveThreads / 32];   // field energy sums of the warps
@@ -332,43 +317,133 @@ __global__ void __launch_bounds__(kClusterSolveThreads) pic_solve_cluster_kernel
 // the converged x is the periodic solution in the Phi_0 = 0 gauge.
 //
 // The nodes are split over the blocks of one cluster, one node per thread,
-// C = ceil(NG/32) <= 16 blocks: float64 issue (2 lanes per clock per SM on
-// GB300) rather than threads bounds an iteration, so the nodes are spread
-// over as many SMs as a cluster holds.  Float64 throughout.  Per iteration two cluster-wide
-// sums (z.v and r.r): block sums, published in shared memory, then every
-// warp adds the C block sums in the same fixed tree, so every thread of every
-// block holds the same scalars.  The two neighbour values of v that A v needs
-// from other blocks are not exchanged after the update: each block publishes
-// its boundary v (before the update) and r (after it) with r.r, and the
-// neighbour forms beta v + r itself -- the same operation on the same numbers
-// as the owner.  So an iteration has two cluster barriers.  A published value
-// is read after the barrier that follows its write and rewritten only after
-// the next barrier, which every reader passes after reading it.  Divisions
-// are done by one lane per warp (float64 division is a long sequence).
+// C = ceil(NG/32) <= 16 blocks, float64 throughout.  An iteration is a chain of
+// dependent operations, and what bounds it is their latency: on GB300 a float64
+// add, multiply or FMA takes 64 clocks, a division 1465, a cluster barrier
+// about 400 and a read of another block's shared memory about 250.  So
+//   * the sums z.v and r.r are taken in integers (warp_sum_fixed): the products
+//     aligned to the warp's largest exponent and added by redux.sync, 200
+//     clocks against 530 for a shuffle tree of float64 adds; they are exact to
+//     2^-57 of the largest product, where the tree rounded each add;
+//   * every warp stores its sum into all blocks' shared memory itself (st.async,
+//     completing on a memory barrier there), so a sum over the cluster takes one
+//     crossing instead of a barrier and a read; every block adds the same
+//     integers, so all hold the same scalars;
+//   * the two neighbour values of v that A v needs from other blocks are not
+//     exchanged after the update: each block sends its boundary v (before the
+//     update) and r (after it) with its part of r.r, and the neighbour forms
+//     beta v + r itself, the same operation on the same numbers as the owner;
+//   * t = c / z.v and beta = d / c are products with reciprocals (recip64), of
+//     which 1/c is formed a whole half iteration before it is needed.
+// A solve of 150 iterations takes 304 us on 1024 nodes, 549 with cluster barriers,
+// float64 trees and divisions; an iteration's 520 instructions a warp, one
+// after the other at 7.4 clocks, are what bounds it now.
+// A block's barrier of one sum cannot complete again before the block has added
+// its own part of the next sum, which it sends only after reading the first, so
+// one buffer per sum is enough.  Every wait has a limit (kCgSpinLimit tries),
+// after which the block sets kErrWait and all blocks leave the loop.
+constexpr unsigned kCgSpinLimit = 1u << 20;    // tries of up to a microsecond
+
+constexpr int kCgParts = kMaxSolveCluster * kClusterSolveThreads / 32;    // warps of a cluster
+
 struct CgExchange {
-    double zv, rr;                // block sums
-    double v0, v1, r0, r1;        // v (before the update) and r (after) at the
-                                  // slice's first and last node
+    double part[2][kCgParts];     // every warp's sum of z.v and of r.r
+    double2 nbr[2];               // (v, r) at the left and the right neighbour's boundary
+    unsigned long long bar[2];    // memory barriers of z.v and of r.r
     double x0, x1;                // Phi at the slice's first and last node
     i128 sr;                      // slice sum of R
 };
 
-__device__ __forceinline__ double warp_div(double num, double den) {
-    double q = 0.0;
-    if ((threadIdx.x & 31) == 0) q = num / den;
-    return __shfl_sync(kFull, q, 0);
+__device__ __forceinline__ unsigned smem_addr(const void *p) {
+    return (unsigned)__cvta_generic_to_shared(p);
+}
+
+__device__ __forceinline__ unsigned peer_addr(const void *p, int rank) {
+    unsigned r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_addr(p)), "r"(rank));
+    return r;
+}
+
+// Into another block's shared memory (peer_addr), counted on its barrier; and
+// the bytes a barrier's phase waits for.  For the lanes with `on`, predicated:
+// a branch around them costs a divergent warp more than they do.
+__device__ __forceinline__ void send8(bool on, unsigned dst, double a, unsigned bar) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %3, 0;\n\t"
+                 "@p st.async.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];\n\t}"
+                 ::"r"(dst), "l"(__double_as_longlong(a)), "r"(bar), "r"((unsigned)on) : "memory");
+}
+
+__device__ __forceinline__ void send16(bool on, unsigned dst, double a, double b, unsigned bar) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %4, 0;\n\t"
+                 "@p st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.b64 [%0], {%1, %2}, [%3];\n\t}"
+                 ::"r"(dst), "l"(__double_as_longlong(a)), "l"(__double_as_longlong(b)), "r"(bar),
+                 "r"((unsigned)on) : "memory");
+}
+
+__device__ __forceinline__ void expect_bytes(bool on, const void *bar, unsigned bytes) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t"
+                 "@p mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n\t}"
+                 ::"r"(smem_addr(bar)), "r"(bytes), "r"((unsigned)on) : "memory");
+}
+
+__device__ __forceinline__ bool wait_phase(const void *bar, unsigned parity) {
+#pragma unroll 1
+    for (unsigned i = 0; i < kCgSpinLimit; i++) {
+        unsigned done;
+        asm volatile("{\n\t.reg .pred p;\n\t"
+                     "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2, 1000;\n\t"
+                     "selp.u32 %0, 1, 0, p;\n\t}"
+                     : "=r"(done) : "r"(smem_addr(bar)), "r"(parity) : "memory");
+        if (done) return true;
+    }
+    return false;
+}
+
+// Sum of float64 values over a warp, in every lane, as integers: 53-bit mantissas
+// with 5 bits below them, aligned to the largest exponent (|m| < 2^58), added
+// in pieces of 27, 27 and 10 bits.  The sum is exact to 2^-57 of the largest
+// value a lane, then rounded once.  (Subnormal values and results are 0.)
+__device__ __forceinline__ double warp_sum_fixed(double p) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(p);
+    const unsigned ex = (unsigned)(b >> 52) & 0x7ffu;
+    const unsigned emax = __reduce_max_sync(kFull, ex);
+    const unsigned long long mant = ((b & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull) << 5;
+    const unsigned sh = emax - ex;
+    long long m = sh < 64u && ex ? (long long)(mant >> sh) : 0ll;
+    m = (long long)b < 0 ? -m : m;
+    const unsigned k = (1u << 27) - 1u;
+    const unsigned s0 = __reduce_add_sync(kFull, (unsigned)m & k);
+    const unsigned s1 = __reduce_add_sync(kFull, (unsigned)(m >> 27) & k);
+    const int s2 = __reduce_add_sync(kFull, (int)(m >> 54));
+    const long long sum = (long long)s0 + ((long long)s1 << 27) + ((long long)s2 << 54);
+    // sum 2^(emax - 1080), by the exponent field
+    const unsigned long long d = (unsigned long long)__double_as_longlong((double)sum);
+    const int ed = (int)((d >> 52) & 0x7ffull) + (int)emax - 1080;
+    const unsigned long long v = (d & 0x800fffffffffffffull) | ((unsigned long long)(unsigned)ed << 52);
+    if (emax == 0x7ffu || ed > 2046) return __longlong_as_double(0x7ff8000000000000ll);
+    return sum == 0 || ed < 1 ? 0.0 : __longlong_as_double((long long)v);
+}
+
+// 1/x: the hardware's approximation y0 (at least 20 bits) and one step of the
+// cubic Newton iteration y0 (1 + e + e^2), e = 1 - x y0: e^3 is below 2^-60,
+// the result within two units of the last place.  Three dependent FMAs.
+__device__ __forceinline__ double recip64(double x) {
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = fma(-x, y, 1.0);
+    return fma(y, fma(e, e, e), y);
 }
 
 template <int MODE>
 __global__ void __launch_bounds__(kClusterSolveThreads) pic_solve_cg_kernel(SolveArgs a) {
     cg::cluster_group cl = cg::this_cluster();
     __shared__ double sv[kClusterSolveThreads + 2];   // v of the slice, ghost-padded
-    __shared__ CgExchange ex;
+    __shared__ __align__(16) CgExchange ex;
     __shared__ ClusterDiag cd;
-    __shared__ double slot[32];
     __shared__ i128 sh[96];
+    __shared__ double scal[2];                        // t and beta; NaN: stop
     const int C = (int)cl.num_blocks(), r = (int)cl.block_rank();
-    const int ng = a.ng, t = threadIdx.x;
+    const int ng = a.ng, t = threadIdx.x, lane = t & 31, w = t >> 5, nw = blockDim.x >> 5;
     const long long step = *a.dstep;
     const double dx = a.dx;
     const int per = (ng + C - 1) / C;
@@ -376,6 +451,10 @@ __global__ void __launch_bounds__(kClusterSolveThreads) pic_solve_cg_kernel(Solv
     const int cnt = min(ng, b0 + per) - b0;
     const int g = b0 + t;
     const bool mine = t < cnt;
+    if (t < 2) {
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&ex.bar[t])) : "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
     double kv[2];
     push_sums_share(a, C, r, kv);
     double rh = 0.0;
@@ -391,68 +470,91 @@ __global__ void __launch_bounds__(kClusterSolveThreads) pic_solve_cg_kernel(Solv
         block_sum3_i128(sr, z1, z2, sh);
         if (t == 0) ex.sr = sr;
     }
+    for (int i = t; i < kClusterSolveThreads + 2; i += blockDim.x) sv[i] = 0.0;
+    cl.sync();                                        // barriers ready in all blocks
+    // lane l of a warp sends the warp's sums to block l
+    const int to = lane < C ? lane : 0;
+    const unsigned dst[2] = {peer_addr(&ex.part[0][r * nw + w], to), peer_addr(&ex.part[1][r * nw + w], to)};
+    const unsigned bar[2] = {peer_addr(&ex.bar[0], to), peer_addr(&ex.bar[1], to)};
+    // the slice's first and last node send their (v, r) to the neighbour (a slice
+    // with neighbours on both sides has at least 17 nodes)
+    const bool first = t == 0 && r > 0, final = t == cnt - 1 && r < C - 1;
+    const int nb = first ? r - 1 : final ? r + 1 : 0;
+    const unsigned ndst = peer_addr(&ex.nbr[first ? 1 : 0], nb), nbar = peer_addr(&ex.bar[1], nb);
+    const unsigned zv_bytes = 8u * (unsigned)(C * nw);
+    const unsigned rr_bytes = zv_bytes + 16u * (unsigned)((r > 0 ? 1 : 0) + (r < C - 1 ? 1 : 0));
     double xg = 0.0;
     double rg = (mine && g >= 1) ? (-rh * dx) * dx : 0.0;
-    double vg = rg;
-    if (mine) sv[t + 1] = vg;
-    if (t == 0) ex.v0 = vg;
-    if (t == cnt - 1) ex.v1 = vg;
-    {
-        const double s = block_sum_f64(rg * rg, slot);
-        if (t == 0) ex.rr = s;
-    }
-    cl.sync();
-    double c = cluster_total(cl, &ex.rr, C);
-    // the neighbours' boundary v (v = r at the start)
-    if (t == 0 && r > 0) sv[0] = cl.map_shared_rank(&ex, r - 1)->v1;
-    if (t == cnt - 1 && r < C - 1) sv[cnt + 1] = cl.map_shared_rank(&ex, r + 1)->v0;
-    __syncthreads();
-    if (sqrt(c) > 1e-16 && ng > 1) {
-        for (int it = 0; it < a.cg_maxit; it++) {
-            double z = 0.0;
-            if (mine) {
-                const double vl = sv[t], vc = sv[t + 1], vr = sv[t + 2];
-                z = g == 0 ? vc : (g == ng - 1 ? vl - 2.0 * vc : (vl - 2.0 * vc) + vr);
+    double vg = 0.0;
+    bool dead = false;                                // a wait ran out
+    // Every warp takes the sums itself where a block has few (no block barrier
+    // between the sum and its use); where it has many, their float64 scalars
+    // would fill the pipe, and warp 0 hands them on.
+    const bool every = nw <= 4;
+    auto publish = [&](int which, double p) {
+        const double f = warp_sum_fixed(p);
+        send8(lane < C, dst[which], f, bar[which]);
+    };
+    auto total = [&](int which, unsigned parity) {
+        dead |= !wait_phase(&ex.bar[which], parity);
+        double v = lane < C * nw ? ex.part[which][lane] : 0.0;
+        for (int i = lane + 32; i < C * nw; i += 32) v += ex.part[which][i];
+        return warp_sum_fixed(v);
+    };
+    const double nan = __longlong_as_double(0x7ff8000000000000ll);
+    double c = 0.0, rc = 0.0, beta = 0.0;
+    for (int it = -1; it < a.cg_maxit; it++) {
+        if (it >= 0) {                                // (it = -1: r.r of the start)
+            const double vc = sv[t + 1];
+            double z = fma(-2.0, vc, sv[t]) + sv[t + 2];      // (Phi_NG = 0: the last ghost stays 0)
+            z = g == 0 ? vc : z;
+            z = mine ? z : 0.0;
+            publish(0, z * vg);
+            expect_bytes(t == 0, &ex.bar[0], zv_bytes);
+            double tk = 0.0;
+            if (every || w == 0) {
+                rc = recip64(c);                      // for beta, while the sums cross
+                const double zv = total(0, (unsigned)it & 1u);
+                tk = c * recip64(zv);
+                // stop where the step would divide by zero
+                tk = dead || zv == 0.0 ? nan : tk;
             }
-            {
-                const double s = block_sum_f64(z * vg, slot);
-                if (t == 0) ex.zv = s;
+            if (!every) {
+                if (t == 0) scal[0] = tk;
+                __syncthreads();
+                tk = scal[0];
             }
-            cl.sync();                                                // S1
-            const double dotzv = cluster_total(cl, &ex.zv, C);
-            if (!(dotzv != 0.0)) break;
-            const double tk = warp_div(c, dotzv);
-            if (!isfinite(tk)) break;
-            if (mine) {
-                xg = fma(tk, vg, xg);
-                rg = fma(-tk, z, rg);
-            }
-            if (t == 0) { ex.v0 = vg; ex.r0 = rg; }
-            if (t == cnt - 1) { ex.v1 = vg; ex.r1 = rg; }
-            {
-                const double s = block_sum_f64(rg * rg, slot);
-                if (t == 0) ex.rr = s;
-            }
-            cl.sync();                                                // S2
-            const double d = cluster_total(cl, &ex.rr, C);
-            if (!(d > 0.0)) break;
-            const double beta = warp_div(d, c);
-            if (mine) {
-                vg = fma(beta, vg, rg);
-                sv[t + 1] = vg;
-            }
-            if (t == 0 && r > 0) {
-                const CgExchange *pl = cl.map_shared_rank(&ex, r - 1);
-                sv[0] = fma(beta, pl->v1, pl->r1);
-            }
-            if (t == cnt - 1 && r < C - 1) {
-                const CgExchange *pr = cl.map_shared_rank(&ex, r + 1);
-                sv[cnt + 1] = fma(beta, pr->v0, pr->r0);
-            }
-            c = d;
-            __syncthreads();
+            if (!isfinite(tk)) break;                 // uniform over the cluster
+            xg = fma(tk, vg, xg);
+            rg = fma(-tk, z, rg);
         }
+        publish(1, rg * rg);
+        send16(first || final, ndst, vg, rg, nbar);
+        expect_bytes(t == 0, &ex.bar[1], rr_bytes);
+        if (every || w == 0) {
+            const double d = total(1, (unsigned)(it + 1) & 1u);
+            beta = it < 0 ? 0.0 : d * rc;
+            // stop where the next step would divide by zero, and at the start where
+            // |r| <= 1e-16
+            if (dead || !(d > 0.0) || (it < 0 && !(sqrt(d) > 1e-16 && ng > 1))) beta = nan;
+            c = d;
+        }
+        if (!every) {
+            if (t == 0) scal[1] = beta;
+            __syncthreads();
+            beta = scal[1];
+        }
+        if (!isfinite(beta)) break;
+        vg = fma(beta, vg, rg);
+        if (mine) sv[t + 1] = vg;
+        // the neighbours' boundary v, formed as they form it
+        const double2 nv = ex.nbr[final ? 1 : 0];
+        const double gv = fma(beta, nv.x, nv.y);
+        if (first || final) sv[final ? cnt + 1 : 0] = gv;
+        if (nw > 1) __syncthreads();
+        else __syncwarp();
     }
+    if (dead && t == 0) atomicOr(a.err, kErrWait);
     // Phi = x; E by Eq. 7 with periodic neighbours (across the blocks)
     __syncthreads();
     if (mine) sv[t + 1] = xg;

@@ -266,6 +266,7 @@ cudaError_t enqueue_solve(pic_run *r, cudaStream_t s, bool after_push) {
     a.k_mode = 2.0 / (double)r->p.ncell;
     a.dx = r->dx;
     a.mass = r->mass;
+    a.err = &r->dev()->err;
     a.solver = r->p.field_solver;
     a.cg_maxit = r->p.cg_iterations ? r->p.cg_iterations : PIC_CG_DEFAULT_ITERATIONS;
     return launch_solve(a, s);

@@ -33,7 +33,7 @@ enum : uint32_t {
     kErrPosition = 1u,   // a position outside [0, L) or not finite
     kErrSortKey = 4u,    // a sort key outside the grid
     kErrInput = 8u,      // an uploaded position outside [0, L) (pic_init, pic_set_state)
-    kErrWait = 16u,      // a grid barrier's wait ran out (steps.cu)
+    kErrWait = 16u,      // a wait ran out (the grid barrier of steps.cu, the CG's sums)
 };
 
 // Float32 constants of the push, formed once on the host.  In the float32
@@ -109,6 +109,7 @@ struct SolveArgs {
     double k_mode;                // 2 / NG: mode amplitude of the mode sums
     double dx;
     double mass;                  // particle mass m = Q0/qm
+    unsigned *err;                // device error word (the CG's waits)
     int solver;                   // PIC_SOLVER_EXACT / PIC_SOLVER_CG
     int cg_maxit;                 // CG: iterations per solve
 };
