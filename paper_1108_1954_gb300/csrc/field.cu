@@ -333,8 +333,8 @@ __global__ void __launch_bounds__(kClusterSolveThreads) pic_solve_cluster_kernel
 //     exchanged after the update: each block sends its boundary v (before the
 //     update) and r (after it) with its part of r.r, and the neighbour forms
 //     beta v + r itself, the same operation on the same numbers as the owner;
-//   * t = c / z.v and beta = d / c are products with reciprocals (recip64), of
-//     which 1/c is formed a whole half iteration before it is needed.
+//   * t = c / z.v and beta = d / c are corrected products with reciprocals
+//     (recip64, divide64), of which 1/c is formed while the sums cross.
 // A solve of 150 iterations takes 304 us on 1024 nodes, 549 with cluster barriers,
 // float64 trees and divisions; an iteration's 520 instructions a warp, one
 // after the other at 7.4 clocks, are what bounds it now.
@@ -400,16 +400,16 @@ __device__ __forceinline__ bool wait_phase(const void *bar, unsigned parity) {
 }
 
 // Sum of float64 values over a warp, in every lane, as integers: 53-bit mantissas
-// with 5 bits below them, aligned to the largest exponent (|m| < 2^58), added
-// in pieces of 27, 27 and 10 bits.  The sum is exact to 2^-57 of the largest
-// value a lane, then rounded once.  (Subnormal values and results are 0.)
+// with 5 bits below them, aligned to the largest exponent (|m| <= 2^58), added
+// in pieces of 27, 27 and 10 bits.  Each lane's value is rounded to 2^-58 of the
+// largest, the sum once more.  (Subnormal values and results are 0.)
 __device__ __forceinline__ double warp_sum_fixed(double p) {
     const unsigned long long b = (unsigned long long)__double_as_longlong(p);
     const unsigned ex = (unsigned)(b >> 52) & 0x7ffu;
     const unsigned emax = __reduce_max_sync(kFull, ex);
-    const unsigned long long mant = ((b & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull) << 5;
+    const unsigned long long mant = ((b & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull) << 6;
     const unsigned sh = emax - ex;
-    long long m = sh < 64u && ex ? (long long)(mant >> sh) : 0ll;
+    long long m = sh < 64u && ex ? (long long)(((mant >> sh) + 1ull) >> 1) : 0ll;    // to nearest
     m = (long long)b < 0 ? -m : m;
     const unsigned k = (1u << 27) - 1u;
     const unsigned s0 = __reduce_add_sync(kFull, (unsigned)m & k);
@@ -432,6 +432,14 @@ __device__ __forceinline__ double recip64(double x) {
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
     const double e = fma(-x, y, 1.0);
     return fma(y, fma(e, e, e), y);
+}
+
+// a / b with y = recip64(b): the product corrected by its residual a - q b, which
+// the FMA gives exactly (Markstein 1990), so that q is off by little more than
+// half a unit of the last place.
+__device__ __forceinline__ double divide64(double a, double b, double y) {
+    const double q = a * y;
+    return fma(fma(-q, b, a), y, q);
 }
 
 template <int MODE>
@@ -515,7 +523,7 @@ __global__ void __launch_bounds__(kClusterSolveThreads) pic_solve_cg_kernel(Solv
             if (every || w == 0) {
                 rc = recip64(c);                      // for beta, while the sums cross
                 const double zv = total(0, (unsigned)it & 1u);
-                tk = c * recip64(zv);
+                tk = divide64(c, zv, recip64(zv));
                 // stop where the step would divide by zero
                 tk = dead || zv == 0.0 ? nan : tk;
             }
@@ -533,7 +541,7 @@ __global__ void __launch_bounds__(kClusterSolveThreads) pic_solve_cg_kernel(Solv
         expect_bytes(t == 0, &ex.bar[1], rr_bytes);
         if (every || w == 0) {
             const double d = total(1, (unsigned)(it + 1) & 1u);
-            beta = it < 0 ? 0.0 : d * rc;
+            beta = it < 0 ? 0.0 : divide64(d, c, rc);
             // stop where the next step would divide by zero, and at the start where
             // |r| <= 1e-16
             if (dead || !(d > 0.0) || (it < 0 && !(sqrt(d) > 1e-16 && ng > 1))) beta = nan;
