@@ -66,9 +66,8 @@ extern "C" {
 #define PIC_ENOMEM (-2)   /* workspace too small / pool budget exhausted      */
 #define PIC_ECUDA (-3)    /* a CUDA runtime call failed                       */
 #define PIC_ETIMEOUT (-4) /* a wait between the blocks of a kernel ran out of
-                             its limit (pic_step_n's many-step launch, the
-                             CG solver); the run needs pic_init or
-                             pic_set_state                                   */
+                             its limit (the many-step launch, the CG
+                             solver); a run needs pic_init or pic_set_state  */
 #define PIC_EDEVICE (-5)  /* a kernel flagged bad particle data                */
 #define PIC_ESTATE (-6)   /* call out of order (e.g. push before init)         */
 
@@ -412,6 +411,10 @@ int pic_tune_sort_interval(pic_run *run, const int32_t *intervals, int32_t count
  * pic_pool_advance, which launches one thread-block-cluster kernel for all
  * runs with steps left: each cluster takes runs from a queue, largest work
  * first, and keeps a run on chip through all of its steps of that launch.
+ * Few active runs, none of them due to sort, take the many-step launch of
+ * pic_step_n side by side instead, where that is faster and free arena space
+ * holds its accumulators (48 NG bytes and 25 KB a run); the particles, the
+ * density and the field are the same bits either way.
  * A run with sort_interval S > 0 sorts its particles by cell before every
  * step n > 0 with n % S == 0, as the single run does (a stable counting sort
  * inside the cluster, into a second pair of particle buffers: 8 N more

@@ -149,6 +149,7 @@ struct pic_pool {
     int variant = kPoolVariant, cluster = 8, block = kPoolBlock, nclusters = 1;
     int wide_clusters = 0;        // > 0: up to so many runs take blocks twice as large
     int sms = 0;
+    int resident_sms = 0;         // SMs of the many-step launch (0: not available)
 
     BatchRun *d_runs() const { return reinterpret_cast<BatchRun *>(arena + tab.runs); }
     int *d_order() const { return reinterpret_cast<int *>(arena + tab.order); }
@@ -245,6 +246,161 @@ int launch(pic_pool *pool, const std::vector<int> &order, bool push) {
     return PIC_OK;
 }
 
+// ---- few active runs: the many-step launch (steps.cu) ---------------------------
+//
+// A cluster of 8 SMs per run leaves most of the GPU idle when few runs are
+// active, and the largest run decides when the launch ends.  The many-step
+// launch gives every run as many SMs as evens out the runs' times.
+
+// Blocks of the runs in `order` on `sms` SMs: one for the diagnostics and at
+// least one worker each, the rest one by one to the run that would take
+// longest.  A step takes about 6 us and 1.5 us per 1024 cells, and a worker
+// 0.4 ns a particle.  *time: of the launch (us); false when there are too many
+// runs.
+bool allot(const pic_pool *pool, const std::vector<int> &order, int sms, std::vector<int> *workers,
+           double *time) {
+    const int spare = sms - 2 * (int)order.size();
+    if (spare < 0) return false;
+    workers->assign(order.size(), 1);
+    auto run_time = [&](size_t i) {
+        const pic_pool::Slot &sl = pool->slots[order[i]];
+        return sl.desc.steps * (6.0 + 1.5 * sl.p.ncell / 1024.0 +
+                                0.4e-3 * (double)sl.p.npart / (*workers)[i]);
+    };
+    std::vector<std::pair<double, size_t>> heap;
+    for (size_t i = 0; i < order.size(); i++) heap.emplace_back(run_time(i), i);
+    std::make_heap(heap.begin(), heap.end());
+    *time = 0.0;                      // of the runs that can use no more workers
+    for (int k = 0; k < spare && !heap.empty();) {
+        std::pop_heap(heap.begin(), heap.end());
+        const double t = heap.back().first;
+        const size_t i = heap.back().second;
+        heap.pop_back();
+        // a worker takes a group of 4 particles per thread at least
+        const int64_t most = (pool->slots[order[i]].p.npart + 4 * kStepsPoolBlock - 1) / (4 * kStepsPoolBlock);
+        if ((*workers)[i] < most && (*workers)[i] < kStepsMaxGrid - 2) {
+            (*workers)[i]++;
+            heap.emplace_back(run_time(i), i);
+            std::push_heap(heap.begin(), heap.end());
+            k++;
+        } else {
+            *time = std::max(*time, t);
+        }
+    }
+    for (const auto &h : heap) *time = std::max(*time, h.first);
+    return true;
+}
+
+// Time of the cluster launch (us): its longest run, on 8 SMs that other clusters
+// share when there are more than fit side by side, or the whole work at the
+// rate of a full GPU.
+double cluster_time(const pic_pool *pool, const std::vector<int> &order) {
+    const double each = 8 * (int)order.size() > pool->sms ? 0.1e-3 : 0.07e-3;
+    double longest = 0.0, work = 0.0;
+    for (int s : order) {
+        const pic_pool::Slot &sl = pool->slots[s];
+        longest = std::max(longest, sl.desc.steps * (14.0 + each * (double)sl.p.npart));
+        work += (double)sl.desc.steps * (double)sl.p.npart;
+    }
+    return std::max(longest, work / 2.3e5);
+}
+
+// Whether the runs of `order` take the many-step launch, and its workers.
+// Measured (us per step of all, cluster launch and this one):
+//   runs of 1e4-1e6: 1 run 13-20, 5.8; 10 runs 51-78, 12; 24 runs 72-81, 23-26;
+//     38 runs 123-135, 36-39; 60 runs 136, 89-96; 76 runs 150, 345
+//   equal runs: 20 of 2e6 210, 133; 40 of 1e6 179, 190; 10 of 4e6 287, 120; 65 of
+//     2e5 55, 78; 60 of 5e4 24, 24; 76 of 1e4 25, 9; 8 of 1.2e7 825, 276
+bool resident(const pic_pool *pool, const std::vector<int> &order, std::vector<int> *workers) {
+    if (!pool->resident_sms) return false;
+    for (int s : order) {
+        const pic_pool::Slot &sl = pool->slots[s];
+        const int64_t S = sl.p.sort_interval;
+        if (S > 0) {                  // a sort falls before a step n > 0 with n % S == 0
+            const int64_t next = sl.done == 0 ? S : (sl.done + S - 1) / S * S;
+            if (next < sl.done + sl.desc.steps) return false;
+        }
+        if (sl.p.ncell > kStepsMaxCells || sl.p.npart > (((int64_t)1 << 38) / sl.p.ncell)) return false;
+    }
+    double time = 0.0;
+    if (!allot(pool, order, pool->resident_sms, workers, &time)) return false;
+    for (size_t i = 0; i < order.size(); i++)       // a worker's counts share words with carries
+        if (pool->slots[order[i]].p.npart / (*workers)[i] >= (1 << 20) - 64) return false;
+    return time < cluster_time(pool, order);
+}
+
+// Advance the runs of `order` by their steps; false (and nothing done) when the
+// arena has no room for the launch's accumulators.
+int launch_resident(pic_pool *pool, const std::vector<int> &order, const std::vector<int> &workers,
+                    bool *done) {
+    *done = false;
+    size_t off = align_up(order.size() * sizeof(StepsArgs)), clear = off;
+    struct Part { size_t acc, sync, partials; };
+    std::vector<Part> parts(order.size());
+    for (size_t i = 0; i < order.size(); i++) {     // what starts at zero, first
+        parts[i].acc = off;
+        off = align_up(off + (size_t)kStepsSlots * pool->slots[order[i]].p.ncell * 8);
+        parts[i].sync = off;
+        off = align_up(off + 4 * sizeof(unsigned));
+    }
+    const size_t cleared = off;
+    for (size_t i = 0; i < order.size(); i++) {
+        parts[i].partials = off;
+        off = align_up(off + (size_t)kStepsSlots * kStepsMaxGrid * 16);
+    }
+    size_t soff = 0, sbytes = 0;
+    if (!pool->idle_space(&soff, &sbytes) || sbytes < off) return PIC_OK;
+    unsigned char *mem = pool->arena + soff;
+    std::vector<StepsArgs> args(order.size());
+    int first = 0, ng_max = 1;
+    for (size_t i = 0; i < order.size(); i++) {
+        const pic_pool::Slot &sl = pool->slots[order[i]];
+        const BatchRun &d = sl.desc;
+        StepsArgs &a = args[i];
+        a.x = d.x;
+        a.v = d.v;
+        a.n = d.n;
+        a.E32 = d.E32;
+        a.E64 = d.E64;
+        a.phi = d.phi;
+        a.rho = d.rho;
+        a.rho_q_last = d.rho_q_last;
+        a.acc = reinterpret_cast<unsigned long long *>(mem + parts[i].acc);
+        a.partials = reinterpret_cast<double *>(mem + parts[i].partials);
+        a.err = pool->d_err();
+        a.sync = reinterpret_cast<unsigned *>(mem + parts[i].sync);
+        a.base[0] = a.base[1] = a.base[2] = 0;
+        a.diag_blocks = 1;
+        a.first_block = first;
+        a.blocks = workers[i] + 1;
+        a.log_copies = steps_pool_copies();
+        a.hist = d.hist;
+        a.hist_len = d.hist_len;
+        a.step0 = sl.done;
+        a.dstep = d.step;
+        a.steps = d.steps;
+        a.c = d.pc;
+        a.weight_total = d.weight_total;
+        a.k_rho = d.k_rho;
+        a.k_e = d.k_e;
+        a.k_phi = d.k_phi;
+        a.k_mode = d.k_mode;
+        a.dx = d.dx;
+        a.mass = d.mass;
+        first += a.blocks;
+        ng_max = std::max(ng_max, sl.p.ncell);
+    }
+    PIC_CUDA(cudaMemcpyAsync(mem, args.data(), args.size() * sizeof(StepsArgs), cudaMemcpyHostToDevice,
+                             pool->stream));
+    PIC_CUDA(cudaMemsetAsync(mem + clear, 0, cleared - clear, pool->stream));
+    PIC_CUDA(launch_steps_pool(reinterpret_cast<const StepsArgs *>(mem), (int)args.size(), first, ng_max,
+                               pool->stream));
+    // the scratch is free again, and the host's arguments read, when this is done
+    PIC_CUDA(cudaStreamSynchronize(pool->stream));
+    *done = true;
+    return PIC_OK;
+}
+
 bool slot_ok(const pic_pool *pool, int32_t slot) {
     return pool && slot >= 0 && slot < (int)pool->slots.size() && pool->slots[slot].used;
 }
@@ -253,6 +409,7 @@ int read_error(pic_pool *pool) {
     unsigned err = 0;
     PIC_CUDA(cudaMemcpyAsync(&err, pool->d_err(), sizeof(err), cudaMemcpyDeviceToHost, pool->stream));
     PIC_CUDA(cudaStreamSynchronize(pool->stream));
+    if (err & kErrWait) return PIC_ETIMEOUT;
     return err ? PIC_EDEVICE : PIC_OK;
 }
 
@@ -303,7 +460,11 @@ int pic_pool_create(const pic_pool_config *cfg, void *arena, size_t arena_bytes,
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&pool->sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess) e = batch_prepare_attributes();
+    int coop = 0, per_sm = 0;
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
+    if (e == cudaSuccess && coop) e = steps_pool_prepare(&per_sm);
     if (e != cudaSuccess) { delete pool; return cuda_fail(e); }
+    if (per_sm > 0) pool->resident_sms = pool->sms;
     rc = set_shape(pool, cfg->variant ? cfg->variant : kPoolVariant,
                    cfg->cluster ? cfg->cluster : 8, cfg->block ? cfg->block : kPoolBlock);
     if (rc) { delete pool; return rc; }
@@ -489,7 +650,11 @@ int pic_pool_advance(pic_pool *pool, int64_t k, int32_t *active) {
         const double wb = (double)pool->slots[b].p.npart * pool->slots[b].desc.steps;
         return wa > wb;
     });
-    int rc = launch(pool, order, true);
+    std::vector<int> workers;
+    bool done = order.empty();
+    int rc = PIC_OK;
+    if (!done && resident(pool, order, &workers)) rc = launch_resident(pool, order, workers, &done);
+    if (!rc && !done) rc = launch(pool, order, true);
     if (rc) return rc;
     for (int i : order) {
         pool->slots[i].done += pool->slots[i].desc.steps;

@@ -428,6 +428,9 @@ int run_steps(pic_run *r, int steps) {
     a.err = &r->dev()->err;
     a.sync = r->dev()->sync;
     for (int i = 0; i < 3; i++) a.base[i] = r->sync_base[i];
+    a.diag_blocks = kStepsDiag;
+    a.first_block = 0;
+    a.blocks = r->steps_grid;
     a.hist = r->at<pic_diag_row>(r->lay.hist);
     a.hist_len = r->lay.hist_len;
     a.step0 = r->step;

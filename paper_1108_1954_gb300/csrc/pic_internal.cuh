@@ -133,6 +133,8 @@ struct StepsArgs {
     unsigned *sync;               // [4], 16-byte aligned: arrivals of the workers, steps
                                   // done by each diagnostics block; never reset ...
     unsigned base[3];             // ... their values before this launch
+    int diag_blocks;              // 1 or 2: the last of the run's blocks, without particles
+    int first_block, blocks;      // the run's part of a pool's grid
     int log_copies;               // copies of a block's tile (set by the launcher)
     pic_diag_row *hist;
     int hist_len;
@@ -145,11 +147,15 @@ struct StepsArgs {
 };
 constexpr int kStepsMaxGrid = 256;
 constexpr int kStepsSlots = 6;     // accumulators in turn
-constexpr int kStepsDiag = 2;      // blocks of the grid without particles
+constexpr int kStepsDiag = 2;      // blocks of a single run's grid without particles
+constexpr int kStepsPoolBlock = 1024;
 constexpr int kStepsMaxCells = 4096;
 constexpr int64_t kStepsMaxParticles = 12500000;   // 100 MB of state
 cudaError_t steps_prepare(int variant, int ng, int block, int *per_sm);
 cudaError_t launch_steps(StepsArgs a, int variant, int grid, int block, cudaStream_t s);
+cudaError_t steps_pool_prepare(int *per_sm);
+int steps_pool_copies();
+cudaError_t launch_steps_pool(const StepsArgs *runs, int nrun, int grid, int ng_max, cudaStream_t s);
 
 // Counting sort by cell.
 template <typename T>

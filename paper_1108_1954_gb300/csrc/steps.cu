@@ -75,9 +75,9 @@ __device__ __forceinline__ void red_release(unsigned *p) {
     asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(p) : "memory");
 }
 
-// Steps t <= last with t mod kStepsDiag == d.
-__device__ __forceinline__ unsigned steps_of(int last, int d) {
-    return last < d ? 0u : (unsigned)((last - d) / kStepsDiag + 1);
+// Steps t <= last with t mod nd == d.
+__device__ __forceinline__ unsigned steps_of(int last, int d, int nd) {
+    return last < d ? 0u : (unsigned)((last - d) / nd + 1);
 }
 
 // Waits until all workers have arrived for step s, and, for a worker, until the
@@ -85,11 +85,11 @@ __device__ __forceinline__ unsigned steps_of(int last, int d) {
 // kStepsSlots.  All threads of the block; false when the wait ran out.
 __device__ __forceinline__ bool wait_step(const StepsArgs &a, int s, int workers, bool worker,
                                           int *dead) {
-    static_assert(kStepsDiag == 2, "two counters");
     if (threadIdx.x == 0) {
+        const int nd = a.diag_blocks;
         const unsigned target = a.base[0] + (unsigned)workers * (unsigned)(s + 1);
-        const unsigned d0 = a.base[1] + steps_of(s + 1 - kStepsSlots, 0);
-        const unsigned d1 = a.base[2] + steps_of(s + 1 - kStepsSlots, 1);
+        const unsigned d0 = a.base[1] + steps_of(s + 1 - kStepsSlots, 0, nd);
+        const unsigned d1 = a.base[2] + (nd > 1 ? steps_of(s + 1 - kStepsSlots, 1, nd) : 0u);
         unsigned polls = 0;
         for (;;) {
             const uint4 v = ld_acquire(a.sync);
@@ -238,9 +238,10 @@ __device__ __forceinline__ void solve_nodes(NodeSolve<K> &s, const StepsArgs &a,
     }
 }
 
+// Block b of a run's workers + nd: all its steps.
 template <int VARIANT, int K>
-__global__ void __launch_bounds__(1024, 1) pic_steps_kernel(StepsArgs a) {
-    extern __shared__ __align__(128) unsigned char smem_raw[];
+__device__ __forceinline__ void run_many_steps(const StepsArgs &a, unsigned char *smem_raw, const int b,
+                                               const int workers) {
     __shared__ long long wr[32];
     __shared__ unsigned long long ws[64];
     __shared__ float4 kvs[32];                    // per warp: (ke, ke low, mom, mom low)
@@ -257,7 +258,7 @@ __global__ void __launch_bounds__(1024, 1) pic_steps_kernel(StepsArgs a) {
     tile.c = tile.n;
     tile.k = a.log_copies;
     const int tid = threadIdx.x, bs = blockDim.x, lane = tid & 31, w = tid >> 5, nw = bs >> 5;
-    const int workers = (int)gridDim.x - kStepsDiag, b = blockIdx.x;
+    const int nd = a.diag_blocks;
     const bool diag = b >= workers;
     const unsigned long long kmant =
         (((unsigned long long)__double_as_longlong(a.k_e) & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull) << 11;
@@ -290,7 +291,7 @@ __global__ void __launch_bounds__(1024, 1) pic_steps_kernel(StepsArgs a) {
         rv[i] = q < q1 ? __ldcg(v4 + q) : zero4;
     }
     __syncthreads();
-    for (int s = diag ? b - workers : 0; s < a.steps; s += diag ? kStepsDiag : 1) {
+    for (int s = diag ? b - workers : 0; s < a.steps; s += diag ? nd : 1) {
         const bool last = s == a.steps - 1;
         const int slot = s % kStepsSlots;
         unsigned long long *acc = a.acc + (size_t)slot * ng;
@@ -495,6 +496,29 @@ __global__ void __launch_bounds__(1024, 1) pic_steps_kernel(StepsArgs a) {
     }
 }
 
+template <int VARIANT, int K>
+__global__ void __launch_bounds__(1024, 1) pic_steps_kernel(StepsArgs a) {
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    run_many_steps<VARIANT, K>(a, smem_raw, blockIdx.x, (int)gridDim.x - a.diag_blocks);
+}
+
+// Several runs side by side, each on its own blocks (a.first_block on), none
+// waiting for another: the pool's few active runs.
+__global__ void __launch_bounds__(1024, 1) pic_steps_pool_kernel(const StepsArgs *runs, int nrun) {
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    __shared__ __align__(16) StepsArgs a;
+    int i = 0;
+    while (i + 1 < nrun && (int)blockIdx.x >= runs[i + 1].first_block) i++;
+    static_assert(sizeof(StepsArgs) % 4 == 0, "copied by words");
+    for (int k = threadIdx.x; k < (int)(sizeof(StepsArgs) / 4); k += blockDim.x)
+        reinterpret_cast<unsigned *>(&a)[k] = reinterpret_cast<const unsigned *>(runs + i)[k];
+    __syncthreads();
+    const int b = (int)blockIdx.x - a.first_block, workers = a.blocks - a.diag_blocks;
+    if (a.c.ng <= 1024) run_many_steps<kDepositCells, 1>(a, smem_raw, b, workers);
+    else if (a.c.ng <= 2048) run_many_steps<kDepositCells, 2>(a, smem_raw, b, workers);
+    else run_many_steps<kDepositCells, 4>(a, smem_raw, b, workers);
+}
+
 using StepsKernel = void (*)(StepsArgs);
 
 template <int V>
@@ -525,6 +549,20 @@ size_t steps_smem(int variant, int ng, int block) {
     return (size_t)(ng + 2) * (4 + (8 << log_copies(variant, block)));
 }
 
+// A launch whose blocks are all resident at once.
+void cooperative(cudaLaunchConfig_t &cfg, cudaLaunchAttribute *attr, int grid, int block, size_t smem,
+                 cudaStream_t s) {
+    cfg = cudaLaunchConfig_t{};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+}
+
 }  // namespace
 
 cudaError_t steps_prepare(int variant, int ng, int block, int *per_sm) {
@@ -542,17 +580,28 @@ cudaError_t launch_steps(StepsArgs a, int variant, int grid, int block, cudaStre
     StepsKernel k = pick_steps(variant, a.c.ng, block);
     if (!k) return cudaErrorInvalidValue;
     a.log_copies = log_copies(variant, block);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3((unsigned)block);
-    cfg.dynamicSmemBytes = steps_smem(variant, a.c.ng, block);
-    cfg.stream = s;
+    cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeCooperative;
-    attr[0].val.cooperative = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cooperative(cfg, attr, grid, block, steps_smem(variant, a.c.ng, block), s);
     return cudaLaunchKernelEx(&cfg, k, a);
+}
+
+cudaError_t steps_pool_prepare(int *per_sm) {
+    const int smem = (int)steps_smem(kDepositCells, kStepsMaxCells, kStepsPoolBlock);
+    cudaError_t e = cudaFuncSetAttribute(&pic_steps_pool_kernel,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, &pic_steps_pool_kernel,
+                                                         kStepsPoolBlock, smem);
+}
+
+int steps_pool_copies() { return log_copies(kDepositCells, kStepsPoolBlock); }
+
+cudaError_t launch_steps_pool(const StepsArgs *runs, int nrun, int grid, int ng_max, cudaStream_t s) {
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr[1];
+    cooperative(cfg, attr, grid, kStepsPoolBlock, steps_smem(kDepositCells, ng_max, kStepsPoolBlock), s);
+    return cudaLaunchKernelEx(&cfg, &pic_steps_pool_kernel, runs, nrun);
 }
 
 }  // namespace pic

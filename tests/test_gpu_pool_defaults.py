@@ -58,3 +58,59 @@ def test_positions_read_back_through_free_space(n, free):
     vt = torch.empty(n, pin_memory=True)
     pool.get_state(slot, xt, vt)
     assert np.array_equal(xt.numpy(), want) and np.array_equal(vt.numpy(), v)
+
+
+def alone(p, seed, steps):
+    run = pic.Run(p, device="cuda:0")
+    run.init(*state(p.npart, seed))
+    run.step_n(steps)
+    return run
+
+
+@pytest.mark.parametrize("variant,cluster,block,ncell_max",
+                         [(1, 8, 256, 2048), (2, 8, 256, 2048), (5, 4, 512, 2048), (6, 2, 512, 1024),
+                          (1 + 16, 8, 256, 2048), (5 + 16, 8, 512, 4096), (6 + 16, 1, 512, 512)])
+def test_many_runs_keep_the_cluster_launch(variant, cluster, block, ncell_max):
+    # more runs than there are SMs: no many-step launch, whatever their sizes
+    n = 160
+    ps = [pic.Params(npart=1000 + 61 * i, ncell=1 + (97 * i) % ncell_max, length=L) for i in range(n)]
+    pool = pic.Pool(max_slots=n, ncell_max=ncell_max, arena_bytes=1 << 27, history=16, variant=variant,
+                    cluster=cluster, block=block, device="cuda:0")
+    slots = [pool.admit(p, *state(p.npart, i), 5) for i, p in enumerate(ps)]
+    pool.advance(2)
+    pool.advance(3)
+    for i in (0, 1, n // 2, n - 1):
+        run = alone(ps[i], i, 5)
+        for a, b in zip(pool.get_cells(slots[i]), run.get_cells()):
+            assert np.array_equal(a, b)
+        f, g = pool.get_field(slots[i]), run.get_field()
+        assert np.array_equal(f["rho_q"], g["rho_q"]) and np.array_equal(f["E"], g["E"])
+
+
+@pytest.mark.parametrize("free", [8 << 20, 0])
+def test_few_uneven_runs_equal_alone(free):
+    # the many-step launch, and without room for its accumulators the clusters;
+    # runs that stop early, one- and two-cell grids, the largest NG it takes
+    specs = [(600001, 4096, 9, 0), (3, 1, 9, 0), (5, 2, 4, 0), (40000, 1025, 9, 0), (70001, 64, 1, 0),
+             (20003, 2049, 7, 50), (20003, 333, 9, 3)]
+    ps = [pic.Params(npart=n, ncell=g, length=L, sort_interval=S) for n, g, _, S in specs]
+    pool = pic.Pool(max_slots=len(ps), ncell_max=4096, variant=5, cluster=8, block=512, history=16,
+                    arena_bytes=(1 << 14) + sum(pic.pool_run_bytes(p, 16) for p in ps) + free,
+                    device="cuda:0")
+    slots = [pool.admit(p, *state(p.npart, i), k) for i, (p, (_, _, k, _)) in enumerate(zip(ps, specs))]
+    assert None not in slots
+    for k in (1, 2, 1, 9):             # the last run sorts before steps 3 and 6
+        pool.advance(k)
+    for i, (p, (_, _, k, _)) in enumerate(zip(ps, specs)):
+        assert pool.step_count(slots[i]) == k
+        run = alone(p, i, k)
+        for a, b in zip(pool.get_cells(slots[i]), run.get_cells()):
+            assert np.array_equal(a, b)
+        f, g = pool.get_field(slots[i]), run.get_field()
+        for key in ("rho_q", "E", "rho"):
+            assert np.array_equal(f[key], g[key])
+        d, e = pool.diagnostics(slots[i], 0, k + 1), run.diagnostics(0, k + 1)
+        assert np.array_equal(d["step"], e["step"]) and np.array_equal(d["charge_q"], e["charge_q"])
+        np.testing.assert_allclose(d["field"], e["field"], rtol=1e-12, atol=1e-300)
+        np.testing.assert_allclose(d["kinetic"][:-1], e["kinetic"][:-1], rtol=1e-5)
+        assert np.isnan(d["kinetic"][-1])
