@@ -159,6 +159,7 @@ struct pic_run {
     int cur = 0;                     // which x/v buffer holds the state
     int grid = 0, block = 0, variant = 0, unroll = 1;
     bool open_shape = true;          // no launch shape asked for
+    bool auto_variant = true;        // nor a deposit variant asked for or tuned
     int steps_grid = 0, steps_block = 0;   // many-step launch (0: not taken)
     unsigned sync_base[3] = {0, 0, 0};   // its counters so far
     int64_t step = 0;
@@ -378,8 +379,13 @@ int default_block(const pic_run *r) {
 }
 
 // Shape of the many-step launch (steps.cu), or none: an exact fixed-point run
-// of one rank whose caller left the push's shape open, whose state stays in L2
-// and whose grid gives a thread at most 4 nodes (both sides measured there).
+// of one rank whose caller left the push's shape open, up to 24e6 particles on
+// up to 2048 cells and 12.5e6 on up to 4096.  Measured (us a step, this launch
+// and push + solve, unsorted after 100 steps / sorted every 20):
+//   cells     1.2e7 particles          1.7e7                    3.4e7
+//    512   34, 48.8 / 41, 48.4   50.8, 60.3 / 57.1, 62.6   97, 102 / 107, 109
+//   2048   38, 47.6 / 43, 48.8   53.1, 59.4 / 59.4, 62.0  100, 101 / 110, 108
+//   4096   45, 48.8 / 51, 51.8   60.3, 61.0 / 67.4, 64.6  107, 102 / 118, 109
 // One group of 4 particles per thread while that takes fewer blocks than SMs.
 // Runs of up to 131072 particles on up to 512 cells take 256 threads a block
 // (5e4 particles, 100 cells: 4.3 us a step against 4.6 with 512 and 5.8 with
@@ -388,7 +394,8 @@ cudaError_t set_steps_shape(pic_run *r) {
     r->steps_grid = 0;
     const pic_params &p = r->p;
     if (p.precision != PIC_FP32_FIXED || p.field_solver != PIC_SOLVER_EXACT || !r->open_shape ||
-        r->npart_total != p.npart || p.npart > kStepsMaxParticles || p.ncell > kStepsMaxCells)
+        r->npart_total != p.npart || p.ncell > kStepsMaxCells ||
+        p.npart > (p.ncell <= 2048 ? kStepsMaxParticles : kStepsMaxParticlesWide))
         return cudaSuccess;
     int coop = 0;
     cudaError_t e = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, r->device);
@@ -590,7 +597,18 @@ int pic_create(const pic_params *p, void *workspace, size_t workspace_bytes,
     set_solve_constants(r, p->npart);
 
     // launch shape of the fused push
-    r->variant = p->deposit_variant ? p->deposit_variant : PIC_DEPOSIT_QUAD;
+    r->open_shape = !p->deposit_variant && !p->block_size && !p->blocks_per_sm && !p->unroll;
+    // A shape left open takes two open runs on 8-particle groups (PAIR8) where
+    // three blocks of 512 threads fit the shared memory; otherwise runs on float4
+    // groups (QUAD).  Measured (us a push, PAIR8 and QUAD, lattice order / after
+    // 400 steps): 2^26 on 4096 cells, sorted every 20, 185/179 and 205/183; 2^25
+    // on 512 cells 113/95 and 184/98; unsorted, 2^25 on 4096, 99/97 and 107/95;
+    // 2^25 on 8192 (two blocks) 110/111 and 101/102.
+    const bool three = 3 * push_smem_bytes(PIC_FP32_FIXED, p->ncell,
+                                           push_wide_tile(p->npart, r->sms)) <= 227 * 1024;
+    r->auto_variant = !p->deposit_variant;
+    r->variant = p->deposit_variant ? p->deposit_variant
+                 : r->open_shape && three ? PIC_DEPOSIT_PAIR8 : PIC_DEPOSIT_QUAD;
     if (p->precision != PIC_FP32_FIXED) r->variant = PIC_DEPOSIT_ATOMIC;
     if (p->shape == PIC_SHAPE_NGP) r->variant = kDepositNgp;
     r->block = p->block_size ? p->block_size : default_block(r);
@@ -598,7 +616,6 @@ int pic_create(const pic_params *p, void *workspace, size_t workspace_bytes,
     if (p->precision != PIC_FP32_FIXED) r->unroll = 1;
     r->grid = push_grid(r, r->variant, r->block, r->unroll, p->blocks_per_sm);
     if (r->grid < 1) { delete r; return PIC_EINVAL; }
-    r->open_shape = !p->deposit_variant && !p->block_size && !p->blocks_per_sm && !p->unroll;
     e = set_steps_shape(r);
     if (e != cudaSuccess) { pic_destroy(r); return cuda_fail(e); }
     *out = r;
@@ -871,7 +888,8 @@ int pic_set_launch(pic_run *run, int32_t variant, int32_t block, int32_t unroll,
     const bool fixed = run->p.precision == PIC_FP32_FIXED;
     const bool ngp = run->p.shape == PIC_SHAPE_NGP;
     if (ngp && variant) return PIC_EINVAL;   // the shape fixes the deposit
-    const int v = variant ? variant : run->variant;
+    // a shape that gives no variant takes QUAD, which has every unroll
+    const int v = variant ? variant : run->auto_variant && !ngp && fixed ? (int)PIC_DEPOSIT_QUAD : run->variant;
     const int b = block ? block : run->block;
     const int u = unroll ? unroll : run->unroll;
     if (!ngp && (!is_variant(v) || (!fixed && v != PIC_DEPOSIT_ATOMIC)))
@@ -886,6 +904,7 @@ int pic_set_launch(pic_run *run, int32_t variant, int32_t block, int32_t unroll,
     run->unroll = u;
     run->grid = g;
     run->open_shape = false;
+    if (variant) run->auto_variant = false;
     PIC_CUDA(set_steps_shape(run));
     destroy_graphs(run);
     return PIC_OK;
@@ -973,6 +992,7 @@ int pic_autotune(pic_run *run, int32_t reps, pic_tune_entry *results,
     run->variant = bv;
     run->block = bb;
     run->unroll = bu;
+    run->auto_variant = false;
     run->grid = bg;                 // (the many-step launch, where taken, is faster than any)
     destroy_graphs(run);
     if (nresults) *nresults = count < max_results || !results ? count : max_results;

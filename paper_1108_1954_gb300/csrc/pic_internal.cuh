@@ -150,7 +150,8 @@ constexpr int kStepsSlots = 6;     // accumulators in turn
 constexpr int kStepsDiag = 2;      // blocks of a single run's grid without particles
 constexpr int kStepsPoolBlock = 1024;
 constexpr int kStepsMaxCells = 4096;
-constexpr int64_t kStepsMaxParticles = 12500000;   // 100 MB of state
+// largest runs: up to 2048 cells, and beyond
+constexpr int64_t kStepsMaxParticles = 24000000, kStepsMaxParticlesWide = 12500000;
 cudaError_t steps_prepare(int variant, int ng, int block, int *per_sm);
 cudaError_t launch_steps(StepsArgs a, int variant, int grid, int block, cudaStream_t s);
 cudaError_t steps_pool_prepare(int *per_sm);

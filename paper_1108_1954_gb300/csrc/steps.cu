@@ -32,13 +32,13 @@
 //   1e6, 1024 cells, sorted every 20           22.5   10.7
 //   3e6, 777 cells, NGP, sorted every 10       27.4   17.8
 //   4.2e6, 2048 cells, sorted every 20         31.0   22.8
-//   1e6, 4096 cells                            24.8   17.5
-//   1.2e7, 2048 cells, sorted every 20         52.9   44.6
+//   1e6, 4096 cells                            24.8   16.0
+//   1.2e7, 2048 cells, sorted every 20         52.9   43.0
 // of which, at 5e4 (clocks): push 2300, sums 380, flush 1040, barrier 2400 (the
 // adds' release and a poll, each a trip to L2), solve 1300 (900 the sums' way
-// from L2), E 510.  Where the state no longer fits L2 (1.7e7 particles: 82
-// against 72 us) or a thread has 8 nodes (1e6 particles on 6000 cells: 31
-// against 28) the two launches are faster and are kept (set_steps_shape).
+// from L2), E 510.  Large runs' pushes stream from memory, for which the two
+// launches have more warps, and a thread with 8 nodes runs out of registers
+// (1e6 particles on 6000 cells: 31 us against 28): set_steps_shape.
 //
 // The solve in 64 bits.  R_g = N 2^24 - NG rho_q[g] and its prefix sums P_g are
 // below N NG 2^24 in magnitude, so they fit 64 bits for N NG <= 2^38 (the
@@ -238,12 +238,165 @@ __device__ __forceinline__ void solve_nodes(NodeSolve<K> &s, const StepsArgs &a,
     }
 }
 
+// The field of a step in a worker's shared copy of E.
+template <int K>
+__device__ __forceinline__ void field_step(const StepsArgs &a, const unsigned long long *acc, float *sE) {
+    __shared__ long long wr[32];
+    __shared__ unsigned long long ws[64];
+    const int ng = a.c.ng, tid = threadIdx.x;
+    const unsigned long long kb = (unsigned long long)__double_as_longlong(a.k_e);
+    const unsigned long long kmant = ((kb & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull) << 11;
+    const int kexp = (int)(kb >> 52) - 1023;
+    NodeSolve<K> ns;
+    solve_nodes<K>(ns, a, acc, ng, wr, ws);
+#pragma unroll
+    for (int j = 0; j < K; j++) {
+        const int g = tid * K + j;
+        if (g >= ng) break;
+        const float e = scaled_f32(ns.m[j], a.k_e, kmant, kexp);
+        sE[g + 1] = e;
+        if (g == ng - 1) sE[0] = e;
+        if (g == 0) sE[ng + 1] = e;
+    }
+    __syncthreads();
+}
+
+// The diagnostics of a step, and after the last one the run's results.
+template <int K>
+__device__ __forceinline__ void diag_step(const StepsArgs &a, int s, int workers,
+                                       const unsigned long long *acc, const float4 *kv,
+                                       unsigned char *smem_raw, unsigned h0) {
+    __shared__ long long wr[32];
+    __shared__ unsigned long long ws[64];
+    const int ng = a.c.ng, tid = threadIdx.x, lane = tid & 31, w = tid >> 5, nw = blockDim.x >> 5;
+    const bool last = s == a.steps - 1;
+    const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
+    NodeSolve<K> ns;
+    solve_nodes<K>(ns, a, acc, ng, wr, ws);
+                    __shared__ float shf[2 * PIC_NMODES][32];
+            __shared__ double shd[8], fchunk[256], tot[2];
+            double *fe = reinterpret_cast<double *>(smem_raw);      // [ng], in the tile
+            NodeDiag d;
+            node_diag_reset(d);
+    #pragma unroll
+            for (int j = 0; j < K; j++) {
+                const int g = tid * K + j;
+                if (g >= ng) break;
+                const double E = a.k_e * i128_to_f64(ns.m[j]);
+                d.fe = 0.0;
+                node_diag(d, g, ng, E, (float)E);
+                fe[g] = d.fe;
+                if (last) {
+                    a.E64[g] = E;
+                    a.E32[g] = (float)E;
+                    a.rho[g] = a.k_rho * i128_to_f64((i128)ns.R[j]);
+                    a.rho_q_last[g] = ns.q[j];
+                }
+            }
+            float md[2 * PIC_NMODES];
+    #pragma unroll
+            for (int m = 0; m < PIC_NMODES; m++) { md[2 * m] = d.re[m]; md[2 * m + 1] = d.im[m]; }
+            static_assert(2 * PIC_NMODES == 16, "16 mode sums per warp");
+            const int used = (ng + 32 * K - 1) / (32 * K);          // warps with nodes
+            if (w < used) {
+                const float msum = warp_sum16_halving(md, lane);
+                if ((lane & 1) == 0) shf[lane >> 1][w] = msum;
+            }
+            __syncthreads();
+            const int chunks = (ng + 31) >> 5;
+            for (int i = w; i < chunks; i += nw) {                  // field energy of 32 nodes
+                const int g = 32 * i + lane;
+                const double sum = warp_sum_f64(g < ng ? fe[g] : 0.0);
+                if (lane == 0) fchunk[i] = sum;
+            }
+            if (w == nw - 1) {                                      // the push's sums
+                float4 p[kStepsMaxGrid / 32];                       // all loads in flight
+    #pragma unroll
+                for (int i = 0; i < kStepsMaxGrid / 32; i++)
+                    p[i] = 32 * i + lane < workers ? __ldcg(kv + 32 * i + lane) : zero4;
+    #pragma unroll
+                for (int i = 1; i < kStepsMaxGrid / 32; i++) {
+                    add_pair(p[0].x, p[0].y, p[i].x, p[i].y);
+                    add_pair(p[0].z, p[0].w, p[i].z, p[i].w);
+                }
+                warp_sum_pairs(p[0], 32);
+                if (lane == 0) {
+                    tot[0] = (double)p[0].x + (double)p[0].y;
+                    tot[1] = (double)p[0].z + (double)p[0].w;
+                }
+            }
+            __syncthreads();
+            const double fe_total = chunk_sum_f64(tid < chunks ? fchunk[tid] : 0.0, chunks, shd);
+            if (w == 0) {
+                const long long n = a.step0 + s + 1;
+                pic_diag_row *prev = &a.hist[(h0 + s) % a.hist_len], *row = &a.hist[(h0 + s + 1) % a.hist_len];
+                // one value per lane: kinetic energy and momentum of the row before,
+                // field energy and charge of this one
+                const double coef = lane == 0 ? 0.5 * a.mass : lane == 1 ? a.mass
+                                    : lane == 2 ? 0.5 * a.dx : a.dx * a.k_rho;
+                const double fe0 = __shfl_sync(kFull, fe_total, 0);
+                const double val = coef * (lane < 2 ? tot[lane] : lane == 2 ? fe0 : (double)ns.SR);
+                if (lane < 4) *(lane == 0 ? &prev->kinetic : lane == 1 ? &prev->momentum
+                                : lane == 2 ? &row->field : &row->charge) = val;
+                if (lane == 4) row->step = n;
+                // sum of rho_q: SR = NG (N 2^24 - it), 0 unless particles were lost
+                if (lane == 5) row->charge_q = ns.SR ? a.weight_total - ns.SR / ng : a.weight_total;
+                if (last && lane >= 6 && lane < 8)       // (otherwise the next step's, perhaps written already)
+                    *(lane == 6 ? &row->kinetic : &row->momentum) = __longlong_as_double(0x7ff8000000000000ll);
+                if (last && lane == 8) *a.dstep = n;
+            } else if (w == 1) {
+                // mode sums: float32 over 8 warps, float64 over those
+                double sum = 0.0;
+                for (int i0 = 0; i0 < used; i0 += 8) {
+                    float part = 0.0f;
+    #pragma unroll
+                    for (int i = 0; i < 8; i++)
+                        part += i0 + i < used ? shf[lane & 15][(i0 + i) & 31] : 0.0f;
+                    sum += (double)part;
+                }
+                const double im = __shfl_down_sync(kFull, sum, 1);
+                if (lane < 2 * PIC_NMODES && !(lane & 1))
+                    a.hist[(h0 + s + 1) % a.hist_len].mode[lane >> 1] =
+                        sqrt(sum * sum + im * im) * a.k_mode;
+            }
+            if (last) {
+                // Phi: sum_{k<g} M_k = NG (g P_g - sum_{j<=g} j R_j) - g SP
+                __shared__ unsigned long long scan64[4 * 32];
+                i128 jr = 0;
+    #pragma unroll
+                for (int j = 0; j < K; j++) jr += (i128)ns.R[j] * (i128)(tid * K + j);
+                i128 run = block_inclusive_scan2_i128(jr, 0, scan64).a - jr;
+    #pragma unroll
+                for (int j = 0; j < K; j++) {
+                    const int g = tid * K + j;
+                    if (g >= ng) break;
+                    run += (i128)ns.R[j] * (i128)g;
+                    const i128 sumM = (i128)ng * ((i128)g * (i128)ns.P[j] - run) - (i128)g * ns.SP;
+                    a.phi[g] = a.k_phi * i128_to_f64(sumM);
+                }
+            }
+}
+
+// With 4 nodes a thread both are called out of line, so that their registers (a
+// node's 128-bit sums, 4 times) are not taken from the push loop: 1.2e7
+// particles on 4096 cells 44.6 us a step, 50.2 inlined.  With 1 or 2 they fit
+// beside it (512 cells 34.4 inlined, 36.0 called).
+template <int K>
+__device__ __noinline__ void field_step_call(const StepsArgs &a, const unsigned long long *acc, float *sE) {
+    field_step<K>(a, acc, sE);
+}
+
+template <int K>
+__device__ __noinline__ void diag_step_call(const StepsArgs &a, int s, int workers,
+                                            const unsigned long long *acc, const float4 *kv,
+                                            unsigned char *smem_raw, unsigned h0) {
+    diag_step<K>(a, s, workers, acc, kv, smem_raw, h0);
+}
+
 // Block b of a run's workers + nd: all its steps.
 template <int VARIANT, int K>
 __device__ __forceinline__ void run_many_steps(const StepsArgs &a, unsigned char *smem_raw, const int b,
                                                const int workers) {
-    __shared__ long long wr[32];
-    __shared__ unsigned long long ws[64];
     __shared__ float4 kvs[32];                    // per warp: (ke, ke low, mom, mom low)
     __shared__ int dead;
     constexpr bool kNgp = VARIANT == kDepositNgp;
@@ -260,9 +413,6 @@ __device__ __forceinline__ void run_many_steps(const StepsArgs &a, unsigned char
     const int tid = threadIdx.x, bs = blockDim.x, lane = tid & 31, w = tid >> 5, nw = bs >> 5;
     const int nd = a.diag_blocks;
     const bool diag = b >= workers;
-    const unsigned long long kmant =
-        (((unsigned long long)__double_as_longlong(a.k_e) & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull) << 11;
-    const int kexp = (int)((unsigned long long)__double_as_longlong(a.k_e) >> 52) - 1023;
     if (tid == 0) dead = 0;
     auto clear_tile = [&] {
         for (int j = tid; j < words; j += bs) {
@@ -361,124 +511,13 @@ __device__ __forceinline__ void run_many_steps(const StepsArgs &a, unsigned char
             clear_tile();                             // while the others arrive
         }
         if (!wait_step(a, s, workers, !diag, &dead)) return;
-        NodeSolve<K> ns;
-        solve_nodes<K>(ns, a, acc, ng, wr, ws);
         if (!diag) {
-#pragma unroll
-            for (int j = 0; j < K; j++) {
-                const int g = tid * K + j;
-                if (g >= ng) break;
-                const float e = scaled_f32(ns.m[j], a.k_e, kmant, kexp);
-                sE[g + 1] = e;
-                if (g == ng - 1) sE[0] = e;
-                if (g == 0) sE[ng + 1] = e;
-            }
-            __syncthreads();
+            if (K >= 4) field_step_call<K>(a, acc, sE);
+            else field_step<K>(a, acc, sE);
             continue;
         }
-        // ---- a diagnostics block: those of the step, beside the workers' next ones
-        __shared__ float shf[2 * PIC_NMODES][32];
-        __shared__ double shd[8], fchunk[256], tot[2];
-        double *fe = reinterpret_cast<double *>(smem_raw);      // [ng], in the tile
-        NodeDiag d;
-        node_diag_reset(d);
-#pragma unroll
-        for (int j = 0; j < K; j++) {
-            const int g = tid * K + j;
-            if (g >= ng) break;
-            const double E = a.k_e * i128_to_f64(ns.m[j]);
-            d.fe = 0.0;
-            node_diag(d, g, ng, E, (float)E);
-            fe[g] = d.fe;
-            if (last) {
-                a.E64[g] = E;
-                a.E32[g] = (float)E;
-                a.rho[g] = a.k_rho * i128_to_f64((i128)ns.R[j]);
-                a.rho_q_last[g] = ns.q[j];
-            }
-        }
-        float md[2 * PIC_NMODES];
-#pragma unroll
-        for (int m = 0; m < PIC_NMODES; m++) { md[2 * m] = d.re[m]; md[2 * m + 1] = d.im[m]; }
-        static_assert(2 * PIC_NMODES == 16, "16 mode sums per warp");
-        const int used = (ng + 32 * K - 1) / (32 * K);          // warps with nodes
-        if (w < used) {
-            const float msum = warp_sum16_halving(md, lane);
-            if ((lane & 1) == 0) shf[lane >> 1][w] = msum;
-        }
-        __syncthreads();
-        const int chunks = (ng + 31) >> 5;
-        for (int i = w; i < chunks; i += nw) {                  // field energy of 32 nodes
-            const int g = 32 * i + lane;
-            const double sum = warp_sum_f64(g < ng ? fe[g] : 0.0);
-            if (lane == 0) fchunk[i] = sum;
-        }
-        if (w == nw - 1) {                                      // the push's sums
-            float4 p[kStepsMaxGrid / 32];                       // all loads in flight
-#pragma unroll
-            for (int i = 0; i < kStepsMaxGrid / 32; i++)
-                p[i] = 32 * i + lane < workers ? __ldcg(kv + 32 * i + lane) : zero4;
-#pragma unroll
-            for (int i = 1; i < kStepsMaxGrid / 32; i++) {
-                add_pair(p[0].x, p[0].y, p[i].x, p[i].y);
-                add_pair(p[0].z, p[0].w, p[i].z, p[i].w);
-            }
-            warp_sum_pairs(p[0], 32);
-            if (lane == 0) {
-                tot[0] = (double)p[0].x + (double)p[0].y;
-                tot[1] = (double)p[0].z + (double)p[0].w;
-            }
-        }
-        __syncthreads();
-        const double fe_total = chunk_sum_f64(tid < chunks ? fchunk[tid] : 0.0, chunks, shd);
-        if (w == 0) {
-            const long long n = a.step0 + s + 1;
-            pic_diag_row *prev = &a.hist[(h0 + s) % a.hist_len], *row = &a.hist[(h0 + s + 1) % a.hist_len];
-            // one value per lane: kinetic energy and momentum of the row before,
-            // field energy and charge of this one
-            const double coef = lane == 0 ? 0.5 * a.mass : lane == 1 ? a.mass
-                                : lane == 2 ? 0.5 * a.dx : a.dx * a.k_rho;
-            const double fe0 = __shfl_sync(kFull, fe_total, 0);
-            const double val = coef * (lane < 2 ? tot[lane] : lane == 2 ? fe0 : (double)ns.SR);
-            if (lane < 4) *(lane == 0 ? &prev->kinetic : lane == 1 ? &prev->momentum
-                            : lane == 2 ? &row->field : &row->charge) = val;
-            if (lane == 4) row->step = n;
-            // sum of rho_q: SR = NG (N 2^24 - it), 0 unless particles were lost
-            if (lane == 5) row->charge_q = ns.SR ? a.weight_total - ns.SR / ng : a.weight_total;
-            if (last && lane >= 6 && lane < 8)       // (otherwise the next step's, perhaps written already)
-                *(lane == 6 ? &row->kinetic : &row->momentum) = __longlong_as_double(0x7ff8000000000000ll);
-            if (last && lane == 8) *a.dstep = n;
-        } else if (w == 1) {
-            // mode sums: float32 over 8 warps, float64 over those
-            double sum = 0.0;
-            for (int i0 = 0; i0 < used; i0 += 8) {
-                float part = 0.0f;
-#pragma unroll
-                for (int i = 0; i < 8; i++)
-                    part += i0 + i < used ? shf[lane & 15][(i0 + i) & 31] : 0.0f;
-                sum += (double)part;
-            }
-            const double im = __shfl_down_sync(kFull, sum, 1);
-            if (lane < 2 * PIC_NMODES && !(lane & 1))
-                a.hist[(h0 + s + 1) % a.hist_len].mode[lane >> 1] =
-                    sqrt(sum * sum + im * im) * a.k_mode;
-        }
-        if (last) {
-            // Phi: sum_{k<g} M_k = NG (g P_g - sum_{j<=g} j R_j) - g SP
-            __shared__ unsigned long long scan64[4 * 32];
-            i128 jr = 0;
-#pragma unroll
-            for (int j = 0; j < K; j++) jr += (i128)ns.R[j] * (i128)(tid * K + j);
-            i128 run = block_inclusive_scan2_i128(jr, 0, scan64).a - jr;
-#pragma unroll
-            for (int j = 0; j < K; j++) {
-                const int g = tid * K + j;
-                if (g >= ng) break;
-                run += (i128)ns.R[j] * (i128)g;
-                const i128 sumM = (i128)ng * ((i128)g * (i128)ns.P[j] - run) - (i128)g * ns.SP;
-                a.phi[g] = a.k_phi * i128_to_f64(sumM);
-            }
-        }
+        if (K >= 4) diag_step_call<K>(a, s, workers, acc, kv, smem_raw, h0);
+        else diag_step<K>(a, s, workers, acc, kv, smem_raw, h0);
         // give the slot back, once no worker reads it any more
         if (!last && !wait_step(a, s + 1, workers, false, &dead)) return;
         for (int g = tid; g < ng; g += bs) acc[g] = 0ull;
@@ -497,7 +536,7 @@ __device__ __forceinline__ void run_many_steps(const StepsArgs &a, unsigned char
 }
 
 template <int VARIANT, int K>
-__global__ void __launch_bounds__(1024, 1) pic_steps_kernel(StepsArgs a) {
+__global__ void __launch_bounds__(1024, 1) pic_steps_kernel(const __grid_constant__ StepsArgs a) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     run_many_steps<VARIANT, K>(a, smem_raw, blockIdx.x, (int)gridDim.x - a.diag_blocks);
 }

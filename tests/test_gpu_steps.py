@@ -74,7 +74,8 @@ def test_sorted_steps_equal_the_two_kernels(n, ng, S, shape):
     assert_same(a, b, n, ng)
 
 
-@pytest.mark.parametrize("n,ng", [(12500000, 512), (12500001, 512), (100003, 4096), (100003, 4097)])
+@pytest.mark.parametrize("n,ng", [(12500000, 2049), (12500001, 2049), (24000000, 512), (24000001, 512),
+                                  (100003, 4096), (100003, 4097)])
 def test_steps_at_the_limits_of_the_launch(n, ng):
     a, b = pair(n, ng)
     a.step_n(3), b.step_n(3)
