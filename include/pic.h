@@ -207,11 +207,12 @@ int pic_push(pic_run *run);
  * their order).  Changes no physical quantity.  Asynchronous. */
 int pic_sort(pic_run *run);
 
-/* n whole steps: [sort if due] + push + solve.  Fixed-point runs with the
- * exact solver, up to 24e6 particles on 2048 cells or 12.5e6 on 4096, whose
- * launch shape is left open (pic_params, pic_set_launch) take many steps per cooperative
- * launch; others replay CUDA graphs.  The results are the same.  While the
- * stream is being captured single launches are enqueued.
+/* n whole steps: [sort if due] + push + solve.  Runs with the exact solver
+ * whose launch shape is left open (pic_params, pic_set_launch) take many steps
+ * per cooperative launch: PIC_FP32_FIXED up to 24e6 particles on 2048 cells or
+ * 12.5e6 on 4096, PIC_FP64 up to 1e6 on 1024.  Others replay CUDA graphs.  The
+ * results are the same.  While the stream is being captured single launches
+ * are enqueued.
  * A step n with n % S == 0 (S = sort_interval > 0, n > 0) sorts first.
  * Asynchronous. */
 int pic_step_n(pic_run *run, int64_t n);

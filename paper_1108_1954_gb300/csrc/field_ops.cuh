@@ -156,6 +156,31 @@ __device__ __forceinline__ double chunk_sum_f64(double v, int chunks, double *sl
     return s;
 }
 
+// Sum of float64 values over a warp, in every lane, as integers: 53-bit mantissas
+// with 5 bits below them, aligned to the largest exponent (|m| <= 2^58), added
+// in pieces of 27, 27 and 10 bits.  Each lane's value is rounded to 2^-58 of the
+// largest, the sum once more.  (Subnormal values and results are 0.)
+__device__ __forceinline__ double warp_sum_fixed(double p) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(p);
+    const unsigned ex = (unsigned)(b >> 52) & 0x7ffu;
+    const unsigned emax = __reduce_max_sync(kFull, ex);
+    const unsigned long long mant = ((b & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull) << 6;
+    const unsigned sh = emax - ex;
+    long long m = sh < 64u && ex ? (long long)(((mant >> sh) + 1ull) >> 1) : 0ll;    // to nearest
+    m = (long long)b < 0 ? -m : m;
+    const unsigned k = (1u << 27) - 1u;
+    const unsigned s0 = __reduce_add_sync(kFull, (unsigned)m & k);
+    const unsigned s1 = __reduce_add_sync(kFull, (unsigned)(m >> 27) & k);
+    const int s2 = __reduce_add_sync(kFull, (int)(m >> 54));
+    const long long sum = (long long)s0 + ((long long)s1 << 27) + ((long long)s2 << 54);
+    // sum 2^(emax - 1080), by the exponent field
+    const unsigned long long d = (unsigned long long)__double_as_longlong((double)sum);
+    const int ed = (int)((d >> 52) & 0x7ffull) + (int)emax - 1080;
+    const unsigned long long v = (d & 0x800fffffffffffffull) | ((unsigned long long)(unsigned)ed << 52);
+    if (emax == 0x7ffu || ed > 2046) return __longlong_as_double(0x7ff8000000000000ll);
+    return sum == 0 || ed < 1 ? 0.0 : __longlong_as_double((long long)v);
+}
+
 // Per-node diagnostics contribution of node g with field E (float64) and its
 // float32 copy: field energy sum and the mode sums (float32 twiddles).
 struct NodeDiag {

@@ -102,6 +102,9 @@ void sort_geometry(int64_t n, int ng, int *nchunk, long long *chunk, int *nseg, 
     *nseg = (int)((nc + *seg_len - 1) / *seg_len);
 }
 
+// A node's density sum in the many-step launch.
+size_t steps_acc_bytes(const pic_params *p) { return p->precision == PIC_FP64 ? 16 : 8; }
+
 void make_layout(const pic_params *p, Layout *L) {
     const size_t n = (size_t)p->npart, ng = (size_t)p->ncell;
     const size_t es = p->precision == PIC_FP64 ? 8 : 4;
@@ -115,7 +118,7 @@ void make_layout(const pic_params *p, Layout *L) {
     L->rho_q_last = take(ng * 8);
     L->rho_f32 = take(ng * 4);
     L->rho_w = take(ng * 16);
-    L->steps_acc = take(kStepsSlots * ng * 8);
+    L->steps_acc = take(kStepsSlots * ng * steps_acc_bytes(p));
     L->rho = take(ng * 8);
     L->phi = take(ng * 8);
     L->E64 = take(ng * 8);
@@ -200,6 +203,23 @@ void destroy_graphs(pic_run *r) {
     if (r->plain) { cudaGraphExecDestroy(r->plain); r->plain = nullptr; }
 }
 
+PushArgs64 push64_args(pic_run *r) {
+    PushArgs64 a;
+    a.x = (double *)r->xs(r->cur);
+    a.v = (double *)r->vs(r->cur);
+    a.n = r->p.npart;
+    a.E64 = r->at<double>(r->lay.E64);
+    a.rho_w = r->at<unsigned long long>(r->lay.rho_w);
+    a.partials = r->at<double>(r->lay.partials);
+    a.err = &r->dev()->err;
+    a.ng = r->p.ncell;
+    a.inv_dx = (double)r->p.ncell / r->p.length;
+    a.length = r->p.length;
+    a.qmdt = r->p.qm * r->p.dt;
+    a.dt = r->p.dt;
+    return a;
+}
+
 cudaError_t enqueue_push(pic_run *r, cudaStream_t s, bool push) {
     const int c = r->cur;
     if (r->p.precision == PIC_FP32_FIXED) {
@@ -226,19 +246,7 @@ cudaError_t enqueue_push(pic_run *r, cudaStream_t s, bool push) {
         a.c = r->pc;
         return launch_push_f32_atomic(a, r->grid, r->block, push, s);
     } else {
-        PushArgs64 a;
-        a.x = (double *)r->xs(c);
-        a.v = (double *)r->vs(c);
-        a.n = r->p.npart;
-        a.E64 = r->at<double>(r->lay.E64);
-        a.rho_w = r->at<unsigned long long>(r->lay.rho_w);
-        a.partials = r->at<double>(r->lay.partials);
-        a.err = &r->dev()->err;
-        a.ng = r->p.ncell;
-        a.inv_dx = (double)r->p.ncell / r->p.length;
-        a.length = r->p.length;
-        a.qmdt = r->p.qm * r->p.dt;
-        a.dt = r->p.dt;
+        const PushArgs64 a = push64_args(r);
         return launch_push_f64(a, r->grid, r->block, push, s);
     }
 }
@@ -378,6 +386,15 @@ int default_block(const pic_run *r) {
     return b;
 }
 
+// Threads of the float64 many-step launch's blocks: one node per thread, and 256
+// or 512 by the particles (us a step with 256, 512 and 1024: 2e4 particles, 64
+// cells 4.8, 5.9, 10.0; 1e5, 512 cells 8.8, 8.7, 12.3; 2e5, 100 cells 9.6, 8.5,
+// 11.8).
+int steps64_block(int64_t npart, int ncell) {
+    const int b = npart <= 65536 && ncell <= 256 ? 256 : 512;
+    return b < ncell ? 1024 : b;
+}
+
 // Shape of the many-step launch (steps.cu), or none: an exact fixed-point run
 // of one rank whose caller left the push's shape open, up to 24e6 particles on
 // up to 2048 cells and 12.5e6 on up to 4096.  Measured (us a step, this launch
@@ -386,6 +403,9 @@ int default_block(const pic_run *r) {
 //    512   34, 48.8 / 41, 48.4   50.8, 60.3 / 57.1, 62.6   97, 102 / 107, 109
 //   2048   38, 47.6 / 43, 48.8   53.1, 59.4 / 59.4, 62.0  100, 101 / 110, 108
 //   4096   45, 48.8 / 51, 51.8   60.3, 61.0 / 67.4, 64.6  107, 102 / 118, 109
+// Float64 runs (steps64.cu) up to 1e6 particles and 1024 cells: 2e4 on 64 cells
+// 4.8 and 15.3 us a step, 5e5 on 1000 20.0 and 26.6, 1e6 27.6 and 30.1; 4e6 on
+// 512 69.8 and 62.0.
 // One group of 4 particles per thread while that takes fewer blocks than SMs.
 // Runs of up to 131072 particles on up to 512 cells take 256 threads a block
 // (5e4 particles, 100 cells: 4.3 us a step against 4.6 with 512 and 5.8 with
@@ -393,20 +413,23 @@ int default_block(const pic_run *r) {
 cudaError_t set_steps_shape(pic_run *r) {
     r->steps_grid = 0;
     const pic_params &p = r->p;
-    if (p.precision != PIC_FP32_FIXED || p.field_solver != PIC_SOLVER_EXACT || !r->open_shape ||
-        r->npart_total != p.npart || p.ncell > kStepsMaxCells ||
-        p.npart > (p.ncell <= 2048 ? kStepsMaxParticles : kStepsMaxParticlesWide))
+    if (p.field_solver != PIC_SOLVER_EXACT || !r->open_shape || r->npart_total != p.npart) return cudaSuccess;
+    const bool f64 = p.precision == PIC_FP64;
+    if (f64 ? p.ncell > 1024 || p.npart > kSteps64MaxParticles
+            : p.precision != PIC_FP32_FIXED || p.ncell > kStepsMaxCells ||
+                  p.npart > (p.ncell <= 2048 ? kStepsMaxParticles : kStepsMaxParticlesWide))
         return cudaSuccess;
     int coop = 0;
     cudaError_t e = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, r->device);
     if (e != cudaSuccess || !coop) return e;
-    const int block = p.npart <= 131072 && p.ncell <= 512 ? 256 : 1024;
+    int block = p.npart <= 131072 && p.ncell <= 512 ? 256 : 1024;
+    if (f64) block = steps64_block(p.npart, p.ncell);
     int per_sm = 0;
-    e = steps_prepare(r->variant, p.ncell, block, &per_sm);
+    e = f64 ? steps64_prepare(p.ncell, block, &per_sm) : steps_prepare(r->variant, p.ncell, block, &per_sm);
     if (e != cudaSuccess || per_sm < 1) return e;
     const int most = (r->sms < kStepsMaxGrid ? r->sms : kStepsMaxGrid) - kStepsDiag;
     if (most < 1) return cudaSuccess;
-    const int64_t need = ((p.npart + 3) / 4 + block - 1) / block;
+    const int64_t need = ((f64 ? p.npart : (p.npart + 3) / 4) + block - 1) / block;
     r->steps_grid = (int)(need < most ? need : most) + kStepsDiag;
     r->steps_block = block;
     return cudaSuccess;
@@ -444,14 +467,17 @@ int run_steps(pic_run *r, int steps) {
     a.dstep = &r->dev()->step;
     a.steps = steps;
     a.c = r->pc;
-    a.weight_total = (long long)r->p.npart << kFixBits;
+    a.d = push64_args(r);
+    a.weight_total = (long long)((unsigned long long)r->p.npart << kFixBits);
     a.k_rho = r->k_rho;
     a.k_e = r->k_e;
     a.k_phi = r->k_phi;
     a.k_mode = 2.0 / (double)r->p.ncell;
     a.dx = r->dx;
     a.mass = r->mass;
-    PIC_CUDA(launch_steps(a, r->variant, r->steps_grid, r->steps_block, r->stream));
+    PIC_CUDA(r->p.precision == PIC_FP64
+                 ? launch_steps64(a, r->steps_grid, r->steps_block, r->stream)
+                 : launch_steps(a, r->variant, r->steps_grid, r->steps_block, r->stream));
     r->sync_base[0] += (unsigned)(r->steps_grid - kStepsDiag) * (unsigned)steps;
     for (int d = 0; d < kStepsDiag; d++)
         r->sync_base[1 + d] += (unsigned)((steps - d + kStepsDiag - 1) / kStepsDiag);
@@ -501,7 +527,7 @@ int prepare_loaded(pic_run *r, int64_t step, Units units, bool aux_copy = false)
     PIC_CUDA(cudaMemsetAsync(r->ws + r->lay.rho_q, 0, (size_t)r->p.ncell * 8, r->stream));
     PIC_CUDA(cudaMemsetAsync(r->ws + r->lay.rho_f32, 0, (size_t)r->p.ncell * 4, r->stream));
     PIC_CUDA(cudaMemsetAsync(r->ws + r->lay.rho_w, 0, (size_t)r->p.ncell * 16, r->stream));
-    PIC_CUDA(cudaMemsetAsync(r->ws + r->lay.steps_acc, 0, (size_t)r->p.ncell * 8 * kStepsSlots, r->stream));
+    PIC_CUDA(cudaMemsetAsync(r->ws + r->lay.steps_acc, 0, (size_t)r->p.ncell * steps_acc_bytes(&r->p) * kStepsSlots, r->stream));
     for (unsigned &v : r->sync_base) v = 0;        // as the counters in ds
     PIC_CUDA(cudaMemsetAsync(r->ws + r->lay.hist, 0xFF, (size_t)r->lay.hist_len * sizeof(pic_diag_row), r->stream));
     PIC_CUDA(enqueue_push(r, r->stream, false));

@@ -126,9 +126,10 @@ struct StepsArgs {
     float *E32;                   // field of the first step in, of the last one out
     double *E64, *phi, *rho;      // of the last step, out
     unsigned long long *rho_q_last; // idem
-    unsigned long long *acc;      // [kStepsSlots][NG] density sums, 0 between launches
-    double *partials;             // [kStepsSlots][kStepsMaxGrid] float4: per-block push sums as
-                                  // float32 pairs (sum v_old v_new and its rest, sum v_new, rest)
+    unsigned long long *acc;      // [kStepsSlots][NG] density sums ([NG][2] in float64, as rho_w),
+                                  // 0 between launches
+    double *partials;             // [kStepsSlots][kStepsMaxGrid][2]: per-block push sums (float32
+                                  // runs: as pairs of float32, sum and rest)
     unsigned *err;
     unsigned *sync;               // [4], 16-byte aligned: arrivals of the workers, steps
                                   // done by each diagnostics block; never reset ...
@@ -142,7 +143,8 @@ struct StepsArgs {
     long long *dstep;             // device step counter
     int steps;
     PushConsts c;
-    long long weight_total;       // N 2^24
+    PushArgs64 d;                 // float64 runs: x, v and the push's constants
+    long long weight_total;       // N 2^24 (fixed point)
     double k_rho, k_e, k_phi, k_mode, dx, mass;   // as SolveArgs
 };
 constexpr int kStepsMaxGrid = 256;
@@ -152,8 +154,11 @@ constexpr int kStepsPoolBlock = 1024;
 constexpr int kStepsMaxCells = 4096;
 // largest runs: up to 2048 cells, and beyond
 constexpr int64_t kStepsMaxParticles = 24000000, kStepsMaxParticlesWide = 12500000;
+constexpr int64_t kSteps64MaxParticles = 1000000;
 cudaError_t steps_prepare(int variant, int ng, int block, int *per_sm);
 cudaError_t launch_steps(StepsArgs a, int variant, int grid, int block, cudaStream_t s);
+cudaError_t steps64_prepare(int ng, int block, int *per_sm);
+cudaError_t launch_steps64(const StepsArgs &a, int grid, int block, cudaStream_t s);
 cudaError_t steps_pool_prepare(int *per_sm);
 int steps_pool_copies();
 cudaError_t launch_steps_pool(const StepsArgs *runs, int nrun, int grid, int ng_max, cudaStream_t s);

@@ -53,58 +53,12 @@
 //
 // Every wait has a limit (kSpinLimit polls, some seconds), after which the block
 // sets kErrWait and all blocks return.
-#include "field_ops.cuh"
-#include "particle_ops.cuh"
+#include "steps_common.cuh"
 
 namespace pic {
 namespace {
 
 constexpr int kResident = 2;               // groups of 4 particles a thread keeps
-constexpr unsigned kSpinLimit = 1u << 23;  // polls of one grid barrier
-
-// The launch's counters, never reset: arrivals of the workers, and the steps
-// that each diagnostics block is done with (StepsArgs::sync, on 16 bytes).
-__device__ __forceinline__ uint4 ld_acquire(const unsigned *p) {
-    uint4 v;
-    asm volatile("ld.acquire.gpu.global.v4.u32 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
-    return v;
-}
-
-__device__ __forceinline__ void red_release(unsigned *p) {
-    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(p) : "memory");
-}
-
-// Steps t <= last with t mod nd == d.
-__device__ __forceinline__ unsigned steps_of(int last, int d, int nd) {
-    return last < d ? 0u : (unsigned)((last - d) / nd + 1);
-}
-
-// Waits until all workers have arrived for step s, and, for a worker, until the
-// slot of step s + 1 has been given back by the diagnostics of step s + 1 -
-// kStepsSlots.  All threads of the block; false when the wait ran out.
-__device__ __forceinline__ bool wait_step(const StepsArgs &a, int s, int workers, bool worker,
-                                          int *dead) {
-    if (threadIdx.x == 0) {
-        const int nd = a.diag_blocks;
-        const unsigned target = a.base[0] + (unsigned)workers * (unsigned)(s + 1);
-        const unsigned d0 = a.base[1] + steps_of(s + 1 - kStepsSlots, 0, nd);
-        const unsigned d1 = a.base[2] + (nd > 1 ? steps_of(s + 1 - kStepsSlots, 1, nd) : 0u);
-        unsigned polls = 0;
-        for (;;) {
-            const uint4 v = ld_acquire(a.sync);
-            if ((int)(v.x - target) >= 0 && (!worker || ((int)(v.y - d0) >= 0 && (int)(v.z - d1) >= 0)))
-                break;
-            if (++polls >= kSpinLimit) {
-                atomicOr(a.err, kErrWait);
-                *dead = 1;
-                break;
-            }
-        }
-    }
-    __syncthreads();
-    return *dead == 0;
-}
 
 // Sum over a warp of 78-bit signed integers, in every lane.
 __device__ __forceinline__ i128 warp_sum_i78(i128 v) {
@@ -264,117 +218,27 @@ __device__ __forceinline__ void field_step(const StepsArgs &a, const unsigned lo
 // The diagnostics of a step, and after the last one the run's results.
 template <int K>
 __device__ __forceinline__ void diag_step(const StepsArgs &a, int s, int workers,
-                                       const unsigned long long *acc, const float4 *kv,
-                                       unsigned char *smem_raw, unsigned h0) {
+                                          const unsigned long long *acc, const float4 *kv,
+                                          unsigned char *smem_raw, unsigned h0) {
     __shared__ long long wr[32];
     __shared__ unsigned long long ws[64];
-    const int ng = a.c.ng, tid = threadIdx.x, lane = tid & 31, w = tid >> 5, nw = blockDim.x >> 5;
-    const bool last = s == a.steps - 1;
-    const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
     NodeSolve<K> ns;
-    solve_nodes<K>(ns, a, acc, ng, wr, ws);
-                    __shared__ float shf[2 * PIC_NMODES][32];
-            __shared__ double shd[8], fchunk[256], tot[2];
-            double *fe = reinterpret_cast<double *>(smem_raw);      // [ng], in the tile
-            NodeDiag d;
-            node_diag_reset(d);
-    #pragma unroll
-            for (int j = 0; j < K; j++) {
-                const int g = tid * K + j;
-                if (g >= ng) break;
-                const double E = a.k_e * i128_to_f64(ns.m[j]);
-                d.fe = 0.0;
-                node_diag(d, g, ng, E, (float)E);
-                fe[g] = d.fe;
-                if (last) {
-                    a.E64[g] = E;
-                    a.E32[g] = (float)E;
-                    a.rho[g] = a.k_rho * i128_to_f64((i128)ns.R[j]);
-                    a.rho_q_last[g] = ns.q[j];
-                }
-            }
-            float md[2 * PIC_NMODES];
-    #pragma unroll
-            for (int m = 0; m < PIC_NMODES; m++) { md[2 * m] = d.re[m]; md[2 * m + 1] = d.im[m]; }
-            static_assert(2 * PIC_NMODES == 16, "16 mode sums per warp");
-            const int used = (ng + 32 * K - 1) / (32 * K);          // warps with nodes
-            if (w < used) {
-                const float msum = warp_sum16_halving(md, lane);
-                if ((lane & 1) == 0) shf[lane >> 1][w] = msum;
-            }
-            __syncthreads();
-            const int chunks = (ng + 31) >> 5;
-            for (int i = w; i < chunks; i += nw) {                  // field energy of 32 nodes
-                const int g = 32 * i + lane;
-                const double sum = warp_sum_f64(g < ng ? fe[g] : 0.0);
-                if (lane == 0) fchunk[i] = sum;
-            }
-            if (w == nw - 1) {                                      // the push's sums
-                float4 p[kStepsMaxGrid / 32];                       // all loads in flight
-    #pragma unroll
-                for (int i = 0; i < kStepsMaxGrid / 32; i++)
-                    p[i] = 32 * i + lane < workers ? __ldcg(kv + 32 * i + lane) : zero4;
-    #pragma unroll
-                for (int i = 1; i < kStepsMaxGrid / 32; i++) {
-                    add_pair(p[0].x, p[0].y, p[i].x, p[i].y);
-                    add_pair(p[0].z, p[0].w, p[i].z, p[i].w);
-                }
-                warp_sum_pairs(p[0], 32);
-                if (lane == 0) {
-                    tot[0] = (double)p[0].x + (double)p[0].y;
-                    tot[1] = (double)p[0].z + (double)p[0].w;
-                }
-            }
-            __syncthreads();
-            const double fe_total = chunk_sum_f64(tid < chunks ? fchunk[tid] : 0.0, chunks, shd);
-            if (w == 0) {
-                const long long n = a.step0 + s + 1;
-                pic_diag_row *prev = &a.hist[(h0 + s) % a.hist_len], *row = &a.hist[(h0 + s + 1) % a.hist_len];
-                // one value per lane: kinetic energy and momentum of the row before,
-                // field energy and charge of this one
-                const double coef = lane == 0 ? 0.5 * a.mass : lane == 1 ? a.mass
-                                    : lane == 2 ? 0.5 * a.dx : a.dx * a.k_rho;
-                const double fe0 = __shfl_sync(kFull, fe_total, 0);
-                const double val = coef * (lane < 2 ? tot[lane] : lane == 2 ? fe0 : (double)ns.SR);
-                if (lane < 4) *(lane == 0 ? &prev->kinetic : lane == 1 ? &prev->momentum
-                                : lane == 2 ? &row->field : &row->charge) = val;
-                if (lane == 4) row->step = n;
-                // sum of rho_q: SR = NG (N 2^24 - it), 0 unless particles were lost
-                if (lane == 5) row->charge_q = ns.SR ? a.weight_total - ns.SR / ng : a.weight_total;
-                if (last && lane >= 6 && lane < 8)       // (otherwise the next step's, perhaps written already)
-                    *(lane == 6 ? &row->kinetic : &row->momentum) = __longlong_as_double(0x7ff8000000000000ll);
-                if (last && lane == 8) *a.dstep = n;
-            } else if (w == 1) {
-                // mode sums: float32 over 8 warps, float64 over those
-                double sum = 0.0;
-                for (int i0 = 0; i0 < used; i0 += 8) {
-                    float part = 0.0f;
-    #pragma unroll
-                    for (int i = 0; i < 8; i++)
-                        part += i0 + i < used ? shf[lane & 15][(i0 + i) & 31] : 0.0f;
-                    sum += (double)part;
-                }
-                const double im = __shfl_down_sync(kFull, sum, 1);
-                if (lane < 2 * PIC_NMODES && !(lane & 1))
-                    a.hist[(h0 + s + 1) % a.hist_len].mode[lane >> 1] =
-                        sqrt(sum * sum + im * im) * a.k_mode;
-            }
-            if (last) {
-                // Phi: sum_{k<g} M_k = NG (g P_g - sum_{j<=g} j R_j) - g SP
-                __shared__ unsigned long long scan64[4 * 32];
-                i128 jr = 0;
-    #pragma unroll
-                for (int j = 0; j < K; j++) jr += (i128)ns.R[j] * (i128)(tid * K + j);
-                i128 run = block_inclusive_scan2_i128(jr, 0, scan64).a - jr;
-    #pragma unroll
-                for (int j = 0; j < K; j++) {
-                    const int g = tid * K + j;
-                    if (g >= ng) break;
-                    run += (i128)ns.R[j] * (i128)g;
-                    const i128 sumM = (i128)ng * ((i128)g * (i128)ns.P[j] - run) - (i128)g * ns.SP;
-                    a.phi[g] = a.k_phi * i128_to_f64(sumM);
-                }
-            }
+    solve_nodes<K>(ns, a, acc, a.c.ng, wr, ws);
+    step_rows<K, true>(a, s, ns, smem_raw, h0, [&](double &k, double &m) {
+        const int lane = threadIdx.x & 31;
+        float4 p[kStepsMaxGrid / 32];                       // all loads in flight
+#pragma unroll
+        for (int i = 0; i < kStepsMaxGrid / 32; i++)
+            p[i] = 32 * i + lane < workers ? __ldcg(kv + 32 * i + lane) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int i = 1; i < kStepsMaxGrid / 32; i++) {
+            add_pair(p[0].x, p[0].y, p[i].x, p[i].y);
+            add_pair(p[0].z, p[0].w, p[i].z, p[i].w);
+        }
+        warp_sum_pairs(p[0], 32);
+        k = (double)p[0].x + (double)p[0].y;
+        m = (double)p[0].z + (double)p[0].w;
+    });
 }
 
 // With 4 nodes a thread both are called out of line, so that their registers (a
@@ -586,20 +450,6 @@ int log_copies(int variant, int block) { return variant != kDepositNgp && block 
 
 size_t steps_smem(int variant, int ng, int block) {
     return (size_t)(ng + 2) * (4 + (8 << log_copies(variant, block)));
-}
-
-// A launch whose blocks are all resident at once.
-void cooperative(cudaLaunchConfig_t &cfg, cudaLaunchAttribute *attr, int grid, int block, size_t smem,
-                 cudaStream_t s) {
-    cfg = cudaLaunchConfig_t{};
-    cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3((unsigned)block);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    attr[0].id = cudaLaunchAttributeCooperative;
-    attr[0].val.cooperative = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
 }
 
 }  // namespace

@@ -127,3 +127,49 @@ def test_a_captured_step_replays():
     b.step_n(4)
     for p, q in zip(c.get_cells(), b.get_cells()):
         assert np.array_equal(p, q)
+
+
+@pytest.mark.parametrize("n", [1, 2, 31, 32, 33, 255, 257, 20000, 100003])
+@pytest.mark.parametrize("ng", [1, 2, 31, 33, 64, 256, 257, 1000, 1024])
+def test_float64_steps_equal_the_two_kernels(n, ng):
+    # the float64 density is exact integers, so the launches agree bit for bit
+    rng = np.random.default_rng(3 * n + ng)
+    x = rng.uniform(0.0, L, n)
+    x[:1] = 0.0
+    x[1:2] = np.nextafter(L, 0.0)
+    v = rng.normal(0.0, 0.4, n)
+    runs = []
+    for kw in (dict(), dict(block_size=256)):
+        r = pic.Run(pic.Params(npart=n, ncell=ng, length=L, precision=pic.PIC_FP64, sort_interval=7, **kw),
+                    device="cuda:0")
+        r.init(x, v)
+        for k in (1, 6, 2, 9):
+            r.step_n(k)
+        runs.append(r)
+    a, b = runs
+    for p, q in zip(a.get_state(), b.get_state()):
+        assert np.array_equal(p, q)
+    f, g = a.get_field(), b.get_field()
+    for k in ("E", "rho", "phi"):
+        assert np.array_equal(f[k], g[k]), k
+    d, e = a.diagnostics(), b.diagnostics()
+    for k in ("step", "charge", "field"):
+        assert np.array_equal(d[k], e[k]), k
+    np.testing.assert_allclose(d["kinetic"][:-1], e["kinetic"][:-1], rtol=1e-13)
+    scale = L / n * np.abs(a.get_state()[1]).sum()
+    assert np.abs(d["momentum"][:-1] - e["momentum"][:-1]).max() <= 1e-13 * scale
+    assert np.isnan(d["kinetic"][-1])
+
+
+@pytest.mark.parametrize("n,ng", [(1000000, 1024), (1000001, 1024), (65537, 256), (1000, 1025)])
+def test_float64_steps_at_the_limits_of_the_launch(n, ng):
+    rng = np.random.default_rng(n)
+    x, v = rng.uniform(0.0, L, n), rng.normal(0.0, 0.2, n)
+    out = []
+    for kw in (dict(), dict(block_size=512)):
+        r = pic.Run(pic.Params(npart=n, ncell=ng, length=L, precision=pic.PIC_FP64, **kw), device="cuda:0")
+        r.init(x, v)
+        r.step_n(3)
+        out.append((*r.get_state(), r.get_field()["E"]))
+    for p, q in zip(*out):
+        assert np.array_equal(p, q)
