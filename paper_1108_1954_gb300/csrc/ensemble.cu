@@ -18,6 +18,7 @@
 #include <vector>
 
 #include "pic_internal.cuh"
+#include "staging.h"
 
 using namespace pic;
 
@@ -27,6 +28,7 @@ constexpr size_t kAlign = 256;
 // least idle arena space for a read-back's device conversion: below it the
 // pieces' launches and copies cost more than the host's own conversion
 constexpr size_t kMinScratch = 256 * 1024;
+constexpr size_t kStageRows = 512;     // history rows that fit the staging memory
 size_t align_up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign; }
 
 struct RunLayout {
@@ -150,6 +152,7 @@ struct pic_pool {
     int wide_clusters = 0;        // > 0: up to so many runs take blocks twice as large
     int sms = 0;
     int resident_sms = 0;         // SMs of the many-step launch (0: not available)
+    pic::Staging stage;
 
     BatchRun *d_runs() const { return reinterpret_cast<BatchRun *>(arena + tab.runs); }
     int *d_order() const { return reinterpret_cast<int *>(arena + tab.order); }
@@ -405,12 +408,21 @@ bool slot_ok(const pic_pool *pool, int32_t slot) {
     return pool && slot >= 0 && slot < (int)pool->slots.size() && pool->slots[slot].used;
 }
 
-int read_error(pic_pool *pool) {
+// Wait for the stream and what was queued into the staging memory; the error
+// word comes with it.  The caller holds the staging's mutex.
+int finish_read(pic_pool *pool) {
     unsigned err = 0;
-    PIC_CUDA(cudaMemcpyAsync(&err, pool->d_err(), sizeof(err), cudaMemcpyDeviceToHost, pool->stream));
-    PIC_CUDA(cudaStreamSynchronize(pool->stream));
+    cudaError_t e = pool->stage.add(&err, pool->d_err(), sizeof(err), pool->stream);
+    const cudaError_t f = pool->stage.finish(pool->stream);
+    if (e == cudaSuccess) e = f;
+    if (e != cudaSuccess) return cuda_fail(e);
     if (err & kErrWait) return PIC_ETIMEOUT;
     return err ? PIC_EDEVICE : PIC_OK;
+}
+
+int read_error(pic_pool *pool) {
+    std::lock_guard<std::mutex> lock(pool->stage.mutex);
+    return finish_read(pool);
 }
 
 }  // namespace
@@ -465,6 +477,7 @@ int pic_pool_create(const pic_pool_config *cfg, void *arena, size_t arena_bytes,
     if (e == cudaSuccess && coop) e = steps_pool_prepare(&per_sm);
     if (e != cudaSuccess) { delete pool; return cuda_fail(e); }
     if (per_sm > 0) pool->resident_sms = pool->sms;
+    pool->stage.create(kStageRows * sizeof(pic_diag_row) + 32 * (size_t)cfg->ncell_max + 1024);
     rc = set_shape(pool, cfg->variant ? cfg->variant : kPoolVariant,
                    cfg->cluster ? cfg->cluster : 8, cfg->block ? cfg->block : kPoolBlock);
     if (rc) { delete pool; return rc; }
@@ -740,12 +753,15 @@ int pic_pool_get_field(pic_pool *pool, int32_t slot, double *rho, double *phi, d
     const pic_pool::Slot &sl = pool->slots[slot];
     if (sl.needs_init) return PIC_ESTATE;
     const size_t nb = (size_t)sl.p.ncell * 8;
-    if (rho) PIC_CUDA(cudaMemcpyAsync(rho, sl.desc.rho, nb, cudaMemcpyDeviceToHost, pool->stream));
-    if (phi) PIC_CUDA(cudaMemcpyAsync(phi, sl.desc.phi, nb, cudaMemcpyDeviceToHost, pool->stream));
-    if (E) PIC_CUDA(cudaMemcpyAsync(E, sl.desc.E64, nb, cudaMemcpyDeviceToHost, pool->stream));
-    if (rho_q)
-        PIC_CUDA(cudaMemcpyAsync(rho_q, sl.desc.rho_q_last, nb, cudaMemcpyDeviceToHost, pool->stream));
-    return read_error(pool);
+    struct { void *dst; const void *src; } const want[] = {
+        {rho, sl.desc.rho}, {phi, sl.desc.phi}, {E, sl.desc.E64}, {rho_q, sl.desc.rho_q_last}};
+    std::lock_guard<std::mutex> lock(pool->stage.mutex);
+    for (const auto &w : want) {
+        if (!w.dst) continue;
+        const cudaError_t e = pool->stage.add(w.dst, w.src, nb, pool->stream);
+        if (e != cudaSuccess) { pool->stage.drop(); return cuda_fail(e); }
+    }
+    return finish_read(pool);
 }
 
 int pic_pool_diagnostics(pic_pool *pool, int32_t slot, int64_t first, int32_t count,
@@ -756,16 +772,18 @@ int pic_pool_diagnostics(pic_pool *pool, int32_t slot, int64_t first, int32_t co
     const int64_t H = pool->cfg.history;
     if (count == 0) return PIC_OK;
     if (first + count - 1 > sl.done || first < sl.done - H + 1) return PIC_EINVAL;
+    std::lock_guard<std::mutex> lock(pool->stage.mutex);
     int64_t got = 0;
     while (got < count) {
         const int64_t pos = (first + got) % H;
         int64_t len = count - got;
         if (pos + len > H) len = H - pos;
-        PIC_CUDA(cudaMemcpyAsync(rows + got, sl.desc.hist + pos, (size_t)len * sizeof(pic_diag_row),
-                                 cudaMemcpyDeviceToHost, pool->stream));
+        const cudaError_t e = pool->stage.add(rows + got, sl.desc.hist + pos,
+                                              (size_t)len * sizeof(pic_diag_row), pool->stream);
+        if (e != cudaSuccess) { pool->stage.drop(); return cuda_fail(e); }
         got += len;
     }
-    return read_error(pool);
+    return finish_read(pool);
 }
 
 int pic_pool_release(pic_pool *pool, int32_t slot) {
@@ -780,7 +798,6 @@ int pic_pool_release(pic_pool *pool, int32_t slot) {
 
 int pic_pool_sync(pic_pool *pool) {
     if (!pool) return PIC_EINVAL;
-    PIC_CUDA(cudaStreamSynchronize(pool->stream));
     return read_error(pool);
 }
 

@@ -13,6 +13,7 @@
 #include <new>
 
 #include "pic_internal.cuh"
+#include "staging.h"
 
 using namespace pic;
 
@@ -23,6 +24,7 @@ constexpr int kMaxPushGrid = 4096;     // per-block partial sums kept
 constexpr int kMaxSortChunks = 1024;
 constexpr int kPlainBlock = 16;        // steps per graph when not sorting
 constexpr int kDefaultHistory = 4096;
+constexpr size_t kStageRows = 512;     // history rows that fit the staging memory
 constexpr int64_t kMaxLaunchSteps = 1 << 20;   // of one many-step launch
 
 size_t align_up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign; }
@@ -115,18 +117,18 @@ void make_layout(const pic_params *p, Layout *L) {
     L->x[1] = take(n * es);
     L->v[1] = take(n * es);
     L->rho_q = take(ng * 8);
-    L->rho_q_last = take(ng * 8);
     L->rho_f32 = take(ng * 4);
     L->rho_w = take(ng * 16);
     L->steps_acc = take(kStepsSlots * ng * steps_acc_bytes(p));
     L->rho = take(ng * 8);
     L->phi = take(ng * 8);
     L->E64 = take(ng * 8);
+    L->rho_q_last = take(ng * 8);
+    L->dev = take(sizeof(DevScalars));
     L->E32 = take(ng * 4);
     L->partials = take((size_t)kMaxPushGrid * 2 * 8);
     L->hist_len = p->history > 0 ? p->history : kDefaultHistory;
     L->hist = take((size_t)L->hist_len * sizeof(pic_diag_row));
-    L->dev = take(sizeof(DevScalars));
     L->tune_rho = take(ng * 8);
     L->phase = take((size_t)kPhaseMaxBins * 4);
     sort_geometry(p->npart, p->ncell, &L->nchunk, &L->chunk, &L->nseg, &L->seg_len);
@@ -169,6 +171,7 @@ struct pic_run {
     bool ready = false, pending_push = false;
     cudaGraphExec_t period[2] = {nullptr, nullptr};   // S steps from x parity 0/1
     cudaGraphExec_t plain = nullptr;                  // kPlainBlock steps, no sort
+    pic::Staging stage;
     PushConsts pc{};
     double dx = 0, mass = 0, k_rho = 0, k_e = 0, k_phi = 0;
     double to_cells = 0, to_phys = 0;  // NG/L and L/NG (float32 positions)
@@ -497,13 +500,25 @@ cudaError_t join_aux(pic_run *r) {
     return e == cudaSuccess ? cudaStreamWaitEvent(r->stream, r->join, 0) : e;
 }
 
-int read_error_word(pic_run *r) {
-    unsigned err = 0;
-    PIC_CUDA(cudaMemcpyAsync(&err, &r->dev()->err, sizeof(err), cudaMemcpyDeviceToHost, r->stream));
-    PIC_CUDA(cudaStreamSynchronize(r->stream));
+int error_code(unsigned err) {
     if (err & kErrInput) return PIC_EINVAL;
     if (err & kErrWait) return PIC_ETIMEOUT;
     return err ? PIC_EDEVICE : PIC_OK;
+}
+
+// Wait for the stream and what was queued into the staging memory; the error
+// word comes with it.  The caller holds the staging's mutex.
+int finish_read(pic_run *r) {
+    unsigned err = 0;
+    cudaError_t e = r->stage.add(&err, &r->dev()->err, sizeof(err), r->stream);
+    const cudaError_t f = r->stage.finish(r->stream);
+    if (e == cudaSuccess) e = f;
+    return e != cudaSuccess ? cuda_fail(e) : error_code(err);
+}
+
+int read_error_word(pic_run *r) {
+    std::lock_guard<std::mutex> lock(r->stage.mutex);
+    return finish_read(r);
 }
 
 // How the positions in buffer 0 are given.
@@ -533,10 +548,9 @@ int prepare_loaded(pic_run *r, int64_t step, Units units, bool aux_copy = false)
     PIC_CUDA(enqueue_push(r, r->stream, false));
     PIC_CUDA(enqueue_solve(r, r->stream, false));
     if (aux_copy) PIC_CUDA(join_aux(r));
-    PIC_CUDA(cudaStreamSynchronize(r->stream));
+    const int rc = read_error_word(r);
     r->step = step;
     r->pending_push = false;
-    const int rc = read_error_word(r);
     r->ready = rc == PIC_OK;       // a rejected upload leaves no usable state
     return rc;
 }
@@ -600,6 +614,7 @@ int pic_create(const pic_params *p, void *workspace, size_t workspace_bytes,
     make_layout(p, &r->lay);
     if (workspace_bytes < r->lay.total) { delete r; return PIC_ENOMEM; }
     r->ws = (unsigned char *)workspace;
+    r->stage.create(kStageRows * sizeof(pic_diag_row) + 32 * (size_t)p->ncell + 1024);
     r->stream = (cudaStream_t)stream;
     cudaError_t e = cudaGetDevice(&r->device);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&r->sms, cudaDevAttrMultiProcessorCount, r->device);
@@ -699,7 +714,6 @@ int pic_get_cells(pic_run *run, float *u, void *v) {
     const size_t bytes = (size_t)run->p.npart * run->elem();
     if (u) PIC_CUDA(cudaMemcpyAsync(u, run->xs(run->cur), bytes, cudaMemcpyDeviceToHost, run->stream));
     if (v) PIC_CUDA(cudaMemcpyAsync(v, run->vs(run->cur), bytes, cudaMemcpyDeviceToHost, run->stream));
-    PIC_CUDA(cudaStreamSynchronize(run->stream));
     return read_error_word(run);
 }
 
@@ -787,7 +801,6 @@ int pic_step_n(pic_run *run, int64_t n) {
 
 int pic_sync(pic_run *run) {
     if (!run) return PIC_EINVAL;
-    PIC_CUDA(cudaStreamSynchronize(run->stream));
     return read_error_word(run);
 }
 
@@ -802,17 +815,18 @@ int pic_diagnostics(pic_run *run, int64_t first, int32_t count, pic_diag_row *ro
     if (count == 0) return PIC_OK;
     if (last > run->step || first < run->step - H + 1) return PIC_EINVAL;
     const pic_diag_row *hist = run->at<pic_diag_row>(run->lay.hist);
+    std::lock_guard<std::mutex> lock(run->stage.mutex);
     int64_t done = 0;
     while (done < count) {
         const int64_t slot = (first + done) % H;
         int64_t len = count - done;
         if (slot + len > H) len = H - slot;
-        PIC_CUDA(cudaMemcpyAsync(rows + done, hist + slot, (size_t)len * sizeof(pic_diag_row),
-                                 cudaMemcpyDeviceToHost, run->stream));
+        const cudaError_t e = run->stage.add(rows + done, hist + slot, (size_t)len * sizeof(pic_diag_row),
+                                             run->stream);
+        if (e != cudaSuccess) { run->stage.drop(); return cuda_fail(e); }
         done += len;
     }
-    PIC_CUDA(cudaStreamSynchronize(run->stream));
-    return read_error_word(run);
+    return finish_read(run);
 }
 
 int pic_get_state(pic_run *run, void *x, void *v) {
@@ -838,7 +852,6 @@ int pic_get_state(pic_run *run, void *x, void *v) {
         PIC_CUDA(cudaMemcpyAsync(x, src, bytes, cudaMemcpyDeviceToHost, run->stream));
     }
     if (v) PIC_CUDA(join_aux(run));
-    PIC_CUDA(cudaStreamSynchronize(run->stream));
     return read_error_word(run);
 }
 
@@ -846,18 +859,18 @@ int pic_get_field(pic_run *run, double *rho, double *phi, double *E, int64_t *rh
     pic::TraceRange trace_("pic_get_field");
     if (!run) return PIC_EINVAL;
     if (!run->ready) return PIC_ESTATE;
-    const size_t ng = (size_t)run->p.ncell;
-    if (rho) PIC_CUDA(cudaMemcpyAsync(rho, run->ws + run->lay.rho, ng * 8, cudaMemcpyDeviceToHost, run->stream));
-    if (phi) PIC_CUDA(cudaMemcpyAsync(phi, run->ws + run->lay.phi, ng * 8, cudaMemcpyDeviceToHost, run->stream));
-    if (E) PIC_CUDA(cudaMemcpyAsync(E, run->ws + run->lay.E64, ng * 8, cudaMemcpyDeviceToHost, run->stream));
-    if (rho_q) {
-        if (run->p.precision == PIC_FP32_FIXED)
-            PIC_CUDA(cudaMemcpyAsync(rho_q, run->ws + run->lay.rho_q_last, ng * 8, cudaMemcpyDeviceToHost, run->stream));
-        else
-            std::memset(rho_q, 0, ng * 8);
+    const size_t nb = (size_t)run->p.ncell * 8;
+    const bool fixed = run->p.precision == PIC_FP32_FIXED;
+    if (rho_q && !fixed) std::memset(rho_q, 0, nb);
+    struct { void *dst; size_t off; } const want[] = {
+        {rho, run->lay.rho}, {phi, run->lay.phi}, {E, run->lay.E64}, {fixed ? rho_q : nullptr, run->lay.rho_q_last}};
+    std::lock_guard<std::mutex> lock(run->stage.mutex);
+    for (const auto &w : want) {
+        if (!w.dst) continue;
+        const cudaError_t e = run->stage.add(w.dst, run->ws + w.off, nb, run->stream);
+        if (e != cudaSuccess) { run->stage.drop(); return cuda_fail(e); }
     }
-    PIC_CUDA(cudaStreamSynchronize(run->stream));
-    return read_error_word(run);
+    return finish_read(run);
 }
 
 int pic_phase_space(pic_run *run, int32_t nx, int32_t nv, double vmin, double vmax,
@@ -885,7 +898,6 @@ int pic_phase_space(pic_run *run, int32_t nx, int32_t nv, double vmin, double vm
         PIC_CUDA(launch_phase(a, run->sms, run->stream));
     }
     PIC_CUDA(cudaMemcpyAsync(counts, d, bytes, cudaMemcpyDeviceToHost, run->stream));
-    PIC_CUDA(cudaStreamSynchronize(run->stream));
     return read_error_word(run);
 }
 
