@@ -5,7 +5,7 @@
 // the error word).  Copies into page-locked memory are queued: they go down
 // together, the caller waits once, and the bytes are moved to where the caller
 // wants them.  What does not fit is copied straight to its place.  A run of 100 steps
-with its rows, field and error word took 851 us a call with pageable copies and 807 so.
+// with its rows, field and error word took 851 us a call with pageable copies and 807 so.
 #pragma once
 
 #include <cstddef>
