@@ -139,7 +139,7 @@ __device__ void cluster_finish(const SolveArgs &a, cg::cluster_group &cl, Cluste
     // the integer charge, with one barrier: warp sums by shuffles (the 16 mode
     // sums by recursive halving), then warp 0 across the warps, each mode sum by
     // one lane in warp order.
-    const double fe = warp_sum_f64(d.fe);
+    const double fe = warp_sum_fast(d.fe);
     unsigned long long cqb = q;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) cqb += __shfl_down_sync(kFull, cqb, o);

@@ -73,6 +73,23 @@ __device__ __forceinline__ I128Pair block_inclusive_scan2_i128(i128 a, i128 b,
     return r;
 }
 
+// The same of one value (w64: 2 x 32 words).
+__device__ __forceinline__ i128 block_inclusive_scan_i128(i128 a, unsigned long long *w64) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const i128 t = shfl_up_i128(a, o);
+        if (lane >= o) a += t;
+    }
+    if (lane == 31) {
+        w64[w] = (unsigned long long)a;
+        w64[32 + w] = (unsigned long long)(a >> 64);
+    }
+    __syncthreads();
+    for (int i = 0; i < w; i++) a += (i128)(((unsigned __int128)w64[32 + i] << 64) | w64[i]);
+    return a;
+}
+
 // Sum of three i128 values over the block (all threads get the sums).
 static __device__ void block_sum3_i128(i128 &a, i128 &b, i128 &c, i128 *sh /*[96]*/) {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -134,28 +151,6 @@ __device__ __forceinline__ double warp_sum_f64(double v) {
     return v;
 }
 
-// Field energy from the sums of 32 consecutive nodes each, of which thread c <
-// 256 holds number c (0 beyond the last): the one order in which the cluster
-// solve and the many-step launch add them, so that a run gives the same value
-// either way.  In thread 0; slot: 8 values; the whole block calls.
-__device__ __forceinline__ double chunk_sum_f64(double v, int chunks, double *slot) {
-    const int w = threadIdx.x >> 5, nw = (chunks + 31) >> 5;
-    if (w < nw) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            if (o >= chunks) continue;        // uniform: zeros only
-            const double u = __shfl_down_sync(kFull, v, o);
-            if ((threadIdx.x & 31) < o) v += u;
-        }
-        if ((threadIdx.x & 31) == 0) slot[w] = v;
-    }
-    __syncthreads();
-    double s = 0.0;
-    if (threadIdx.x == 0)
-        for (int i = 0; i < nw; i++) s += slot[i];
-    return s;
-}
-
 // Sum of float64 values over a warp, in every lane, as integers: 53-bit mantissas
 // with 5 bits below them, aligned to the largest exponent (|m| <= 2^58), added
 // in pieces of 27, 27 and 10 bits.  Each lane's value is rounded to 2^-58 of the
@@ -179,6 +174,25 @@ __device__ __forceinline__ double warp_sum_fixed(double p) {
     const unsigned long long v = (d & 0x800fffffffffffffull) | ((unsigned long long)(unsigned)ed << 52);
     if (emax == 0x7ffu || ed > 2046) return __longlong_as_double(0x7ff8000000000000ll);
     return sum == 0 || ed < 1 ? 0.0 : __longlong_as_double((long long)v);
+}
+
+// The same; sums that are infinite or not numbers as plain addition gives them.
+__device__ __forceinline__ double warp_sum_fast(double v) {
+    const double s = warp_sum_fixed(v);
+    return s == s ? s : __shfl_sync(kFull, warp_sum_f64(v), 0);         // uniform
+}
+
+// Field energy from the sums of 32 consecutive nodes each, of which thread c <
+// 256 holds number c (0 beyond the last): the one order in which the cluster
+// solve and the many-step launch add them, so that a run gives the same value
+// either way.  In warp 0; slot: 8 values; the whole block calls.
+__device__ __forceinline__ double chunk_sum_f64(double v, int chunks, double *slot) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = (chunks + 31) >> 5;
+    double s = w < nw ? warp_sum_fast(v) : 0.0;
+    if (nw == 1) return s;                            // uniform
+    if (w < nw && lane == 0) slot[w] = s;
+    __syncthreads();
+    return w == 0 ? warp_sum_fast(lane < nw ? slot[lane] : 0.0) : 0.0;
 }
 
 // Per-node diagnostics contribution of node g with field E (float64) and its

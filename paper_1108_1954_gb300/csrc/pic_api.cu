@@ -166,6 +166,7 @@ struct pic_run {
     bool open_shape = true;          // no launch shape asked for
     bool auto_variant = true;        // nor a deposit variant asked for or tuned
     int steps_grid = 0, steps_block = 0;   // many-step launch (0: not taken)
+    bool steps_small = false;              // one particle per lane
     unsigned sync_base[3] = {0, 0, 0};   // its counters so far
     int64_t step = 0;
     bool ready = false, pending_push = false;
@@ -409,10 +410,23 @@ int steps64_block(int64_t npart, int ncell) {
 // Float64 runs (steps64.cu) up to 1e6 particles and 1024 cells: 2e4 on 64 cells
 // 4.8 and 15.3 us a step, 5e5 on 1000 20.0 and 26.6, 1e6 27.6 and 30.1; 4e6 on
 // 512 69.8 and 62.0.
-// One group of 4 particles per thread while that takes fewer blocks than SMs.
-// Runs of up to 131072 particles on up to 512 cells take 256 threads a block
-// (5e4 particles, 100 cells: 4.3 us a step against 4.6 with 512 and 5.8 with
-// 1024; 2e5 particles, 1500 cells: 10.0 with 1024, 10.7 and 17.2).
+// Runs of few particles take them one per lane (steps_small; a lane's 4 in turn
+// are a chain 4 times as long), and small blocks, whose barriers cost less.  us
+// per step, groups of 4 in blocks of 256 (512) 1024 threads, and one per lane in
+// 256, 512, 1024 (unsorted, lattice start | Maxwellian):
+//   2e4 on 64      3.64 (3.80) 4.84   2.87  3.14  3.88 | 3.61 (3.79) 4.89  2.90  3.14  3.86
+//   5e4 on 100     3.59 (3.86) 4.95   3.08  3.11  3.89 | 3.59 (3.83) 4.92  3.60  3.32  3.89
+//   1.3e5 on 512   4.62 (4.47) 5.15    -    3.85  4.17 | 4.99 (4.50) 5.17   -    4.49  4.80
+//   3e5 on 300     5.16 (4.28) 5.10    -    4.37  4.35 | 5.65 (4.91) 5.15   -    5.05  5.05
+//   3e5 on 1000    6.89 (5.44) 6.23    -     -    5.34 | 7.38 (5.94) 6.32   -     -    5.91
+//   6e5 on 512     7.47 (5.45) 5.28    -    5.41  5.27 | 8.06 (6.06) 6.07   -    6.10  6.08
+//   1e6 on 1024    12.1 (8.48) 7.24    -     -    7.22
+// As many blocks as one group per thread takes, up to the SMs.
+void steps_shape(int64_t n, int ng, bool *small, int *block) {
+    *small = n <= 600000 && ng <= 1024;           // (one node per thread)
+    *block = !*small || ng > 512 || n > 400000 ? 1024 : ng > 256 || n > 40000 ? 512 : 256;
+}
+
 cudaError_t set_steps_shape(pic_run *r) {
     r->steps_grid = 0;
     const pic_params &p = r->p;
@@ -425,14 +439,15 @@ cudaError_t set_steps_shape(pic_run *r) {
     int coop = 0;
     cudaError_t e = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, r->device);
     if (e != cudaSuccess || !coop) return e;
-    int block = p.npart <= 131072 && p.ncell <= 512 ? 256 : 1024;
+    int block = 0, per_sm = 0;
     if (f64) block = steps64_block(p.npart, p.ncell);
-    int per_sm = 0;
-    e = f64 ? steps64_prepare(p.ncell, block, &per_sm) : steps_prepare(r->variant, p.ncell, block, &per_sm);
+    else steps_shape(p.npart, p.ncell, &r->steps_small, &block);
+    e = f64 ? steps64_prepare(p.ncell, block, &per_sm)
+            : steps_prepare(r->variant, p.ncell, block, r->steps_small, &per_sm);
     if (e != cudaSuccess || per_sm < 1) return e;
     const int most = (r->sms < kStepsMaxGrid ? r->sms : kStepsMaxGrid) - kStepsDiag;
     if (most < 1) return cudaSuccess;
-    const int64_t need = ((f64 ? p.npart : (p.npart + 3) / 4) + block - 1) / block;
+    const int64_t need = ((f64 || r->steps_small ? p.npart : (p.npart + 3) / 4) + block - 1) / block;
     r->steps_grid = (int)(need < most ? need : most) + kStepsDiag;
     r->steps_block = block;
     return cudaSuccess;
@@ -480,7 +495,7 @@ int run_steps(pic_run *r, int steps) {
     a.mass = r->mass;
     PIC_CUDA(r->p.precision == PIC_FP64
                  ? launch_steps64(a, r->steps_grid, r->steps_block, r->stream)
-                 : launch_steps(a, r->variant, r->steps_grid, r->steps_block, r->stream));
+                 : launch_steps(a, r->variant, r->steps_grid, r->steps_block, r->steps_small, r->stream));
     r->sync_base[0] += (unsigned)(r->steps_grid - kStepsDiag) * (unsigned)steps;
     for (int d = 0; d < kStepsDiag; d++)
         r->sync_base[1 + d] += (unsigned)((steps - d + kStepsDiag - 1) / kStepsDiag);

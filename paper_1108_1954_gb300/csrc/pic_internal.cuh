@@ -155,8 +155,8 @@ constexpr int kStepsMaxCells = 4096;
 // largest runs: up to 2048 cells, and beyond
 constexpr int64_t kStepsMaxParticles = 24000000, kStepsMaxParticlesWide = 12500000;
 constexpr int64_t kSteps64MaxParticles = 1000000;
-cudaError_t steps_prepare(int variant, int ng, int block, int *per_sm);
-cudaError_t launch_steps(StepsArgs a, int variant, int grid, int block, cudaStream_t s);
+cudaError_t steps_prepare(int variant, int ng, int block, bool small, int *per_sm);
+cudaError_t launch_steps(StepsArgs a, int variant, int grid, int block, bool small, cudaStream_t s);
 cudaError_t steps64_prepare(int ng, int block, int *per_sm);
 cudaError_t launch_steps64(const StepsArgs &a, int grid, int block, cudaStream_t s);
 cudaError_t steps_pool_prepare(int *per_sm);

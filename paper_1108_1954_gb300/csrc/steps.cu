@@ -8,7 +8,7 @@
 //
 //   push     each block pushes its contiguous part of the particles and deposits
 //            into its own tile (the device code of push.cu).  A thread keeps its
-//            first kResident groups of 4 particles in registers from step to step;
+//            first kResident groups of particles in registers from step to step;
 //   flush    the tile is added to one of kStepsSlots global accumulators, used
 //            in turn;
 //   barrier  arrivals counted in global memory, a bounded spin;
@@ -20,25 +20,33 @@
 // Two more blocks have no particles.  They take the steps in turn and, while
 // the workers go on, compute a step's diagnostics (float64 work that would hold
 // the workers up: at 64 clocks a dependent float64 add and 840 a square root,
-// a step's take 8 to 16 thousand clocks, up to twice a worker's step), then
+// a step's take 5 to 10 thousand clocks, up to twice a worker's step), then
 // clear the step's accumulator and give it back; a worker waits only if the
 // diagnostics fall kStepsSlots - 1 steps behind.  After the last step they
 // write E, Phi, rho and the consumed sums.
 //
+// Up to 6e5 particles on up to 1024 cells the lanes take particles one by one
+// (SMALL), beyond that in groups of 4 (16-byte loads; in a small run only a
+// longer chain per lane: pic_api.cu, steps_shape).
+//
 // What a step costs (GB300, us): launches of push and solve before, and here
-//   2e4 particles, 64 cells, one step a call   16.4   11.0
-//   5e4, 100 cells                             14.0    4.3
-//   5e5, 300 cells                             18.5    7.1
-//   1e6, 1024 cells, sorted every 20           22.5   10.7
-//   3e6, 777 cells, NGP, sorted every 10       27.4   17.8
-//   4.2e6, 2048 cells, sorted every 20         31.0   22.8
-//   1e6, 4096 cells                            24.8   16.0
-//   1.2e7, 2048 cells, sorted every 20         52.9   43.0
-// of which, at 5e4 (clocks): push 2300, sums 380, flush 1040, barrier 2400 (the
+//   2e4 particles, 64 cells, one step a call   16.4   10.2
+//   2e4, 64 cells                              13.4    2.9
+//   5e4, 100 cells                             14.0    3.1
+//   5e5, 300 cells                             18.5    5.2
+//   1e6, 1024 cells, sorted every 20           22.5    9.0
+//   3e6, 777 cells, NGP, sorted every 10       27.4   14.0
+//   4.2e6, 2048 cells, sorted every 20         31.0   19.2
+//   1e6, 4096 cells                            24.8   11.4
+//   1.2e7, 2048 cells, sorted every 20         52.9   41.3
+// of which, at 5e4 (clocks): push 700, sums 380, flush 1040, barrier 2400 (the
 // adds' release and a poll, each a trip to L2), solve 1300 (900 the sums' way
-// from L2), E 510.  Large runs' pushes stream from memory, for which the two
-// launches have more warps, and a thread with 8 nodes runs out of registers
-// (1e6 particles on 6000 cells: 31 us against 28): set_steps_shape.
+// from L2), E 510.  Counting a node's arrivals in the upper bits of its sum, so
+// that a block waits for the sums themselves, saves the release's trip but the
+// polls of all nodes hold up the adds: 4.1 us a step at 5e4.  Large runs' pushes
+// stream from memory, for which the two launches have more warps, and a thread
+// with 8 nodes runs out of registers (1e6 particles on 6000 cells: 31 us against
+// 28): set_steps_shape.
 //
 // The solve in 64 bits.  R_g = N 2^24 - NG rho_q[g] and its prefix sums P_g are
 // below N NG 2^24 in magnitude, so they fit 64 bits for N NG <= 2^38 (the
@@ -58,7 +66,7 @@
 namespace pic {
 namespace {
 
-constexpr int kResident = 2;               // groups of 4 particles a thread keeps
+constexpr int kResident = 2;               // groups of particles a thread keeps
 
 // Sum over a warp of 78-bit signed integers, in every lane.
 __device__ __forceinline__ i128 warp_sum_i78(i128 v) {
@@ -119,21 +127,29 @@ __device__ __forceinline__ void warp_sum_pairs(float4 &p, int n) {
     }
 }
 
-// Push and deposit the first m of a group's 4 particles.
-template <bool NGP>
-__device__ __forceinline__ void step4(float4 &x, float4 &v, int m, const float *sE, const Tile &t,
-                                      const PushConsts &c, unsigned *err, float &ke, float &mom) {
-    float xs[4] = {x.x, x.y, x.z, x.w}, vs[4] = {v.x, v.y, v.z, v.w};
+// The W particles of a lane's group, as one word.
+template <int W> struct Group { using T = float4; };
+template <> struct Group<1> { using T = float; };
+
+// Push and deposit the first m of a group's W particles.
+template <bool NGP, int W>
+__device__ __forceinline__ void step_group(typename Group<W>::T &x, typename Group<W>::T &v, int m,
+                                           const float *sE, const Tile &t, const PushConsts &c,
+                                           unsigned *err, float &ke, float &mom) {
+    using T = typename Group<W>::T;
+    alignas(16) float xs[W], vs[W];
+    *reinterpret_cast<T *>(xs) = x;
+    *reinterpret_cast<T *>(vs) = v;
 #pragma unroll
-    for (int k = 0; k < 4; k++) {
+    for (int k = 0; k < W; k++) {
         if (k >= m) continue;
         if (NGP) push_particle_ngp(xs[k], vs[k], sE, c, ke, mom);
         else push_particle(xs[k], vs[k], sE, c, ke, mom);
     }
-    if (NGP) deposit_ngp<4>(t, xs, m, c, err);
-    else deposit_cells<4>(t, xs, m, c, err);
-    x = make_float4(xs[0], xs[1], xs[2], xs[3]);
-    v = make_float4(vs[0], vs[1], vs[2], vs[3]);
+    if (NGP) deposit_ngp<W>(t, xs, m, c, err);
+    else deposit_cells<W>(t, xs, m, c, err);
+    x = *reinterpret_cast<const T *>(xs);
+    v = *reinterpret_cast<const T *>(vs);
 }
 
 // The field of the whole grid, in thread t's K nodes K t ... K t + K - 1.
@@ -258,12 +274,14 @@ __device__ __noinline__ void diag_step_call(const StepsArgs &a, int s, int worke
 }
 
 // Block b of a run's workers + nd: all its steps.
-template <int VARIANT, int K>
+template <int VARIANT, int K, bool SMALL>
 __device__ __forceinline__ void run_many_steps(const StepsArgs &a, unsigned char *smem_raw, const int b,
                                                const int workers) {
     __shared__ float4 kvs[32];                    // per warp: (ke, ke low, mom, mom low)
     __shared__ int dead;
     constexpr bool kNgp = VARIANT == kDepositNgp;
+    constexpr int kW = SMALL ? 1 : 4;             // particles of a group
+    using G = typename Group<kW>::T;
     const PushConsts c = a.c;
     const int ng = c.ng;
     const int words = (ng + 2) << a.log_copies, K_ = 1 << a.log_copies;
@@ -287,22 +305,21 @@ __device__ __forceinline__ void run_many_steps(const StepsArgs &a, unsigned char
     clear_tile();
     for (int j = tid; j < ng + 2; j += bs) sE[j] = a.E32[j == 0 ? ng - 1 : (j == ng + 1 ? 0 : j - 1)];
     // this block's groups [q0, q1); the thread's groups q0 + tid + i bs, the first
-    // kResident of them in registers.  The run's last group may hold fewer than 4
+    // kResident of them in registers.  The run's last group may hold fewer than kW
     // particles; its other words are padding of the arrays.
-    const int n4 = (int)((a.n + 3) >> 2), left = (int)(a.n - 4ll * (n4 - 1));    // n4 <= 2^30
-    const int q0 = diag ? 0 : (int)((long long)n4 * b / workers);
-    const int q1 = diag ? 0 : (int)((long long)n4 * (b + 1) / workers);
+    const int nq = (int)((a.n + kW - 1) / kW), left = (int)(a.n - (long long)kW * (nq - 1));  // nq <= 2^30
+    const int q0 = diag ? 0 : (int)((long long)nq * b / workers);
+    const int q1 = diag ? 0 : (int)((long long)nq * (b + 1) / workers);
     const unsigned h0 = diag ? (unsigned)(a.step0 % a.hist_len) : 0u;     // history slot of the first step
-    auto members = [&](int q) { return q >= q1 ? 0 : q == n4 - 1 ? left : 4; };
-    float4 *x4 = reinterpret_cast<float4 *>(a.x);
-    float4 *v4 = reinterpret_cast<float4 *>(a.v);
-    const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
-    float4 rx[kResident], rv[kResident];
+    auto members = [&](int q) { return q >= q1 ? 0 : q == nq - 1 ? left : kW; };
+    G *xg = reinterpret_cast<G *>(a.x);
+    G *vg = reinterpret_cast<G *>(a.v);
+    G rx[kResident], rv[kResident];
 #pragma unroll
     for (int i = 0; i < kResident; i++) {
         const int q = q0 + tid + i * bs;
-        rx[i] = q < q1 ? __ldcg(x4 + q) : zero4;
-        rv[i] = q < q1 ? __ldcg(v4 + q) : zero4;
+        rx[i] = q < q1 ? __ldcg(xg + q) : G{};
+        rv[i] = q < q1 ? __ldcg(vg + q) : G{};
     }
     __syncthreads();
     for (int s = diag ? b - workers : 0; s < a.steps; s += diag ? nd : 1) {
@@ -313,27 +330,27 @@ __device__ __forceinline__ void run_many_steps(const StepsArgs &a, unsigned char
         if (!diag) {
             float ke = 0.0f, mom = 0.0f;
             const int qs = q0 + tid + kResident * bs;
-            float4 cx = qs < q1 ? __ldcg(x4 + qs) : zero4, cv = qs < q1 ? __ldcg(v4 + qs) : zero4;
+            G cx = qs < q1 ? __ldcg(xg + qs) : G{}, cv = qs < q1 ? __ldcg(vg + qs) : G{};
 #pragma unroll
             for (int i = 0; i < kResident; i++) {
                 const int m = members(q0 + tid + i * bs);
-                if (m) step4<kNgp>(rx[i], rv[i], m, sE, tile, c, a.err, ke, mom);
+                if (m) step_group<kNgp, kW>(rx[i], rv[i], m, sE, tile, c, a.err, ke, mom);
             }
             for (int q = qs; q < q1; q += bs) {
-                float4 xx = cx, vv = cv;
+                G xx = cx, vv = cv;
                 const int qn = q + bs;
-                cx = qn < q1 ? __ldcg(x4 + qn) : zero4;
-                cv = qn < q1 ? __ldcg(v4 + qn) : zero4;
-                step4<kNgp>(xx, vv, members(q), sE, tile, c, a.err, ke, mom);
-                __stcg(x4 + q, xx);
-                __stcg(v4 + q, vv);
+                cx = qn < q1 ? __ldcg(xg + qn) : G{};
+                cv = qn < q1 ? __ldcg(vg + qn) : G{};
+                step_group<kNgp, kW>(xx, vv, members(q), sE, tile, c, a.err, ke, mom);
+                __stcg(xg + q, xx);
+                __stcg(vg + q, vv);
             }
             float4 sums = make_float4(ke, 0.0f, mom, 0.0f);
             warp_sum_pairs(sums, 32);
             if (lane == 0) kvs[w] = sums;
             __syncthreads();
             if (w == nw - 1) {                        // the block's sums, still as pairs
-                float4 p = lane < nw ? kvs[lane] : zero4;
+                float4 p = lane < nw ? kvs[lane] : make_float4(0.f, 0.f, 0.f, 0.f);
                 warp_sum_pairs(p, nw);
                 if (lane == 0) kv[b] = p;
             }
@@ -393,16 +410,16 @@ __device__ __forceinline__ void run_many_steps(const StepsArgs &a, unsigned char
         for (int i = 0; i < kResident; i++) {
             const int q = q0 + tid + i * bs;
             if (q >= q1) break;
-            __stcg(x4 + q, rx[i]);
-            __stcg(v4 + q, rv[i]);
+            __stcg(xg + q, rx[i]);
+            __stcg(vg + q, rv[i]);
         }
     }
 }
 
-template <int VARIANT, int K>
+template <int VARIANT, int K, bool SMALL>
 __global__ void __launch_bounds__(1024, 1) pic_steps_kernel(const __grid_constant__ StepsArgs a) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    run_many_steps<VARIANT, K>(a, smem_raw, blockIdx.x, (int)gridDim.x - a.diag_blocks);
+    run_many_steps<VARIANT, K, SMALL>(a, smem_raw, blockIdx.x, (int)gridDim.x - a.diag_blocks);
 }
 
 // Several runs side by side, each on its own blocks (a.first_block on), none
@@ -417,27 +434,30 @@ __global__ void __launch_bounds__(1024, 1) pic_steps_pool_kernel(const StepsArgs
         reinterpret_cast<unsigned *>(&a)[k] = reinterpret_cast<const unsigned *>(runs + i)[k];
     __syncthreads();
     const int b = (int)blockIdx.x - a.first_block, workers = a.blocks - a.diag_blocks;
-    if (a.c.ng <= 1024) run_many_steps<kDepositCells, 1>(a, smem_raw, b, workers);
-    else if (a.c.ng <= 2048) run_many_steps<kDepositCells, 2>(a, smem_raw, b, workers);
-    else run_many_steps<kDepositCells, 4>(a, smem_raw, b, workers);
+    // a lane's 4 particles or fewer: one by one (pic_api.cu, steps_shape)
+    if (a.c.ng <= 1024 && a.n <= 4ll * workers * kStepsPoolBlock)
+        run_many_steps<kDepositCells, 1, true>(a, smem_raw, b, workers);
+    else if (a.c.ng <= 1024) run_many_steps<kDepositCells, 1, false>(a, smem_raw, b, workers);
+    else if (a.c.ng <= 2048) run_many_steps<kDepositCells, 2, false>(a, smem_raw, b, workers);
+    else run_many_steps<kDepositCells, 4, false>(a, smem_raw, b, workers);
 }
 
 using StepsKernel = void (*)(StepsArgs);
 
 template <int V>
-StepsKernel pick_nodes(int per_thread) {
+StepsKernel pick_nodes(int per_thread, bool small) {
     switch (per_thread) {
-        case 1: return &pic_steps_kernel<V, 1>;
-        case 2: return &pic_steps_kernel<V, 2>;
-        case 4: return &pic_steps_kernel<V, 4>;
+        case 1: return small ? &pic_steps_kernel<V, 1, true> : &pic_steps_kernel<V, 1, false>;
+        case 2: return &pic_steps_kernel<V, 2, false>;
+        case 4: return &pic_steps_kernel<V, 4, false>;
         default: return nullptr;
     }
 }
 
-StepsKernel pick_steps(int variant, int ng, int block) {
+StepsKernel pick_steps(int variant, int ng, int block, bool small) {
     int k = 1;
     while (k * block < ng) k *= 2;
-    return variant == kDepositNgp ? pick_nodes<kDepositNgp>(k) : pick_nodes<kDepositCells>(k);
+    return variant == kDepositNgp ? pick_nodes<kDepositNgp>(k, small) : pick_nodes<kDepositCells>(k, small);
 }
 
 // Copies of a block's tile, lanes alternating between them: lanes of one cell
@@ -454,9 +474,9 @@ size_t steps_smem(int variant, int ng, int block) {
 
 }  // namespace
 
-cudaError_t steps_prepare(int variant, int ng, int block, int *per_sm) {
+cudaError_t steps_prepare(int variant, int ng, int block, bool small, int *per_sm) {
     *per_sm = 0;
-    StepsKernel k = pick_steps(variant, ng, block);
+    StepsKernel k = pick_steps(variant, ng, block, small);
     if (!k) return cudaSuccess;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)steps_smem(variant, kStepsMaxCells, block));
@@ -465,8 +485,8 @@ cudaError_t steps_prepare(int variant, int ng, int block, int *per_sm) {
                                                          steps_smem(variant, ng, block));
 }
 
-cudaError_t launch_steps(StepsArgs a, int variant, int grid, int block, cudaStream_t s) {
-    StepsKernel k = pick_steps(variant, a.c.ng, block);
+cudaError_t launch_steps(StepsArgs a, int variant, int grid, int block, bool small, cudaStream_t s) {
+    StepsKernel k = pick_steps(variant, a.c.ng, block, small);
     if (!k) return cudaErrorInvalidValue;
     a.log_copies = log_copies(variant, block);
     cudaLaunchConfig_t cfg;

@@ -66,6 +66,14 @@ __device__ __forceinline__ void step_rows(const StepsArgs &a, int s, const Solve
     __shared__ float shf[2 * PIC_NMODES][32];
     __shared__ double shd[8], fchunk[256], tot[2];
     double *fe = reinterpret_cast<double *>(smem_raw);      // [ng], in the tile
+    if (w == nw - 1) {       // the push's sums: the warp without nodes, where there is one
+        double k, m;
+        sums(k, m);
+        if (lane == 0) {
+            tot[0] = k;
+            tot[1] = m;
+        }
+    }
     NodeDiag d;
     node_diag_reset(d);
 #pragma unroll
@@ -96,16 +104,8 @@ __device__ __forceinline__ void step_rows(const StepsArgs &a, int s, const Solve
     const int chunks = (ng + 31) >> 5;
     for (int i = w; i < chunks; i += nw) {                  // field energy of 32 nodes
         const int g = 32 * i + lane;
-        const double sum = warp_sum_f64(g < ng ? fe[g] : 0.0);
+        const double sum = warp_sum_fast(g < ng ? fe[g] : 0.0);
         if (lane == 0) fchunk[i] = sum;
-    }
-    if (w == nw - 1) {                                      // the push's sums
-        double k, m;
-        sums(k, m);
-        if (lane == 0) {
-    tot[0] = k;
-    tot[1] = m;
-        }
     }
     __syncthreads();
     const double fe_total = chunk_sum_f64(tid < chunks ? fchunk[tid] : 0.0, chunks, shd);
@@ -126,7 +126,8 @@ __device__ __forceinline__ void step_rows(const StepsArgs &a, int s, const Solve
         if (last && lane >= 6 && lane < 8)       // (otherwise the next step's, perhaps written already)
             *(lane == 6 ? &row->kinetic : &row->momentum) = __longlong_as_double(0x7ff8000000000000ll);
         if (last && lane == 8) *a.dstep = n;
-    } else if (w == 1) {
+    }
+    if (w == nw - 1) {
         // mode sums: float32 over 8 warps, float64 over those
         double sum = 0.0;
         for (int i0 = 0; i0 < used; i0 += 8) {
@@ -143,11 +144,11 @@ __device__ __forceinline__ void step_rows(const StepsArgs &a, int s, const Solve
     }
     if (last) {
         // Phi: sum_{k<g} M_k = NG (g P_g - sum_{j<=g} j R_j) - g SP
-        __shared__ unsigned long long scan64[4 * 32];
+        __shared__ unsigned long long scan64[2 * 32];
         i128 jr = 0;
 #pragma unroll
         for (int j = 0; j < K; j++) jr += (i128)ns.R[j] * (i128)(tid * K + j);
-        i128 run = block_inclusive_scan2_i128(jr, 0, scan64).a - jr;
+        i128 run = block_inclusive_scan_i128(jr, scan64) - jr;
 #pragma unroll
         for (int j = 0; j < K; j++) {
             const int g = tid * K + j;

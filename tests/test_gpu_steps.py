@@ -173,3 +173,15 @@ def test_float64_steps_at_the_limits_of_the_launch(n, ng):
         out.append((*r.get_state(), r.get_field()["E"]))
     for p, q in zip(*out):
         assert np.array_equal(p, q)
+
+
+@pytest.mark.parametrize("n,ng", [(40000, 256), (40001, 256), (40000, 257), (400000, 512), (400001, 512),
+                                  (400001, 513), (600000, 1024), (600001, 1024), (600000, 1025)])
+@pytest.mark.parametrize("shape", [pic.PIC_SHAPE_CIC, pic.PIC_SHAPE_NGP])
+def test_steps_at_the_limits_of_one_particle_per_lane(n, ng, shape):
+    # where the lanes' groups and the block size change; integers, so bit for bit
+    a, b = pair(n, ng, shape=shape)
+    for k in (1, 7):
+        a.step_n(k), b.step_n(k)
+        assert_same(a, b, n, ng)
+    a.close(), b.close()
