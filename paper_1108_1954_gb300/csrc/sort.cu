@@ -35,6 +35,21 @@ __device__ __forceinline__ unsigned cell_key(T x, T inv_dx, int ng) {
     return (unsigned)u;
 }
 
+// The same for float64: one float64 instruction, the product, and the clamps and
+// the truncation on its bits.  The comparisons and the conversion take the
+// float64 pipe too, at 16 clocks a warp each, and bounded both passes (2^24
+// particles: count 148 us, 42 so; scatter 162, 122 so).
+__device__ __forceinline__ unsigned cell_key(double x, double inv_dx, int ng) {
+    const double u = x * inv_dx;
+    const int hi = __double2hiint(u);
+    const unsigned top = (unsigned)(ng - 1);
+    if (hi < 0x3ff00000) return 0u;                       // u < 1, negative
+    if (hi >= 0x7ff00000) return hi == 0x7ff00000 && __double2loint(u) == 0 ? top : 0u;  // inf, NaN
+    const int e = (hi >> 20) - 1023;
+    const unsigned j = e > 20 ? top : (((unsigned)hi & 0xfffffu) | 0x100000u) >> (20 - e);
+    return j < top ? j : top;
+}
+
 template <typename T>
 __global__ void __launch_bounds__(kSortThreads) sort_count_kernel(SortArgs<T> a) {
     extern __shared__ unsigned sh_count[];

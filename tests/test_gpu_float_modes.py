@@ -96,3 +96,21 @@ def test_a_particle_thrown_out_of_the_box_is_flagged(precision, bad):
     with pytest.raises(pic.PicError) as e:
         run.sync()
     assert e.value.code == pic.PIC_EDEVICE
+
+
+@pytest.mark.parametrize("n,ng", [(1, 1), (7, 2), (1000, 3), (100003, 100), (100003, 1024), (300001, 8192)])
+def test_float64_sort_is_the_stable_order_by_cell(n, ng):
+    # cell edges and their neighbours among the positions; the key is that of
+    # plain float64 arithmetic, so the order is the same particle for particle
+    rng = np.random.default_rng(n + ng)
+    x, v = state(n, ng, n)
+    k = n // 2
+    edge = rng.integers(0, ng + 1, k) / (ng / L)
+    x[n - k:] = np.clip(np.nextafter(edge, edge + rng.choice([-1.0, 0.0, 1.0], k)), 0.0, np.nextafter(L, 0.0))
+    run = pic.Run(pic.Params(npart=n, ncell=ng, length=L, precision=pic.PIC_FP64, sort_interval=4),
+                  device="cuda:0")
+    run.init(x, v)
+    run.sort()
+    order = np.argsort(np.minimum((x * (ng / L)).astype(np.int64), ng - 1), kind="stable")
+    assert np.array_equal(run.get_state()[0], x[order])
+    run.close()
