@@ -5,18 +5,27 @@
 // field reads broadcasts and lets its deposit aggregate equal nodes before the
 // shared-memory atomics.  It changes no physical quantity.
 //
-// Five passes, all deterministic and stable (particles of one cell keep their
-// relative order):
+// Four passes (five beyond 1024 cells), all deterministic and stable (particles
+// of one cell keep their relative order):
 //   count    block b counts the cells of its contiguous chunk -> hist[b][g]
 //   colscan  per (segment of chunks, cell): exclusive prefix over the chunks
 //            of the segment, in place, and the segment total
-//   segscan  per cell: exclusive prefix over the segments, in place, and the
-//            cell total
-//   base     exclusive prefix of the cell totals over the cells -> base[g]
+//   base     per cell: exclusive prefix over the segments, in place, and the
+//            cell total (many cells: a pass of its own, segscan); exclusive prefix
+//            of those over the cells -> base[g]
 //   scatter  block b walks its chunk in order, 512 particles at a time
 //            (64 consecutive per warp); the warps take their slots from the
 //            per-cell cursors one after the other, so the order within a
 //            cell is the original order.
+// A small sort is launches, not work (1e6 particles, 1024 cells: passes of 3, 3, 2
+// and 8 us), so each pass but the first is launched with programmatic
+// serialisation: its blocks come up while the pass ahead still runs, and wait
+// for that pass (and so for all before it: each waits before it ends) where
+// they first read its results.  The scatter has loaded its first particles by
+// then; those are complete before the count begins, which waits for everything
+// ahead of it in the stream.  A sort, us, five plain launches before and here: 2e4
+// particles on 64 cells 24.5, 13.5; 1e6 on 1024 27.2, 19.9; 4.2e6 on 2048 47.3,
+// 37.4; 1.2e7 on 4096 115.5, 108.7; 2^26 on 4096 390, 388.
 // The destination index is bounds-checked; a violation sets the device error
 // word instead of writing.
 #include "pic_internal.cuh"
@@ -53,6 +62,7 @@ __device__ __forceinline__ unsigned cell_key(double x, double inv_dx, int ng) {
 template <typename T>
 __global__ void __launch_bounds__(kSortThreads) sort_count_kernel(SortArgs<T> a) {
     extern __shared__ unsigned sh_count[];
+    cudaTriggerProgrammaticLaunchCompletion();
     const int ng = a.ng;
     for (int g = threadIdx.x; g < ng; g += blockDim.x) sh_count[g] = 0u;
     __syncthreads();
@@ -135,6 +145,8 @@ __device__ __forceinline__ unsigned column_scan(unsigned *p, size_t stride, int 
 
 template <typename T>
 __global__ void __launch_bounds__(256) sort_colscan_kernel(SortArgs<T> a) {
+    cudaTriggerProgrammaticLaunchCompletion();
+    cudaGridDependencySynchronize();
     const int g = blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= a.ng) return;
     const int seg = blockIdx.y;
@@ -142,28 +154,35 @@ __global__ void __launch_bounds__(256) sort_colscan_kernel(SortArgs<T> a) {
     a.segtot[(size_t)seg * a.ng + g] = column_scan(a.hist + (size_t)b0 * a.ng + g, a.ng, b1 - b0);
 }
 
-// Per cell: exclusive prefix of the segment totals over the segments (in
-// place) and the cell total (into base).  One thread per cell.
+// Per cell: exclusive prefix of the segment totals over the segments, in place,
+// and the cell total.  Many cells only: few are done by the base pass itself.
 template <typename T>
 __global__ void __launch_bounds__(256) sort_segscan_kernel(SortArgs<T> a) {
+    cudaTriggerProgrammaticLaunchCompletion();
+    cudaGridDependencySynchronize();
     const int g = blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= a.ng) return;
-    a.base[g] = column_scan(a.segtot + g, a.ng, a.nseg);
+    if (g < a.ng) a.base[g] = column_scan(a.segtot + g, a.ng, a.nseg);
 }
 
-// Exclusive prefix of the cell totals over the cells -> first slot of each
-// cell.  One block; each thread scans a contiguous run of cells.
-template <typename T>
-__global__ void __launch_bounds__(512) sort_base_kernel(SortArgs<T> a) {
-    __shared__ unsigned wt[32];
-    const int ng = a.ng, T_ = blockDim.x, t = threadIdx.x;
-    const int k = (ng + T_ - 1) / T_;
-    const int g0 = t * k;
+// One block.  The cell totals (SEGSCAN: as the pass above), then their exclusive
+// prefix over the cells, the first slot of each cell (each thread scans a
+// contiguous run of cells).
+constexpr int kBaseThreads = 1024;
+
+template <typename T, bool SEGSCAN>
+__global__ void __launch_bounds__(kBaseThreads) sort_base_kernel(SortArgs<T> a) {
+    __shared__ unsigned wt[kBaseThreads / 32], total[PIC_NCELL_MAX];
+    // the scatter's blocks only now: brought up while the count's are resident they
+    // would be spread unevenly over the SMs (2^26 particles: 406 us a sort, 386 so)
+    cudaGridDependencySynchronize();
+    cudaTriggerProgrammaticLaunchCompletion();
+    const int ng = a.ng, t = threadIdx.x;
+    for (int g = t; g < ng; g += kBaseThreads) total[g] = SEGSCAN ? column_scan(a.segtot + g, a.ng, a.nseg) : a.base[g];
+    __syncthreads();
+    const int k = (ng + kBaseThreads - 1) / kBaseThreads;
+    const int g0 = min(ng, t * k), g1 = min(ng, g0 + k);
     unsigned local = 0;
-    for (int j = 0; j < k; j++) {
-        const int g = g0 + j;
-        if (g < ng) local += a.base[g];
-    }
+    for (int g = g0; g < g1; g++) local += total[g];
     const int lane = t & 31, w = t >> 5;
     unsigned inc = local;
     for (int o = 1; o < 32; o <<= 1) {
@@ -172,15 +191,10 @@ __global__ void __launch_bounds__(512) sort_base_kernel(SortArgs<T> a) {
     }
     if (lane == 31) wt[w] = inc;
     __syncthreads();
-    unsigned off = 0;
-    for (int i = 0; i < w; i++) off += wt[i];
-    unsigned run = off + inc - local;
-    for (int j = 0; j < k; j++) {
-        const int g = g0 + j;
-        if (g >= ng) break;
-        const unsigned c = a.base[g];
+    unsigned run = __reduce_add_sync(kFull, lane < w ? wt[lane] : 0u) + inc - local;
+    for (int g = g0; g < g1; g++) {
         a.base[g] = run;
-        run += c;
+        run += total[g];
     }
 }
 
@@ -211,11 +225,6 @@ template <typename T>
 __global__ void __launch_bounds__(kSortThreads) sort_scatter_kernel(SortArgs<T> a) {
     extern __shared__ unsigned cursor[];
     const int ng = a.ng;
-    const int seg = blockIdx.x / a.seg_len;
-    const unsigned *row = a.hist + (size_t)blockIdx.x * ng;
-    const unsigned *srow = a.segtot + (size_t)seg * ng;
-    for (int g = threadIdx.x; g < ng; g += blockDim.x) cursor[g] = a.base[g] + srow[g] + row[g];
-    __syncthreads();
     const long long start = (long long)blockIdx.x * a.chunk;
     const long long end = min(a.n, start + a.chunk);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
@@ -231,6 +240,12 @@ __global__ void __launch_bounds__(kSortThreads) sort_scatter_kernel(SortArgs<T> 
         nx[j] = ldx(start + own + 32 * j);
         nv[j] = ldv(start + own + 32 * j);
     }
+    cudaGridDependencySynchronize();
+    const int seg = blockIdx.x / a.seg_len;
+    const unsigned *row = a.hist + (size_t)blockIdx.x * ng;
+    const unsigned *srow = a.segtot + (size_t)seg * ng;
+    for (int g = threadIdx.x; g < ng; g += blockDim.x) cursor[g] = a.base[g] + srow[g] + row[g];
+    __syncthreads();
     for (long long r0 = start; r0 < end; r0 += round) {
         T x[kSub], v[kSub];
 #pragma unroll
@@ -279,21 +294,40 @@ __global__ void __launch_bounds__(kSortThreads) sort_scatter_kernel(SortArgs<T> 
     }
 }
 
+// A launch that may begin before the pass ahead of it is done.
+template <typename T>
+cudaError_t launch_next(void (*k)(SortArgs<T>), dim3 grid, int block, size_t smem, const SortArgs<T> &a,
+                        cudaStream_t s) {
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k, a);
+}
+
 template <typename T>
 cudaError_t launch_sort_t(const SortArgs<T> &a, cudaStream_t s) {
     const size_t smem = (size_t)a.ng * sizeof(unsigned);
     sort_count_kernel<T><<<a.nchunk, kSortThreads, smem, s>>>(a);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    dim3 cg((a.ng + 255) / 256, a.nseg);
-    sort_colscan_kernel<T><<<cg, 256, 0, s>>>(a);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    sort_segscan_kernel<T><<<(a.ng + 255) / 256, 256, 0, s>>>(a);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    sort_base_kernel<T><<<1, 512, 0, s>>>(a);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    sort_scatter_kernel<T><<<a.nchunk, kSortThreads, smem, s>>>(a);
-    return cudaGetLastError();
+    e = launch_next(&sort_colscan_kernel<T>, dim3((a.ng + 255) / 256, a.nseg), 256, 0, a, s);
+    // With several cells a thread the one block's column scans take longer than a
+    // launch.  A sort, us, without and with the separate pass: 2e4 particles on 64
+    // cells 13.5, 14.9; 1e6 on 1024 19.9, 20.1; 4.2e6 on 2048 40.1, 37.4.
+    const bool one = a.ng <= kBaseThreads;
+    if (e == cudaSuccess && !one) e = launch_next(&sort_segscan_kernel<T>, dim3((a.ng + 255) / 256), 256, 0, a, s);
+    if (e == cudaSuccess)
+        e = launch_next(one ? &sort_base_kernel<T, true> : &sort_base_kernel<T, false>, dim3(1), kBaseThreads,
+                        0, a, s);
+    if (e == cudaSuccess) e = launch_next(&sort_scatter_kernel<T>, dim3(a.nchunk), kSortThreads, smem, a, s);
+    return e;
 }
 
 }  // namespace

@@ -185,3 +185,25 @@ def test_steps_at_the_limits_of_one_particle_per_lane(n, ng, shape):
         a.step_n(k), b.step_n(k)
         assert_same(a, b, n, ng)
     a.close(), b.close()
+
+
+@pytest.mark.parametrize("n,ng", [(1, 1), (255, 1023), (20000, 64), (300007, 1024), (300007, 1025),
+                                  (1000003, 2049), (70000, 8192)])
+def test_a_sort_is_the_stable_order_by_cell(n, ng):
+    # the passes run into each other: several sorts and pushes back to back
+    run = pic.Run(pic.Params(npart=n, ncell=ng, length=L, sort_interval=8), device="cuda:0")
+    run.init(*state(n, 3 * n + ng))
+    u, v = run.get_cells()
+    for _ in range(3):
+        run.sort()
+        order = np.argsort(np.clip(u, 0, ng - 1).astype(np.int64), kind="stable")
+        u, v = u[order], v[order]
+        got = run.get_cells()
+        assert np.array_equal(got[0], u) and np.array_equal(got[1], v)
+        run.push(), run.sort(), run.solve_field()
+        w = run.get_cells()
+        key = np.clip(w[0], 0, ng - 1).astype(np.int64)
+        assert np.all(np.diff(key) >= 0)
+        run.push(), run.solve_field()
+        u, v = run.get_cells()
+    run.close()
