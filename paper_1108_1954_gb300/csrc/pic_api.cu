@@ -378,13 +378,18 @@ int push_grid(const pic_run *r, int variant, int block, int unroll, int bps_cap)
 // Threads per block of the push when the caller leaves them open.  Every
 // block stages E and flushes a tile of NG nodes with one or two global adds
 // each, so large runs take few large blocks (512 threads; 1024 where the
-// float64 tile leaves room for one block per SM); a run with less than a
+// float64 tile leaves room for one block per SM, and where the float32-atomic
+// tile then takes more copies: push.cu); a run with less than a
 // block of 512 for every SM takes smaller ones, down to 64 threads, so that
 // all SMs share it.
 int default_block(const pic_run *r) {
     if (r->p.precision == PIC_FP32_FIXED) return 512;
     const long long groups = (r->p.npart + 3) / 4;
-    const int most = push_smem_bytes(r->p.precision, r->p.ncell, false) > 100 * 1024 ? 1024 : 512;
+    const int mode = r->p.precision, ng = r->p.ncell;
+    const size_t small = push_smem_bytes(mode, ng, false, 512);
+    const bool one = mode == PIC_FP32_ATOMIC ? push_smem_bytes(mode, ng, false, 1024) > small
+                                             : small > 100 * 1024;
+    const int most = one ? 1024 : 512;
     int b = 64;
     while (b < most && groups > (long long)b * r->sms) b *= 2;
     return b;
@@ -661,7 +666,7 @@ int pic_create(const pic_params *p, void *workspace, size_t workspace_bytes,
     // on 512 cells 113/95 and 184/98; unsorted, 2^25 on 4096, 99/97 and 107/95;
     // 2^25 on 8192 (two blocks) 110/111 and 101/102.
     const bool three = 3 * push_smem_bytes(PIC_FP32_FIXED, p->ncell,
-                                           push_wide_tile(p->npart, r->sms)) <= 227 * 1024;
+                                           push_wide_tile(p->npart, r->sms), 512) <= 227 * 1024;
     r->auto_variant = !p->deposit_variant;
     r->variant = p->deposit_variant ? p->deposit_variant
                  : r->open_shape && three ? PIC_DEPOSIT_PAIR8 : PIC_DEPOSIT_QUAD;

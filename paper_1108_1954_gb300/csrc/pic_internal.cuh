@@ -277,7 +277,7 @@ cudaError_t launch_push_f32_atomic(PushArgsF32Atomic a, int grid, int block, boo
                                    cudaStream_t s);
 cudaError_t launch_push_f64(const PushArgs64 &a, int grid, int block,
                             bool push, cudaStream_t s);
-size_t push_smem_bytes(int mode, int ng, bool wide);
+size_t push_smem_bytes(int mode, int ng, bool wide, int block);
 bool push_wide_tile(long long n, int sms);
 cudaError_t push_prepare_attributes(int mode);
 int push_max_blocks_per_sm(int mode, int variant, int unroll, int block, int ng, bool wide);

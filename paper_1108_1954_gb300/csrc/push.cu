@@ -248,17 +248,25 @@ __global__ void __launch_bounds__(512) pic_push_oct_kernel(PushArgs a) {
 // So two open runs per thread are summed in registers first (PAIR), and the
 // block keeps `copies` sums per node, side by side, lane l adding to copy
 // l mod copies: lanes of one cell then meet on an address copies times less
-// often.  As many copies as fit beside E in kAtomicTile bytes, at most 32 (one
-// per lane).  Measured (2^24 particles, 1024 cells, 16 copies): 61 us a push,
-// the mean over sort periods, against 295 us with one copy and a shuffle sum
+// often, and with 32 copies a warp's lanes never meet and use a bank each.
+// Measured (2^24 particles, 1024 cells, the mean over sort periods): 60 us a push
+// with 32 copies, 68 with 16, against 295 us with one copy and a shuffle sum
 // where a whole warp holds one run, and 140 us (sorted) to 380 us (lattice
 // order) with two adds per particle.
-// (72 KB: two 512-thread blocks of 53 registers per SM keep their place.)
-constexpr size_t kAtomicTile = 72 * 1024;
+// As many copies as fit beside E, at most 32: in 216 KB for a block of 1024
+// threads (its 53 registers leave room for one per SM), in 72 KB for smaller
+// ones, so that two of 512 keep their place; open shapes take the large block
+// where it holds more copies.  us a push, 2^24 particles sorted every 20 steps, in
+// two blocks of 512 and one of 1024: 256 cells (32 copies either way) 58.9, 62.3;
+// 1024 66.9, 59.6; 1600 78.5, 62.8; 2048 77.2, 65.1; 4096 83.5, 70.3; 8192 82.7,
+// 72.1; 4e6 on 1600 28.1, 25.1; 1e6 on 4096 18.1, 18.1.  (Three of 512 threads and
+// 40 registers: 10 us more on 1024 cells, the loops fail more often.)
+constexpr size_t kAtomicShared = 216 * 1024, kAtomicSharedSmall = 72 * 1024;
 
-int atomic_copies(int ng) {
+int atomic_copies(int ng, int block) {
+    const size_t most = block > 512 ? kAtomicShared - 4 * (size_t)(ng + 2) : kAtomicSharedSmall;
     int k = 32;
-    while (k > 1 && (size_t)(ng + 2) * 4 * k > kAtomicTile) k /= 2;
+    while (k > 1 && (size_t)(ng + 2) * 4 * k > most) k /= 2;
     return k;
 }
 
@@ -531,16 +539,15 @@ bool push_wide_tile(long long n, int sms) {
     return n / sms > kPackedCount - 512 * 32;
 }
 
-size_t push_smem_bytes(int mode, int ng, bool wide) {
+size_t push_smem_bytes(int mode, int ng, bool wide, int block) {
     if (mode == PIC_FP64) return (size_t)(ng + 1) * 16 + (size_t)(ng + 2) * 12;
-    if (mode == PIC_FP32_ATOMIC) return (size_t)(ng + 2) * 4 * (1 + atomic_copies(ng));
+    if (mode == PIC_FP32_ATOMIC) return (size_t)(ng + 2) * 4 * (1 + atomic_copies(ng, block));
     return (size_t)(ng + 2) * (wide ? 16 : 12);
 }
 
 cudaError_t push_prepare_attributes(int mode) {
-    // the atomic tile is largest where 32 copies just fit
-    const int bytes = mode == PIC_FP32_ATOMIC ? (int)(2 * kAtomicTile)
-                                              : (int)push_smem_bytes(mode, PIC_NCELL_MAX, true);
+    const int bytes = mode == PIC_FP32_ATOMIC ? (int)kAtomicShared
+                                              : (int)push_smem_bytes(mode, PIC_NCELL_MAX, true, 0);
     cudaError_t e = cudaSuccess;
     if (mode == PIC_FP32_FIXED) {
         const int unrolls[3] = {1, 2, 4};
@@ -573,7 +580,7 @@ cudaError_t push_prepare_attributes(int mode) {
 
 int push_max_blocks_per_sm(int mode, int variant, int unroll, int block, int ng, bool wide) {
     int nb = 0;
-    const size_t smem = push_smem_bytes(mode, ng, wide);
+    const size_t smem = push_smem_bytes(mode, ng, wide, block);
     cudaError_t e;
     if (mode == PIC_FP32_FIXED) {
         FixedKernel k = pick_fixed(variant, true, unroll);
@@ -595,14 +602,14 @@ cudaError_t launch_push_fixed(const PushArgs &a, int grid, int block, int varian
                               int unroll, bool push, cudaStream_t s) {
     FixedKernel k = pick_fixed(variant, push, unroll);
     if (!k) return cudaErrorInvalidValue;
-    k<<<grid, block, push_smem_bytes(PIC_FP32_FIXED, a.c.ng, a.wide), s>>>(a);
+    k<<<grid, block, push_smem_bytes(PIC_FP32_FIXED, a.c.ng, a.wide, block), s>>>(a);
     return cudaGetLastError();
 }
 
 cudaError_t launch_push_f32_atomic(PushArgsF32Atomic a, int grid, int block, bool push,
                                    cudaStream_t s) {
-    const size_t smem = push_smem_bytes(PIC_FP32_ATOMIC, a.c.ng, false);
-    a.copies = atomic_copies(a.c.ng);
+    const size_t smem = push_smem_bytes(PIC_FP32_ATOMIC, a.c.ng, false, block);
+    a.copies = atomic_copies(a.c.ng, block);
     if (push) pic_push_f32atomic_kernel<true><<<grid, block, smem, s>>>(a);
     else pic_push_f32atomic_kernel<false><<<grid, block, smem, s>>>(a);
     return cudaGetLastError();
@@ -610,7 +617,7 @@ cudaError_t launch_push_f32_atomic(PushArgsF32Atomic a, int grid, int block, boo
 
 cudaError_t launch_push_f64(const PushArgs64 &a, int grid, int block, bool push,
                             cudaStream_t s) {
-    const size_t smem = push_smem_bytes(PIC_FP64, a.ng, false);
+    const size_t smem = push_smem_bytes(PIC_FP64, a.ng, false, block);
     if (push) pic_push_f64_kernel<true><<<grid, block, smem, s>>>(a);
     else pic_push_f64_kernel<false><<<grid, block, smem, s>>>(a);
     return cudaGetLastError();

@@ -114,3 +114,25 @@ def test_float64_sort_is_the_stable_order_by_cell(n, ng):
     order = np.argsort(np.minimum((x * (ng / L)).astype(np.int64), ng - 1), kind="stable")
     assert np.array_equal(run.get_state()[0], x[order])
     run.close()
+
+
+@pytest.mark.parametrize("n", [311295, 311300, 400003])       # below and at a block of 1024 for every SM
+@pytest.mark.parametrize("ng", [574, 575, 1674, 1675, 8192])  # copies 32/32, 16/32, 8/32, 8/16, 2/4
+def test_atomic_deposit_in_large_blocks(n, ng):
+    # the density and the next step's against blocks of 512 threads: two orders of
+    # the same float32 adds, each within the bound above of the exact sum
+    x, v = state(n, ng, n + ng)
+    x32 = np.minimum(x.astype(np.float32), np.nextafter(np.float32(L), np.float32(0)))
+    rho = []
+    for block in (0, 512):
+        run = pic.Run(pic.Params(npart=n, ncell=ng, length=L, precision=pic.PIC_FP32_ATOMIC, block_size=block),
+                      device="cuda:0")
+        run.init(x32, v.astype(np.float32))
+        rho.append([run.get_field()["rho"]])
+        run.step_n(1)
+        rho[-1].append(run.get_field()["rho"])
+        run.close()
+    for a, b in zip(*rho):
+        most = float((1.0 - np.minimum(a, b)).max() / (ng / n))
+        assert np.abs(a - b).max() <= 2 * (ng / n) * 2.0 ** -24 * (2.0 * (most + 1) ** 2 + 2.0 * ng * (most + 1))
+        assert abs(a.sum()) <= 2 * ng * (ng / n) * 2.0 ** -24 * 2.0 * (most + 1) ** 2
