@@ -501,7 +501,7 @@ int run_steps(pic_run *r, int steps) {
     PIC_CUDA(r->p.precision == PIC_FP64
                  ? launch_steps64(a, r->steps_grid, r->steps_block, r->stream)
                  : launch_steps(a, r->variant, r->steps_grid, r->steps_block, r->steps_small, r->stream));
-    r->sync_base[0] += (unsigned)(r->steps_grid - kStepsDiag) * (unsigned)steps;
+    r->sync_base[0] += (unsigned)(r->steps_grid - kStepsDiag) * ((unsigned)steps + 1u);
     for (int d = 0; d < kStepsDiag; d++)
         r->sync_base[1 + d] += (unsigned)((steps - d + kStepsDiag - 1) / kStepsDiag);
     r->step += steps;

@@ -22,8 +22,8 @@
 // the workers up: at 64 clocks a dependent float64 add and 840 a square root,
 // a step's take 5 to 10 thousand clocks, up to twice a worker's step), then
 // clear the step's accumulator and give it back; a worker waits only if the
-// diagnostics fall kStepsSlots - 1 steps behind.  After the last step they
-// write E, Phi, rho and the consumed sums.
+// diagnostics fall kStepsSlots - 1 steps behind.  After the last step the
+// workers write E, Phi, rho and the consumed sums, each of some nodes.
 //
 // Up to 6e5 particles on up to 1024 cells the lanes take particles one by one
 // (SMALL), beyond that in groups of 4 (16-byte loads; in a small run only a
@@ -31,14 +31,16 @@
 //
 // What a step costs (GB300, us): launches of push and solve before, and here
 //   2e4 particles, 64 cells, one step a call   16.4   10.2
+//   3e5, 500 cells, one step a call             -     12.3
+//   1e6, 2048 cells, one step a call            -     21.9
 //   2e4, 64 cells                              13.4    2.9
 //   5e4, 100 cells                             14.0    3.1
-//   5e5, 300 cells                             18.5    5.2
-//   1e6, 1024 cells, sorted every 20           22.5    9.0
-//   3e6, 777 cells, NGP, sorted every 10       27.4   14.0
-//   4.2e6, 2048 cells, sorted every 20         31.0   19.2
-//   1e6, 4096 cells                            24.8   11.4
-//   1.2e7, 2048 cells, sorted every 20         52.9   41.3
+//   5e5, 300 cells                             18.5    5.1
+//   1e6, 1024 cells, sorted every 20           22.5    8.4
+//   3e6, 777 cells, NGP, sorted every 10       27.4   13.1
+//   4.2e6, 2048 cells, sorted every 20         31.0   18.3
+//   1e6, 4096 cells                            24.8   11.3
+//   1.2e7, 2048 cells, sorted every 20         52.9   39.9
 // of which, at 5e4 (clocks): push 700, sums 380, flush 1040, barrier 2400 (the
 // adds' release and a poll, each a trip to L2), solve 1300 (900 the sums' way
 // from L2), E 510.  Counting a node's arrivals in the upper bits of its sum, so
@@ -231,7 +233,20 @@ __device__ __forceinline__ void field_step(const StepsArgs &a, const unsigned lo
     __syncthreads();
 }
 
-// The diagnostics of a step, and after the last one the run's results.
+// After the last step: the results, once the sums have been read (a worker's last
+// arrival).
+template <int K>
+__device__ __forceinline__ void last_step(const StepsArgs &a, const unsigned long long *acc, int b,
+                                          int workers) {
+    __shared__ long long wr[32];
+    __shared__ unsigned long long ws[64];
+    NodeSolve<K> ns;
+    solve_nodes<K>(ns, a, acc, a.c.ng, wr, ws);
+    if (threadIdx.x == 0) red_release(a.sync);
+    step_results<K, true>(a, ns, b, workers);
+}
+
+// The diagnostics of a step.
 template <int K>
 __device__ __forceinline__ void diag_step(const StepsArgs &a, int s, int workers,
                                           const unsigned long long *acc, const float4 *kv,
@@ -388,11 +403,11 @@ __device__ __forceinline__ void run_many_steps(const StepsArgs &a, unsigned char
             }
             __syncthreads();
             if (tid == 0) red_release(a.sync);        // the whole block's adds: after the barrier
-            if (last) break;                          // a diagnostics block writes the results
-            clear_tile();                             // while the others arrive
+            if (!last) clear_tile();                  // while the others arrive
         }
         if (!wait_step(a, s, workers, !diag, &dead)) return;
         if (!diag) {
+            if (last) break;
             if (K >= 4) field_step_call<K>(a, acc, sE);
             else field_step<K>(a, acc, sE);
             continue;
@@ -400,7 +415,7 @@ __device__ __forceinline__ void run_many_steps(const StepsArgs &a, unsigned char
         if (K >= 4) diag_step_call<K>(a, s, workers, acc, kv, smem_raw, h0);
         else diag_step<K>(a, s, workers, acc, kv, smem_raw, h0);
         // give the slot back, once no worker reads it any more
-        if (!last && !wait_step(a, s + 1, workers, false, &dead)) return;
+        if (!wait_step(a, s + 1, workers, false, &dead)) return;
         for (int g = tid; g < ng; g += bs) acc[g] = 0ull;
         __syncthreads();
         if (tid == 0) red_release(a.sync + 1 + (b - workers));
@@ -413,6 +428,8 @@ __device__ __forceinline__ void run_many_steps(const StepsArgs &a, unsigned char
             __stcg(xg + q, rx[i]);
             __stcg(vg + q, rv[i]);
         }
+        const int slot = (a.steps - 1) % kStepsSlots;
+        last_step<K>(a, a.acc + (size_t)slot * ng, b, workers);
     }
 }
 

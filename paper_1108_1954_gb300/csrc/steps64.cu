@@ -171,12 +171,16 @@ __global__ void __launch_bounds__(1024, 1) pic_steps64_kernel(const __grid_const
             }
             __syncthreads();
             if (tid == 0) red_release(a.sync);        // the whole block's adds: after the barrier
-            if (last) break;
-            clear_tile();                             // while the others arrive
+            if (!last) clear_tile();                  // while the others arrive
         }
         if (!wait_step(a, s, workers, !diag, &dead)) return;
         Solved64 ns;
         solve_nodes64(ns, a, acc, ng, scan64);
+        if (!diag && last) {
+            if (tid == 0) red_release(a.sync);        // the sums have been read
+            step_results<1, false>(a, ns, b, workers);
+            break;
+        }
         if (!diag) {
             if (tid < ng) {
                 const double e = a.k_e * i128_to_f64(ns.m[0]);
@@ -205,7 +209,7 @@ __global__ void __launch_bounds__(1024, 1) pic_steps64_kernel(const __grid_const
             m = warp_sum_fixed(m);
         });
         // give the slot back, once no worker reads it any more
-        if (!last && !wait_step(a, s + 1, workers, false, &dead)) return;
+        if (!wait_step(a, s + 1, workers, false, &dead)) return;
         for (int g = tid; g < 2 * ng; g += bs) acc[g] = 0ull;
         __syncthreads();
         if (tid == 0) red_release(a.sync + 1 + (b - workers));
