@@ -46,9 +46,11 @@ namespace pic {
 namespace {
 
 constexpr int kClusterSolveThreads = 512;   // most nodes per block (one per thread)
-// nodes per block of the exact solve: its per-node float64 conversions and
-// diagnostics are the critical path, so spread them over up to 16 SMs
-constexpr int kSolveNodesPerBlock = 256;
+// Nodes per block of the exact solve: its per-node float64 conversions and
+// diagnostics are the critical path, so spread them over up to 16 SMs.  us a
+// solve with 256, 128 and 64: 1024 nodes 9.4, 8.6, 8.5; 2048 9.2, 8.4, 8.4; 4096
+// 8.9 each.
+constexpr int kSolveNodesPerBlock = 128;
 constexpr int kMaxSolveCluster = 16;        // blocks per cluster (16: non-portable)
 
 // ---- the density as integers --------------------------------------------------
@@ -236,6 +238,8 @@ __global__ void __launch_bounds__(kClusterSolveThreads) pic_solve_cluster_kernel
     __shared__ __align__(16) unsigned long long scan64[4 * 32];
     const int C = (int)cl.num_blocks(), r = (int)cl.block_rank();
     const int ng = a.ng, t = threadIdx.x;
+    cudaGridDependencySynchronize();
+    cudaTriggerProgrammaticLaunchCompletion();      // the next push may come up
     const long long step = *a.dstep;
     const i128 ntot = whole_density<MODE>(a);
     const int per = (int)blockDim.x;              // whole warps of nodes
@@ -427,6 +431,8 @@ __global__ void __launch_bounds__(kClusterSolveThreads) pic_solve_cg_kernel(Solv
     __shared__ double scal[2];                        // t and beta; NaN: stop
     const int C = (int)cl.num_blocks(), r = (int)cl.block_rank();
     const int ng = a.ng, t = threadIdx.x, lane = t & 31, w = t >> 5, nw = blockDim.x >> 5;
+    cudaGridDependencySynchronize();
+    cudaTriggerProgrammaticLaunchCompletion();      // the next push may come up
     const long long step = *a.dstep;
     const double dx = a.dx;
     const int per = (ng + C - 1) / C;
@@ -584,7 +590,7 @@ SolveKernel pick_solve(int mode, int solver) {
 
 // Cluster shape of the solves: C = ceil(NG / per_block) blocks (at most 16),
 // ceil(NG / C) nodes each, rounded up to whole warps.  The exact solve takes
-// up to 256 nodes per block, the CG 32 (both are float64-bound on GB300).  The
+// up to 128 nodes per block, the CG 32 (both are float64-bound on GB300).  The
 // exact solve's blocks take as many nodes as they have threads, so that every
 // warp holds 32 nodes from a multiple of 32 on.
 void solve_cluster_shape(int ng, int per_block, int *C, int *threads) {
@@ -608,19 +614,7 @@ cudaError_t solve_prepare_attributes() {
 cudaError_t launch_solve(const SolveArgs &a, cudaStream_t s) {
     int C = 1, threads = 32;
     solve_cluster_shape(a.ng, a.solver == PIC_SOLVER_CG ? 32 : kSolveNodesPerBlock, &C, &threads);
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr[1];
-    cfg.gridDim = dim3((unsigned)C, 1, 1);
-    cfg.blockDim = dim3((unsigned)threads, 1, 1);
-    cfg.dynamicSmemBytes = 0;
-    cfg.stream = s;
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)C;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, pick_solve(a.mode, a.solver), a);
+    return launch_after(pick_solve(a.mode, a.solver), dim3((unsigned)C), threads, 0, s, C, a);
 }
 
 }  // namespace pic

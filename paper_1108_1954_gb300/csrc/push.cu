@@ -77,12 +77,15 @@ __global__ void __launch_bounds__(512) pic_push_fixed_kernel(PushArgs a) {
     float *sE = reinterpret_cast<float *>(smem_raw);                 // ng + 2
     const Tile tile = make_tile(smem_raw + 4 * (ng + 2), ng + 2, a.wide);
     const int tid = threadIdx.x, bs = blockDim.x, lane = tid & 31;
+    cudaTriggerProgrammaticLaunchCompletion();
     for (int j = tid; j < ng + 2; j += bs) {
         tile.w[j] = 0u;
         tile.n[j] = 0u;
         tile.c[j] = 0u;
-        if (PUSH) sE[j] = a.E32[j == 0 ? ng - 1 : (j == ng + 1 ? 0 : j - 1)];
     }
+    cudaGridDependencySynchronize();
+    if (PUSH)
+        for (int j = tid; j < ng + 2; j += bs) sE[j] = a.E32[j == 0 ? ng - 1 : (j == ng + 1 ? 0 : j - 1)];
     __syncthreads();
 
     float ke = 0.0f, mom = 0.0f;
@@ -178,12 +181,15 @@ __global__ void __launch_bounds__(512) pic_push_oct_kernel(PushArgs a) {
     float *sE = reinterpret_cast<float *>(smem_raw);                 // ng + 2
     const Tile tile = make_tile(smem_raw + 4 * (ng + 2), ng + 2, a.wide);
     const int tid = threadIdx.x, bs = blockDim.x, lane = tid & 31;
+    cudaTriggerProgrammaticLaunchCompletion();
     for (int j = tid; j < ng + 2; j += bs) {
         tile.w[j] = 0u;
         tile.n[j] = 0u;
         tile.c[j] = 0u;
-        if (PUSH) sE[j] = a.E32[j == 0 ? ng - 1 : (j == ng + 1 ? 0 : j - 1)];
     }
+    cudaGridDependencySynchronize();
+    if (PUSH)
+        for (int j = tid; j < ng + 2; j += bs) sE[j] = a.E32[j == 0 ? ng - 1 : (j == ng + 1 ? 0 : j - 1)];
     __syncthreads();
 
     float ke = 0.0f, mom = 0.0f;
@@ -279,9 +285,11 @@ __global__ void __launch_bounds__(1024) pic_push_f32atomic_kernel(PushArgsF32Ato
     float *sE = reinterpret_cast<float *>(smem_raw);      // ng + 2, ghost-padded
     float *sRho = sE + ng + 2;                            // [ng + 2][copies], ghost-padded
     const int tid = threadIdx.x, bs = blockDim.x, K = a.copies;
+    cudaTriggerProgrammaticLaunchCompletion();
+    for (int j = tid; j < (ng + 2) * K; j += bs) sRho[j] = 0.0f;
+    cudaGridDependencySynchronize();
     for (int j = tid; j < ng + 2; j += bs)
         if (PUSH) sE[j] = a.E32[j == 0 ? ng - 1 : (j == ng + 1 ? 0 : j - 1)];
-    for (int j = tid; j < (ng + 2) * K; j += bs) sRho[j] = 0.0f;
     __syncthreads();
     float *mine = sRho + (tid & (K - 1));                 // this lane's copy
     auto add = [&](unsigned key, float l, float r) {
@@ -415,10 +423,14 @@ __global__ void __launch_bounds__(1024) pic_push_f64_kernel(PushArgs64 a) {
     t.lo = reinterpret_cast<unsigned *>(pair + ng + 1);
     t.mid = t.lo + ng + 2;
     t.hi = t.mid + ng + 2;
+    cudaTriggerProgrammaticLaunchCompletion();
     for (int j = tid; j < ng + 2; j += bs) {
         t.lo[j] = 0u;
         t.mid[j] = 0u;
         t.hi[j] = 0u;
+    }
+    cudaGridDependencySynchronize();
+    for (int j = tid; j < ng + 2; j += bs) {
         if (PUSH && j <= ng) {
             const double el = a.E64[j == 0 ? ng - 1 : j - 1], er = a.E64[j == ng ? 0 : j];
             const double de = er - el;
@@ -602,25 +614,22 @@ cudaError_t launch_push_fixed(const PushArgs &a, int grid, int block, int varian
                               int unroll, bool push, cudaStream_t s) {
     FixedKernel k = pick_fixed(variant, push, unroll);
     if (!k) return cudaErrorInvalidValue;
-    k<<<grid, block, push_smem_bytes(PIC_FP32_FIXED, a.c.ng, a.wide, block), s>>>(a);
-    return cudaGetLastError();
+    return launch_after(k, dim3(grid), block, push_smem_bytes(PIC_FP32_FIXED, a.c.ng, a.wide, block), s, 0, a);
 }
 
 cudaError_t launch_push_f32_atomic(PushArgsF32Atomic a, int grid, int block, bool push,
                                    cudaStream_t s) {
     const size_t smem = push_smem_bytes(PIC_FP32_ATOMIC, a.c.ng, false, block);
     a.copies = atomic_copies(a.c.ng, block);
-    if (push) pic_push_f32atomic_kernel<true><<<grid, block, smem, s>>>(a);
-    else pic_push_f32atomic_kernel<false><<<grid, block, smem, s>>>(a);
-    return cudaGetLastError();
+    return launch_after(push ? &pic_push_f32atomic_kernel<true> : &pic_push_f32atomic_kernel<false>, dim3(grid),
+                        block, smem, s, 0, a);
 }
 
 cudaError_t launch_push_f64(const PushArgs64 &a, int grid, int block, bool push,
                             cudaStream_t s) {
     const size_t smem = push_smem_bytes(PIC_FP64, a.ng, false, block);
-    if (push) pic_push_f64_kernel<true><<<grid, block, smem, s>>>(a);
-    else pic_push_f64_kernel<false><<<grid, block, smem, s>>>(a);
-    return cudaGetLastError();
+    return launch_after(push ? &pic_push_f64_kernel<true> : &pic_push_f64_kernel<false>, dim3(grid), block, smem,
+                        s, 0, a);
 }
 
 }  // namespace pic

@@ -294,39 +294,22 @@ __global__ void __launch_bounds__(kSortThreads) sort_scatter_kernel(SortArgs<T> 
     }
 }
 
-// A launch that may begin before the pass ahead of it is done.
-template <typename T>
-cudaError_t launch_next(void (*k)(SortArgs<T>), dim3 grid, int block, size_t smem, const SortArgs<T> &a,
-                        cudaStream_t s) {
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr[1];
-    cfg.gridDim = grid;
-    cfg.blockDim = dim3((unsigned)block);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k, a);
-}
-
 template <typename T>
 cudaError_t launch_sort_t(const SortArgs<T> &a, cudaStream_t s) {
     const size_t smem = (size_t)a.ng * sizeof(unsigned);
     sort_count_kernel<T><<<a.nchunk, kSortThreads, smem, s>>>(a);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    e = launch_next(&sort_colscan_kernel<T>, dim3((a.ng + 255) / 256, a.nseg), 256, 0, a, s);
+    e = launch_after(&sort_colscan_kernel<T>, dim3((a.ng + 255) / 256, a.nseg), 256, 0, s, 0, a);
     // With several cells a thread the one block's column scans take longer than a
     // launch.  A sort, us, without and with the separate pass: 2e4 particles on 64
     // cells 13.5, 14.9; 1e6 on 1024 19.9, 20.1; 4.2e6 on 2048 40.1, 37.4.
     const bool one = a.ng <= kBaseThreads;
-    if (e == cudaSuccess && !one) e = launch_next(&sort_segscan_kernel<T>, dim3((a.ng + 255) / 256), 256, 0, a, s);
+    if (e == cudaSuccess && !one) e = launch_after(&sort_segscan_kernel<T>, dim3((a.ng + 255) / 256), 256, 0, s, 0, a);
     if (e == cudaSuccess)
-        e = launch_next(one ? &sort_base_kernel<T, true> : &sort_base_kernel<T, false>, dim3(1), kBaseThreads,
-                        0, a, s);
-    if (e == cudaSuccess) e = launch_next(&sort_scatter_kernel<T>, dim3(a.nchunk), kSortThreads, smem, a, s);
+        e = launch_after(one ? &sort_base_kernel<T, true> : &sort_base_kernel<T, false>, dim3(1), kBaseThreads,
+                         0, s, 0, a);
+    if (e == cudaSuccess) e = launch_after(&sort_scatter_kernel<T>, dim3(a.nchunk), kSortThreads, smem, s, 0, a);
     return e;
 }
 
