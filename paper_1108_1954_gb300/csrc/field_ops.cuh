@@ -44,8 +44,9 @@ __device__ __forceinline__ double i128_to_f64(i128 v) {
 struct I128Pair {
     i128 a, b;
 };
-__device__ __forceinline__ I128Pair block_inclusive_scan2_i128(i128 a, i128 b,
-                                                               unsigned long long *w64) {
+// Warps from `used` on hold zeros and get no meaningful result.
+__device__ __forceinline__ I128Pair block_inclusive_scan2_i128(i128 a, i128 b, unsigned long long *w64,
+                                                               int used = 32) {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -63,7 +64,7 @@ __device__ __forceinline__ I128Pair block_inclusive_scan2_i128(i128 a, i128 b,
     }
     __syncthreads();
     i128 oa = 0, ob = 0;
-    for (int i = 0; i < w; i++) {
+    for (int i = 0; i < min(w, used); i++) {
         oa += (i128)(((unsigned __int128)w64[32 + i] << 64) | w64[i]);
         ob += (i128)(((unsigned __int128)w64[96 + i] << 64) | w64[64 + i]);
     }

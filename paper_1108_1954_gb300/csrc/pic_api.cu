@@ -413,7 +413,7 @@ int steps64_block(int64_t npart, int ncell) {
 //   2048   38, 47.6 / 43, 48.8   53.1, 59.4 / 59.4, 62.0  100, 101 / 110, 108
 //   4096   45, 48.8 / 51, 51.8   60.3, 61.0 / 67.4, 64.6  107, 102 / 118, 109
 // Float64 runs (steps64.cu) up to 1e6 particles and 1024 cells: 2e4 on 64 cells
-// 4.8 and 15.3 us a step, 5e5 on 1000 20.0 and 26.6, 1e6 27.6 and 30.1; 4e6 on
+// 4.1 and 15.3 us a step, 5e5 on 1000 17.6 and 26.6, 1e6 27.6 and 30.1; 4e6 on
 // 512 69.8 and 62.0.
 // Runs of few particles take them one per lane (steps_small; a lane's 4 in turn
 // are a chain 4 times as long), and small blocks, whose barriers cost less.  us

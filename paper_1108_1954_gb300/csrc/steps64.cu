@@ -15,7 +15,7 @@
 //     field.cu) with one node per thread, and E stays float64;
 //   * the sums of v_old v_new and v_new are taken over a warp as aligned integers
 //     (warp_sum_fixed), 200 clocks against 700 for a tree of float64 adds.
-// 2e4 particles, 64 cells: 4.8 us a step, 15.3 with the two kernels.  The float64
+// 2e4 particles, 64 cells: 4.1 us a step, 15.3 with the two kernels.  The float64
 // solve of all nodes by every block (6 instructions a warp of nodes) bounds large
 // grids and the push's five instructions a particle large runs; those keep the
 // two kernels (pic_api.cu, set_steps_shape).
@@ -36,16 +36,17 @@ struct Solved64 {
 __device__ __forceinline__ void solve_nodes64(Solved64 &s, const StepsArgs &a,
                                               const unsigned long long *acc, int ng,
                                               unsigned long long *scan64) {
-    const int g = threadIdx.x, nw = blockDim.x >> 5;
+    const int g = threadIdx.x;
     const bool in = g < ng;
     ulonglong2 w = make_ulonglong2(0ull, 0ull);
     if (in) w = __ldcg(reinterpret_cast<const ulonglong2 *>(acc) + g);
     s.q[0] = (i128)w.x + ((i128)w.y << 40);
     s.R[0] = in ? ((i128)a.n << 53) - (i128)ng * s.q[0] : (i128)0;
-    const I128Pair sc = block_inclusive_scan2_i128(s.R[0], s.R[0] * (i128)g, scan64);
+    const int used = (ng + 31) >> 5;                  // warps with nodes
+    const I128Pair sc = block_inclusive_scan2_i128(s.R[0], s.R[0] * (i128)g, scan64, used);
     i128 S1 = 0;
     s.SR = 0;
-    for (int i = 0; i < nw; i++) {
+    for (int i = 0; i < used; i++) {
         s.SR += (i128)(((unsigned __int128)scan64[32 + i] << 64) | scan64[i]);
         S1 += (i128)(((unsigned __int128)scan64[96 + i] << 64) | scan64[64 + i]);
     }
