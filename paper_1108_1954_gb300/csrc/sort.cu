@@ -25,7 +25,8 @@
 // then; those are complete before the count begins, which waits for everything
 // ahead of it in the stream.  A sort, us, five plain launches before and here: 2e4
 // particles on 64 cells 24.5, 13.5; 1e6 on 1024 27.2, 19.9; 4.2e6 on 2048 47.3,
-// 37.4; 1.2e7 on 4096 115.5, 108.7; 2^26 on 4096 390, 388.
+// 37.4; 1.2e7 on 4096 115.5, 108.7; 2^26 on 4096 390, 388 (353 with the long
+// chunks' scatter, below).
 // The destination index is bounds-checked; a violation sets the device error
 // word instead of writing.
 #include "pic_internal.cuh"
@@ -198,31 +199,43 @@ __global__ void __launch_bounds__(kBaseThreads) sort_base_kernel(SortArgs<T> a) 
     }
 }
 
-// Scatter: block b walks its chunk in order, 256 particles at a time (one
-// per thread, with the loads four iterations ahead).  Lanes of
-// one cell within a warp are ranked by __match_any_sync; the warps take their
-// slots from the chunk's per-cell cursors one after the other (a barrier per
-// warp), so the order within a cell is the original order.  Measured on
-// GB300 against tile-wise variants (eight groups per warp turn, per-warp
-// window histograms, one warp per chunk, a shared-memory radix sort of each
-// 2048-particle tile with coalesced writes), this plain form was the fastest
-// over the config-2 run: the others either lowered the number of resident
-// blocks whose turns interleave, or spent ~175 instructions per particle.
 // The scatter walks its chunk in rounds of kSub x 256 particles: warp w owns
 // the round's particles [32 kSub w, 32 kSub (w + 1)) as kSub steps of 32
 // (lane l takes particle 32 j + l of step j).  Lanes of one cell in a step are
 // ranked by __match_any_sync; in its turn a warp's leaders take their slots
 // from the per-cell cursors, step after step; the warps take their turns in
-// order, so a cell's particles keep their order in the chunk.  One round of
-// turns (a block barrier per warp) serves kSub x 256 particles; the next
-// round's particles are loaded a round ahead.  Measured on GB300 (2^25
-// particles after two sorts): kSub = 2, 30 registers, 134-147 us against 179
-// us for one step per turn; kSub = 3, 4 and 8 take more registers and fewer
-// blocks per SM and were slower (185, 147-152 and 199 us).
-constexpr int kSub = 2;
+// order, so a cell's particles keep their order in the chunk.  The next round's
+// particles are loaded a round ahead.  The turns are a serial chain, which is
+// what bounds the pass (2^25 particles: warps wait at barriers 3/4 of the time);
+// what differs is what the other warps do meanwhile.
+//   short chunks  the warps step through the turns together, a block barrier each;
+//                 kSub = 2 (30 registers; 3, 4 and 8 leave fewer blocks per SM)
+//   LONG          a warp hands its turn to the next over a barrier of the two and
+//                 goes on to its stores and its next particles' keys; kSub = 4
+//                 (2, 3 and 6 on 2^26 particles: 395, 373 and 383 us a sort against
+//                 353).  The shorter the chunk, the more of it is the way to the
+//                 last warp's first turn.
+// us a sort, short and LONG: 3e6 particles on 777 cells 30.4, 31.9; 4.2e6 on 2048
+// 37.6, 41.5; 8.4e6 on 512 51.6, 51.6, on 4096 85.6, 81.4; 1.2e7 on 4096 109, 102;
+// 2^24 on 8192 246, 197; 2^26 on 4096 385, 353; float64 8.4e6 on 1024 94, 82, 2^24
+// 174, 140.  Slots taken by fetch-adds: 379 on 2^26.
+constexpr long long kLongChunk = 8192;
 
-template <typename T>
+// A warp's turn: handed from one warp to the next over a barrier of their two (of
+// the next one's number + 1; both threads' worth of one warp wait, the other's
+// only arrive).  No barrier is used again before the turn has gone all round.
+static_assert(kSortThreads / 32 <= 15, "a named barrier per warp");
+__device__ __forceinline__ void turn_wait(int warp) {
+    asm volatile("bar.sync %0, 64;" ::"r"(warp + 1) : "memory");
+}
+__device__ __forceinline__ void turn_pass(int warp) {
+    __threadfence_block();
+    asm volatile("bar.arrive %0, 64;" ::"r"(warp + 1) : "memory");
+}
+
+template <typename T, bool LONG>
 __global__ void __launch_bounds__(kSortThreads) sort_scatter_kernel(SortArgs<T> a) {
+    constexpr int kSub = LONG ? 4 : 2;
     extern __shared__ unsigned cursor[];
     const int ng = a.ng;
     const long long start = (long long)blockIdx.x * a.chunk;
@@ -265,18 +278,26 @@ __global__ void __launch_bounds__(kSortThreads) sort_scatter_kernel(SortArgs<T> 
             leader[j] = __ffs(peers[j]) - 1;
             base[j] = 0u;
         }
-        for (int w = 0; w < nwarp; w++) {
-            if (w == warp) {
+        auto take = [&] {
 #pragma unroll
-                for (int j = 0; j < kSub; j++) {
-                    if (key[j] != kNoKey && lane == leader[j]) {
-                        base[j] = cursor[key[j]];
-                        cursor[key[j]] = base[j] + (unsigned)__popc(peers[j]);
-                    }
-                    __syncwarp();
+            for (int j = 0; j < kSub; j++) {
+                if (key[j] != kNoKey && lane == leader[j]) {
+                    base[j] = cursor[key[j]];
+                    cursor[key[j]] = base[j] + (unsigned)__popc(peers[j]);
                 }
+                __syncwarp();
             }
-            __syncthreads();
+        };
+        if (LONG) {
+            if (warp > 0 || r0 > start) turn_wait(warp);
+            take();
+            if (warp < nwarp - 1) turn_pass(warp + 1);
+            else if (r0 + round < end) turn_pass(0);
+        } else {
+            for (int w = 0; w < nwarp; w++) {
+                if (w == warp) take();
+                __syncthreads();
+            }
         }
 #pragma unroll
         for (int j = 0; j < kSub; j++) {
@@ -309,7 +330,9 @@ cudaError_t launch_sort_t(const SortArgs<T> &a, cudaStream_t s) {
     if (e == cudaSuccess)
         e = launch_after(one ? &sort_base_kernel<T, true> : &sort_base_kernel<T, false>, dim3(1), kBaseThreads,
                          0, s, 0, a);
-    if (e == cudaSuccess) e = launch_after(&sort_scatter_kernel<T>, dim3(a.nchunk), kSortThreads, smem, s, 0, a);
+    if (e == cudaSuccess)
+        e = launch_after(a.chunk >= kLongChunk ? &sort_scatter_kernel<T, true> : &sort_scatter_kernel<T, false>,
+                         dim3(a.nchunk), kSortThreads, smem, s, 0, a);
     return e;
 }
 
@@ -320,9 +343,12 @@ cudaError_t sort_prepare_attributes(int ng) {
     const int bytes = PIC_NCELL_MAX * (int)sizeof(unsigned);
     cudaError_t e;
     if ((e = cudaFuncSetAttribute(&sort_count_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes))) return e;
-    if ((e = cudaFuncSetAttribute(&sort_scatter_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes))) return e;
     if ((e = cudaFuncSetAttribute(&sort_count_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes))) return e;
-    return cudaFuncSetAttribute(&sort_scatter_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    for (auto *k : {&sort_scatter_kernel<float, false>, &sort_scatter_kernel<float, true>})
+        if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes))) return e;
+    for (auto *k : {&sort_scatter_kernel<double, false>, &sort_scatter_kernel<double, true>})
+        if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes))) return e;
+    return cudaSuccess;
 }
 
 cudaError_t launch_sort_f32(const SortArgs<float> &a, cudaStream_t s) { return launch_sort_t(a, s); }

@@ -207,3 +207,22 @@ def test_a_sort_is_the_stable_order_by_cell(n, ng):
         run.push(), run.solve_field()
         u, v = run.get_cells()
     run.close()
+
+
+@pytest.mark.parametrize("n,ng", [(8388608, 4096), (8388609, 64), (8389631, 777), (9000001, 8192)])
+@pytest.mark.parametrize("precision", [pic.PIC_FP32_FIXED, pic.PIC_FP64])
+def test_a_sort_of_long_chunks_is_the_stable_order_by_cell(n, ng, precision):
+    run = pic.Run(pic.Params(npart=n, ncell=ng, length=L, precision=precision, sort_interval=8), device="cuda:0")
+    rng = np.random.default_rng(n)
+    x = np.minimum(rng.uniform(0.0, L, n).astype(run.p.dtype), np.nextafter(run.p.dtype(L), run.p.dtype(0)))
+    run.init(x, np.arange(n, dtype=run.p.dtype) * run.p.dtype(1e-9))
+    if precision == pic.PIC_FP64:
+        u, key = x, np.minimum((x * (ng / L)).astype(np.int64), ng - 1)
+        take = lambda: run.get_state()[0]
+    else:
+        u = run.get_cells()[0]
+        key = np.clip(u, 0, ng - 1).astype(np.int64)
+        take = lambda: run.get_cells()[0]
+    run.sort()
+    assert np.array_equal(take(), u[np.argsort(key, kind="stable")])
+    run.close()
