@@ -28,7 +28,6 @@ constexpr size_t kAlign = 256;
 // least idle arena space for a read-back's device conversion: below it the
 // pieces' launches and copies cost more than the host's own conversion
 constexpr size_t kMinScratch = 256 * 1024;
-constexpr size_t kStageRows = 512;     // history rows that fit the staging memory
 size_t align_up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign; }
 
 struct RunLayout {
@@ -477,7 +476,6 @@ int pic_pool_create(const pic_pool_config *cfg, void *arena, size_t arena_bytes,
     if (e == cudaSuccess && coop) e = steps_pool_prepare(&per_sm);
     if (e != cudaSuccess) { delete pool; return cuda_fail(e); }
     if (per_sm > 0) pool->resident_sms = pool->sms;
-    pool->stage.create(kStageRows * sizeof(pic_diag_row) + 32 * (size_t)cfg->ncell_max + 1024);
     rc = set_shape(pool, cfg->variant ? cfg->variant : kPoolVariant,
                    cfg->cluster ? cfg->cluster : 8, cfg->block ? cfg->block : kPoolBlock);
     if (rc) { delete pool; return rc; }

@@ -24,7 +24,6 @@ constexpr int kMaxPushGrid = 4096;     // per-block partial sums kept
 constexpr int kMaxSortChunks = 1024;
 constexpr int kPlainBlock = 16;        // steps per graph when not sorting
 constexpr int kDefaultHistory = 4096;
-constexpr size_t kStageRows = 512;     // history rows that fit the staging memory
 constexpr int64_t kMaxLaunchSteps = 1 << 20;   // of one many-step launch
 
 size_t align_up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign; }
@@ -634,7 +633,6 @@ int pic_create(const pic_params *p, void *workspace, size_t workspace_bytes,
     make_layout(p, &r->lay);
     if (workspace_bytes < r->lay.total) { delete r; return PIC_ENOMEM; }
     r->ws = (unsigned char *)workspace;
-    r->stage.create(kStageRows * sizeof(pic_diag_row) + 32 * (size_t)p->ncell + 1024);
     r->stream = (cudaStream_t)stream;
     cudaError_t e = cudaGetDevice(&r->device);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&r->sms, cudaDevAttrMultiProcessorCount, r->device);
