@@ -239,7 +239,6 @@ __global__ void __launch_bounds__(kClusterSolveThreads) pic_solve_cluster_kernel
     const int C = (int)cl.num_blocks(), r = (int)cl.block_rank();
     const int ng = a.ng, t = threadIdx.x;
     cudaGridDependencySynchronize();
-    cudaTriggerProgrammaticLaunchCompletion();      // the next push may come up
     const long long step = *a.dstep;
     const i128 ntot = whole_density<MODE>(a);
     const int per = (int)blockDim.x;              // whole warps of nodes
@@ -432,7 +431,6 @@ __global__ void __launch_bounds__(kClusterSolveThreads) pic_solve_cg_kernel(Solv
     const int C = (int)cl.num_blocks(), r = (int)cl.block_rank();
     const int ng = a.ng, t = threadIdx.x, lane = t & 31, w = t >> 5, nw = blockDim.x >> 5;
     cudaGridDependencySynchronize();
-    cudaTriggerProgrammaticLaunchCompletion();      // the next push may come up
     const long long step = *a.dstep;
     const double dx = a.dx;
     const int per = (ng + C - 1) / C;

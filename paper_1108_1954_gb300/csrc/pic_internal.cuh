@@ -301,11 +301,13 @@ cudaError_t batch_prepare_attributes();
 // or writes what that one, or any before it, works on
 // (cudaGridDependencySynchronize; all before it too, as each such kernel waits
 // itself before it ends).  A kernel lets the next one's blocks come up with
-// cudaTriggerProgrammaticLaunchCompletion.  A push comes up while the solve before
-// it runs on a few SMs, clears its tile and waits; the solve comes up as the
-// push's blocks end.  us a step, plain launches and these: from a graph, 2e4
-// particles on 64 cells 12.3, 11.5, 1e6 on 1024 21.6, 20.0; launched one by one,
-// 2e6 on 1024 26.6, 22.3; float32 atomic, 2^24 on 1024 68.2, 63.1.
+// cudaTriggerProgrammaticLaunchCompletion.  The solve does not: a push that comes up
+// while the solve's blocks still hold some SMs is spread unevenly where its own
+// shape leaves room (2^25 particles, one block of 512 per SM: 166 us a step, 121
+// without).  So a push follows as the solve's blocks end, a solve as the push's
+// do.  us a step, plain launches and these: from a graph, 2e4 particles on 64 cells
+// 12.3, 12.0, 1e6 on 1024 21.6, 20.5; launched one by one, 2e6 on 1024 26.6, 22.3;
+// float32 atomic, 2^24 on 1024 68.2, 63.
 template <class... P>
 cudaError_t launch_after(void (*k)(P...), dim3 grid, int block, size_t smem, cudaStream_t s, int cluster,
                          const P &...args) {
