@@ -338,7 +338,7 @@ __global__ void __launch_bounds__(kClusterSolveThreads) pic_solve_cluster_kernel
 //     beta v + r itself, the same operation on the same numbers as the owner;
 //   * t = c / z.v and beta = d / c are corrected products with reciprocals
 //     (recip64, divide64), of which 1/c is formed while the sums cross.
-// A solve of 150 iterations takes 304 us on 1024 nodes, 549 with cluster barriers,
+// A solve of 150 iterations takes 333 us on 1024 nodes, 549 with cluster barriers,
 // float64 trees and divisions; an iteration's 520 instructions a warp, one
 // after the other at 7.4 clocks, are what bounds it now.
 // A block's barrier of one sum cannot complete again before the block has added
