@@ -449,10 +449,11 @@ cudaError_t set_steps_shape(pic_run *r) {
     e = f64 ? steps64_prepare(p.ncell, block, &per_sm)
             : steps_prepare(r->variant, p.ncell, block, r->steps_small, &per_sm);
     if (e != cudaSuccess || per_sm < 1) return e;
-    const int most = (r->sms < kStepsMaxGrid ? r->sms : kStepsMaxGrid) - kStepsDiag;
+    const int nd = steps_diag_blocks(r->lay.hist_len);
+    const int most = (r->sms < kStepsMaxGrid ? r->sms : kStepsMaxGrid) - nd;
     if (most < 1) return cudaSuccess;
     const int64_t need = ((f64 || r->steps_small ? p.npart : (p.npart + 3) / 4) + block - 1) / block;
-    r->steps_grid = (int)(need < most ? need : most) + kStepsDiag;
+    r->steps_grid = (int)(need < most ? need : most) + nd;
     r->steps_block = block;
     return cudaSuccess;
 }
@@ -480,7 +481,8 @@ int run_steps(pic_run *r, int steps) {
     a.err = &r->dev()->err;
     a.sync = r->dev()->sync;
     for (int i = 0; i < 3; i++) a.base[i] = r->sync_base[i];
-    a.diag_blocks = kStepsDiag;
+    const int nd = steps_diag_blocks(r->lay.hist_len);
+    a.diag_blocks = nd;
     a.first_block = 0;
     a.blocks = r->steps_grid;
     a.hist = r->at<pic_diag_row>(r->lay.hist);
@@ -500,9 +502,8 @@ int run_steps(pic_run *r, int steps) {
     PIC_CUDA(r->p.precision == PIC_FP64
                  ? launch_steps64(a, r->steps_grid, r->steps_block, r->stream)
                  : launch_steps(a, r->variant, r->steps_grid, r->steps_block, r->steps_small, r->stream));
-    r->sync_base[0] += (unsigned)(r->steps_grid - kStepsDiag) * ((unsigned)steps + 1u);
-    for (int d = 0; d < kStepsDiag; d++)
-        r->sync_base[1 + d] += (unsigned)((steps - d + kStepsDiag - 1) / kStepsDiag);
+    r->sync_base[0] += (unsigned)(r->steps_grid - nd) * ((unsigned)steps + 1u);
+    for (int d = 0; d < nd; d++) r->sync_base[1 + d] += (unsigned)((steps - d + nd - 1) / nd);
     r->step += steps;
     return PIC_OK;
 }

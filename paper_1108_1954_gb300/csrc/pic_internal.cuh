@@ -149,7 +149,11 @@ struct StepsArgs {
 };
 constexpr int kStepsMaxGrid = 256;
 constexpr int kStepsSlots = 6;     // accumulators in turn
-constexpr int kStepsDiag = 2;      // blocks of a single run's grid without particles
+constexpr int kStepsDiag = 2;      // blocks of a single run's grid without particles, at most
+// Two of them write the rows of steps up to kStepsSlots - 1 apart in no fixed
+// order, each step its own row and the one before: up to kStepsSlots rows, where
+// those can be one slot of the ring, a run has one.
+constexpr int steps_diag_blocks(int hist_len) { return hist_len > kStepsSlots ? kStepsDiag : 1; }
 constexpr int kStepsPoolBlock = 1024;
 constexpr int kStepsMaxCells = 4096;
 // largest runs: up to 2048 cells, and beyond

@@ -17,7 +17,8 @@
 //            integer arithmetic, so all blocks get the same bits, and with one
 //            node per thread its cost hardly depends on NG.
 //
-// Two more blocks have no particles.  They take the steps in turn and, while
+// Two more blocks (one where the history ring is short: pic_internal.cuh,
+// steps_diag_blocks) have no particles.  They take the steps in turn and, while
 // the workers go on, compute a step's diagnostics (float64 work that would hold
 // the workers up: at 64 clocks a dependent float64 add and 840 a square root,
 // a step's take 5 to 10 thousand clocks, up to twice a worker's step), then

@@ -113,8 +113,9 @@ __device__ __forceinline__ void step_rows(const StepsArgs &a, int s, const Solve
                             : lane == 2 ? 0.5 * a.dx : a.dx * a.k_rho;
         const double fe0 = __shfl_sync(kFull, fe_total, 0);
         const double val = coef * (lane < 2 ? tot[lane] : lane == 2 ? fe0 : i128_to_f64((i128)ns.SR));
-        if (lane < 4) *(lane == 0 ? &prev->kinetic : lane == 1 ? &prev->momentum
-                        : lane == 2 ? &row->field : &row->charge) = val;
+        if (lane < 4 && (lane >= 2 || prev != row))       // (a ring of one row: only the new one)
+            *(lane == 0 ? &prev->kinetic : lane == 1 ? &prev->momentum
+              : lane == 2 ? &row->field : &row->charge) = val;
         if (lane == 4) row->step = n;
         // sum of rho_q: SR = NG (N 2^24 - it), 0 unless particles were lost
         if (lane == 5) row->charge_q = !FIXED ? 0 : ns.SR ? a.weight_total - (long long)ns.SR / ng : a.weight_total;

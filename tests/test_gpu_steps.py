@@ -226,3 +226,54 @@ def test_a_sort_of_long_chunks_is_the_stable_order_by_cell(n, ng, precision):
     run.sort()
     assert np.array_equal(take(), u[np.argsort(key, kind="stable")])
     run.close()
+
+
+@pytest.mark.parametrize("H", [1, 2, 3, 4, 5, 6, 7, 8])
+@pytest.mark.parametrize("n,ng,precision", [(20000, 64, pic.PIC_FP32_FIXED), (300007, 777, pic.PIC_FP32_FIXED),
+                                            (5001, 1025, pic.PIC_FP32_FIXED), (20000, 64, pic.PIC_FP64)])
+def test_short_history_rings_hold_the_last_rows(H, n, ng, precision):
+    # rows that share a slot of the ring are written in the steps' order
+    rng = np.random.default_rng(H)
+    dt = np.float64 if precision == pic.PIC_FP64 else np.float32
+    x, v = rng.uniform(0.0, 0.999 * L, n).astype(dt), rng.normal(0.0, 0.4, n).astype(dt)
+    runs = []
+    for kw in (dict(), dict(block_size=256)):
+        r = pic.Run(pic.Params(npart=n, ncell=ng, length=L, precision=precision, history=H, **kw), device="cuda:0")
+        r.init(x, v)
+        runs.append(r)
+    for k in (1, 2, 5, 6, 7, 40):
+        rows = []
+        for r in runs:
+            r.step_n(k)
+            rows.append(r.diagnostics(max(0, r.step - H + 1), min(H, r.step + 1)))
+        d, e = rows
+        for key in ("step", "charge_q", "charge", "field"):
+            assert np.array_equal(d[key], e[key]), key
+        for key in ("kinetic", "momentum"):
+            assert np.isnan(d[key][-1]) and np.all(np.isfinite(d[key][:-1]))
+        np.testing.assert_allclose(d["kinetic"][:-1], e["kinetic"][:-1], rtol=1e-5)
+        np.testing.assert_allclose(d["mode"], e["mode"], rtol=0, atol=64 * 2.0 ** -24 * 2.0 / ng *
+                                   np.abs(runs[0].get_field()["E"]).sum() + 1e-12)
+    for r in runs:
+        r.close()
+
+
+@pytest.mark.parametrize("H", [1, 2, 3])
+def test_short_history_rings_of_a_pool(H):
+    n, ng = 20000, 64
+    p = pic.Params(npart=n, ncell=ng, length=L, history=H)
+    x, v = state(n, 5)
+    pool = pic.Pool(max_slots=1, ncell_max=ng, arena_bytes=1 << 24, history=H, device="cuda:0")
+    slot = pool.admit(p, x, v, 30)
+    run = pic.Run(pic.Params(npart=n, ncell=ng, length=L, history=H, block_size=256), device="cuda:0")
+    run.init(x, v)
+    for k in (1, 2, 7, 20):
+        pool.advance(k)
+        run.step_n(k)
+        first, count = max(0, run.step - H + 1), min(H, run.step + 1)
+        d, e = pool.diagnostics(slot, first, count), run.diagnostics(first, count)
+        for key in ("step", "charge_q"):
+            assert np.array_equal(d[key], e[key]), key
+        np.testing.assert_allclose(d["field"], e["field"], rtol=1e-12)
+        assert np.isnan(d["kinetic"][-1]) and np.all(np.isfinite(d["kinetic"][:-1]))
+    pool.close()
