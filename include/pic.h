@@ -308,6 +308,15 @@ int pic_device_arrays(pic_run *run, void **x, void **v, void **E32);
 int pic_launch_shape(const pic_run *run, int32_t *grid, int32_t *block,
                      int32_t *variant, int32_t *unroll);
 
+/* The waits between the blocks of a kernel (the many-step launch, the CG solver):
+ * each gives up after `polls` tries (>= PIC_WAIT_LIMIT_MIN; 0: the default, some
+ * seconds), the kernel returns, and the next synchronising call reports
+ * PIC_ETIMEOUT.  missing (0 or 1): arrivals that a wait expects beyond those that
+ * come.  With 1 the waits of the steps that follow run out, which is how the
+ * handling of a time-out is tested; nothing else is changed. */
+#define PIC_WAIT_LIMIT_MIN 4096
+int pic_set_wait_limit(pic_run *run, int32_t polls, int32_t missing);
+
 /* Device-side initial loading of a two-stream plasma (Sec. 2, the initial set-up;
  * Appendix A; the Sec. 4 beams).  Particle j of N:
  *   x = (j + 1/2) L/N - sum_m (eps_m/k_m) sin(k_m x0 + phase_m), k_m = 2 pi m/L,

@@ -100,6 +100,7 @@ _SIG = {
     "pic_launch_shape": (C.c_int, [_VP, C.POINTER(C.c_int32), C.POINTER(C.c_int32),
                                    C.POINTER(C.c_int32), C.POINTER(C.c_int32)]),
     "pic_autotune": (C.c_int, [_VP, C.c_int32, _VP, C.c_int32, C.POINTER(C.c_int32)]),
+    "pic_set_wait_limit": (C.c_int, [_VP, C.c_int32, C.c_int32]),
     "pic_set_launch": (C.c_int, [_VP, C.c_int32, C.c_int32, C.c_int32, C.c_int32]),
     "pic_set_shard": (C.c_int, [_VP, C.c_int64]),
     "pic_device_density": (C.c_int, [_VP, C.POINTER(_VP)]),
@@ -358,6 +359,12 @@ class Run:
                    blocks_per_sm: int = 0):
         _check(_lib.pic_set_launch(self._h, int(variant), int(block), int(unroll),
                                    int(blocks_per_sm)), "pic_set_launch")
+
+    def set_wait_limit(self, polls: int = 0, missing: int = 0):
+        """Polls after which a wait between a kernel's blocks gives up (0: the
+        default); missing = 1 makes the waits of the steps that follow run
+        out (for tests of what comes after)."""
+        _check(_lib.pic_set_wait_limit(self._h, int(polls), int(missing)), "pic_set_wait_limit")
 
     def autotune(self, reps: int = 5, cache: str | None = None) -> np.ndarray:
         """Time the candidate push shapes on a copy of the state and adopt

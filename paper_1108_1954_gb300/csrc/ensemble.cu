@@ -372,6 +372,7 @@ int launch_resident(pic_pool *pool, const std::vector<int> &order, const std::ve
         a.err = pool->d_err();
         a.sync = reinterpret_cast<unsigned *>(mem + parts[i].sync);
         a.base[0] = a.base[1] = a.base[2] = 0;
+        a.wait_limit = kStepsWaitLimit;
         a.diag_blocks = 1;
         a.first_block = first;
         a.blocks = workers[i] + 1;

@@ -338,14 +338,16 @@ __global__ void __launch_bounds__(kClusterSolveThreads) pic_solve_cluster_kernel
 //     beta v + r itself, the same operation on the same numbers as the owner;
 //   * t = c / z.v and beta = d / c are corrected products with reciprocals
 //     (recip64, divide64), of which 1/c is formed while the sums cross.
-// A solve of 150 iterations takes 333 us on 1024 nodes, 549 with cluster barriers,
+// A step of 150 iterations takes 311 us on 1024 nodes, 549 with cluster barriers,
 // float64 trees and divisions; an iteration's 520 instructions a warp, one
 // after the other at 7.4 clocks, are what bounds it now.
 // A block's barrier of one sum cannot complete again before the block has added
 // its own part of the next sum, which it sends only after reading the first, so
-// one buffer per sum is enough.  Every wait has a limit (kCgSpinLimit tries),
-// after which the block sets kErrWait and all blocks leave the loop.
-constexpr unsigned kCgSpinLimit = 1u << 20;    // tries of up to a microsecond
+// one buffer per sum is enough.  Every wait has a limit (SolveArgs::wait_limit
+// tries of up to a microsecond), after which the thread sets kErrWait and its sum is
+// no number, with which its warp, the block at the end of the iteration (the only
+// way out of the loop, so that the barriers of all warps match) and, for want of
+// its sums, the other blocks stop.  What a block sent last has arrived by then.
 
 constexpr int kCgParts = kMaxSolveCluster * kClusterSolveThreads / 32;    // warps of a cluster
 
@@ -389,9 +391,9 @@ __device__ __forceinline__ void expect_bytes(bool on, const void *bar, unsigned 
                  ::"r"(smem_addr(bar)), "r"(bytes), "r"((unsigned)on) : "memory");
 }
 
-__device__ __forceinline__ bool wait_phase(const void *bar, unsigned parity) {
+__device__ __forceinline__ bool wait_phase(const void *bar, unsigned parity, unsigned limit) {
 #pragma unroll 1
-    for (unsigned i = 0; i < kCgSpinLimit; i++) {
+    for (unsigned i = 0; i < limit; i++) {
         unsigned done;
         asm volatile("{\n\t.reg .pred p;\n\t"
                      "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2, 1000;\n\t"
@@ -468,29 +470,30 @@ __global__ void __launch_bounds__(kClusterSolveThreads) pic_solve_cg_kernel(Solv
     const bool first = t == 0 && r > 0, final = t == cnt - 1 && r < C - 1;
     const int nb = first ? r - 1 : final ? r + 1 : 0;
     const unsigned ndst = peer_addr(&ex.nbr[first ? 1 : 0], nb), nbar = peer_addr(&ex.bar[1], nb);
-    const unsigned zv_bytes = 8u * (unsigned)(C * nw);
+    const unsigned zv_bytes = 8u * ((unsigned)(C * nw) + a.wait_missing);
     const unsigned rr_bytes = zv_bytes + 16u * (unsigned)((r > 0 ? 1 : 0) + (r < C - 1 ? 1 : 0));
     double xg = 0.0;
     double rg = (mine && g >= 1) ? (-rh * dx) * dx : 0.0;
     double vg = 0.0;
-    bool dead = false;                                // a wait ran out
+    bool dead = false;                                // a wait of this thread ran out
     // Every warp takes the sums itself where a block has few (no block barrier
     // between the sum and its use); where it has many, their float64 scalars
     // would fill the pipe, and warp 0 hands them on.
     const bool every = nw <= 4;
+    const double nan = __longlong_as_double(0x7ff8000000000000ll);
     auto publish = [&](int which, double p) {
         const double f = warp_sum_fixed(p);
         send8(lane < C, dst[which], f, bar[which]);
     };
     auto total = [&](int which, unsigned parity) {
-        dead |= !wait_phase(&ex.bar[which], parity);
+        dead |= !wait_phase(&ex.bar[which], parity, a.wait_limit);
         double v = lane < C * nw ? ex.part[which][lane] : 0.0;
         for (int i = lane + 32; i < C * nw; i += 32) v += ex.part[which][i];
-        return warp_sum_fixed(v);
+        return warp_sum_fixed(dead ? nan : v);        // in all lanes
     };
-    const double nan = __longlong_as_double(0x7ff8000000000000ll);
     double c = 0.0, rc = 0.0, beta = 0.0;
     for (int it = -1; it < a.cg_maxit; it++) {
+        bool stop = false;                            // uniform over the warp, if not `every` the block
         if (it >= 0) {                                // (it = -1: r.r of the start)
             const double vc = sv[t + 1];
             double z = fma(-2.0, vc, sv[t]) + sv[t + 2];      // (Phi_NG = 0: the last ghost stays 0)
@@ -504,44 +507,52 @@ __global__ void __launch_bounds__(kClusterSolveThreads) pic_solve_cg_kernel(Solv
                 const double zv = total(0, (unsigned)it & 1u);
                 tk = divide64(c, zv, recip64(zv));
                 // stop where the step would divide by zero
-                tk = dead || zv == 0.0 ? nan : tk;
+                tk = zv == 0.0 ? nan : tk;
             }
             if (!every) {
                 if (t == 0) scal[0] = tk;
                 __syncthreads();
                 tk = scal[0];
             }
-            if (!isfinite(tk)) break;                 // uniform over the cluster
-            xg = fma(tk, vg, xg);
-            rg = fma(-tk, z, rg);
+            stop = !isfinite(tk);
+            if (!stop) {
+                xg = fma(tk, vg, xg);
+                rg = fma(-tk, z, rg);
+            }
         }
-        publish(1, rg * rg);
-        send16(first || final, ndst, vg, rg, nbar);
-        expect_bytes(t == 0, &ex.bar[1], rr_bytes);
-        if (every || w == 0) {
-            const double d = total(1, (unsigned)(it + 1) & 1u);
-            beta = it < 0 ? 0.0 : divide64(d, c, rc);
-            // stop where the next step would divide by zero, and at the start where
-            // |r| <= 1e-16
-            if (dead || !(d > 0.0) || (it < 0 && !(sqrt(d) > 1e-16 && ng > 1))) beta = nan;
-            c = d;
+        if (!stop) {
+            publish(1, rg * rg);
+            send16(first || final, ndst, vg, rg, nbar);
+            expect_bytes(t == 0, &ex.bar[1], rr_bytes);
+            if (every || w == 0) {
+                const double d = total(1, (unsigned)(it + 1) & 1u);
+                beta = it < 0 ? 0.0 : divide64(d, c, rc);
+                // stop where the next step would divide by zero, and at the start where
+                // |r| <= 1e-16
+                if (!(d > 0.0) || (it < 0 && !(sqrt(d) > 1e-16 && ng > 1))) beta = nan;
+                c = d;
+            }
+            if (!every) {
+                if (t == 0) scal[1] = beta;
+                __syncthreads();
+                beta = scal[1];
+            }
+            stop = !isfinite(beta);
         }
-        if (!every) {
-            if (t == 0) scal[1] = beta;
-            __syncthreads();
-            beta = scal[1];
+        if (!stop) {
+            vg = fma(beta, vg, rg);
+            if (mine) sv[t + 1] = vg;
+            // the neighbours' boundary v, formed as they form it
+            const double2 nv = ex.nbr[final ? 1 : 0];
+            const double gv = fma(beta, nv.x, nv.y);
+            if (first || final) sv[final ? cnt + 1 : 0] = gv;
         }
-        if (!isfinite(beta)) break;
-        vg = fma(beta, vg, rg);
-        if (mine) sv[t + 1] = vg;
-        // the neighbours' boundary v, formed as they form it
-        const double2 nv = ex.nbr[final ? 1 : 0];
-        const double gv = fma(beta, nv.x, nv.y);
-        if (first || final) sv[final ? cnt + 1 : 0] = gv;
-        if (nw > 1) __syncthreads();
-        else __syncwarp();
+        if (nw == 1) __syncwarp();
+        else if (every) stop = __syncthreads_or(stop);
+        else __syncthreads();
+        if (stop) break;
     }
-    if (dead && t == 0) atomicOr(a.err, kErrWait);
+    if (dead) atomicOr(a.err, kErrWait);
     // Phi = x; E by Eq. 7 with periodic neighbours (across the blocks)
     __syncthreads();
     if (mine) sv[t + 1] = xg;

@@ -167,6 +167,7 @@ struct pic_run {
     int steps_grid = 0, steps_block = 0;   // many-step launch (0: not taken)
     bool steps_small = false;              // one particle per lane
     unsigned sync_base[3] = {0, 0, 0};   // its counters so far
+    unsigned wait_limit = 0, wait_missing = 0;   // pic_set_wait_limit
     int64_t step = 0;
     bool ready = false, pending_push = false;
     cudaGraphExec_t period[2] = {nullptr, nullptr};   // S steps from x parity 0/1
@@ -279,6 +280,8 @@ cudaError_t enqueue_solve(pic_run *r, cudaStream_t s, bool after_push) {
     a.dx = r->dx;
     a.mass = r->mass;
     a.err = &r->dev()->err;
+    a.wait_limit = r->wait_limit ? r->wait_limit : kCgWaitLimit;
+    a.wait_missing = r->wait_missing;
     a.solver = r->p.field_solver;
     a.cg_maxit = r->p.cg_iterations ? r->p.cg_iterations : PIC_CG_DEFAULT_ITERATIONS;
     return launch_solve(a, s);
@@ -481,6 +484,8 @@ int run_steps(pic_run *r, int steps) {
     a.err = &r->dev()->err;
     a.sync = r->dev()->sync;
     for (int i = 0; i < 3; i++) a.base[i] = r->sync_base[i];
+    a.base[0] += r->wait_missing;
+    a.wait_limit = r->wait_limit ? r->wait_limit : kStepsWaitLimit;
     const int nd = steps_diag_blocks(r->lay.hist_len);
     a.diag_blocks = nd;
     a.first_block = 0;
@@ -1058,6 +1063,14 @@ done:
     if (rc) return rc;
     PIC_CUDA(cudaMemsetAsync(run->ws + run->lay.tune_rho, 0, (size_t)run->p.ncell * 8, run->stream));
     return read_error_word(run);
+}
+
+int pic_set_wait_limit(pic_run *run, int32_t polls, int32_t missing) {
+    if (!run || (polls != 0 && polls < PIC_WAIT_LIMIT_MIN) || missing < 0 || missing > 1) return PIC_EINVAL;
+    run->wait_limit = (unsigned)polls;
+    run->wait_missing = (unsigned)missing;
+    destroy_graphs(run);
+    return PIC_OK;
 }
 
 int pic_set_shard(pic_run *run, int64_t npart_total) {

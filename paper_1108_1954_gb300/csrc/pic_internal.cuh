@@ -110,6 +110,8 @@ struct SolveArgs {
     double dx;
     double mass;                  // particle mass m = Q0/qm
     unsigned *err;                // device error word (the CG's waits)
+    unsigned wait_limit;          // CG: tries of a wait ...
+    unsigned wait_missing;        // ... and values it expects beyond those sent (0; tests)
     int solver;                   // PIC_SOLVER_EXACT / PIC_SOLVER_CG
     int cg_maxit;                 // CG: iterations per solve
 };
@@ -134,6 +136,7 @@ struct StepsArgs {
     unsigned *sync;               // [4], 16-byte aligned: arrivals of the workers, steps
                                   // done by each diagnostics block; never reset ...
     unsigned base[3];             // ... their values before this launch
+    unsigned wait_limit;          // polls of a wait
     int diag_blocks;              // 1 or 2: the last of the run's blocks, without particles
     int first_block, blocks;      // the run's part of a pool's grid
     int log_copies;               // copies of a block's tile (set by the launcher)
@@ -147,12 +150,15 @@ struct StepsArgs {
     long long weight_total;       // N 2^24 (fixed point)
     double k_rho, k_e, k_phi, k_mode, dx, mass;   // as SolveArgs
 };
+// Limits of the waits (some seconds, and about one) when the caller sets none.
+constexpr unsigned kStepsWaitLimit = 1u << 23, kCgWaitLimit = 1u << 20;
 constexpr int kStepsMaxGrid = 256;
 constexpr int kStepsSlots = 6;     // accumulators in turn
 constexpr int kStepsDiag = 2;      // blocks of a single run's grid without particles, at most
 // Two of them write the rows of steps up to kStepsSlots - 1 apart in no fixed
 // order, each step its own row and the one before: up to kStepsSlots rows, where
-// those can be one slot of the ring, a run has one.
+// those can be one slot of the ring, a run has one (us a step with one and two: 2e4
+// particles on 64 cells 3.9, 2.8; 1e6 on 1024 7.7, 8.0; 1e6 on 4096 17.7, 12.3).
 constexpr int steps_diag_blocks(int hist_len) { return hist_len > kStepsSlots ? kStepsDiag : 1; }
 constexpr int kStepsPoolBlock = 1024;
 constexpr int kStepsMaxCells = 4096;

@@ -62,7 +62,7 @@
 // 2^-64 of a rounding boundary of float32, where the chain's own three
 // roundings (each 2^-53) could matter, the chain itself is evaluated.
 //
-// Every wait has a limit (kSpinLimit polls, some seconds), after which the block
+// Every wait has a limit (kStepsWaitLimit polls, some seconds), after which the block
 // sets kErrWait and all blocks return.
 #include "steps_common.cuh"
 

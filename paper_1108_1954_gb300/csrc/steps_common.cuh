@@ -9,8 +9,6 @@
 namespace pic {
 namespace {
 
-constexpr unsigned kSpinLimit = 1u << 23;  // polls of one grid barrier
-
 // The launch's counters, never reset: arrivals of the workers (one a step, and one
 // when the last step's sums have been read), and the steps that each diagnostics
 // block is done with (StepsArgs::sync, on 16 bytes).
@@ -45,7 +43,7 @@ __device__ __forceinline__ bool wait_step(const StepsArgs &a, int s, int workers
             const uint4 v = ld_acquire(a.sync);
             if ((int)(v.x - target) >= 0 && (!worker || ((int)(v.y - d0) >= 0 && (int)(v.z - d1) >= 0)))
                 break;
-            if (++polls >= kSpinLimit) {
+            if (++polls >= a.wait_limit) {
                 atomicOr(a.err, kErrWait);
                 *dead = 1;
                 break;
