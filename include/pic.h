@@ -67,7 +67,8 @@ extern "C" {
 #define PIC_ECUDA (-3)    /* a CUDA runtime call failed                       */
 #define PIC_ETIMEOUT (-4) /* a wait between the blocks of a kernel ran out of
                              its limit (the many-step launch, the CG
-                             solver); a run needs pic_init or pic_set_state  */
+                             solver); a run needs pic_init or pic_set_state,
+                             a pool's run is lost (pic_pool_advance)         */
 #define PIC_EDEVICE (-5)  /* a kernel flagged bad particle data                */
 #define PIC_ESTATE (-6)   /* call out of order (e.g. push before init)         */
 
@@ -480,8 +481,14 @@ int pic_pool_admit_loaded(pic_pool *pool, const pic_params *p, const pic_loading
 
 /* Advance every admitted run by min(k, steps left) steps (set-up first for
  * newly admitted runs).  *active receives the number of runs that took part.
- * Asynchronous. */
+ * PIC_ETIMEOUT: a wait of the many-step launch ran out.  The runs that were to take
+ * part are lost: their steps are not counted, they are not advanced or reported
+ * finished any more, reading them returns PIC_ETIMEOUT, and pic_pool_release frees
+ * their place.  The pool and its other runs go on. */
 int pic_pool_advance(pic_pool *pool, int64_t k, int32_t *active);
+
+/* pic_set_wait_limit for the pool's many-step launches. */
+int pic_pool_set_wait_limit(pic_pool *pool, int32_t polls, int32_t missing);
 
 /* Slots whose runs have done all their steps (host bookkeeping; the results
  * are ready once the stream has reached the advance that finished them). */

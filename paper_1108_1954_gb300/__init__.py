@@ -114,6 +114,7 @@ _SIG = {
     "pic_pool_table_bytes": (C.c_int, [_VP, C.POINTER(C.c_size_t)]),
     "pic_pool_create": (C.c_int, [_VP, _VP, C.c_size_t, _VP, C.POINTER(_VP)]),
     "pic_pool_destroy": (None, [_VP]),
+    "pic_pool_set_wait_limit": (C.c_int, [_VP, C.c_int32, C.c_int32]),
     "pic_pool_configure": (C.c_int, [_VP, C.c_int32, C.c_int32, C.c_int32]),
     "pic_pool_admit": (C.c_int, [_VP, _P, _VP, _VP, C.c_int64, C.POINTER(C.c_int32)]),
     "pic_pool_advance": (C.c_int, [_VP, C.c_int64, C.POINTER(C.c_int32)]),
@@ -519,6 +520,11 @@ class Pool:
     def configure(self, variant: int, cluster: int, block: int):
         _check(_lib.pic_pool_configure(self._h, int(variant), int(cluster), int(block)),
                "pic_pool_configure")
+
+    def set_wait_limit(self, polls: int = 0, missing: int = 0):
+        """Run.set_wait_limit for the pool's many-step launches."""
+        _check(_lib.pic_pool_set_wait_limit(self._h, int(polls), int(missing)),
+               "pic_pool_set_wait_limit")
 
     def admit(self, p: Params, x0, v0, steps: int):
         """Slot of the admitted run, or None when the arena or slots are full."""

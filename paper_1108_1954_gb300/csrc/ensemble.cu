@@ -125,6 +125,7 @@ struct pic_pool {
     size_t used = 0;
     struct Slot {
         bool used = false, needs_init = false;
+        bool lost = false;            // in a launch whose wait ran out
         pic_params p{};
         size_t off = 0, size = 0;
         RunLayout lay{};
@@ -151,6 +152,7 @@ struct pic_pool {
     int wide_clusters = 0;        // > 0: up to so many runs take blocks twice as large
     int sms = 0;
     int resident_sms = 0;         // SMs of the many-step launch (0: not available)
+    unsigned wait_limit = 0, wait_missing = 0;   // pic_pool_set_wait_limit
     pic::Staging stage;
 
     BatchRun *d_runs() const { return reinterpret_cast<BatchRun *>(arena + tab.runs); }
@@ -331,8 +333,11 @@ bool resident(const pic_pool *pool, const std::vector<int> &order, std::vector<i
     return time < cluster_time(pool, order);
 }
 
-// Advance the runs of `order` by their steps; false (and nothing done) when the
-// arena has no room for the launch's accumulators.
+int read_error_word(pic_pool *pool, unsigned *err);
+
+// Advance the runs of `order` by their steps; *done false (and nothing done) when
+// the arena has no room for the launch's accumulators.  PIC_ETIMEOUT: a wait ran out;
+// the runs of the launch are lost, the others are as before.
 int launch_resident(pic_pool *pool, const std::vector<int> &order, const std::vector<int> &workers,
                     bool *done) {
     *done = false;
@@ -371,8 +376,9 @@ int launch_resident(pic_pool *pool, const std::vector<int> &order, const std::ve
         a.partials = reinterpret_cast<double *>(mem + parts[i].partials);
         a.err = pool->d_err();
         a.sync = reinterpret_cast<unsigned *>(mem + parts[i].sync);
-        a.base[0] = a.base[1] = a.base[2] = 0;
-        a.wait_limit = kStepsWaitLimit;
+        a.base[0] = pool->wait_missing;
+        a.base[1] = a.base[2] = 0;
+        a.wait_limit = pool->wait_limit ? pool->wait_limit : kStepsWaitLimit;
         a.diag_blocks = 1;
         a.first_block = first;
         a.blocks = workers[i] + 1;
@@ -399,25 +405,47 @@ int launch_resident(pic_pool *pool, const std::vector<int> &order, const std::ve
     PIC_CUDA(launch_steps_pool(reinterpret_cast<const StepsArgs *>(mem), (int)args.size(), first, ng_max,
                                pool->stream));
     // the scratch is free again, and the host's arguments read, when this is done
-    PIC_CUDA(cudaStreamSynchronize(pool->stream));
+    unsigned err = 0;
+    const int rc = read_error_word(pool, &err);
+    if (rc) return rc;
     *done = true;
-    return PIC_OK;
+    if (!(err & kErrWait)) return PIC_OK;
+    // the word is the pool's: what the other runs have set stays
+    for (int s : order) pool->slots[s].lost = true;
+    err &= ~kErrWait;
+    PIC_CUDA(cudaMemcpyAsync(pool->d_err(), &err, sizeof(err), cudaMemcpyHostToDevice, pool->stream));
+    PIC_CUDA(cudaStreamSynchronize(pool->stream));
+    return PIC_ETIMEOUT;
 }
 
 bool slot_ok(const pic_pool *pool, int32_t slot) {
     return pool && slot >= 0 && slot < (int)pool->slots.size() && pool->slots[slot].used;
 }
 
+// Whether a run has results to read.
+int readable(const pic_pool::Slot &sl) {
+    return sl.lost ? PIC_ETIMEOUT : sl.needs_init ? PIC_ESTATE : PIC_OK;
+}
+
 // Wait for the stream and what was queued into the staging memory; the error
 // word comes with it.  The caller holds the staging's mutex.
-int finish_read(pic_pool *pool) {
-    unsigned err = 0;
-    cudaError_t e = pool->stage.add(&err, pool->d_err(), sizeof(err), pool->stream);
+int finish_read(pic_pool *pool, unsigned *err) {
+    *err = 0;
+    cudaError_t e = pool->stage.add(err, pool->d_err(), sizeof(*err), pool->stream);
     const cudaError_t f = pool->stage.finish(pool->stream);
     if (e == cudaSuccess) e = f;
-    if (e != cudaSuccess) return cuda_fail(e);
-    if (err & kErrWait) return PIC_ETIMEOUT;
-    return err ? PIC_EDEVICE : PIC_OK;
+    return e == cudaSuccess ? PIC_OK : cuda_fail(e);
+}
+
+int finish_read(pic_pool *pool) {
+    unsigned err;
+    const int rc = finish_read(pool, &err);
+    return rc ? rc : err ? PIC_EDEVICE : PIC_OK;
+}
+
+int read_error_word(pic_pool *pool, unsigned *err) {
+    std::lock_guard<std::mutex> lock(pool->stage.mutex);
+    return finish_read(pool, err);
 }
 
 int read_error(pic_pool *pool) {
@@ -649,7 +677,7 @@ int pic_pool_advance(pic_pool *pool, int64_t k, int32_t *active) {
     order.clear();
     for (int i = 0; i < (int)pool->slots.size(); i++) {
         pic_pool::Slot &sl = pool->slots[i];
-        if (!sl.used) continue;
+        if (!sl.used || sl.lost) continue;
         const int64_t left = sl.target - sl.done;
         const int64_t take = left < k ? left : k;
         // one launch advances at most INT_MAX steps (the descriptor's int)
@@ -676,12 +704,19 @@ int pic_pool_advance(pic_pool *pool, int64_t k, int32_t *active) {
     return PIC_OK;
 }
 
+int pic_pool_set_wait_limit(pic_pool *pool, int32_t polls, int32_t missing) {
+    if (!pool || (polls != 0 && polls < PIC_WAIT_LIMIT_MIN) || missing < 0 || missing > 1) return PIC_EINVAL;
+    pool->wait_limit = (unsigned)polls;
+    pool->wait_missing = (unsigned)missing;
+    return PIC_OK;
+}
+
 int pic_pool_finished(const pic_pool *pool, int32_t *slots, int32_t max, int32_t *n) {
     if (!pool || !n || max < 0) return PIC_EINVAL;
     int c = 0;
     for (int i = 0; i < (int)pool->slots.size(); i++) {
         const pic_pool::Slot &sl = pool->slots[i];
-        if (sl.used && !sl.needs_init && sl.done >= sl.target) {
+        if (sl.used && !sl.needs_init && !sl.lost && sl.done >= sl.target) {
             if (slots && c < max) slots[c] = i;
             c++;
         }
@@ -700,7 +735,7 @@ int pic_pool_get_cells(pic_pool *pool, int32_t slot, float *u, float *v) {
     pic::TraceRange trace_("pic_pool_get_cells");
     if (!slot_ok(pool, slot)) return PIC_EINVAL;
     const pic_pool::Slot &sl = pool->slots[slot];
-    if (sl.needs_init) return PIC_ESTATE;
+    if (const int rc = readable(sl)) return rc;
     const size_t pb = (size_t)sl.p.npart * 4;
     if (u) PIC_CUDA(cudaMemcpyAsync(u, sl.desc.x, pb, cudaMemcpyDeviceToHost, pool->stream));
     if (v) PIC_CUDA(cudaMemcpyAsync(v, sl.desc.v, pb, cudaMemcpyDeviceToHost, pool->stream));
@@ -711,7 +746,7 @@ int pic_pool_get_state(pic_pool *pool, int32_t slot, void *x, void *v) {
     pic::TraceRange trace_("pic_pool_get_state");
     if (!slot_ok(pool, slot)) return PIC_EINVAL;
     const pic_pool::Slot &sl = pool->slots[slot];
-    if (sl.needs_init) return PIC_ESTATE;
+    if (const int rc = readable(sl)) return rc;
     const size_t pb = (size_t)sl.p.npart * 4;
     const double to_phys = sl.p.length / (double)sl.p.ncell;
     const float Lf = (float)sl.p.length;
@@ -750,7 +785,7 @@ int pic_pool_get_field(pic_pool *pool, int32_t slot, double *rho, double *phi, d
     pic::TraceRange trace_("pic_pool_get_field");
     if (!slot_ok(pool, slot)) return PIC_EINVAL;
     const pic_pool::Slot &sl = pool->slots[slot];
-    if (sl.needs_init) return PIC_ESTATE;
+    if (const int rc = readable(sl)) return rc;
     const size_t nb = (size_t)sl.p.ncell * 8;
     struct { void *dst; const void *src; } const want[] = {
         {rho, sl.desc.rho}, {phi, sl.desc.phi}, {E, sl.desc.E64}, {rho_q, sl.desc.rho_q_last}};
@@ -768,6 +803,7 @@ int pic_pool_diagnostics(pic_pool *pool, int32_t slot, int64_t first, int32_t co
     pic::TraceRange trace_("pic_pool_diagnostics");
     if (!slot_ok(pool, slot) || !rows || count < 0 || first < 0) return PIC_EINVAL;
     const pic_pool::Slot &sl = pool->slots[slot];
+    if (sl.lost) return PIC_ETIMEOUT;
     const int64_t H = pool->cfg.history;
     if (count == 0) return PIC_OK;
     if (first + count - 1 > sl.done || first < sl.done - H + 1) return PIC_EINVAL;

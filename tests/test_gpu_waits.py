@@ -63,3 +63,39 @@ def test_wait_limits_are_checked():
         assert e.value.code == pic.PIC_EINVAL
     r.set_wait_limit(4096, 0)
     r.close()
+
+
+def test_a_pool_loses_the_runs_of_a_launch_whose_wait_ran_out():
+    ps = [pic.Params(npart=n, ncell=ng, length=L) for n, ng in ((20000, 64), (300007, 1025), (5001, 300))]
+    pool = pic.Pool(max_slots=4, ncell_max=2048, arena_bytes=1 << 26, history=16, device="cuda:0")
+    first = pool.admit(ps[2], *state(5001, 2), 4)          # done before the others come
+    pool.advance(4)
+    kept = pool.get_state(first)
+    slots = [pool.admit(p, *state(p.npart, i), 9) for i, p in enumerate(ps[:2])]
+    pool.advance(3)
+    pool.set_wait_limit(POLLS, 1)
+    with pytest.raises(pic.PicError) as e:
+        pool.advance(6)
+    assert e.value.code == pic.PIC_ETIMEOUT
+    pool.set_wait_limit()
+    assert pool.finished() == [first]
+    for s in slots:
+        assert pool.step_count(s) == 3
+        for read in (pool.get_state, pool.get_cells, pool.get_field, lambda s: pool.diagnostics(s, 3, 1)):
+            with pytest.raises(pic.PicError) as e:
+                read(s)
+            assert e.value.code == pic.PIC_ETIMEOUT
+    pool.sync()                                            # the word is clear, the other run readable
+    for a, b in zip(pool.get_state(first), kept):
+        assert np.array_equal(a, b)
+    assert pool.advance(6) == 0
+    for s in slots:
+        pool.release(s)
+    again = pool.admit(ps[1], *state(300007, 1), 5)
+    assert pool.advance(9) == 1 and sorted(pool.finished()) == sorted([first, again])
+    run = pic.Run(ps[1], device="cuda:0")
+    run.init(*state(300007, 1))
+    run.step_n(5)
+    for a, b in zip(pool.get_cells(again), run.get_cells()):
+        assert np.array_equal(a, b)
+    assert np.array_equal(pool.get_field(again)["E"], run.get_field()["E"])
