@@ -211,9 +211,11 @@ int pic_sort(pic_run *run);
 /* n whole steps: [sort if due] + push + solve.  Runs with the exact solver
  * whose launch shape is left open (pic_params, pic_set_launch) take many steps
  * per cooperative launch: PIC_FP32_FIXED up to 24e6 particles on 2048 cells or
- * 12.5e6 on 4096, PIC_FP64 up to 1e6 on 1024.  Others replay CUDA graphs.  The
- * results are the same.  While the stream is being captured single launches
- * are enqueued.
+ * 12.5e6 on 4096, PIC_FP64 up to 1e6 on 1024.  Others replay CUDA graphs.  While
+ * the stream is being captured single launches are enqueued.  The particles, the
+ * density, the field, charge, charge_q and the field energy are the same bits
+ * whichever it is; the kinetic, momentum and mode entries of the rows are sums in
+ * another order and agree to rounding.
  * A step n with n % S == 0 (S = sort_interval > 0, n > 0) sorts first.
  * Asynchronous. */
 int pic_step_n(pic_run *run, int64_t n);

@@ -461,11 +461,14 @@ cudaError_t set_steps_shape(pic_run *r) {
     return cudaSuccess;
 }
 
-// Whether the run's stream is being captured into a graph: a replay would not
-// advance the host's copy of the many-step launch's counters.
+// Whether the run's stream is being captured into a graph.  Then single launches are
+// enqueued: a replay would not advance the host's copy of the many-step launch's
+// counters, and the run's own graphs cannot be made (instantiated) meanwhile.
 bool capturing(const pic_run *r) {
     cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-    return cudaStreamIsCapturing(r->stream, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(r->stream, &st) == cudaSuccess) return st != cudaStreamCaptureStatusNone;
+    (void)cudaGetLastError();
+    return true;
 }
 
 int run_steps(pic_run *r, int steps) {
@@ -785,7 +788,7 @@ int pic_step_n(pic_run *run, int64_t n) {
     if (!run || n < 0) return PIC_EINVAL;
     if (!run->ready || run->pending_push) return PIC_ESTATE;
     const int64_t S = run->p.sort_interval;
-    const bool resident = run->steps_grid && !capturing(run);
+    const bool cap = capturing(run), resident = run->steps_grid && !cap;
     while (n > 0) {
         const bool sort_due = S > 0 && run->step > 0 && run->step % S == 0;
         if (resident) {
@@ -796,7 +799,7 @@ int pic_step_n(pic_run *run, int64_t n) {
             const int rc = run_steps(run, (int)k);
             if (rc) return rc;
             n -= k;
-        } else if (sort_due && n >= S) {
+        } else if (!cap && sort_due && n >= S) {
             cudaGraphExec_t &g = run->period[run->cur];
             if (!g) {
                 int rc = capture(run, run->cur, true, (int)S, &g);
@@ -806,7 +809,7 @@ int pic_step_n(pic_run *run, int64_t n) {
             run->cur = 1 - run->cur;
             run->step += S;
             n -= S;
-        } else if (S == 0 && n >= kPlainBlock) {
+        } else if (!cap && S == 0 && n >= kPlainBlock) {
             if (!run->plain) {
                 int rc = capture(run, run->cur, false, kPlainBlock, &run->plain);
                 if (rc) return rc;

@@ -277,3 +277,30 @@ def test_short_history_rings_of_a_pool(H):
         np.testing.assert_allclose(d["field"], e["field"], rtol=1e-12)
         assert np.isnan(d["kinetic"][-1]) and np.all(np.isfinite(d["kinetic"][:-1]))
     pool.close()
+
+
+@pytest.mark.parametrize("n", [1, 20, 45])
+@pytest.mark.parametrize("kw", [{}, dict(sort_interval=3), dict(precision=pic.PIC_FP64), dict(block_size=128),
+                                dict(block_size=128, sort_interval=20)])
+def test_captured_steps_replay_and_the_run_goes_on(n, kw):
+    # many steps in a capture, of runs that replay graphs of their own, too
+    dt = np.float64 if kw.get("precision") == pic.PIC_FP64 else np.float32
+    rng = np.random.default_rng(n)
+    x, v = rng.uniform(0.0, 0.999 * L, 20000).astype(dt), rng.normal(0.0, 0.4, 20000).astype(dt)
+    s = torch.cuda.Stream()
+    a = pic.Run(pic.Params(npart=20000, ncell=64, length=L, **kw), device="cuda:0", stream=s)
+    b = pic.Run(pic.Params(npart=20000, ncell=64, length=L, **{**kw, "block_size": 256}), device="cuda:0")
+    a.init(x, v), b.init(x, v)
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s):
+        a.step_n(n)
+    # a sort swaps the buffers that the graph was captured with
+    replays = 1 if "sort_interval" in kw else 3
+    for _ in range(replays):
+        g.replay()
+    torch.cuda.synchronize()
+    b.step_n(n * replays)
+    a.step_n(7), b.step_n(7)
+    for p, q in zip(a.get_state(), b.get_state()):
+        assert np.array_equal(p, q)
+    a.close(), b.close()
