@@ -212,7 +212,10 @@ int pic_sort(pic_run *run);
  * whose launch shape is left open (pic_params, pic_set_launch) take many steps
  * per cooperative launch: PIC_FP32_FIXED up to 24e6 particles on 2048 cells or
  * 12.5e6 on 4096, PIC_FP64 up to 1e6 on 1024.  Others replay CUDA graphs.  While
- * the stream is being captured single launches are enqueued.  The particles, the
+ * the stream is being captured single launches are enqueued; a replay advances the
+ * device's state, its count of steps and the rows, but not pic_step_count or the
+ * steps that sort_interval and pic_diagnostics go by, and from a capture on the run
+ * takes no many-step launch.  The particles, the
  * density, the field, charge, charge_q and the field energy are the same bits
  * whichever it is; the kinetic, momentum and mode entries of the rows are sums in
  * another order and agree to rounding.

@@ -170,6 +170,7 @@ struct pic_run {
     unsigned wait_limit = 0, wait_missing = 0;   // pic_set_wait_limit
     int64_t step = 0;
     bool ready = false, pending_push = false;
+    bool captured = false;           // steps of this run are in a graph of the caller's
     cudaGraphExec_t period[2] = {nullptr, nullptr};   // S steps from x parity 0/1
     cudaGraphExec_t plain = nullptr;                  // kPlainBlock steps, no sort
     pic::Staging stage;
@@ -760,6 +761,7 @@ int pic_solve_field(pic_run *run) {
     pic::TraceRange trace_("pic_solve_field");
     if (!run) return PIC_EINVAL;
     if (!run->ready) return PIC_ESTATE;
+    if (run->pending_push && run->steps_grid && !run->captured) run->captured = capturing(run);
     PIC_CUDA(enqueue_solve(run, run->stream, run->pending_push));
     if (run->pending_push) run->step++;
     run->pending_push = false;
@@ -788,7 +790,12 @@ int pic_step_n(pic_run *run, int64_t n) {
     if (!run || n < 0) return PIC_EINVAL;
     if (!run->ready || run->pending_push) return PIC_ESTATE;
     const int64_t S = run->p.sort_interval;
-    const bool cap = capturing(run), resident = run->steps_grid && !cap;
+    const bool cap = capturing(run);
+    // Replays advance the device's count of steps and not the host's, which the
+    // many-step launch goes by (read on the device it cost 1-5% of a step): from the
+    // first capture on a run takes the kernels that go by the device's.
+    if (cap) run->captured = true;
+    const bool resident = run->steps_grid && !run->captured;
     while (n > 0) {
         const bool sort_due = S > 0 && run->step > 0 && run->step % S == 0;
         if (resident) {

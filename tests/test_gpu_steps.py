@@ -303,4 +303,40 @@ def test_captured_steps_replay_and_the_run_goes_on(n, kw):
     a.step_n(7), b.step_n(7)
     for p, q in zip(a.get_state(), b.get_state()):
         assert np.array_equal(p, q)
+    # the host counted the captured steps once; the device's rows are those of b
+    rows = a.diagnostics(0, a.step + 1)
+    want = b.diagnostics(0, a.step + 1)
+    assert a.step == n + 7
+    for key in ("step", "charge_q", "charge", "field"):
+        assert np.array_equal(rows[key], want[key]), key
     a.close(), b.close()
+
+
+@pytest.mark.parametrize("steps", [1, 2, 3, 20])
+@pytest.mark.parametrize("H", [4, 64])
+@pytest.mark.parametrize("phases", [False, True])
+def test_steps_after_replays_continue_the_devices_count(steps, H, phases):
+    # a short and a long ring; the device's step counter, read through the rows
+    s = torch.cuda.Stream()
+    a = pic.Run(pic.Params(npart=5001, ncell=64, length=L, history=H), device="cuda:0", stream=s)
+    a.init(*state(5001, 9))
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s):
+        if phases:
+            a.push(), a.solve_field()
+        else:
+            a.step_n(1)
+    a.set_state(*state(5001, 9), 0)           # the graph is still there
+    a.step_n(1)
+    with torch.cuda.stream(s):                # a replay goes to the current stream
+        for _ in range(H + 1):
+            g.replay()
+    a.step_n(steps)
+    torch.cuda.synchronize()
+    first = max(0, a.step - H + 1)
+    held = a.diagnostics(first, a.step - first + 1)["step"]
+    last = 1 + H + 1 + steps
+    # the ring holds the device's last H rows
+    slots = {r % H: r for r in range(max(0, last - H + 1), last + 1)}
+    assert held.tolist() == [slots[r % H] for r in range(first, a.step + 1)]
+    a.close()
