@@ -429,10 +429,11 @@ int steps64_block(int64_t npart, int ncell) {
 //   3e5 on 1000    6.89 (5.44) 6.23    -     -    5.34 | 7.38 (5.94) 6.32   -     -    5.91
 //   6e5 on 512     7.47 (5.45) 5.28    -    5.41  5.27 | 8.06 (6.06) 6.07   -    6.10  6.08
 //   1e6 on 1024    12.1 (8.48) 7.24    -     -    7.22
-// As many blocks as one group per thread takes, up to the SMs.
+// As many blocks as one group per thread takes, up to the SMs.  (So a lane's float32
+// sums are of 4 particles at most, as those of a push of so few particles are.)
 void steps_shape(int64_t n, int ng, bool *small, int *block) {
     *small = n <= 600000 && ng <= 1024;           // (one node per thread)
-    *block = !*small || ng > 512 || n > 400000 ? 1024 : ng > 256 || n > 40000 ? 512 : 256;
+    *block = !*small || ng > 512 || n > 300000 ? 1024 : ng > 256 || n > 40000 ? 512 : 256;
 }
 
 cudaError_t set_steps_shape(pic_run *r) {

@@ -134,23 +134,32 @@ __device__ __forceinline__ void warp_sum_pairs(float4 &p, int n) {
 template <int W> struct Group { using T = float4; };
 template <> struct Group<1> { using T = float; };
 
-// Push and deposit the first m of a group's W particles.
+// Push and deposit a group's W particles.  The v_old v_new and v_new of a group of 4
+// are summed before they join the thread's sums, whose chain of
+// float32 adds, the longest part of the rows' error, is so a quarter as long
+// (kinetic energy against float64 sums, rms: 2.3e7 Maxwellian particles 1.1e-9
+// without and 2.8e-10 so, 5.6e-10 in the push kernel's chains, of two thirds the
+// length, without).
 template <bool NGP, int W>
-__device__ __forceinline__ void step_group(typename Group<W>::T &x, typename Group<W>::T &v, int m,
+__device__ __forceinline__ void step_group(typename Group<W>::T &x, typename Group<W>::T &v,
                                            const float *sE, const Tile &t, const PushConsts &c,
                                            unsigned *err, float &ke, float &mom) {
     using T = typename Group<W>::T;
     alignas(16) float xs[W], vs[W];
     *reinterpret_cast<T *>(xs) = x;
     *reinterpret_cast<T *>(vs) = v;
+    float gke = 0.0f, gmom = 0.0f;
 #pragma unroll
     for (int k = 0; k < W; k++) {
-        if (k >= m) continue;
-        if (NGP) push_particle_ngp(xs[k], vs[k], sE, c, ke, mom);
-        else push_particle(xs[k], vs[k], sE, c, ke, mom);
+        if (NGP) push_particle_ngp(xs[k], vs[k], sE, c, W > 1 ? gke : ke, W > 1 ? gmom : mom);
+        else push_particle(xs[k], vs[k], sE, c, W > 1 ? gke : ke, W > 1 ? gmom : mom);
     }
-    if (NGP) deposit_ngp<W>(t, xs, m, c, err);
-    else deposit_cells<W>(t, xs, m, c, err);
+    if (W > 1) {
+        ke += gke;
+        mom += gmom;
+    }
+    if (NGP) deposit_ngp<W>(t, xs, W, c, err);
+    else deposit_cells<W>(t, xs, W, c, err);
     x = *reinterpret_cast<const T *>(xs);
     v = *reinterpret_cast<const T *>(vs);
 }
@@ -273,20 +282,14 @@ __device__ __forceinline__ void diag_step(const StepsArgs &a, int s, int workers
     });
 }
 
-// With 4 nodes a thread both are called out of line, so that their registers (a
-// node's 128-bit sums, 4 times) are not taken from the push loop: 1.2e7
-// particles on 4096 cells 44.6 us a step, 50.2 inlined.  With 1 or 2 they fit
-// beside it (512 cells 34.4 inlined, 36.0 called).
+// With 4 nodes a thread it is called out of line, so that its registers (a node's
+// 128-bit sums, 4 times) are not taken from the push loop: 1.2e7 particles on 4096
+// cells 44.6 us a step, 50.2 inlined.  With 1 or 2 they fit beside it (512 cells 34.4
+// inlined, 36.0 called).  The diagnostics have a loop of their own for the same
+// reason.
 template <int K>
 __device__ __noinline__ void field_step_call(const StepsArgs &a, const unsigned long long *acc, float *sE) {
     field_step<K>(a, acc, sE);
-}
-
-template <int K>
-__device__ __noinline__ void diag_step_call(const StepsArgs &a, int s, int workers,
-                                            const unsigned long long *acc, const float4 *kv,
-                                            unsigned char *smem_raw, unsigned h0) {
-    diag_step<K>(a, s, workers, acc, kv, smem_raw, h0);
 }
 
 // Block b of a run's workers + nd: all its steps.
@@ -320,14 +323,28 @@ __device__ __forceinline__ void run_many_steps(const StepsArgs &a, unsigned char
     };
     clear_tile();
     for (int j = tid; j < ng + 2; j += bs) sE[j] = a.E32[j == 0 ? ng - 1 : (j == ng + 1 ? 0 : j - 1)];
+    if (diag) {
+        __syncthreads();
+        const unsigned h0 = (unsigned)(a.step0 % a.hist_len);             // history slot of the first step
+        for (int s = b - workers; s < a.steps; s += nd) {
+            const int slot = s % kStepsSlots;
+            unsigned long long *acc = a.acc + (size_t)slot * ng;
+            const float4 *kv = reinterpret_cast<const float4 *>(a.partials) + (size_t)slot * kStepsMaxGrid;
+            if (!wait_step(a, s, workers, false, &dead)) return;
+            diag_step<K>(a, s, workers, acc, kv, smem_raw, h0);
+            // give the slot back, once no worker reads it any more
+            if (!wait_step(a, s + 1, workers, false, &dead)) return;
+            for (int g = tid; g < ng; g += bs) acc[g] = 0ull;
+            __syncthreads();
+            if (tid == 0) red_release(a.sync + 1 + (b - workers));
+        }
+        return;
+    }
     // this block's groups [q0, q1); the thread's groups q0 + tid + i bs, the first
-    // kResident of them in registers.  The run's last group may hold fewer than kW
-    // particles; its other words are padding of the arrays.
-    const int nq = (int)((a.n + kW - 1) / kW), left = (int)(a.n - (long long)kW * (nq - 1));  // nq <= 2^30
-    const int q0 = diag ? 0 : (int)((long long)nq * b / workers);
-    const int q1 = diag ? 0 : (int)((long long)nq * (b + 1) / workers);
-    const unsigned h0 = diag ? (unsigned)(a.step0 % a.hist_len) : 0u;     // history slot of the first step
-    auto members = [&](int q) { return q >= q1 ? 0 : q == nq - 1 ? left : kW; };
+    // kResident of them in registers.  The last N mod kW particles are block 0's.
+    const int nq = (int)(a.n / kW), left = (int)(a.n % kW);                     // nq <= 2^30
+    const int q0 = (int)((long long)nq * b / workers);
+    const int q1 = (int)((long long)nq * (b + 1) / workers);
     G *xg = reinterpret_cast<G *>(a.x);
     G *vg = reinterpret_cast<G *>(a.v);
     G rx[kResident], rv[kResident];
@@ -338,100 +355,92 @@ __device__ __forceinline__ void run_many_steps(const StepsArgs &a, unsigned char
         rv[i] = q < q1 ? __ldcg(vg + q) : G{};
     }
     __syncthreads();
-    for (int s = diag ? b - workers : 0; s < a.steps; s += diag ? nd : 1) {
+    for (int s = 0; s < a.steps; s++) {
         const bool last = s == a.steps - 1;
         const int slot = s % kStepsSlots;
         unsigned long long *acc = a.acc + (size_t)slot * ng;
         float4 *kv = reinterpret_cast<float4 *>(a.partials) + (size_t)slot * kStepsMaxGrid;
-        if (!diag) {
-            float ke = 0.0f, mom = 0.0f;
-            const int qs = q0 + tid + kResident * bs;
-            G cx = qs < q1 ? __ldcg(xg + qs) : G{}, cv = qs < q1 ? __ldcg(vg + qs) : G{};
-#pragma unroll
-            for (int i = 0; i < kResident; i++) {
-                const int m = members(q0 + tid + i * bs);
-                if (m) step_group<kNgp, kW>(rx[i], rv[i], m, sE, tile, c, a.err, ke, mom);
-            }
-            for (int q = qs; q < q1; q += bs) {
-                G xx = cx, vv = cv;
-                const int qn = q + bs;
-                cx = qn < q1 ? __ldcg(xg + qn) : G{};
-                cv = qn < q1 ? __ldcg(vg + qn) : G{};
-                step_group<kNgp, kW>(xx, vv, members(q), sE, tile, c, a.err, ke, mom);
-                __stcg(xg + q, xx);
-                __stcg(vg + q, vv);
-            }
-            float4 sums = make_float4(ke, 0.0f, mom, 0.0f);
-            warp_sum_pairs(sums, 32);
-            if (lane == 0) kvs[w] = sums;
-            __syncthreads();
-            if (w == nw - 1) {                        // the block's sums, still as pairs
-                float4 p = lane < nw ? kvs[lane] : make_float4(0.f, 0.f, 0.f, 0.f);
-                warp_sum_pairs(p, nw);
-                if (lane == 0) kv[b] = p;
-            }
-            // node g: the left weights of cell g + 1 and the right ones of cell g
-            // (held by the lane below: a warp's first lane only reads them), node
-            // NG - 1 also cell 0's left ones, node 0 cell NG's right ones (NGP: the
-            // counts of word g + 1; word NG + 1 is node 0, word 0 stays empty)
-            auto cell = [&](int j) {
-                u64 n = 0ull, W = 0ull;
-#pragma unroll 4
-                for (int i = 0; i < K_; i++) {
-                    const int at = (j << a.log_copies) + ((i + lane) & (K_ - 1));
-                    if (kNgp) {
-                        n += tile0.n[at];
-                    } else {
-                        const CellSum cs = cell_sum(tile0.w[at], tile0.n[at], 0u, false);
-                        n += cs.n;
-                        W += cs.W;
-                    }
-                }
-                return ulonglong2{n, W};
-            };
-            constexpr int kPer = kNgp ? 32 : 31;                // nodes a warp
-            for (int g0 = kPer * w; g0 < ng; g0 += kPer * nw) {
-                const int g = kNgp ? g0 + lane : g0 + lane - 1;
-                const ulonglong2 own = g < ng ? cell(g + 1) : ulonglong2{0ull, 0ull};
-                u64 val = (own.x << kFixBits) - own.y;
-                if (!kNgp) val += __shfl_up_sync(kFull, own.y, 1);
-                if (g == (kNgp ? 0 : ng - 1)) {
-                    const ulonglong2 e = cell(kNgp ? ng + 1 : 0);
-                    val += (e.x << kFixBits) - e.y;
-                }
-                if (!kNgp && g == 0) val += cell(ng).y;
-                if ((kNgp || lane > 0) && g < ng && val) atomicAdd(&acc[g], val);
-            }
-            __syncthreads();
-            if (tid == 0) red_release(a.sync);        // the whole block's adds: after the barrier
-            if (!last) clear_tile();                  // while the others arrive
-        }
-        if (!wait_step(a, s, workers, !diag, &dead)) return;
-        if (!diag) {
-            if (last) break;
-            if (K >= 4) field_step_call<K>(a, acc, sE);
-            else field_step<K>(a, acc, sE);
-            continue;
-        }
-        if (K >= 4) diag_step_call<K>(a, s, workers, acc, kv, smem_raw, h0);
-        else diag_step<K>(a, s, workers, acc, kv, smem_raw, h0);
-        // give the slot back, once no worker reads it any more
-        if (!wait_step(a, s + 1, workers, false, &dead)) return;
-        for (int g = tid; g < ng; g += bs) acc[g] = 0ull;
-        __syncthreads();
-        if (tid == 0) red_release(a.sync + 1 + (b - workers));
-    }
-    if (!diag) {
+        float ke = 0.0f, mom = 0.0f;
+        const int qs = q0 + tid + kResident * bs;
+        G cx = qs < q1 ? __ldcg(xg + qs) : G{}, cv = qs < q1 ? __ldcg(vg + qs) : G{};
 #pragma unroll
         for (int i = 0; i < kResident; i++) {
-            const int q = q0 + tid + i * bs;
-            if (q >= q1) break;
-            __stcg(xg + q, rx[i]);
-            __stcg(vg + q, rv[i]);
+            if (q0 + tid + i * bs < q1) step_group<kNgp, kW>(rx[i], rv[i], sE, tile, c, a.err, ke, mom);
         }
-        const int slot = (a.steps - 1) % kStepsSlots;
-        last_step<K>(a, a.acc + (size_t)slot * ng, b, workers);
+        for (int q = qs; q < q1; q += bs) {
+            G xx = cx, vv = cv;
+            const int qn = q + bs;
+            cx = qn < q1 ? __ldcg(xg + qn) : G{};
+            cv = qn < q1 ? __ldcg(vg + qn) : G{};
+            step_group<kNgp, kW>(xx, vv, sE, tile, c, a.err, ke, mom);
+            __stcg(xg + q, xx);
+            __stcg(vg + q, vv);
+        }
+        if (kW > 1 && b == 0 && tid < left) {
+            float *px = a.x + (long long)kW * nq + tid, *pv = a.v + (long long)kW * nq + tid;
+            float x1 = __ldcg(px), v1 = __ldcg(pv);
+            step_group<kNgp, 1>(x1, v1, sE, tile, c, a.err, ke, mom);
+            __stcg(px, x1);
+            __stcg(pv, v1);
+        }
+        float4 sums = make_float4(ke, 0.0f, mom, 0.0f);
+        warp_sum_pairs(sums, 32);
+        if (lane == 0) kvs[w] = sums;
+        __syncthreads();
+        if (w == nw - 1) {                        // the block's sums, still as pairs
+            float4 p = lane < nw ? kvs[lane] : make_float4(0.f, 0.f, 0.f, 0.f);
+            warp_sum_pairs(p, nw);
+            if (lane == 0) kv[b] = p;
+        }
+        // node g: the left weights of cell g + 1 and the right ones of cell g
+        // (held by the lane below: a warp's first lane only reads them), node
+        // NG - 1 also cell 0's left ones, node 0 cell NG's right ones (NGP: the
+        // counts of word g + 1; word NG + 1 is node 0, word 0 stays empty)
+        auto cell = [&](int j) {
+            u64 n = 0ull, W = 0ull;
+#pragma unroll 4
+            for (int i = 0; i < K_; i++) {
+                const int at = (j << a.log_copies) + ((i + lane) & (K_ - 1));
+                if (kNgp) {
+                    n += tile0.n[at];
+                } else {
+                    const CellSum cs = cell_sum(tile0.w[at], tile0.n[at], 0u, false);
+                    n += cs.n;
+                    W += cs.W;
+                }
+            }
+            return ulonglong2{n, W};
+        };
+        constexpr int kPer = kNgp ? 32 : 31;                // nodes a warp
+        for (int g0 = kPer * w; g0 < ng; g0 += kPer * nw) {
+            const int g = kNgp ? g0 + lane : g0 + lane - 1;
+            const ulonglong2 own = g < ng ? cell(g + 1) : ulonglong2{0ull, 0ull};
+            u64 val = (own.x << kFixBits) - own.y;
+            if (!kNgp) val += __shfl_up_sync(kFull, own.y, 1);
+            if (g == (kNgp ? 0 : ng - 1)) {
+                const ulonglong2 e = cell(kNgp ? ng + 1 : 0);
+                val += (e.x << kFixBits) - e.y;
+            }
+            if (!kNgp && g == 0) val += cell(ng).y;
+            if ((kNgp || lane > 0) && g < ng && val) atomicAdd(&acc[g], val);
+        }
+        __syncthreads();
+        if (tid == 0) red_release(a.sync);        // the whole block's adds: after the barrier
+        if (!last) clear_tile();                  // while the others arrive
+        if (!wait_step(a, s, workers, true, &dead)) return;
+        if (last) break;
+        if (K >= 4) field_step_call<K>(a, acc, sE);
+        else field_step<K>(a, acc, sE);
     }
+#pragma unroll
+    for (int i = 0; i < kResident; i++) {
+        const int q = q0 + tid + i * bs;
+        if (q >= q1) break;
+        __stcg(xg + q, rx[i]);
+        __stcg(vg + q, rv[i]);
+    }
+    const int slot = (a.steps - 1) % kStepsSlots;
+    last_step<K>(a, a.acc + (size_t)slot * ng, b, workers);
 }
 
 template <int VARIANT, int K, bool SMALL>

@@ -340,3 +340,40 @@ def test_steps_after_replays_continue_the_devices_count(steps, H, phases):
     slots = {r % H: r for r in range(max(0, last - H + 1), last + 1)}
     assert held.tolist() == [slots[r % H] for r in range(first, a.step + 1)]
     a.close()
+
+
+@pytest.mark.parametrize("n,ng", [(300000, 512), (300001, 512), (600002, 1024), (600003, 1025), (600005, 100), (2, 1026),
+                                  (3, 2049), (6, 4096)])
+@pytest.mark.parametrize("shape", [pic.PIC_SHAPE_CIC, pic.PIC_SHAPE_NGP])
+def test_the_last_particles_of_a_run_and_another_block_size(n, ng, shape):
+    # 1 to 3 particles beyond the last group of 4, no group at all, and the lines of
+    # steps_shape
+    a, b = pair(n, ng, shape=shape, sort_interval=5)
+    for k in (1, 3, 8):
+        a.step_n(k), b.step_n(k)
+        assert_same(a, b, n, ng)
+    a.close(), b.close()
+
+
+# Rows against float64 sums of the same particles.  Products and group sums are
+# rounded to 2^-24 of themselves, a thread's sum once a group, at random: an error of
+# the total of 2^-24 / 2 sqrt(adds in a chain / threads) rms, taken 8 times; chains
+# and threads of the push kernels' sums, which the launch's may not exceed.
+@pytest.mark.parametrize("n,ng", [(20000, 64), (300007, 300), (1024003, 1024), (4200001, 2048), (12345679, 4096),
+                                  (23000003, 2000)])
+@pytest.mark.parametrize("shape", [pic.PIC_SHAPE_CIC, pic.PIC_SHAPE_NGP])
+def test_kinetic_energy_and_momentum_against_float64_sums(n, ng, shape):
+    run = pic.Run(pic.Params(npart=n, ncell=ng, length=L, shape=shape), device="cuda:0")
+    run.init(*state(n, 11))
+    m = L / n
+    threads = min(n / 4.0, 1536.0 * 152)
+    tol = 8 * 2.0 ** -25 * math.sqrt(max(4.0, n / threads) / threads)
+    old = run.get_cells()[1].astype(np.float64)
+    for _ in range(4):
+        run.step_n(1)
+        new = run.get_cells()[1].astype(np.float64)
+        row = run.diagnostics(run.step - 1, 1)[0]
+        assert abs(row["kinetic"] - 0.5 * m * (old * new).sum()) <= tol * 0.5 * m * np.abs(old * new).sum()
+        assert abs(row["momentum"] - m * new.sum()) <= tol * m * np.abs(new).sum()
+        old = new
+    run.close()
