@@ -377,3 +377,23 @@ def test_kinetic_energy_and_momentum_against_float64_sums(n, ng, shape):
         assert abs(row["momentum"] - m * new.sum()) <= tol * m * np.abs(new).sum()
         old = new
     run.close()
+
+
+# Mode amplitudes against float64 sums: P = NG/256 parts are summed in float32, 13 adds
+# deep, each rounding at random to 2^-25 of the part (rms 2^-25 / sqrt 3), at most
+# 1/P of sum |E|; the parts' errors add in squares.
+@pytest.mark.parametrize("n,ng", [(1000003, 2048), (4000001, 4096)])
+def test_mode_amplitudes_against_float64_sums(n, ng):
+    run = pic.Run(pic.Params(npart=n, ncell=ng, length=L), device="cuda:0")
+    run.init(*state(n, 12))
+    theta = 2.0 * math.pi * np.arange(ng) / ng
+    parts, err = ng / 256.0, []
+    for _ in range(12):
+        run.step_n(1)
+        E = run.get_field()["E"]
+        row = run.diagnostics(run.step, 1)[0]
+        for m in range(8):
+            want = 2.0 / ng * abs(np.sum(E * np.exp(-1j * (m + 1) * theta)))
+            err.append((row["mode"][m] - want) / (2.0 / ng * np.abs(E).sum()))
+    assert np.sqrt(np.mean(np.square(err))) <= math.sqrt(13.0 / parts) * 2.0 ** -25 / math.sqrt(3.0)
+    run.close()
