@@ -133,6 +133,34 @@ __device__ __forceinline__ void push_particle_ngp(float &u, float &v, const floa
     kick_drift_wrap(u, v, ep, c, ke, mom);
 }
 
+// s + e = a + b exactly (Knuth's two-sum); pairs (h, l) added over a warp
+__device__ __forceinline__ void add_pair(float &h, float &l, float h2, float l2) {
+    const float s = __fadd_rn(h, h2);
+    const float t = __fsub_rn(s, h);
+    const float e = __fadd_rn(__fsub_rn(h, __fsub_rn(s, t)), __fsub_rn(h2, t));
+    l = __fadd_rn(__fadd_rn(l, l2), e);
+    h = s;
+}
+
+// The same for one value and three adds less, exact where |h| >= |v| (Dekker's fast
+// two-sum); otherwise off by a rounding of v at most.
+__device__ __forceinline__ void add_fast(float &h, float &l, float v) {
+    const float s = __fadd_rn(h, v);
+    l = __fadd_rn(l, __fsub_rn(v, __fsub_rn(s, h)));
+    h = s;
+}
+
+// (x, y) and (z, w) summed over the first n lanes of a warp (the others hold
+// zeros), in lane 0.
+__device__ __forceinline__ void warp_sum_pairs(float4 &p, int n) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        if (o >= n) continue;                         // uniform
+        add_pair(p.x, p.y, __shfl_down_sync(kFull, p.x, o), __shfl_down_sync(kFull, p.y, o));
+        add_pair(p.z, p.w, __shfl_down_sync(kFull, p.z, o), __shfl_down_sync(kFull, p.w, o));
+    }
+}
+
 // Shared-memory density tiles.  GB300 has no single-instruction 64-bit integer
 // add on shared memory (it is a compare-and-swap loop), so sums are kept in 32
 // bits by fetch-adds, and the one add that wraps a word counts a carry.

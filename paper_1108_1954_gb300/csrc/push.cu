@@ -276,10 +276,19 @@ int atomic_copies(int ng, int block) {
     return k;
 }
 
-template <bool PUSH>
+// A thread takes 4 particles at a time where one block of 256 had one, so plain
+// float32 sums of v_old v_new and v_new have longer chains, and more of their rounding
+// in the rows.  The sums are therefore pairs of float32, to which few particles are
+// added one by one (EXACT), many in groups of 4.  Kinetic energy against exact sums, rms: 2e4
+// particles 1.3e-10 (4.9e-10 with plain chains, 2.2e-10 with one particle a thread),
+// 1e6 2.8e-11 (1.0e-10, 8.2e-11), 2^24 1.9e-11 (3.8e-10, 1.5e-10).  us a step, one by one
+// and in groups: 1e6 on 1024 cells 17.9, 17.4; 4e6 29.4, 27.9; 2^24 67.4, 63.2.
+constexpr long long kAtomicExact = 1 << 21;
+
+template <bool PUSH, bool EXACT>
 __global__ void __launch_bounds__(1024) pic_push_f32atomic_kernel(PushArgsF32Atomic a) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    __shared__ double red[64];
+    __shared__ float4 red[32];                            // per warp: (ke, ke low, mom, mom low)
     const PushConsts c = a.c;
     const int ng = c.ng;
     float *sE = reinterpret_cast<float *>(smem_raw);      // ng + 2, ghost-padded
@@ -296,7 +305,22 @@ __global__ void __launch_bounds__(1024) pic_push_f32atomic_kernel(PushArgsF32Ato
         atomicAdd(&mine[key * K], l);
         atomicAdd(&mine[(key + 1) * K], r);
     };
-    float ke = 0.0f, mom = 0.0f;
+    float4 sums = make_float4(0.f, 0.f, 0.f, 0.f);        // (ke, ke low, mom, mom low)
+    float gke = 0.0f, gmom = 0.0f;                        // of a group
+    auto join = [&] {
+        if (EXACT) {
+            add_pair(sums.x, sums.y, gke, 0.0f);
+            add_pair(sums.z, sums.w, gmom, 0.0f);
+        } else {
+            add_fast(sums.x, sums.y, gke);
+            add_fast(sums.z, sums.w, gmom);
+        }
+        gke = gmom = 0.0f;
+    };
+    auto push = [&](float &x, float &v) {
+        push_particle(x, v, sE, c, gke, gmom);
+        if (EXACT) join();
+    };
     const long long n4 = a.n >> 2;
     const long long stride = (long long)gridDim.x * bs;
     float4 *x4 = reinterpret_cast<float4 *>(a.x);
@@ -315,7 +339,7 @@ __global__ void __launch_bounds__(1024) pic_push_f32atomic_kernel(PushArgsF32Ato
         bool bad = false;
 #pragma unroll
         for (int k = 0; k < 4; k++) {
-            if (PUSH) push_particle(xs[k], vs[k], sE, c, ke, mom);
+            if (PUSH) push(xs[k], vs[k]);
             const Loc l = locate(xs[k]);
             const bool ok = l.j <= (unsigned)ng;
             bad |= !ok;
@@ -334,6 +358,7 @@ __global__ void __launch_bounds__(1024) pic_push_f32atomic_kernel(PushArgsF32Ato
             }
         }
         if (PUSH) {
+            if (!EXACT) join();
             __stcs(x4 + q, make_float4(xs[0], xs[1], xs[2], xs[3]));
             __stcs(v4 + q, make_float4(vs[0], vs[1], vs[2], vs[3]));
         }
@@ -347,16 +372,21 @@ __global__ void __launch_bounds__(1024) pic_push_f32atomic_kernel(PushArgsF32Ato
     if (blockIdx.x == 0 && tid < (int)(a.n & 3)) {
         const long long i = n4 * 4 + tid;
         float x = a.x[i], v = PUSH ? a.v[i] : 0.0f;
-        if (PUSH) push_particle(x, v, sE, c, ke, mom);
+        if (PUSH) push(x, v);
         const Loc l = locate(x);
         if (l.j <= (unsigned)ng) add(l.j, 1.0f - l.f, l.f);
         else atomicOr(a.err, kErrPosition);
         if (PUSH) { a.x[i] = x; a.v[i] = v; }
     }
     if (PUSH) {
-        double dke = ke, dmom = mom;
+        join();                                           // (block 0's last particles)
+        // the block's sums as pairs: the float64 pipe would take 2.5 us
+        warp_sum_pairs(sums, 32);
+        if ((tid & 31) == 0) red[tid >> 5] = sums;
         __syncthreads();
-        block_sum2(dke, dmom, red);
+        float4 p = tid < 32 && tid < ((bs + 31) >> 5) ? red[tid & 31] : make_float4(0.f, 0.f, 0.f, 0.f);
+        if (tid < 32) warp_sum_pairs(p, 32);
+        const double dke = (double)p.x + (double)p.y, dmom = (double)p.z + (double)p.w;
         if (tid == 0) {
             a.partials[2 * blockIdx.x] = dke;
             a.partials[2 * blockIdx.x + 1] = dmom;
@@ -508,6 +538,13 @@ __global__ void __launch_bounds__(1024) pic_push_f64_kernel(PushArgs64 a) {
     }
 }
 
+using AtomicKernel = void (*)(PushArgsF32Atomic);
+
+AtomicKernel atomic_kernel(bool push, long long n) {
+    if (!push) return &pic_push_f32atomic_kernel<false, false>;
+    return n <= kAtomicExact ? &pic_push_f32atomic_kernel<true, true> : &pic_push_f32atomic_kernel<true, false>;
+}
+
 using FixedKernel = void (*)(PushArgs);
 
 template <int V>
@@ -575,11 +612,10 @@ cudaError_t push_prepare_attributes(int mode) {
                     if (e != cudaSuccess) return e;
                 }
     } else if (mode == PIC_FP32_ATOMIC) {
-        e = cudaFuncSetAttribute(&pic_push_f32atomic_kernel<true>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(&pic_push_f32atomic_kernel<false>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+        for (AtomicKernel k : {atomic_kernel(true, 1), atomic_kernel(true, kAtomicExact + 1), atomic_kernel(false, 1)}) {
+            e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+            if (e != cudaSuccess) return e;
+        }
     } else {
         e = cudaFuncSetAttribute(&pic_push_f64_kernel<true>,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
@@ -600,7 +636,7 @@ int push_max_blocks_per_sm(int mode, int variant, int unroll, int block, int ng,
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, block, smem);
     }
     else if (mode == PIC_FP32_ATOMIC)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, &pic_push_f32atomic_kernel<true>, block, smem);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, &pic_push_f32atomic_kernel<true, false>, block, smem);
     else
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, &pic_push_f64_kernel<true>, block, smem);
     if (e != cudaSuccess) {
@@ -621,8 +657,7 @@ cudaError_t launch_push_f32_atomic(PushArgsF32Atomic a, int grid, int block, boo
                                    cudaStream_t s) {
     const size_t smem = push_smem_bytes(PIC_FP32_ATOMIC, a.c.ng, false, block);
     a.copies = atomic_copies(a.c.ng, block);
-    return launch_after(push ? &pic_push_f32atomic_kernel<true> : &pic_push_f32atomic_kernel<false>, dim3(grid),
-                        block, smem, s, 0, a);
+    return launch_after(atomic_kernel(push, a.n), dim3(grid), block, smem, s, 0, a);
 }
 
 cudaError_t launch_push_f64(const PushArgs64 &a, int grid, int block, bool push,

@@ -110,26 +110,6 @@ __device__ __forceinline__ float scaled_f32(i128 m, double k, unsigned long long
     return __uint_as_float(bits | (neg ? 0x80000000u : 0u));
 }
 
-// s + e = a + b exactly (Knuth's two-sum); pairs (h, l) added over a warp
-__device__ __forceinline__ void add_pair(float &h, float &l, float h2, float l2) {
-    const float s = __fadd_rn(h, h2);
-    const float t = __fsub_rn(s, h);
-    const float e = __fadd_rn(__fsub_rn(h, __fsub_rn(s, t)), __fsub_rn(h2, t));
-    l = __fadd_rn(__fadd_rn(l, l2), e);
-    h = s;
-}
-
-// (x, y) and (z, w) summed over the first n lanes of a warp (the others hold
-// zeros), in lane 0.
-__device__ __forceinline__ void warp_sum_pairs(float4 &p, int n) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        if (o >= n) continue;                         // uniform
-        add_pair(p.x, p.y, __shfl_down_sync(kFull, p.x, o), __shfl_down_sync(kFull, p.y, o));
-        add_pair(p.z, p.w, __shfl_down_sync(kFull, p.z, o), __shfl_down_sync(kFull, p.w, o));
-    }
-}
-
 // The W particles of a lane's group, as one word.
 template <int W> struct Group { using T = float4; };
 template <> struct Group<1> { using T = float; };
