@@ -429,8 +429,11 @@ int pic_tune_sort_interval(pic_run *run, const int32_t *intervals, int32_t count
  * first, and keeps a run on chip through all of its steps of that launch.
  * Few active runs, none of them due to sort, take the many-step launch of
  * pic_step_n side by side instead, where that is faster and free arena space
- * holds its accumulators (48 NG bytes and 25 KB a run); the particles, the
- * density and the field are the same bits either way.
+ * holds its accumulators (48 NG bytes and 25 KB a run), in a pool whose launch
+ * shape is left open, or where pic_pool_many_step allows it.  The particles, the
+ * density, the field and charge_q are the same bits either way; the other entries
+ * of the rows are sums in another order and agree to rounding, so their last bits
+ * depend on which runs are active together.
  * A run with sort_interval S > 0 sorts its particles by cell before every
  * step n > 0 with n % S == 0, as the single run does (a stable counting sort
  * inside the cluster, into a second pair of particle buffers: 8 N more
@@ -468,8 +471,14 @@ int pic_pool_create(const pic_pool_config *cfg, void *arena, size_t arena_bytes,
                     void *stream, pic_pool **out);
 void pic_pool_destroy(pic_pool *pool);
 
-/* Change the launch shape (variant, cluster, block) of later advances. */
+/* Change the launch shape (variant, cluster, block) of later advances.  The shape
+ * is then chosen: few runs take it too. */
 int pic_pool_configure(pic_pool *pool, int32_t variant, int32_t cluster, int32_t block);
+
+/* Whether few active runs may take the many-step launch.  At first on where
+ * pic_pool_config leaves variant, cluster and block open (0), otherwise off;
+ * pic_pool_configure turns it off. */
+int pic_pool_many_step(pic_pool *pool, int32_t on);
 
 /* Admit a run: copy its initial state x0, v0 (host, N float32 each, positions
  * in [0, L)) into the arena and queue its set-up (deposit + solve of E^0,

@@ -115,6 +115,7 @@ _SIG = {
     "pic_pool_create": (C.c_int, [_VP, _VP, C.c_size_t, _VP, C.POINTER(_VP)]),
     "pic_pool_destroy": (None, [_VP]),
     "pic_pool_set_wait_limit": (C.c_int, [_VP, C.c_int32, C.c_int32]),
+    "pic_pool_many_step": (C.c_int, [_VP, C.c_int32]),
     "pic_pool_configure": (C.c_int, [_VP, C.c_int32, C.c_int32, C.c_int32]),
     "pic_pool_admit": (C.c_int, [_VP, _P, _VP, _VP, C.c_int64, C.POINTER(C.c_int32)]),
     "pic_pool_advance": (C.c_int, [_VP, C.c_int64, C.POINTER(C.c_int32)]),
@@ -520,6 +521,11 @@ class Pool:
     def configure(self, variant: int, cluster: int, block: int):
         _check(_lib.pic_pool_configure(self._h, int(variant), int(cluster), int(block)),
                "pic_pool_configure")
+
+    def many_step(self, on: bool):
+        """Whether few active runs may take the many-step launch instead of the
+        pool's shape (at first where the shape is left open)."""
+        _check(_lib.pic_pool_many_step(self._h, int(bool(on))), "pic_pool_many_step")
 
     def set_wait_limit(self, polls: int = 0, missing: int = 0):
         """Run.set_wait_limit for the pool's many-step launches."""

@@ -152,6 +152,7 @@ struct pic_pool {
     int wide_clusters = 0;        // > 0: up to so many runs take blocks twice as large
     int sms = 0;
     int resident_sms = 0;         // SMs of the many-step launch (0: not available)
+    bool many_step = true;        // few runs may take it (pic_pool_many_step)
     unsigned wait_limit = 0, wait_missing = 0;   // pic_pool_set_wait_limit
     pic::Staging stage;
 
@@ -316,7 +317,7 @@ double cluster_time(const pic_pool *pool, const std::vector<int> &order) {
 //   equal runs: 20 of 2e6 210, 133; 40 of 1e6 179, 190; 10 of 4e6 287, 120; 65 of
 //     2e5 55, 78; 60 of 5e4 24, 24; 76 of 1e4 25, 9; 8 of 1.2e7 825, 276
 bool resident(const pic_pool *pool, const std::vector<int> &order, std::vector<int> *workers) {
-    if (!pool->resident_sms) return false;
+    if (!pool->resident_sms || !pool->many_step) return false;
     for (int s : order) {
         const pic_pool::Slot &sl = pool->slots[s];
         const int64_t S = sl.p.sort_interval;
@@ -508,6 +509,7 @@ int pic_pool_create(const pic_pool_config *cfg, void *arena, size_t arena_bytes,
     rc = set_shape(pool, cfg->variant ? cfg->variant : kPoolVariant,
                    cfg->cluster ? cfg->cluster : 8, cfg->block ? cfg->block : kPoolBlock);
     if (rc) { delete pool; return rc; }
+    pool->many_step = !cfg->variant && !cfg->cluster && !cfg->block;
     if (!cfg->block)
         pool->wide_clusters = batch_max_clusters(pool->variant, pool->cluster, 2 * kPoolBlock,
                                                  pool->cfg.ncell_max);
@@ -521,7 +523,15 @@ void pic_pool_destroy(pic_pool *pool) { delete pool; }
 
 int pic_pool_configure(pic_pool *pool, int32_t variant, int32_t cluster, int32_t block) {
     if (!pool) return PIC_EINVAL;
-    return set_shape(pool, variant, cluster, block);
+    const int rc = set_shape(pool, variant, cluster, block);
+    if (!rc) pool->many_step = false;
+    return rc;
+}
+
+int pic_pool_many_step(pic_pool *pool, int32_t on) {
+    if (!pool) return PIC_EINVAL;
+    pool->many_step = on != 0;
+    return PIC_OK;
 }
 
 }  // extern "C"

@@ -112,9 +112,13 @@ class Server:
             raise ValueError("advance_steps must be at least 1")
 
         def make_pool():
-            return Pool(max_slots=max_slots, ncell_max=ncell_max, arena_bytes=arena_bytes,
+            # the shape is that of the cluster launches; few resident runs
+            # take the many-step launch
+            pool = Pool(max_slots=max_slots, ncell_max=ncell_max, arena_bytes=arena_bytes,
                         history=history, variant=variant, cluster=cluster, block=block,
                         device=device)
+            pool.many_step(True)
+            return pool
         self.make_pool = make_pool
         self.pool = make_pool()
         self.k = int(advance_steps)

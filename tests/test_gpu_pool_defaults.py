@@ -114,3 +114,91 @@ def test_few_uneven_runs_equal_alone(free):
         np.testing.assert_allclose(d["field"], e["field"], rtol=1e-12, atol=1e-300)
         np.testing.assert_allclose(d["kinetic"][:-1], e["kinetic"][:-1], rtol=1e-5)
         assert np.isnan(d["kinetic"][-1])
+
+
+def two_kernels(p, seed, steps):
+    """The run alone by push and solve kernels (a shape of its own)."""
+    q = pic.Params(npart=p.npart, ncell=p.ncell, length=L, sort_interval=p.sort_interval, block_size=256)
+    return alone(q, seed, steps)
+
+
+def assert_equal_runs(pool, slot, run):
+    for a, b in zip(pool.get_cells(slot), run.get_cells()):
+        assert np.array_equal(a, b)
+    f, g = pool.get_field(slot), run.get_field()
+    for key in ("rho_q", "E", "rho"):
+        assert np.array_equal(f[key], g[key])
+
+
+def many_step_launched(pool):
+    """Whether an advance takes the many-step launch: its waits are made to run out."""
+    pool.set_wait_limit(4096, 1)
+    try:
+        pool.advance(1)
+        return False
+    except pic.PicError as e:
+        assert e.code == pic.PIC_ETIMEOUT
+        return True
+    finally:
+        pool.set_wait_limit()
+
+
+@pytest.mark.parametrize("how,many", [("open", True), ("config", False), ("block", False), ("configured", False),
+                                      ("allowed", True), ("forbidden", False)])
+def test_a_chosen_shape_is_taken(how, many):
+    kw = dict(config=dict(variant=5, cluster=2, block=512), allowed=dict(variant=5, cluster=2, block=512),
+              block=dict(block=256)).get(how, {})
+    pool = pic.Pool(max_slots=1, ncell_max=64, arena_bytes=1 << 24, history=16, device="cuda:0", **kw)
+    if how == "configured":
+        pool.configure(17, 4, 256)
+    elif how in ("allowed", "forbidden"):
+        pool.many_step(how == "allowed")
+    p = pic.Params(npart=20000, ncell=64, length=L)
+    slot = pool.admit(p, *state(20000, 1), 5)
+    pool.advance(2)
+    assert many_step_launched(pool) == many
+    if not many:
+        pool.advance(2)
+        assert_equal_runs(pool, slot, two_kernels(p, 1, 5))
+
+
+@pytest.mark.parametrize("variant,cluster,block,ncell_max",
+                         [(2, 8, 256, 2048), (1, 8, 256, 2048), (5, 4, 512, 2048), (2, 2, 512, 1024), (2, 1, 512, 512),
+                          (1, 4, 256, 1024), (2 + 16, 8, 512, 4096), (5 + 16, 8, 256, 2048)])
+def test_chosen_shapes_equal_the_two_kernels(variant, cluster, block, ncell_max):
+    sizes = [(20000, 64), (100003, 2048), (5, 16), (1, 1), (77777, 512), (250001, 1024), (65537, 4096)]
+    ps = [pic.Params(npart=n, ncell=g, length=L) for n, g in sizes if g <= ncell_max]
+    pool = pic.Pool(max_slots=len(ps), ncell_max=ncell_max, arena_bytes=1 << 27, history=32, variant=variant,
+                    cluster=cluster, block=block, device="cuda:0")
+    slots = [pool.admit(p, *state(p.npart, i), 12) for i, p in enumerate(ps)]
+    pool.advance(5)
+    pool.advance(7)
+    for i, p in enumerate(ps):
+        assert_equal_runs(pool, slots[i], two_kernels(p, i, 12))
+
+
+@pytest.mark.parametrize("runs", [1, 37, 38, 39, 90])
+def test_open_clusters_on_both_sides_of_the_block_size_equal_the_two_kernels(runs):
+    # blocks of 512 threads while every run has a cluster of its own, then of 256
+    ps = [pic.Params(npart=2000 + 37 * i, ncell=1 + (53 * i) % 2048, length=L) for i in range(runs)]
+    pool = pic.Pool(max_slots=runs, ncell_max=2048, arena_bytes=1 << 26, history=16, device="cuda:0")
+    pool.many_step(False)
+    slots = [pool.admit(p, *state(p.npart, i), 6) for i, p in enumerate(ps)]
+    pool.advance(6)
+    for i in (0, runs // 2, runs - 1):
+        assert_equal_runs(pool, slots[i], two_kernels(ps[i], i, 6))
+
+
+def test_many_step_runs_of_a_pool_equal_the_two_kernels():
+    specs = [(600001, 2048, 9, 0), (3, 1, 9, 0), (5, 2, 4, 0), (40000, 1025, 9, 0), (70001, 64, 1, 0), (20003, 1024, 7, 50)]
+    ps = [pic.Params(npart=n, ncell=g, length=L, sort_interval=S) for n, g, _, S in specs]
+    pool = pic.Pool(max_slots=len(ps), ncell_max=2048, history=16, arena_bytes=1 << 26, device="cuda:0")
+    slots = [pool.admit(p, *state(p.npart, i), k) for i, (p, (_, _, k, _)) in enumerate(zip(ps, specs))]
+    for k in (1, 2, 1, 9):
+        pool.advance(k)
+    for i, (p, (_, _, k, _)) in enumerate(zip(ps, specs)):
+        assert pool.step_count(slots[i]) == k
+        assert_equal_runs(pool, slots[i], two_kernels(p, i, k))
+    pool.release(slots[0])
+    pool.admit(ps[1], *state(3, 1), 5)
+    assert many_step_launched(pool)
