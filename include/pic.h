@@ -352,9 +352,15 @@ int pic_init_loaded(pic_run *run, const pic_loading *ld);
 
 /* Set the launch shape of the fused push (deposit variant, block size, unroll,
  * resident blocks per SM; 0 keeps the current value / picks the default).
- * Drops the captured graphs.  PIC_EINVAL for a shape the kernel cannot run. */
+ * Drops the captured graphs.  PIC_EINVAL for a shape the kernel cannot run.  The
+ * run's shape is then chosen: pic_step_n takes no many-step launch. */
 int pic_set_launch(pic_run *run, int32_t variant, int32_t block, int32_t unroll,
                    int32_t blocks_per_sm);
+
+/* Take a shape that pic_autotune adopted for another run of this kind (all three
+ * values as pic_launch_shape gave them): the run is left as pic_autotune leaves
+ * it, its shape open if it was. */
+int pic_adopt_launch(pic_run *run, int32_t variant, int32_t block, int32_t unroll);
 
 /* One timed candidate of pic_autotune. */
 typedef struct pic_tune_entry {
@@ -373,7 +379,8 @@ typedef struct pic_tune_entry {
  * velocities), and the fastest shape changes with it: tune after those.
  * Writes up to
  * max_results entries to results (may be NULL) and their count to *nresults.
- * Synchronises.  PIC_ESTATE before pic_init or between pic_push and
+ * A run whose shape was open goes on to take the many-step launch where
+ * pic_step_n does.  Synchronises.  PIC_ESTATE before pic_init or between pic_push and
  * pic_solve_field. */
 int pic_autotune(pic_run *run, int32_t reps, pic_tune_entry *results,
                  int32_t max_results, int32_t *nresults);

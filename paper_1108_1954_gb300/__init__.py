@@ -100,6 +100,7 @@ _SIG = {
     "pic_launch_shape": (C.c_int, [_VP, C.POINTER(C.c_int32), C.POINTER(C.c_int32),
                                    C.POINTER(C.c_int32), C.POINTER(C.c_int32)]),
     "pic_autotune": (C.c_int, [_VP, C.c_int32, _VP, C.c_int32, C.POINTER(C.c_int32)]),
+    "pic_adopt_launch": (C.c_int, [_VP, C.c_int32, C.c_int32, C.c_int32]),
     "pic_set_wait_limit": (C.c_int, [_VP, C.c_int32, C.c_int32]),
     "pic_set_launch": (C.c_int, [_VP, C.c_int32, C.c_int32, C.c_int32, C.c_int32]),
     "pic_set_shard": (C.c_int, [_VP, C.c_int64]),
@@ -383,7 +384,8 @@ class Run:
                                self.p.shape)
             hit = tune_cache.lookup(cache, k)
             if hit is not None:
-                self.set_launch(hit["variant"], hit["block"], hit["unroll"])
+                _check(_lib.pic_adopt_launch(self._h, int(hit["variant"]), int(hit["block"]),
+                                             int(hit["unroll"])), "pic_adopt_launch")
                 return np.zeros(0, dtype=TUNE_DTYPE)
         out = np.zeros(64, dtype=TUNE_DTYPE)
         n = C.c_int32(0)

@@ -954,13 +954,14 @@ int pic_launch_shape(const pic_run *run, int32_t *grid, int32_t *block, int32_t 
     return PIC_OK;
 }
 
-int pic_set_launch(pic_run *run, int32_t variant, int32_t block, int32_t unroll,
-                   int32_t blocks_per_sm) {
-    if (!run) return PIC_EINVAL;
-    if (run->pending_push) return PIC_ESTATE;
+}  // extern "C"
+
+namespace {
+
+// The push's shape; open: whether the run's shape counts as left open after it.
+int take_launch(pic_run *run, int32_t variant, int32_t block, int32_t unroll, int32_t blocks_per_sm, bool open) {
     const bool fixed = run->p.precision == PIC_FP32_FIXED;
     const bool ngp = run->p.shape == PIC_SHAPE_NGP;
-    if (ngp && variant) return PIC_EINVAL;   // the shape fixes the deposit
     // a shape that gives no variant takes QUAD, which has every unroll
     const int v = variant ? variant : run->auto_variant && !ngp && fixed ? (int)PIC_DEPOSIT_QUAD : run->variant;
     const int b = block ? block : run->block;
@@ -976,11 +977,31 @@ int pic_set_launch(pic_run *run, int32_t variant, int32_t block, int32_t unroll,
     run->block = b;
     run->unroll = u;
     run->grid = g;
-    run->open_shape = false;
+    run->open_shape = open;
     if (variant) run->auto_variant = false;
     PIC_CUDA(set_steps_shape(run));
     destroy_graphs(run);
     return PIC_OK;
+}
+
+}  // namespace
+
+extern "C" {
+
+int pic_set_launch(pic_run *run, int32_t variant, int32_t block, int32_t unroll,
+                   int32_t blocks_per_sm) {
+    if (!run) return PIC_EINVAL;
+    if (run->pending_push) return PIC_ESTATE;
+    if (run->p.shape == PIC_SHAPE_NGP && variant) return PIC_EINVAL;   // the shape fixes the deposit
+    return take_launch(run, variant, block, unroll, blocks_per_sm, false);
+}
+
+int pic_adopt_launch(pic_run *run, int32_t variant, int32_t block, int32_t unroll) {
+    if (!run) return PIC_EINVAL;
+    if (run->pending_push) return PIC_ESTATE;
+    if (variant < 1 || block < 1 || unroll < 1) return PIC_EINVAL;
+    if (run->p.shape == PIC_SHAPE_NGP && variant != kDepositNgp) return PIC_EINVAL;
+    return take_launch(run, variant, block, unroll, run->p.blocks_per_sm, run->open_shape);
 }
 
 int pic_autotune(pic_run *run, int32_t reps, pic_tune_entry *results,

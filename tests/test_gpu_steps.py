@@ -397,3 +397,39 @@ def test_mode_amplitudes_against_float64_sums(n, ng):
             err.append((row["mode"][m] - want) / (2.0 / ng * np.abs(E).sum()))
     assert np.sqrt(np.mean(np.square(err))) <= math.sqrt(13.0 / parts) * 2.0 ** -25 / math.sqrt(3.0)
     run.close()
+
+
+def many_step_launched(run):
+    """Whether pic_step_n takes the many-step launch: its waits are made to run out
+    (the run needs a new state afterwards)."""
+    run.set_wait_limit(4096, 1)
+    run.step_n(2)
+    try:
+        run.sync()
+        return False
+    except pic.PicError as e:
+        assert e.code == pic.PIC_ETIMEOUT
+        return True
+    finally:
+        run.set_wait_limit()
+
+
+@pytest.mark.parametrize("shape", [pic.PIC_SHAPE_CIC, pic.PIC_SHAPE_NGP])
+@pytest.mark.parametrize("open_shape", [True, False])
+def test_a_shape_from_the_tuning_cache_leaves_the_run_as_tuning_does(tmp_path, shape, open_shape):
+    n, ng, path = 200003, 1024, str(tmp_path / "shapes.json")
+    kw = dict() if open_shape else dict(block_size=128)
+    runs = [pic.Run(pic.Params(npart=n, ncell=ng, length=L, shape=shape, **kw), device="cuda:0") for _ in range(2)]
+    for i, r in enumerate(runs):
+        r.init(*state(n, 4))
+        assert (len(r.autotune(reps=2, cache=path)) == 0) == (i == 1)
+        r.step_n(5)
+    assert runs[0].launch_shape() == runs[1].launch_shape()
+    assert_same(runs[0], runs[1], n, ng)
+    assert [many_step_launched(r) for r in runs] == [open_shape, open_shape]
+    r = pic.Run(pic.Params(npart=n, ncell=ng, length=L, shape=shape), device="cuda:0")
+    r.init(*state(n, 4))
+    r.set_launch(block=256)
+    assert not many_step_launched(r)
+    for bad in ((0, 256, 1), (3, 256, 1), (1, 0, 1), (1, 256, 3), (9, 512, 4)):
+        assert pic._lib.pic_adopt_launch(r._h, *bad) == pic.PIC_EINVAL
