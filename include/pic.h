@@ -417,7 +417,10 @@ int pic_device_density(pic_run *run, void **rho_q);
  * run's push shape: the sort of the state is timed, then the sorted copy is
  * pushed max(S) times with the current field, each push timed (t(k), k pushes
  * after a sort); cost(S) = (t_sort + sum_{k<S} t(k)) / S, cost(0) = the mean
- * of the last quarter of t(k).  ms_per_step[count] (may be NULL) receives the
+ * of the last quarter of t(k).  A run that takes the many-step launch
+ * (pic_step_n) is timed in it: a launch of S whole steps takes the place of the
+ * pushes, and cost(0) is a step of a launch of the drifted copy.
+ * ms_per_step[count] (may be NULL) receives the
  * costs, *best (may be NULL) the cheapest candidate; adopt != 0 sets the
  * run's sort interval to it (dropping the captured graphs).  The run's state
  * is untouched.  Synchronises.  PIC_ESTATE as for pic_autotune. */

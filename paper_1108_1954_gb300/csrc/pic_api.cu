@@ -473,7 +473,8 @@ bool capturing(const pic_run *r) {
     return true;
 }
 
-int run_steps(pic_run *r, int steps) {
+// The many-step launch of the run's state (but for the counters' values).
+StepsArgs steps_args(pic_run *r) {
     const int c = r->cur;
     StepsArgs a;
     a.x = (float *)r->xs(c);
@@ -488,18 +489,14 @@ int run_steps(pic_run *r, int steps) {
     a.partials = r->at<double>(r->lay.partials);
     a.err = &r->dev()->err;
     a.sync = r->dev()->sync;
-    for (int i = 0; i < 3; i++) a.base[i] = r->sync_base[i];
-    a.base[0] += r->wait_missing;
     a.wait_limit = r->wait_limit ? r->wait_limit : kStepsWaitLimit;
-    const int nd = steps_diag_blocks(r->lay.hist_len);
-    a.diag_blocks = nd;
+    a.diag_blocks = steps_diag_blocks(r->lay.hist_len);
     a.first_block = 0;
     a.blocks = r->steps_grid;
     a.hist = r->at<pic_diag_row>(r->lay.hist);
     a.hist_len = r->lay.hist_len;
     a.step0 = r->step;
     a.dstep = &r->dev()->step;
-    a.steps = steps;
     a.c = r->pc;
     a.d = push64_args(r);
     a.weight_total = (long long)((unsigned long long)r->p.npart << kFixBits);
@@ -509,11 +506,25 @@ int run_steps(pic_run *r, int steps) {
     a.k_mode = 2.0 / (double)r->p.ncell;
     a.dx = r->dx;
     a.mass = r->mass;
-    PIC_CUDA(r->p.precision == PIC_FP64
-                 ? launch_steps64(a, r->steps_grid, r->steps_block, r->stream)
-                 : launch_steps(a, r->variant, r->steps_grid, r->steps_block, r->steps_small, r->stream));
+    return a;
+}
+
+cudaError_t enqueue_steps(pic_run *r, StepsArgs a, int steps) {
+    const int nd = a.diag_blocks;
+    for (int i = 0; i < 3; i++) a.base[i] = r->sync_base[i];
+    a.base[0] += r->wait_missing;
+    a.steps = steps;
+    const cudaError_t e = r->p.precision == PIC_FP64
+        ? launch_steps64(a, r->steps_grid, r->steps_block, r->stream)
+        : launch_steps(a, r->variant, r->steps_grid, r->steps_block, r->steps_small, r->stream);
+    if (e != cudaSuccess) return e;
     r->sync_base[0] += (unsigned)(r->steps_grid - nd) * ((unsigned)steps + 1u);
     for (int d = 0; d < nd; d++) r->sync_base[1 + d] += (unsigned)((steps - d + nd - 1) / nd);
+    return cudaSuccess;
+}
+
+int run_steps(pic_run *r, int steps) {
+    PIC_CUDA(enqueue_steps(r, steps_args(r), steps));
     r->step += steps;
     return PIC_OK;
 }
@@ -1131,6 +1142,9 @@ int pic_device_density(pic_run *run, void **rho_q) {
 // S > 0 the cost is (t_sort + sum_{k<S} t(k)) / S; for S = 0 (never sort) it
 // is the mean of the last quarter of t(k), the drifted state.  The run's own
 // state is untouched (the copy's pushes deposit into the tuning density).
+// A run that takes the many-step launch is timed in it: (t_sort + T(S)) / S with T(S)
+// a launch of S steps of the sorted copy, and for S = 0 a step of a launch that
+// goes on from kmax steps after the sort.
 int pic_tune_sort_interval(pic_run *run, const int32_t *intervals, int32_t count,
                            float *ms_per_step, int32_t *best, int32_t adopt) {
     pic::TraceRange trace_("pic_tune_sort_interval");
@@ -1152,6 +1166,7 @@ int pic_tune_sort_interval(pic_run *run, const int32_t *intervals, int32_t count
     if (e == cudaSuccess) e = cudaEventRecord(ev[0], run->stream);
     if (e == cudaSuccess) e = enqueue_sort_into(run, c, run->stream);
     if (e == cudaSuccess) e = cudaEventRecord(ev[1], run->stream);
+    const bool resident = run->steps_grid && !run->captured;
     PushArgs a;
     a.x = (float *)run->xs(1 - c);
     a.v = (float *)run->vs(1 - c);
@@ -1162,7 +1177,7 @@ int pic_tune_sort_interval(pic_run *run, const int32_t *intervals, int32_t count
     a.err = &run->dev()->err;
     a.wide = push_wide_tile(run->p.npart, run->sms);
     a.c = run->pc;
-    for (int k = 0; k < kmax && e == cudaSuccess; k++) {
+    for (int k = 0; k < kmax && e == cudaSuccess && !resident; k++) {
         e = cudaEventRecord(ev[2 + 2 * k], run->stream);
         if (e == cudaSuccess)
             e = launch_push_fixed(a, run->grid, run->block, run->variant, run->unroll, true,
@@ -1172,23 +1187,64 @@ int pic_tune_sort_interval(pic_run *run, const int32_t *intervals, int32_t count
     if (e == cudaSuccess) e = cudaStreamSynchronize(run->stream);
     float tsort = 0.0f, t[256];
     if (e == cudaSuccess) e = cudaEventElapsedTime(&tsort, ev[0], ev[1]);
-    for (int k = 0; k < kmax && e == cudaSuccess; k++)
+    for (int k = 0; k < kmax && e == cudaSuccess && !resident; k++)
         e = cudaEventElapsedTime(&t[k], ev[2 + 2 * k], ev[3 + 2 * k]);
+    float launch[64];
+    if (resident) {
+        // what the launch writes beside the copy goes to memory that a fixed-point run
+        // uses for nothing else, or not between calls
+        StepsArgs b = steps_args(run);
+        const size_t ng = (size_t)run->p.ncell;
+        b.x = a.x;
+        b.v = a.v;
+        b.E32 = run->at<float>(run->lay.rho_f32);
+        b.E64 = run->at<double>(run->lay.rho_w);
+        b.phi = b.E64 + ng;
+        b.rho = run->at<double>(run->lay.tune_rho);
+        unsigned char *mem = run->ws + run->lay.phase;
+        static_assert((kStepsMaxCells + 1) * 8 + (kStepsSlots + 1) * sizeof(pic_diag_row) <= (size_t)kPhaseMaxBins * 4,
+                      "the launch's outputs in the histogram's place");
+        b.rho_q_last = reinterpret_cast<unsigned long long *>(mem);
+        b.dstep = reinterpret_cast<long long *>(mem + ng * 8);
+        b.hist = reinterpret_cast<pic_diag_row *>(mem + (ng + 1) * 8);
+        b.hist_len = kStepsSlots + 1;
+        b.diag_blocks = steps_diag_blocks(run->lay.hist_len);      // as steps_grid counts them
+        // the copy sorted anew (or as it is), and one launch of it; ms of the launch
+        auto time_steps = [&](bool sort, int steps, float *ms) {
+            cudaError_t f = sort ? enqueue_sort_into(run, c, run->stream) : cudaSuccess;
+            if (f == cudaSuccess)
+                f = cudaMemcpyAsync(b.E32, run->ws + run->lay.E32, ng * 4, cudaMemcpyDeviceToDevice, run->stream);
+            if (f == cudaSuccess) f = cudaEventRecord(ev[2], run->stream);
+            if (f == cudaSuccess) f = enqueue_steps(run, b, steps);
+            if (f == cudaSuccess) f = cudaEventRecord(ev[3], run->stream);
+            if (f == cudaSuccess) f = cudaEventSynchronize(ev[3]);
+            if (f == cudaSuccess) f = cudaEventElapsedTime(ms, ev[2], ev[3]);
+            return f;
+        };
+        float ms = 0.0f;
+        if (e == cudaSuccess) e = time_steps(true, kmax, &ms);            // warm
+        if (e == cudaSuccess) e = time_steps(false, 64, &launch[0]);
+        const float drifted = launch[0] / 64.0f;
+        for (int i = 0; i < count && e == cudaSuccess; i++) {
+            if (intervals[i] > 0) e = time_steps(true, intervals[i], &launch[i]);
+            else launch[i] = drifted;
+        }
+    }
     if (e != cudaSuccess) rc = cuda_fail(e);
     for (int i = 0; i < made; i++) cudaEventDestroy(ev[i]);
     if (rc) return rc;
     float drift = 0.0f;
     const int q0 = kmax - kmax / 4;
-    for (int k = q0; k < kmax; k++) drift += t[k];
+    for (int k = q0; k < kmax && !resident; k++) drift += t[k];
     drift /= (float)(kmax - q0);
     int bi = 0;
     float bcost = 0.0f;
     for (int i = 0; i < count; i++) {
         const int S = intervals[i];
-        float cost = drift;
+        float cost = resident ? launch[i] : drift;
         if (S > 0) {
-            cost = tsort;
-            for (int k = 0; k < S; k++) cost += t[k];
+            cost = tsort + (resident ? launch[i] : 0.0f);
+            for (int k = 0; k < S && !resident; k++) cost += t[k];
             cost /= (float)S;
         }
         if (ms_per_step) ms_per_step[i] = cost;

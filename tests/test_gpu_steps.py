@@ -433,3 +433,42 @@ def test_a_shape_from_the_tuning_cache_leaves_the_run_as_tuning_does(tmp_path, s
     assert not many_step_launched(r)
     for bad in ((0, 256, 1), (3, 256, 1), (1, 0, 1), (1, 256, 3), (9, 512, 4)):
         assert pic._lib.pic_adopt_launch(r._h, *bad) == pic.PIC_EINVAL
+
+
+@pytest.mark.parametrize("n,ng,shape,H", [(20000, 64, pic.PIC_SHAPE_CIC, 256), (300007, 777, pic.PIC_SHAPE_NGP, 256),
+                                          (700001, 4096, pic.PIC_SHAPE_CIC, 3), (5, 1, pic.PIC_SHAPE_CIC, 1)])
+def test_the_sort_interval_is_tuned_on_the_launch_that_the_run_takes(n, ng, shape, H):
+    a, b = pair(n, ng, shape=shape, history=H)
+    for r in (a, b):
+        r.step_n(9)
+    intervals = (0, 1, 20, 5)
+    best, ms = a.tune_sort_interval(intervals)
+    assert list(ms) == list(intervals) and all(t > 0 for t in ms.values())
+    assert ms[best] == min(ms.values())
+    # the state, the rows and the launch's own accumulators and counters are as before
+    for _ in range(2):
+        a.step_n(7), b.step_n(7)
+        for p, q in zip(a.get_cells(), b.get_cells()):
+            assert np.array_equal(p, q)
+        f, g = a.get_field(), b.get_field()
+        for k in ("rho_q", "E", "rho", "phi"):
+            assert np.array_equal(f[k], g[k]), k
+        first, count = max(0, a.step - H + 1), min(H, a.step + 1)
+        d, e = a.diagnostics(first, count), b.diagnostics(first, count)
+        for k in ("step", "charge_q", "field"):
+            assert np.array_equal(d[k], e[k]), k
+    a.phase_space(8, 8, -1.0, 1.0)
+    a.tune_sort_interval((0, 10), adopt=True)
+    a.step_n(25)
+    a.sync()
+    # timed in the launch that pic_step_n takes: its waits run out there too, and a
+    # run whose shape is chosen has none
+    for r, takes in ((a, True), (b, False)):
+        r.set_wait_limit(4096, 1)
+        if takes:
+            with pytest.raises(pic.PicError) as e:
+                r.tune_sort_interval(intervals)
+            assert e.value.code == pic.PIC_ETIMEOUT
+        else:
+            r.tune_sort_interval(intervals)
+    a.close(), b.close()
