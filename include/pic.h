@@ -46,7 +46,10 @@
  * sets a device error word, which the synchronising calls (pic_sync,
  * pic_diagnostics, pic_get_state, pic_get_field) report as PIC_EDEVICE.
  *
- * Threading.  Calls on one run are not thread-safe; different runs are.
+ * Threading.  Calls on one run are not thread-safe; different runs are.  The
+ * read-backs of a pool (pic_pool_get_state, _get_cells, _get_field, _diagnostics)
+ * may come from several threads, and beside admissions and releases of other
+ * slots; its other calls are not thread-safe.
  */
 #ifndef PIC_H
 #define PIC_H
@@ -220,6 +223,10 @@ int pic_sort(pic_run *run);
  * whichever it is; the kinetic, momentum and mode entries of the rows are sums in
  * another order and agree to rounding.
  * A step n with n % S == 0 (S = sort_interval > 0, n > 0) sorts first.
+ * Runs on streams of their own share the SMs: many-step launches that together need
+ * more than all of them take turns.  From some 1e6 particles a run on, 8 or more
+ * runs at once then give more steps in all with a chosen shape (16 runs of 3e6 on
+ * 777 cells: 12.0 us a step of one run, 10.1 with push and solve kernels).
  * Asynchronous. */
 int pic_step_n(pic_run *run, int64_t n);
 

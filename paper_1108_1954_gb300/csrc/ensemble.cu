@@ -14,6 +14,7 @@
 #include <cstdio>
 #include <cstring>
 #include <map>
+#include <mutex>
 #include <new>
 #include <vector>
 
@@ -155,6 +156,8 @@ struct pic_pool {
     bool many_step = true;        // few runs may take it (pic_pool_many_step)
     unsigned wait_limit = 0, wait_missing = 0;   // pic_pool_set_wait_limit
     pic::Staging stage;
+    // what is handed out of the arena, or used of its idle space
+    std::mutex arena_mutex;
 
     BatchRun *d_runs() const { return reinterpret_cast<BatchRun *>(arena + tab.runs); }
     int *d_order() const { return reinterpret_cast<int *>(arena + tab.order); }
@@ -357,6 +360,7 @@ int launch_resident(pic_pool *pool, const std::vector<int> &order, const std::ve
         off = align_up(off + (size_t)kStepsSlots * kStepsMaxGrid * 16);
     }
     size_t soff = 0, sbytes = 0;
+    std::lock_guard<std::mutex> lock(pool->arena_mutex);          // till the launch is done
     if (!pool->idle_space(&soff, &sbytes) || sbytes < off) return PIC_OK;
     unsigned char *mem = pool->arena + soff;
     std::vector<StepsArgs> args(order.size());
@@ -547,7 +551,10 @@ int admit_common(pic_pool *pool, const pic_params *p, int64_t steps, int32_t *sl
     if (s < 0) return PIC_ENOMEM;
     const RunLayout L = run_layout(p, pool->cfg.history);
     size_t off;
-    if (!pool->alloc(L.total, &off)) return PIC_ENOMEM;
+    {
+        std::lock_guard<std::mutex> lock(pool->arena_mutex);
+        if (!pool->alloc(L.total, &off)) return PIC_ENOMEM;
+    }
     pic_pool::Slot &sl = pool->slots[s];
     sl.used = true;
     sl.needs_init = true;
@@ -593,6 +600,7 @@ int admit_common(pic_pool *pool, const pic_params *p, int64_t steps, int32_t *sl
         e = cudaMemsetAsync(d.hist, 0xFF, (size_t)pool->cfg.history * sizeof(pic_diag_row), pool->stream);
     if (e != cudaSuccess) {
         sl = pic_pool::Slot();
+        std::lock_guard<std::mutex> lock(pool->arena_mutex);
         pool->release(off, L.total);
         return cuda_fail(e);
     }
@@ -610,6 +618,7 @@ int check_admit(const pic_pool *pool, const pic_params *p) {
 
 void drop_slot(pic_pool *pool, int s) {
     pic_pool::Slot &sl = pool->slots[s];
+    std::lock_guard<std::mutex> lock(pool->arena_mutex);
     pool->release(sl.off, sl.size);
     sl = pic_pool::Slot();
 }
@@ -761,8 +770,10 @@ int pic_pool_get_state(pic_pool *pool, int32_t slot, void *x, void *v) {
     const double to_phys = sl.p.length / (double)sl.p.ncell;
     const float Lf = (float)sl.p.length;
     size_t soff = 0, sbytes = 0;
+    std::unique_lock<std::mutex> lock(pool->arena_mutex);         // till the copies are queued
     const bool scratch = x && pool->idle_space(&soff, &sbytes) && sbytes >= std::min(pb, kMinScratch);
     if (!scratch) {
+        lock.unlock();
         // the arena is full: cell coordinates down, converted here with the
         // same two float64-rounded steps as the device conversion
         const int rc = pic_pool_get_cells(pool, slot, (float *)x, (float *)v);
@@ -786,6 +797,7 @@ int pic_pool_get_state(pic_pool *pool, int32_t slot, void *x, void *v) {
         PIC_CUDA(cudaMemcpyAsync((float *)x + i, tmp, (size_t)m * 4, cudaMemcpyDeviceToHost,
                                  pool->stream));
     }
+    lock.unlock();
     if (v) PIC_CUDA(cudaMemcpyAsync(v, sl.desc.v, pb, cudaMemcpyDeviceToHost, pool->stream));
     return read_error(pool);
 }
@@ -836,6 +848,7 @@ int pic_pool_release(pic_pool *pool, int32_t slot) {
     pic_pool::Slot &sl = pool->slots[slot];
     // the arena space may be reused by the next admission: its uploads are
     // stream-ordered after every launch already enqueued
+    std::lock_guard<std::mutex> lock(pool->arena_mutex);
     pool->release(sl.off, sl.size);
     sl = pic_pool::Slot();
     return PIC_OK;

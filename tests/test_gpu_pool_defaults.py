@@ -202,3 +202,46 @@ def test_many_step_runs_of_a_pool_equal_the_two_kernels():
     pool.release(slots[0])
     pool.admit(ps[1], *state(3, 1), 5)
     assert many_step_launched(pool)
+
+
+def test_read_backs_from_several_threads_beside_admissions():
+    # the threads' conversions share the arena's idle space, which an admission takes from
+    import threading
+    sizes = [300007, 200003, 90001, 50021]
+    ps = [pic.Params(npart=n, ncell=300, length=L) for n in sizes]
+    extra = pic.Params(npart=70001, ncell=100, length=L)
+    need = (1 << 14) + sum(pic.pool_run_bytes(p, 16) for p in ps) + pic.pool_run_bytes(extra, 16)
+    pool = pic.Pool(max_slots=8, ncell_max=512, arena_bytes=need + (600 << 10), history=16, device="cuda:0")
+    slots = [pool.admit(p, *state(p.npart, i), 3) for i, p in enumerate(ps)]
+    pool.advance(3)
+    want = [pool.get_state(s) for s in slots]
+    x, v = state(extra.npart, 9)
+    errors = []
+
+    def read(i):
+        try:
+            for _ in range(40):
+                a, b = pool.get_state(slots[i])
+                assert np.array_equal(a, want[i][0]) and np.array_equal(b, want[i][1])
+                assert np.array_equal(pool.get_field(slots[i])["rho_q"], fields[i])
+        except BaseException as e:
+            errors.append(e)
+
+    fields = [pool.get_field(s)["rho_q"] for s in slots]
+    threads = [threading.Thread(target=read, args=(i,)) for i in range(len(ps))]
+    [t.start() for t in threads]
+    for _ in range(20):
+        s = pool.admit(extra, x, v, 1)
+        pool.release(s)
+    s = pool.admit(extra, x, v, 2)
+    [t.join() for t in threads]
+    assert not errors, errors[0]
+    pool.advance(2)
+    assert_equal_runs(pool, s, two_kernels_of(extra, x, v, 2))
+
+
+def two_kernels_of(p, x, v, steps):
+    run = pic.Run(pic.Params(npart=p.npart, ncell=p.ncell, length=L, block_size=256), device="cuda:0")
+    run.init(x, v)
+    run.step_n(steps)
+    return run
