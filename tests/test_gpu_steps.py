@@ -472,3 +472,42 @@ def test_the_sort_interval_is_tuned_on_the_launch_that_the_run_takes(n, ng, shap
         else:
             r.tune_sort_interval(intervals)
     a.close(), b.close()
+
+
+@pytest.mark.parametrize("threads", [False, True])
+def test_runs_on_streams_of_their_own_equal_the_two_kernels(threads):
+    # many-step launches of several runs in flight at once, one by one and from threads
+    specs = [(20000, 64, 0), (300007, 500, 7), (1000003, 1024, 0), (700001, 4096, 0), (50021, 100, 3), (20000, 100, 0),
+             (3, 1, 0), (131073, 2048, 5)]
+    runs = []
+    for i, (n, ng, S) in enumerate(specs):
+        kw = dict(precision=pic.PIC_FP64) if i == 5 else {}
+        r = pic.Run(pic.Params(npart=n, ncell=ng, length=L, sort_interval=S, **kw), device="cuda:0",
+                    stream=torch.cuda.Stream())
+        x, v = state(n, i)
+        r.init(x.astype(r.p.dtype), v.astype(r.p.dtype))
+        runs.append(r)
+
+    def go(r):
+        for k in (1, 30, 2, 17):
+            r.step_n(k)
+        r.sync()
+
+    if threads:
+        import threading
+        ts = [threading.Thread(target=go, args=(r,)) for r in runs]
+        [t.start() for t in ts], [t.join() for t in ts]
+    else:
+        for k in (1, 30, 2, 17):
+            for r in runs:
+                r.step_n(k)
+    for i, (r, (n, ng, S)) in enumerate(zip(runs, specs)):
+        q = pic.Run(pic.Params(npart=n, ncell=ng, length=L, sort_interval=S, precision=r.p.precision, block_size=256),
+                    device="cuda:0")
+        x, v = state(n, i)
+        q.init(x.astype(q.p.dtype), v.astype(q.p.dtype))
+        q.step_n(50)
+        for a, b in zip(r.get_state(), q.get_state()):
+            assert np.array_equal(a, b)
+        assert np.array_equal(r.get_field()["E"], q.get_field()["E"])
+        r.close(), q.close()
