@@ -815,7 +815,7 @@ int pic_pool_get_field(pic_pool *pool, int32_t slot, double *rho, double *phi, d
     for (const auto &w : want) {
         if (!w.dst) continue;
         const cudaError_t e = pool->stage.add(w.dst, w.src, nb, pool->stream);
-        if (e != cudaSuccess) { pool->stage.drop(); return cuda_fail(e); }
+        if (e != cudaSuccess) { pool->stage.abandon(pool->stream); return cuda_fail(e); }
     }
     return finish_read(pool);
 }
@@ -837,7 +837,7 @@ int pic_pool_diagnostics(pic_pool *pool, int32_t slot, int64_t first, int32_t co
         if (pos + len > H) len = H - pos;
         const cudaError_t e = pool->stage.add(rows + got, sl.desc.hist + pos,
                                               (size_t)len * sizeof(pic_diag_row), pool->stream);
-        if (e != cudaSuccess) { pool->stage.drop(); return cuda_fail(e); }
+        if (e != cudaSuccess) { pool->stage.abandon(pool->stream); return cuda_fail(e); }
         got += len;
     }
     return finish_read(pool);

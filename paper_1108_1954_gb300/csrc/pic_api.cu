@@ -869,7 +869,7 @@ int pic_diagnostics(pic_run *run, int64_t first, int32_t count, pic_diag_row *ro
         if (slot + len > H) len = H - slot;
         const cudaError_t e = run->stage.add(rows + done, hist + slot, (size_t)len * sizeof(pic_diag_row),
                                              run->stream);
-        if (e != cudaSuccess) { run->stage.drop(); return cuda_fail(e); }
+        if (e != cudaSuccess) { run->stage.abandon(run->stream); return cuda_fail(e); }
         done += len;
     }
     return finish_read(run);
@@ -914,7 +914,7 @@ int pic_get_field(pic_run *run, double *rho, double *phi, double *E, int64_t *rh
     for (const auto &w : want) {
         if (!w.dst) continue;
         const cudaError_t e = run->stage.add(w.dst, run->ws + w.off, nb, run->stream);
-        if (e != cudaSuccess) { run->stage.drop(); return cuda_fail(e); }
+        if (e != cudaSuccess) { run->stage.abandon(run->stream); return cuda_fail(e); }
     }
     return finish_read(run);
 }

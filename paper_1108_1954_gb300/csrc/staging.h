@@ -21,6 +21,21 @@
 
 namespace pic {
 
+// Page-locked memory is made and freed while another stream may be captured into a
+// graph, which either call would end in the default capture mode.
+class RelaxedCapture {
+public:
+    RelaxedCapture() { ok_ = cudaThreadExchangeStreamCaptureMode(&mode_) == cudaSuccess; }
+    ~RelaxedCapture() {
+        if (ok_) (void)cudaThreadExchangeStreamCaptureMode(&mode_);
+    }
+    bool ok() const { return ok_; }
+
+private:
+    cudaStreamCaptureMode mode_ = cudaStreamCaptureModeRelaxed;
+    bool ok_;
+};
+
 class Slabs {
 public:
     static constexpr int kSlabs = 8;
@@ -40,14 +55,12 @@ public:
         }
         void *p = nullptr;
         if (!make) return p;
-        // another thread may be capturing a graph
-        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-        if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) return p;
+        RelaxedCapture relaxed;
+        if (!relaxed.ok()) return p;
         if (cudaMallocHost(&p, kSlabBytes) != cudaSuccess) {
             p = nullptr;
             (void)cudaGetLastError();
         }
-        (void)cudaThreadExchangeStreamCaptureMode(&mode);
         return p;
     }
 
@@ -60,7 +73,8 @@ public:
                 return;
             }
         }
-        cudaFreeHost(p);
+        RelaxedCapture relaxed;
+        (void)cudaFreeHost(p);
     }
 
 private:
@@ -112,9 +126,15 @@ public:
         return e;
     }
 
-    void drop() { n_ = 0, used_ = 0; }
+    // Start afresh after an error, when what was queued before it has arrived.
+    void abandon(cudaStream_t s) {
+        (void)cudaStreamSynchronize(s);
+        drop();
+    }
 
 private:
+    void drop() { n_ = 0, used_ = 0; }
+
     static constexpr int kItems = 8, kDirect = 32;
     struct Item {
         void *dst;

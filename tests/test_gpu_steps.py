@@ -511,3 +511,32 @@ def test_runs_on_streams_of_their_own_equal_the_two_kernels(threads):
             assert np.array_equal(a, b)
         assert np.array_equal(r.get_field()["E"], q.get_field()["E"])
         r.close(), q.close()
+
+
+def test_handles_close_while_another_stream_is_captured():
+    # more handles with page-locked slabs than are kept: the rest are freed
+    runs = []
+    for i in range(12):
+        r = pic.Run(pic.Params(npart=1000, ncell=16, length=L), device="cuda:0")
+        r.init(*state(1000, i))
+        for _ in range(40):
+            r.sync()
+        runs.append(r)
+    x = torch.zeros(16, device="cuda")
+    s, g = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(g, stream=s):                  # "global" capture mode
+        x.add_(1.0)
+        for r in runs:
+            pic._lib.pic_destroy(r._h)
+            r._h = None
+        x.add_(1.0)
+    g.replay()
+    torch.cuda.synchronize()
+    assert torch.all(x == 2.0)
+    r = pic.Run(pic.Params(npart=1000, ncell=16, length=L), device="cuda:0")
+    r.init(*state(1000, 0))
+    for _ in range(40):
+        r.sync()
+    assert len(r.diagnostics()) == 1
+    r.close()
