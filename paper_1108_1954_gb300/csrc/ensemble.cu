@@ -333,7 +333,7 @@ bool resident(const pic_pool *pool, const std::vector<int> &order, std::vector<i
     double time = 0.0;
     if (!allot(pool, order, pool->resident_sms, workers, &time)) return false;
     for (size_t i = 0; i < order.size(); i++)       // a worker's counts share words with carries
-        if (pool->slots[order[i]].p.npart / (*workers)[i] >= (1 << 20) - 64) return false;
+        if (pool->slots[order[i]].p.npart / (*workers)[i] >= kPackedCount - 64) return false;
     return time < cluster_time(pool, order);
 }
 

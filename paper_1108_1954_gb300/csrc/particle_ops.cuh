@@ -199,10 +199,6 @@ struct Tile {
     unsigned k;             // cell j's word is j << k (2^k copies of the tile, steps.cu)
 };
 
-constexpr int kCountBits = 20;
-// The most particles of a tile whose carries share the counts' words.
-constexpr long long kPackedCount = (1ll << kCountBits) - 1;
-
 // A tile of `words` words per array at mem; 8 or (wide) 12 bytes per word.
 __device__ __forceinline__ Tile make_tile(unsigned char *mem, int words, bool wide) {
     Tile t;

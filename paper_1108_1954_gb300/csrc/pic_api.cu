@@ -458,7 +458,11 @@ cudaError_t set_steps_shape(pic_run *r) {
     const int most = (r->sms < kStepsMaxGrid ? r->sms : kStepsMaxGrid) - nd;
     if (most < 1) return cudaSuccess;
     const int64_t need = ((f64 || r->steps_small ? p.npart : (p.npart + 3) / 4) + block - 1) / block;
-    r->steps_grid = (int)(need < most ? need : most) + nd;
+    const int workers = (int)(need < most ? need : most);
+    // a worker's counts share words with carries, as in a push's tile (fixed point; the
+    // limits above are far from it on a GPU with more than 24 SMs)
+    if (!f64 && p.npart / workers >= kPackedCount - 64) return cudaSuccess;
+    r->steps_grid = workers + nd;
     r->steps_block = block;
     return cudaSuccess;
 }

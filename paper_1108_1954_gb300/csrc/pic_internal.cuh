@@ -121,6 +121,11 @@ __host__ __device__ constexpr int density_bits(int mode) {
     return mode == PIC_FP32_FIXED ? kFixBits : mode == PIC_FP32_ATOMIC ? 30 : 53;
 }
 
+// The most particles of a density tile whose carries share the counts' words
+// (particle_ops.cuh).
+constexpr int kCountBits = 20;
+constexpr long long kPackedCount = (1ll << kCountBits) - 1;
+
 // Many steps of a fixed-point run in one cooperative launch (steps.cu).
 struct StepsArgs {
     float *x, *v;                 // N each, 16-byte aligned
