@@ -141,3 +141,59 @@ def test_pool_rejects_cg():
         pool.admit(pic.Params(npart=1000, ncell=64, length=4 * math.pi,
                               field_solver=pic.PIC_SOLVER_CG), x32, v32, 10)
     pool.close()
+
+
+def test_cg_on_one_warp_is_the_iteration_with_rounded_divisions():
+    # Up to 32 nodes every sum is one warp's, so the whole iteration can be followed bit
+    # for bit: products and FMAs rounded once, sums as aligned integers, t and beta the
+    # rounded quotients.
+    from fractions import Fraction as F
+
+    def fma(a, b, c):
+        return float(F(a) * F(b) + F(c))
+
+    def warp_sum(values):
+        # 2^-58 of the largest exponent's power of two is the last place (to nearest,
+        # halves away from zero)
+        top = max((math.frexp(p)[1] for p in values if p), default=None)
+        if top is None:
+            return 0.0
+        unit, total = F(2) ** (top - 58), 0
+        for p in values:
+            m = int(abs(F(p)) / unit * 2)
+            total += (1 if p > 0 else -1) * ((m + 1) >> 1)
+        return float(total * unit)
+
+    for ng, n, iters in ((2, 100, 150), (3, 1000, 7), (8, 4099, 150), (17, 20000, 30), (31, 3000, 150), (32, 50021, 60)):
+        length = 4.0 * math.pi
+        run = pic.Run(pic.Params(npart=n, ncell=ng, length=length, field_solver=pic.PIC_SOLVER_CG, cg_iterations=iters),
+                      device="cuda:0")
+        rng = np.random.default_rng(ng)
+        run.init(rng.uniform(0.0, 0.999 * length, n).astype(np.float32), np.zeros(n, np.float32))
+        f = run.get_field()
+        run.close()
+        dx = length / ng
+        k_rho = 1.0 / math.ldexp(float(n), 24)
+        rho = [k_rho * float((n << 24) - ng * int(q)) for q in f["rho_q"]]
+        assert rho == f["rho"].tolist()
+        r = [0.0] + [(-v * dx) * dx for v in rho[1:]]
+        x, v, c = [0.0] * ng, [0.0] * ng, 0.0
+        for it in range(-1, iters):
+            if it >= 0:
+                z = []
+                for g in range(ng):
+                    left, right = (v[g - 1] if g else 0.0), (v[g + 1] if g + 1 < ng else 0.0)
+                    z.append(v[0] if g == 0 else fma(-2.0, v[g], left) + right)
+                zv = warp_sum([a * b for a, b in zip(z, v)])
+                if zv == 0.0:
+                    break
+                t = c / zv
+                x = [fma(t, b, a) for a, b in zip(x, v)]
+                r = [fma(-t, b, a) for a, b in zip(r, z)]
+            d = warp_sum([a * a for a in r])
+            if not d > 0.0 or (it < 0 and not (math.sqrt(d) > 1e-16 and ng > 1)):
+                break
+            beta = 0.0 if it < 0 else d / c
+            c = d
+            v = [fma(beta, a, b) for a, b in zip(v, r)]
+        assert f["phi"].tolist() == x, (ng, iters)
