@@ -282,7 +282,7 @@ int atomic_copies(int ng, int block) {
 // added one by one (EXACT), many in groups of 4.  Kinetic energy against exact sums, rms: 2e4
 // particles 1.3e-10 (4.9e-10 with plain chains, 2.2e-10 with one particle a thread),
 // 1e6 2.8e-11 (1.0e-10, 8.2e-11), 2^24 1.9e-11 (3.8e-10, 1.5e-10).  us a step, one by one
-// and in groups: 1e6 on 1024 cells 17.9, 17.4; 4e6 29.4, 27.9; 2^24 67.4, 63.2.
+// and in groups: 1e6 on 1024 cells 18.2, 17.4; 4e6 29.4, 27.9; 2^24 67.4, 63.4.
 constexpr long long kAtomicExact = 1 << 21;
 
 template <bool PUSH, bool EXACT>
@@ -338,8 +338,11 @@ __global__ void __launch_bounds__(1024) pic_push_f32atomic_kernel(PushArgsF32Ato
         float la = 0.0f, ra = 0.0f, lb = 0.0f, rb = 0.0f;
         bool bad = false;
 #pragma unroll
-        for (int k = 0; k < 4; k++) {
+        for (int k = 0; k < 4; k++)
             if (PUSH) push(xs[k], vs[k]);
+        if (PUSH && !EXACT) join();
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
             const Loc l = locate(xs[k]);
             const bool ok = l.j <= (unsigned)ng;
             bad |= !ok;
@@ -358,7 +361,6 @@ __global__ void __launch_bounds__(1024) pic_push_f32atomic_kernel(PushArgsF32Ato
             }
         }
         if (PUSH) {
-            if (!EXACT) join();
             __stcs(x4 + q, make_float4(xs[0], xs[1], xs[2], xs[3]));
             __stcs(v4 + q, make_float4(vs[0], vs[1], vs[2], vs[3]));
         }
