@@ -536,7 +536,7 @@ def tune_pool(states, steps, history):
 
 def time_batched(args):
     """Config 3: the ensemble in one persistent cluster launch vs the same
-    runs one per launch (each through pic_step_n, CUDA graphs)."""
+    runs one after another (each through pic_step_n: the many-step launch)."""
     import torch
     import paper_1108_1954_gb300 as pic
     K, H = args.batched_steps, 16
@@ -572,7 +572,7 @@ def time_batched(args):
         r = pic.Run(pic.Params(npart=p.npart, ncell=p.ncell, length=p.length, dt=p.dt,
                                sort_interval=S, history=max(64, K + 1)))
         r.init(x, v)
-        r.step_n(3 * S if S else 16)    # capture its graphs outside the timed region
+        r.step_n(3 * S if S else 16)    # warm, outside the timed region
         runs.append(r)
     torch.cuda.synchronize()
     s = torch.cuda.current_stream()
@@ -700,10 +700,12 @@ def variant_scan(args):
 
 def time_c1(args):
     """Config 1 (20,000 electrons, 64 cells, 200 steps): launch-bound, so
-    reported as microseconds per step -- through pic_step_n (CUDA graphs of
-    16 steps) and as a one-run pool (all 200 steps in one cluster launch; the
-    fastest of clusters of 1, 2, 4 and 8 blocks); and in the configuration's
-    own float64 precision through pic_step_n."""
+    reported as microseconds per step -- through pic_step_n (the many-step
+    launch, in the configuration's own float64 precision too), as a one-run
+    pool whose shape is left open (the many-step launch there), and as a
+    one-run pool in one cluster launch (the fastest of clusters of 1, 2, 4 and
+    8 blocks).  The keys' names (graphs, one_launch) are those of the launches
+    that these once were."""
     import numpy as np
     import torch
     import workloads as W
@@ -713,7 +715,7 @@ def time_c1(args):
     x32, v32 = W.to_f32_state(x, v, L)
     run = pic.Run(pic.Params(npart=n, ncell=ng, length=L, dt=0.1, history=K + 1))
     run.init(x32, v32)
-    run.step_n(32)                    # capture the graph
+    run.step_n(32)                    # warm
     run.init(x32, v32)
     s = run.stream
     e0, e1 = torch.cuda.Event(True), torch.cuda.Event(True)
@@ -737,10 +739,10 @@ def time_c1(args):
     torch.cuda.synchronize()
     t_fp64 = e0.elapsed_time(e1) / 1e3
     run.close()
-    best = None
-    for cluster in (1, 2, 4, 8):
-        pool = pic.Pool(max_slots=1, ncell_max=64, arena_bytes=1 << 24, history=K + 1,
-                        variant=5, cluster=cluster, block=256)
+    best = t_open = None
+    for cluster in (0, 1, 2, 4, 8):          # 0: the shape left open
+        shape = dict(variant=5, cluster=cluster, block=256) if cluster else {}
+        pool = pic.Pool(max_slots=1, ncell_max=64, arena_bytes=1 << 24, history=K + 1, **shape)
         for rep in range(2):                 # the first pass warms up
             slot = pool.admit(pic.Params(npart=n, ncell=ng, length=L, dt=0.1), x32, v32, K)
             pool.advance(0)
@@ -751,13 +753,15 @@ def time_c1(args):
             pool.sync()
             t = e0.elapsed_time(e1) / 1e3
             pool.release(slot)
-        if best is None or t < best[0]:
+        if not cluster:
+            t_open = t
+        elif best is None or t < best[0]:
             best = (t, cluster)
         pool.close()
     t_pool, cluster = best
     return {"npart": n, "ncell": ng, "steps": K,
             "us_per_step_graphs": 1e6 * t_graph / K, "us_per_step_one_launch": 1e6 * t_pool / K,
-            "us_per_step_graphs_fp64": 1e6 * t_fp64 / K,
+            "us_per_step_graphs_fp64": 1e6 * t_fp64 / K, "us_per_step_pool_open": 1e6 * t_open / K,
             "one_launch_shape": {"variant": 5, "cluster": cluster, "block": 256},
             "value_graphs": n * K / t_graph, "value_one_launch": n * K / t_pool,
             "unit": "particle-steps/s"}
@@ -818,6 +822,7 @@ def time_weak(args):
     per = pic.pool_run_bytes(pic.Params(npart=n, ncell=ng, length=L), 8)
     pool = pic.Pool(max_slots=R, ncell_max=ng, arena_bytes=R * per + (64 << 20), history=8,
                     variant=getattr(args, "pool_variant", 5), cluster=8, block=512)
+    pool.many_step(True)                         # where that is faster
     for r in range(R):
         slot = pool.admit_loaded(pic.Params(npart=n, ncell=ng, length=L, dt=0.1),
                                  pic.Loading(v0=0.0, vth=0.2, seed=5000 + r), steps + 40)

@@ -468,8 +468,6 @@ __device__ void run_steps(const BatchArgs &a, const BatchRun &R, cg::cluster_gro
                 unsigned long long t = 0;
                 for (int j = 0; j < nw; j++) t += cqw[j];
                 ex.cq = t;
-                ex.diag[kDiagKE] = 0.0;
-                ex.diag[kDiagMom] = 0.0;
                 ex.diag[kDiagCharge] = r == 0 ? R.dx * R.k_rho * i128_to_f64(SR) : 0.0;
             }
         }

@@ -168,9 +168,7 @@ __device__ void cluster_finish(const SolveArgs &a, cg::cluster_group &cl, Cluste
             cd.cq = sc;
             cd.kv[0] = kv[0];
             cd.kv[1] = kv[1];
-            cd.diag[kDiagFE] = 0.0;
-            cd.diag[kDiagKE] = 0.0;
-            cd.diag[kDiagMom] = 0.0;
+            cd.diag[kDiagFE] = 0.0;               // (block 0 adds the warps' sums, below)
             cd.diag[kDiagCharge] = charge;
         }
     }

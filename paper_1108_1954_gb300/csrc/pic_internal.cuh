@@ -84,7 +84,7 @@ struct PushArgsF32Atomic {
 };
 
 // Per-block share of the step diagnostics.
-enum { kDiagFE = 0, kDiagKE, kDiagMom, kDiagCharge, kDiagModes,
+enum { kDiagFE = 0, kDiagCharge, kDiagModes,
        kDiagFields = kDiagModes + 2 * PIC_NMODES };
 
 // Field solve (one cluster of up to 16 blocks).
