@@ -17,7 +17,8 @@
  * Precision (PIC_FP32_FIXED, the default): positions and velocities are
  * float32; the deposit is exact integer arithmetic on 2^-24 fractions of a
  * particle (below), so the density is the same integer for any launch shape
- * or particle order; the field solve and all diagnostics are float64.
+ * or particle order; the field solve is float64, and so are the diagnostics (but
+ * for the terms of the push's sums and of the mode amplitudes, which are float32).
  *
  * Cell units.  In the float32 modes the device keeps each position as its
  * cell coordinate u = x NG / L in [0, NG) (node g at u = g + 1/2), so the box
@@ -37,14 +38,17 @@
  * Ownership.  The caller owns all device memory: it allocates one workspace
  * of pic_workspace_size() bytes (any allocator; 256-byte alignment) and the
  * library carves every device array out of it.  The library allocates no
- * device memory.  It keeps a small host-side handle (pic_run) and CUDA graphs.
+ * device memory.  It keeps a small host-side handle (pic_run), CUDA graphs, and
+ * page-locked host memory for read-backs (384 KB a handle that reads often; up to 8
+ * such pieces are kept for later handles when theirs are closed).
  * All work is enqueued on the caller's stream; calls return before the GPU
  * finishes, except those documented as synchronising.
  *
  * Errors.  Every int-returning call returns PIC_OK (0) or a negative code.
  * Kernels never trap: a particle with a non-finite or out-of-range position
  * sets a device error word, which the synchronising calls (pic_sync,
- * pic_diagnostics, pic_get_state, pic_get_field) report as PIC_EDEVICE.
+ * pic_diagnostics, pic_get_state, pic_get_field) report as PIC_EDEVICE.  Kernels whose
+ * blocks wait for one another give up after some seconds (PIC_ETIMEOUT).
  *
  * Threading.  Calls on one run are not thread-safe; different runs are.  The
  * read-backs of a pool (pic_pool_get_state, _get_cells, _get_field, _diagnostics)

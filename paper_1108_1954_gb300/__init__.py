@@ -490,7 +490,8 @@ def pool_run_bytes(p: Params, history: int) -> int:
 
 class Pool:
     """An ensemble of independent runs advanced together by one persistent
-    cluster launch per advance (the batched and served forms)."""
+    cluster launch per advance (the batched and served forms), or, few of
+    them in a pool whose shape is left open, by one many-step launch."""
 
     def __init__(self, max_slots: int, ncell_max: int, arena_bytes: int, history: int = 256,
                  variant: int = 0, cluster: int = 0, block: int = 0, device=None, stream=None):

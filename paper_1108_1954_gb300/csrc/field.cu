@@ -59,10 +59,10 @@ constexpr int kMaxSolveCluster = 16;        // blocks per cluster (16: non-porta
 // units of 2^-B of a particle, and rho_g = K R_g with R_g = N 2^B - NG q_g and
 // K = rho_ion / (N 2^B).
 //   fixed point     B = 24: the deposit's own integers
-//   float32 atomic  B = 30: the float32 sum to the nearest 2^-30 (a sum of at
-//                   least 2^-6 converts exactly)
+//   float32 atomic  B = 30: the float32 sum, exactly: locate's fractions, and so all
+//                   weights and their sums, are multiples of 2^-24
 //   float64         B = 53: the deposit's own integers, kept as two 64-bit sums
-//                   of the low 40 bits and of the rest (push.cu)
+//                   of the low 40 bits and of the rest (push64.cuh)
 // Bounds of the 128-bit arithmetic below, worst at B = 53, N < 2^32, NG = 2^13
 // with every particle in one cell: |P_g| <= NG N 2^53 < 2^98, |sum P| < 2^111,
 // |M_g| < 2^112 and the two terms of sum M below 2^125 each.
@@ -337,8 +337,8 @@ __global__ void __launch_bounds__(kClusterSolveThreads) pic_solve_cluster_kernel
 //   * t = c / z.v and beta = d / c are corrected products with reciprocals
 //     (recip64, divide64), of which 1/c is formed while the sums cross.
 // A step of 150 iterations takes 311 us on 1024 nodes, 549 with cluster barriers,
-// float64 trees and divisions; an iteration's 520 instructions a warp, one
-// after the other at 7.4 clocks, are what bounds it now.
+// float64 trees and divisions; an iteration's instructions, one after the other
+// in 4200 clocks, are what bounds it now.
 // A block's barrier of one sum cannot complete again before the block has added
 // its own part of the next sum, which it sends only after reading the first, so
 // one buffer per sum is enough.  Every wait has a limit (SolveArgs::wait_limit

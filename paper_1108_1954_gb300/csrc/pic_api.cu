@@ -411,17 +411,20 @@ int steps64_block(int64_t npart, int ncell) {
 // of one rank whose caller left the push's shape open, up to 24e6 particles on
 // up to 2048 cells and 12.5e6 on up to 4096.  Measured (us a step, this launch
 // and push + solve, unsorted after 100 steps / sorted every 20):
-//   cells     1.2e7 particles          1.7e7                    3.4e7
-//    512   34, 48.8 / 41, 48.4   50.8, 60.3 / 57.1, 62.6   97, 102 / 107, 109
-//   2048   38, 47.6 / 43, 48.8   53.1, 59.4 / 59.4, 62.0  100, 101 / 110, 108
-//   4096   45, 48.8 / 51, 51.8   60.3, 61.0 / 67.4, 64.6  107, 102 / 118, 109
+//   cells     1.2e7 particles              1.7e7                      2.4e7
+//    512   31.6, 43.3 / 39.5, 44.2   48.6, 58.6 / 55.8, 61.6   67.3, 76.4 / 76.5, 80.5
+//   2048   33.9, 43.6 / 40.4, 46.2   50.7, 58.6 / 57.1, 62.5   69.5, 75.9 / 77.7, 80.7
+//   4096   37.4, 46.4 / 43.4, 49.1
+// (With an older, slower form of the launch 3.4e7 took 97, 102 / 107, 109 on 512 cells
+// and 107, 102 / 118, 109 on 4096, 1.7e7 60.3, 61.0 / 67.4, 64.6 on 4096.)
 // Float64 runs (steps64.cu) up to 1e6 particles and 1024 cells: 2e4 on 64 cells
 // 4.1 and 15.3 us a step, 5e5 on 1000 17.6 and 26.6, 1e6 27.6 and 30.1; 4e6 on
 // 512 69.8 and 62.0.
 // Runs of few particles take them one per lane (steps_small; a lane's 4 in turn
 // are a chain 4 times as long), and small blocks, whose barriers cost less.  us
 // per step, groups of 4 in blocks of 256 (512) 1024 threads, and one per lane in
-// 256, 512, 1024 (unsorted, lattice start | Maxwellian):
+// 256, 512, 1024 (unsorted, lattice start | Maxwellian; groups then of up to 4, a
+// twentieth slower):
 //   2e4 on 64      3.64 (3.80) 4.84   2.87  3.14  3.88 | 3.61 (3.79) 4.89  2.90  3.14  3.86
 //   5e4 on 100     3.59 (3.86) 4.95   3.08  3.11  3.89 | 3.59 (3.83) 4.92  3.60  3.32  3.89
 //   1.3e5 on 512   4.62 (4.47) 5.15    -    3.85  4.17 | 4.99 (4.50) 5.17   -    4.49  4.80

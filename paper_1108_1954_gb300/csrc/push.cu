@@ -15,7 +15,8 @@
 // shape, the particle order or the deposit variant.
 //
 // Deposit variants (all give the same integers):
-//   ATOMIC        two shared-memory atomics per particle;
+//   ATOMIC        per cell, a count and a sum of right weights: an add of 1 and one
+//                 fetch-add per particle (particle_ops.cuh, cell tiles);
 //   MATCH         lanes of a warp whose particles share a left node are
 //                 grouped by __match_any_sync; the group's weights are summed
 //                 by __reduce_add_sync and its first lane does two atomics;
@@ -25,7 +26,7 @@
 //                 interleaved cells (the two beams before the first sort)
 //                 still combine.
 // The nearest-grid-point shape (PIC_SHAPE_NGP) uses the same loop with the
-// NGP gather and a QUAD-style deposit of whole particles to the cell's node.
+// NGP gather and counts the particles of each cell.
 // The tiles hold exact 64-bit sums in two 32-bit words (particle_ops.cuh).
 #include "particle_ops.cuh"
 #include "push64.cuh"
@@ -256,11 +257,11 @@ __global__ void __launch_bounds__(512) pic_push_oct_kernel(PushArgs a) {
 // l mod copies: lanes of one cell then meet on an address copies times less
 // often, and with 32 copies a warp's lanes never meet and use a bank each.
 // Measured (2^24 particles, 1024 cells, the mean over sort periods): 60 us a push
-// with 32 copies, 68 with 16, against 295 us with one copy and a shuffle sum
+// with 32 copies (2^24 on 4096 cells, 8 copies: 73), 68 with 16, against 295 us with one copy and a shuffle sum
 // where a whole warp holds one run, and 140 us (sorted) to 380 us (lattice
 // order) with two adds per particle.
 // As many copies as fit beside E, at most 32: in 216 KB for a block of 1024
-// threads (its 53 registers leave room for one per SM), in 72 KB for smaller
+// threads (its 56 registers leave room for one per SM), in 72 KB for smaller
 // ones, so that two of 512 keep their place; open shapes take the large block
 // where it holds more copies.  us a push, 2^24 particles sorted every 20 steps, in
 // two blocks of 512 and one of 1024: 256 cells (32 copies either way) 58.9, 62.3;

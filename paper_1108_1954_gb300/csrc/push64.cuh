@@ -1,5 +1,5 @@
 // push64.cuh -- the per-particle arithmetic of the float64 mode, shared by the
-// push kernel (push.cu) and the many-step launch (steps.cu).
+// push kernel (push.cu) and the many-step launch (steps64.cu).
 //
 // GB300 issues float64 at 2 lanes per clock per SM, so a float64 instruction
 // of a warp takes the pipe for 16 clocks, the time of some 40 integer
@@ -12,9 +12,9 @@
 //   gather    E_l + f (E_r - E_l) = fma(1 + f, dE, E_l - dE): 1 + f is the
 //             fraction's bits under the exponent of 1, dE and E_l - dE are
 //             kept as pairs in shared memory;
-//   deposit   the weights are integers of 2^-53 (f to within 2^-54, which a
-//             float64 sum of one particle or more does not resolve either),
-//             summed exactly: runs of equal cell in registers (two open runs
+//   deposit   the weights are integers of 2^-53, f truncated to F bits and those
+//             (the fraction of a float64 u + 1/2 >= 1/2 is a multiple of 2^-53
+//             at best, and of NG 2^-53 at the far end of the box), summed exactly: runs of equal cell in registers (two open runs
 //             of a thread's 4 particles, as PAIR), then in a tile of three
 //             32-bit words per node.  Native 32-bit shared adds take the place
 //             of float64 compare-and-swap loops, and the density no longer

@@ -14,7 +14,7 @@
 //            cell total (many cells: a pass of its own, segscan); exclusive prefix
 //            of those over the cells -> base[g]
 //   scatter  block b walks its chunk in order, 512 particles at a time
-//            (64 consecutive per warp); the warps take their slots from the
+//            (64 consecutive per warp; long chunks 1024, 128); the warps take their slots from the
 //            per-cell cursors one after the other, so the order within a
 //            cell is the original order.
 // A small sort is launches, not work (1e6 particles, 1024 cells: passes of 3, 3, 2

@@ -28,20 +28,21 @@
 //
 // Up to 6e5 particles on up to 1024 cells the lanes take particles one by one
 // (SMALL), beyond that in groups of 4 (16-byte loads; in a small run only a
-// longer chain per lane: pic_api.cu, steps_shape).
+// longer chain per lane: pic_api.cu, steps_shape).  Groups are whole, which saves the
+// loop its tests (3e6 particles, NGP, 13.3 us a step with them, 12.3 so).
 //
 // What a step costs (GB300, us): launches of push and solve before, and here
-//   2e4 particles, 64 cells, one step a call   16.4   10.2
-//   3e5, 500 cells, one step a call             -     12.3
-//   1e6, 2048 cells, one step a call            -     21.9
-//   2e4, 64 cells                              13.4    2.9
-//   5e4, 100 cells                             14.0    3.1
-//   5e5, 300 cells                             18.5    5.1
-//   1e6, 1024 cells, sorted every 20           22.5    8.4
-//   3e6, 777 cells, NGP, sorted every 10       27.4   13.1
-//   4.2e6, 2048 cells, sorted every 20         31.0   18.3
-//   1e6, 4096 cells                            24.8   11.3
-//   1.2e7, 2048 cells, sorted every 20         52.9   39.9
+//   2e4 particles, 64 cells, one step a call   16.4    9.9
+//   3e5, 500 cells, one step a call             -     12.4
+//   1e6, 2048 cells, one step a call            -     20.5
+//   2e4, 64 cells                              13.4    2.8
+//   5e4, 100 cells                             14.0    3.0
+//   5e5, 300 cells                             18.5    4.9
+//   1e6, 1024 cells, sorted every 20           22.5    8.1
+//   3e6, 777 cells, NGP, sorted every 10       27.4   12.3
+//   4.2e6, 2048 cells, sorted every 20         31.0   18.1
+//   1e6, 4096 cells                            24.8   11.1
+//   1.2e7, 2048 cells, sorted every 20         52.9   40.0
 // of which, at 5e4 (clocks): push 700, sums 380, flush 1040, barrier 2400 (the
 // adds' release and a poll, each a trip to L2), solve 1300 (900 the sums' way
 // from L2), E 510.  Counting a node's arrivals in the upper bits of its sum, so
