@@ -473,11 +473,17 @@ cudaError_t set_steps_shape(pic_run *r) {
 // Whether the run's stream is being captured into a graph.  Then single launches are
 // enqueued: a replay would not advance the host's copy of the many-step launch's
 // counters, and the run's own graphs cannot be made (instantiated) meanwhile.
-bool capturing(const pic_run *r) {
+bool capturing(pic_run *r) {
     cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(r->stream, &st) == cudaSuccess) return st != cudaStreamCaptureStatusNone;
-    (void)cudaGetLastError();
-    return true;
+    if (cudaStreamIsCapturing(r->stream, &st) != cudaSuccess) {      // (the legacy stream beside
+        (void)cudaGetLastError();                                   // a capture: nothing can run)
+        return true;
+    }
+    // Replays advance the device's count of steps and not the host's, which the
+    // many-step launch goes by (read on the device it cost 1-5% of a step): from the
+    // first capture on a run takes the kernels that go by the device's.
+    if (st != cudaStreamCaptureStatusNone) r->captured = true;
+    return st != cudaStreamCaptureStatusNone;
 }
 
 // The many-step launch of the run's state (but for the counters' values).
@@ -780,7 +786,7 @@ int pic_solve_field(pic_run *run) {
     pic::TraceRange trace_("pic_solve_field");
     if (!run) return PIC_EINVAL;
     if (!run->ready) return PIC_ESTATE;
-    if (run->pending_push && run->steps_grid && !run->captured) run->captured = capturing(run);
+    if (run->pending_push && run->steps_grid && !run->captured) (void)capturing(run);
     PIC_CUDA(enqueue_solve(run, run->stream, run->pending_push));
     if (run->pending_push) run->step++;
     run->pending_push = false;
@@ -809,12 +815,7 @@ int pic_step_n(pic_run *run, int64_t n) {
     if (!run || n < 0) return PIC_EINVAL;
     if (!run->ready || run->pending_push) return PIC_ESTATE;
     const int64_t S = run->p.sort_interval;
-    const bool cap = capturing(run);
-    // Replays advance the device's count of steps and not the host's, which the
-    // many-step launch goes by (read on the device it cost 1-5% of a step): from the
-    // first capture on a run takes the kernels that go by the device's.
-    if (cap) run->captured = true;
-    const bool resident = run->steps_grid && !run->captured;
+    const bool cap = capturing(run), resident = run->steps_grid && !cap && !run->captured;
     while (n > 0) {
         const bool sort_due = S > 0 && run->step > 0 && run->step % S == 0;
         if (resident) {

@@ -540,3 +540,28 @@ def test_handles_close_while_another_stream_is_captured():
         r.sync()
     assert len(r.diagnostics()) == 1
     r.close()
+
+
+def test_a_call_beside_another_streams_capture_does_not_count_as_captured():
+    # a run on the legacy stream cannot step while another stream is captured in the
+    # default mode; afterwards it is as it was
+    a, b = pair(20000, 64)
+    s, g = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    x = torch.zeros(4, device="cuda")
+    torch.cuda.synchronize()
+    failed = None
+    try:
+        with torch.cuda.graph(g, stream=s):
+            x.add_(1.0)
+            try:
+                a.step_n(2)
+            except pic.PicError as e:
+                failed = e.code
+    except RuntimeError:
+        pass                                           # the capture is lost
+    torch.cuda.synchronize()
+    if failed is None:                                 # (where it can, it has stepped)
+        b.step_n(2)
+    a.step_n(3), b.step_n(3)
+    assert_same(a, b, 20000, 64)
+    assert many_step_launched(a)
