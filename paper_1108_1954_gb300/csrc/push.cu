@@ -261,7 +261,7 @@ __global__ void __launch_bounds__(512) pic_push_oct_kernel(PushArgs a) {
 // where a whole warp holds one run, and 140 us (sorted) to 380 us (lattice
 // order) with two adds per particle.
 // As many copies as fit beside E, at most 32: in 216 KB for a block of 1024
-// threads (its 56 registers leave room for one per SM), in 72 KB for smaller
+// threads (its 50 registers leave room for one per SM), in 72 KB for smaller
 // ones, so that two of 512 keep their place; open shapes take the large block
 // where it holds more copies.  us a push, 2^24 particles sorted every 20 steps, in
 // two blocks of 512 and one of 1024: 256 cells (32 copies either way) 58.9, 62.3;
@@ -280,11 +280,12 @@ int atomic_copies(int ng, int block) {
 // A thread takes 4 particles at a time where one block of 256 had one, so plain
 // float32 sums of v_old v_new and v_new have longer chains, and more of their rounding
 // in the rows.  The sums are therefore pairs of float32, to which few particles are
-// added one by one (EXACT), many in groups of 4.  Kinetic energy against exact sums, rms: 2e4
-// particles 1.3e-10 (4.9e-10 with plain chains, 2.2e-10 with one particle a thread),
-// 1e6 2.8e-11 (1.0e-10, 8.2e-11), 2^24 1.9e-11 (3.8e-10, 1.5e-10).  us a step, one by one
-// and in groups: 1e6 on 1024 cells 18.2, 17.4; 4e6 29.4, 27.9; 2^24 67.4, 63.4.
-constexpr long long kAtomicExact = 1 << 21;
+// added one by one (EXACT), many in groups of 4.  Kinetic energy against exact sums,
+// rms: 2e4 particles 1.3e-10 (4.9e-10 with plain chains, 2.2e-10 with one particle a
+// thread), 1e6 2.8e-11 (1.0e-10, 8.2e-11), 2^22 1.9e-11 (1.8e-10, 1.2e-10), in groups
+// 3e-11, 2^24 2.2e-11 (3.8e-10, 1.5e-10).  us a step, one by one and in groups: 4e6 on
+// 1600 cells 28.2, 26.4; 2^24 on 1024 (in an older loop) 67.4, 63.4.
+constexpr long long kAtomicExact = 1 << 22;
 
 template <bool PUSH, bool EXACT>
 __global__ void __launch_bounds__(1024) pic_push_f32atomic_kernel(PushArgsF32Atomic a) {
@@ -322,16 +323,15 @@ __global__ void __launch_bounds__(1024) pic_push_f32atomic_kernel(PushArgsF32Ato
         push_particle(x, v, sE, c, gke, gmom);
         if (EXACT) join();
     };
-    const long long n4 = a.n >> 2;
-    const long long stride = (long long)gridDim.x * bs;
+    const unsigned n4 = (unsigned)(a.n >> 2), stride = gridDim.x * (unsigned)bs;     // N < 2^32
     float4 *x4 = reinterpret_cast<float4 *>(a.x);
     float4 *v4 = reinterpret_cast<float4 *>(a.v);
     const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
-    const long long q00 = (long long)blockIdx.x * bs;
-    float4 cx = q00 + tid < n4 ? __ldcs(x4 + q00 + tid) : zero4;
-    float4 cv = PUSH && q00 + tid < n4 ? __ldcs(v4 + q00 + tid) : zero4;
-    for (long long q = q00 + tid; q < n4; q += stride) {
-        const long long qn = q + stride;
+    const unsigned q0 = blockIdx.x * (unsigned)bs + (unsigned)tid;
+    float4 cx = q0 < n4 ? __ldcs(x4 + q0) : zero4;
+    float4 cv = PUSH && q0 < n4 ? __ldcs(v4 + q0) : zero4;
+    for (unsigned q = q0; q < n4; q += stride) {
+        const unsigned qn = q + stride;
         const float4 nx = qn < n4 ? __ldcs(x4 + qn) : zero4;
         const float4 nv = PUSH && qn < n4 ? __ldcs(v4 + qn) : zero4;
         float xs[4] = {cx.x, cx.y, cx.z, cx.w}, vs[4] = {cv.x, cv.y, cv.z, cv.w};
@@ -373,7 +373,7 @@ __global__ void __launch_bounds__(1024) pic_push_f32atomic_kernel(PushArgsF32Ato
     }
     // the last N mod 4 particles
     if (blockIdx.x == 0 && tid < (int)(a.n & 3)) {
-        const long long i = n4 * 4 + tid;
+        const long long i = 4ll * n4 + tid;
         float x = a.x[i], v = PUSH ? a.v[i] : 0.0f;
         if (PUSH) push(x, v);
         const Loc l = locate(x);

@@ -140,9 +140,9 @@ def test_atomic_deposit_in_large_blocks(n, ng):
 
 # Rows of the float32-atomic mode against float64 sums of the same particles.  A
 # float32 rounding of p is off by p 2^-24 / sqrt 3 rms at most; what is rounded is each
-# product, and beyond 2^21 particles the sums of 2, 3 and 4 of a group: for particles
+# product, and beyond 2^22 particles the sums of 2, 3 and 4 of a group: for particles
 # of one size sqrt(1 + 4 + 9 + 16) / 2 times as much.  The rows' rms over 12 steps.
-@pytest.mark.parametrize("n,ng", [(20001, 64), (1000003, 1024), (1 << 21, 512), ((1 << 21) + 1, 512), ((1 << 23) + 3, 1024)])
+@pytest.mark.parametrize("n,ng", [(20001, 64), (1000003, 1024), (1 << 22, 512), ((1 << 22) + 1, 512), ((1 << 23) + 3, 1024)])
 def test_atomic_rows_against_float64_sums(n, ng):
     rng = np.random.default_rng(n)
     run = pic.Run(pic.Params(npart=n, ncell=ng, length=L, precision=pic.PIC_FP32_ATOMIC), device="cuda:0")
@@ -154,7 +154,7 @@ def test_atomic_rows_against_float64_sums(n, ng):
         new = run.get_cells()[1].astype(np.float64)
         row = run.diagnostics(run.step - 1, 1)[0]
         for key, p, k in (("kinetic", old * new, 0.5 * L / n), ("momentum", new, L / n)):
-            rounding = 2.0 ** -24 / math.sqrt(3.0) * math.sqrt((p * p).sum()) * (1.0 if n <= 1 << 21 else 30 ** 0.5 / 2)
+            rounding = 2.0 ** -24 / math.sqrt(3.0) * math.sqrt((p * p).sum()) * (1.0 if n <= 1 << 22 else 30 ** 0.5 / 2)
             err[key].append((row[key] / k - p.sum()) / rounding)
         old = new
     assert np.sqrt(np.mean(np.square(err["kinetic"]))) <= 1.0
